@@ -275,35 +275,94 @@ __global__ void k_init(Lattice L, int cur, int inst, const double *phi, const do
     }
 }
 
+// rho/rho0 = 1 + sum_i w_i F_i in FP64, from 36 sum_i w_i F_i =
+// 12 F_0 + 2 sum_axis F + sum_diagonal F.
+//
+// Double-precision instructions issue at a small fraction of the FP32 rate on
+// this GPU, so single-precision offsets are summed in FP32 by error-free
+// transformations: TwoSum (Knuth, The Art of Computer Programming 2, 4.2.2)
+// carries each addition's exact error into a second sum, whose own errors go
+// into a third (the K-fold summation of Ogita, Rump and Oishi, "Accurate sum
+// and dot product", 2005, K = 3).  What is dropped is of the order of
+// (20 2^-24)^3 sum |F|, below the rounding of an FP64 sum of values near 1; the
+// powers of two that weight the terms are exact.  Only the three partial sums
+// are converted.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+__device__ __forceinline__ double density(const float (&F)[Q])
+{
+    float s = 8.0f * F[0], c = 0.0f, d = 0.0f;
+    auto add = [&](float v) {
+        float e, f;
+        two_sum(s, v, s, e);
+        two_sum(c, e, c, f);
+        d += f;
+    };
+    add(4.0f * F[0]);
+#pragma unroll
+    for (int i = 1; i < Q; i++) add(csq(i) == 1 ? 2.0f * F[i] : F[i]);
+    double t = (double)s;
+    // an infinite partial sum has no error term (inf - inf)
+    if (isfinite(s)) t += (double)c + (double)d;
+    return (36.0 + t) * (1.0 / 36.0);  // exactly 0 where every offset is -1
+}
+
+__device__ __forceinline__ double density(const double (&F)[Q])
+{
+    double a = 0.0, b = 0.0;
+#pragma unroll
+    for (int i = 1; i < Q; i++) (csq(i) == 1 ? a : b) += F[i];
+    return (36.0 + (12.0 * F[0] + 2.0 * a + b)) * (1.0 / 36.0);
+}
+
+// The colour offsets G_i = phi (1 + F_i) + (c_i . a)/|c_i| of a node sum to
+// phi (1 + sum w F) (the directions cancel pairwise), so its component
+// densities are rho (1 +- phi)/2 and its order parameter is the record's.
+//
+// The read is bound by FP64 issue unless that work is kept this short: with
+// each direction's populations formed in FP64 (some 270 FP64 instructions a
+// node) the densities and phi of 256x128x128 FP32 nodes took 1304 us for 0.5 GB of
+// traffic; with the sums above (8 FP64 instructions a node) about 110 us
 template <class S>
-__global__ void k_read(Lattice L, int cur, int inst, unsigned mask, double *out, AbiMap map)
+__global__ void __launch_bounds__(256) k_read(Lattice L, int cur, int inst, unsigned mask, double *out, AbiMap map)
 {
     using R = typename Store<S>::real;
     const InstDev &I = L.inst[inst];
     const long long N = I.N;
     const Pop<S> pop(L.pop[cur], I);
     const ColourOf<S> C(L, I);
+    const bool dens = mask & (LBM_FIELD_RHO_A | LBM_FIELD_RHO_B | LBM_FIELD_PHI);
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
         const uint8_t f = L.flags[I.node_off + n];
         const bool fluid = (f & OWNER_MASK) == OWN_FLUID;
-        const NodeState<S> ns{pop, C, (int)n};
-        double ra = 0.0, rb = 0.0;
-        if (fluid)
-            for (int i = 0; i < Q; i++) {
-                const double w = wgt<double>(i) * I.rho0, Fv = ns.F(i), Gv = ns.G(i);
-                ra += 0.5 * w * (1.0 + Fv + Gv);
-                rb += 0.5 * w * (1.0 + Fv - Gv);
-            }
+        double ra = 0.0, rb = 0.0, ph = 0.0;
+        if (dens && fluid) {
+            R F[Q];
+#pragma unroll
+            for (int i = 0; i < Q; i++) F[i] = pop.F(i, (int)n);
+            const double p = (double)C.at((int)n).p, rr = density(F);
+            const double h = 0.5 * I.rho0 * rr;
+            ra = h + h * p;
+            rb = h - h * p;
+            // 0/0 and the like keep their NaN
+            ph = isfinite(rr) && rr != 0.0 ? p : p * rr / rr;
+        }
         long long off = 0;
         if (mask & LBM_FIELD_RHO_A) { out[off + n] = ra; off += N; }
         if (mask & LBM_FIELD_RHO_B) { out[off + n] = rb; off += N; }
-        if (mask & LBM_FIELD_PHI) { out[off + n] = fluid ? (ra - rb) / (ra + rb) : 0.0; off += N; }
+        if (mask & LBM_FIELD_PHI) { out[off + n] = ph; off += N; }
         if (mask & LBM_FIELD_U) {
             const R *U = (const R *)L.u;
             for (int a = 0; a < 3; a++) out[off + a * N + n] = (double)U[a * L.Ntot + I.node_off + n];
             off += 3 * N;
         }
         if (mask & LBM_FIELD_POPS) {
+            const NodeState<S> ns{pop, C, (int)n};
             for (int a = 0; a < Q; a++) {
                 const int i = map.dev[a];
                 const double w = wgt<double>(i) * I.rho0;
@@ -329,12 +388,13 @@ __global__ void k_mass_partial(Lattice L, int cur, int inst, double *part)
     double sa = 0.0, sb = 0.0;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
         if ((L.flags[I.node_off + n] & OWNER_MASK) != OWN_FLUID) continue;
-        const NodeState<S> ns{pop, C, (int)n};
-        for (int i = 0; i < Q; i++) {
-            const double w = wgt<double>(i) * I.rho0, Fv = ns.F(i), Gv = ns.G(i);
-            sa += 0.5 * w * (1.0 + Fv + Gv);
-            sb += 0.5 * w * (1.0 + Fv - Gv);
-        }
+        typename Store<S>::real F[Q];
+#pragma unroll
+        for (int i = 0; i < Q; i++) F[i] = pop.F(i, (int)n);
+        // rho (1 +- phi)/2, as in k_read
+        const double p = (double)C.at((int)n).p, h = 0.5 * I.rho0 * density(F);
+        sa += h + h * p;
+        sb += h - h * p;
     }
     __shared__ double sh[2][256];
     sh[0][threadIdx.x] = sa;
