@@ -323,7 +323,8 @@ lbm_status lbm_diagnostics(lbm_ctx *ctx, int inst, double *out);
  * tile 0 (default): with 16-bit storage and an even nx in every instance the
  * bulk collision takes two nodes of a row per thread (pair loads and stores),
  * one node per thread otherwise; tile 1: one node per thread always.
- * zchunk: z-planes per work item of the gradient pass (0: 16).  Every shape
+ * zchunk: z-planes per work item of the gradient pass (0: chosen from the
+ * size of the grid).  Every shape
  * computes the same update; the node-pair collision agrees with the one-node
  * collision to the rounding of the storage type (the code generator may fuse
  * a different set of multiply-adds), the z-chunk gives the same bits.  Invalid

@@ -14,6 +14,8 @@
 
 using namespace lbmg;
 
+static_assert(MAX_PART == LBM_MAX_PARTICLES, "particles of an instance");
+
 struct lbm_ctx {
     lbm_precision prec;
     int n_inst;
@@ -30,7 +32,7 @@ struct lbm_ctx {
     // (phi, b n) of the current state, one per node
     void *phi = nullptr, *col = nullptr;
     size_t col_sz = 32;  // bytes of one colour record
-    void *grad = nullptr, *gmag = nullptr, *kap = nullptr, *u = nullptr;
+    void *grad = nullptr, *u = nullptr;
     std::vector<PartDev> parts_h;
     PartDev *parts_d = nullptr;
     double *mem_part = nullptr, *cap_part = nullptr, *hist = nullptr;
@@ -73,7 +75,7 @@ struct lbm_ctx {
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_pairs;
     cudaEvent_t ev_open[N_STAGES] = {};
     // launch variant of the fluid update
-    FluidLaunch fz = {0, 0, 0, false};
+    FluidLaunch fz = {0, 0, 0, 8, false};
     int zc_request = 0;        // z-planes per gradient work item, 0: automatic
     std::vector<int> zc_inst;  // per instance (the autotuner's size classes), 0: zc_request
     // drop-speed control: per instance integral (3) and last U_a (3); block partials
@@ -99,7 +101,7 @@ struct lbm_ctx {
 // when every row has an even length
 static void plan_launch(lbm_ctx *c)
 {
-    c->fz.gc_items = plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst);
+    plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, c->prec == LBM_FP64, &c->fz);
     c->fz.rows = plan_rows(c->inst_h);
     bool even = true;
     for (const auto &I : c->inst_h) even = even && I.nx % 2 == 0;
@@ -145,8 +147,6 @@ static Lattice make_lattice(const lbm_ctx *c)
     L.phi = c->phi;
     L.col = c->col;
     L.grad = c->grad;
-    L.gmag = c->gmag;
-    L.kap = c->kap;
     L.u = c->u;
     L.Ntot = c->Ntot;
     L.parts = c->parts_d;
@@ -858,8 +858,6 @@ void lbm_destroy(lbm_ctx *ctx)
     cudaFree(ctx->phi);
     cudaFree(ctx->col);
     cudaFree(ctx->grad);
-    cudaFree(ctx->gmag);
-    cudaFree(ctx->kap);
     cudaFree(ctx->static_list);
     cudaFree(ctx->static_bfl);
     cudaFree(ctx->speed_d);
@@ -996,6 +994,12 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
     }
     ctx->Ntot = node_off;
     ctx->pop_bytes = (size_t)pop_off;
+    {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+            ctx->n_sm = sms;
+    }
     plan_launch(ctx);
     if (stream) {
         ctx->stream = (cudaStream_t)stream;
@@ -1010,12 +1014,6 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
     // bulk fluid kernels: at the highest priority their CTAs are dispatched as
     // soon as bulk CTAs retire instead of after the whole bulk grid (at the
     // lowest priority the 256x128x128 step measured 452 against 390 us)
-    {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
-            ctx->n_sm = sms;
-    }
     int prio_least = 0, prio_greatest = 0;
     cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
     if (cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, prio_greatest) != cudaSuccess ||
@@ -1041,7 +1039,8 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
         (st = alloc((void **)&ctx->flags, Nt + FLAG_PAD)) || (st = alloc(&ctx->pop[0], ctx->pop_bytes)) ||
         (st = alloc(&ctx->pop[1], ctx->pop_bytes)) || (st = alloc(&ctx->phi, Nt * ctx->real_sz)) ||
         (st = alloc(&ctx->col, Nt * ctx->col_sz)) ||
-        (st = alloc(&ctx->grad, 3 * Nt * ctx->real_sz)) || (st = alloc(&ctx->gmag, Nt * ctx->real_sz)) || (st = alloc(&ctx->kap, Nt * ctx->real_sz)) || (st = alloc((void **)&ctx->status, sizeof(unsigned))) ||
+        (st = alloc(&ctx->grad, 4 * Nt * ctx->real_sz)) ||
+        (st = alloc((void **)&ctx->status, sizeof(unsigned))) ||
         (st = alloc((void **)&ctx->diag_d, sizeof(double) * 2 * n_instances)) ||
         (st = alloc((void **)&ctx->diag_part, sizeof(double) * 2 * DIAG_BLOCKS)) ||
         (st = alloc((void **)&ctx->speed_d, sizeof(double) * 6 * n_instances)) ||
@@ -1075,9 +1074,7 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
     cudaMemsetAsync(ctx->status, 0, sizeof(unsigned), ctx->stream);
     cudaMemsetAsync(ctx->phi, 0, Nt * ctx->real_sz, ctx->stream);
     cudaMemsetAsync(ctx->col, 0, Nt * ctx->col_sz, ctx->stream);
-    cudaMemsetAsync(ctx->grad, 0, 3 * Nt * ctx->real_sz, ctx->stream);
-    cudaMemsetAsync(ctx->gmag, 0, Nt * ctx->real_sz, ctx->stream);
-    cudaMemsetAsync(ctx->kap, 0, Nt * ctx->real_sz, ctx->stream);
+    cudaMemsetAsync(ctx->grad, 0, 4 * Nt * ctx->real_sz, ctx->stream);
     cudaMemsetAsync(ctx->flags + Nt, 0, FLAG_PAD, ctx->stream);
     cudaMemsetAsync(ctx->diag_d, 0, sizeof(double) * 2 * n_instances, ctx->stream);
     cudaMemsetAsync(ctx->speed_d, 0, sizeof(double) * 6 * n_instances, ctx->stream);

@@ -20,6 +20,8 @@
 // (lbm_internal.cuh); the collision needs the colour offsets only through phi.
 // Storage type S in {double, float, __half, __nv_bfloat16}; arithmetic in
 // double for S = double and float otherwise.
+#include <algorithm>
+
 #include "lbm_node.cuh"
 
 // CTAs of 256 threads per SM the single-precision order-parameter and
@@ -243,8 +245,6 @@ __device__ __forceinline__ void collide_bound_node(const Lattice &L, int cur, co
     if ((fl & OWNER_MASK) != OWN_FLUID || !(fl & BOUND_BIT)) return;
     const Pop<S> in(L.pop[cur], *I);
     const Pop<S> out(L.pop[cur ^ 1], *I);
-    const R *Nn = (const R *)L.grad + I->node_off;
-    const long long Nt = L.Ntot;
     R *U = I->store_u ? (R *)L.u + I->node_off : nullptr;
     GlobalNbr nb;
     nb.nb.init(x, y, z, I->nx, I->ny, I->nz);
@@ -253,11 +253,8 @@ __device__ __forceinline__ void collide_bound_node(const Lattice &L, int cur, co
     gather_all<S>(*I, L.parts, nb, in, (const ColourOf<S> *)nullptr, n, F, (R *)nullptr, x, y, z);
     FluidPar<R> P;
     load_par(*I, P);
-    const R m = ((const R *)L.gmag)[g];
-    const R gr[3] = {Nn[n] * m, Nn[Nt + n] * m, Nn[2 * Nt + n] * m};
-    const R nn[3] = {Nn[n], Nn[Nt + n], Nn[2 * Nt + n]};
-    collide_store_phi<S>(P, F, ((const R *)L.phi)[g], gr, nn, ((const R *)L.kap)[g], out, n,
-                         col_slot<S>(L, g), U, L.Ntot, L.status);
+    collide_store_phi<S>(P, F, ((const R *)L.phi)[g], ((const GradRec<R> *)L.grad)[g], out, n, col_slot<S>(L, g), U,
+                         L.Ntot, L.status);
 }
 
 template <class S>
@@ -297,11 +294,7 @@ __device__ __forceinline__ void collide_body(const Lattice &L, const InstDev &I,
     const Pop<S> out(L.pop[cur ^ 1], I);
     // every load of an interior fluid node is issued before the flag is tested
     const uint8_t fl = L.flags[g];
-    const R *Nn = (const R *)L.grad + I.node_off;
-    const long long Nt = L.Ntot;
-    const R nn[3] = {Nn[n], Nn[Nt + n], Nn[2 * Nt + n]};
-    const R m = ((const R *)L.gmag)[g];
-    const R kap = ((const R *)L.kap)[g];
+    const GradRec<R> gr = ((const GradRec<R> *)L.grad)[g];
     const R phi = ((const R *)L.phi)[g];
     Nbr nb;
     nb.init(x, y, z, I.nx, I.ny, I.nz);
@@ -319,8 +312,7 @@ __device__ __forceinline__ void collide_body(const Lattice &L, const InstDev &I,
     if (fl & BOUND_BIT) return;
     FluidPar<R> P;
     load_par(I, P);
-    const R gr[3] = {nn[0] * m, nn[1] * m, nn[2] * m};
-    collide_store_phi<S>(P, F, phi, gr, nn, kap, out, n, col_slot<S>(L, g), U, L.Ntot, L.status);
+    collide_store_phi<S>(P, F, phi, gr, out, n, col_slot<S>(L, g), U, L.Ntot, L.status);
 }
 
 // Node pairs (x even, x + 1) of one row per thread, for 16-bit storage: the
@@ -342,13 +334,8 @@ __device__ __forceinline__ void collide_body2(const Lattice &L, const InstDev &I
     const Pop<S> out(L.pop[cur ^ 1], I);
     const int N = in.N;
     const uint8_t fl0 = L.flags[g], fl1 = L.flags[g + 1];
-    const R *Nn = (const R *)L.grad + I.node_off;
     const long long Nt = L.Ntot;
-    const float2 n0 = *reinterpret_cast<const float2 *>(Nn + n);
-    const float2 n1 = *reinterpret_cast<const float2 *>(Nn + Nt + n);
-    const float2 n2 = *reinterpret_cast<const float2 *>(Nn + 2 * Nt + n);
-    const float2 mv = *reinterpret_cast<const float2 *>((const R *)L.gmag + g);
-    const float2 kv = *reinterpret_cast<const float2 *>((const R *)L.kap + g);
+    const GradRec<R> grA = ((const GradRec<R> *)L.grad)[g], grB = ((const GradRec<R> *)L.grad)[g + 1];
     const float2 pv = *reinterpret_cast<const float2 *>((const R *)L.phi + g);
     Nbr nb;
     nb.init(x, y, z, I.nx, I.ny, I.nz);
@@ -382,11 +369,9 @@ __device__ __forceinline__ void collide_body2(const Lattice &L, const InstDev &I
     if (!a0 && !a1) return;
     FluidPar<R> P;
     load_par(I, P);
-    const R grA[3] = {n0.x * mv.x, n1.x * mv.x, n2.x * mv.x};
-    const R grB[3] = {n0.y * mv.y, n1.y * mv.y, n2.y * mv.y};
     const R phA = pv.x, phB = pv.y;
-    const CollideState<R> cA = collide_state(P, F0, phA, grA, kv.x);
-    const CollideState<R> cB = collide_state(P, F1, phB, grB, kv.y);
+    const CollideState<R> cA = collide_state(P, F0, phA, grA);
+    const CollideState<R> cB = collide_state(P, F1, phB, grB);
     if ((a0 && (!(cA.rr > R(0)) || !(phA == phA))) || (a1 && (!(cB.rr > R(0)) || !(phB == phB))))
         atomicOr(L.status, ST_UNSTABLE);
     if (U) {
@@ -406,8 +391,8 @@ __device__ __forceinline__ void collide_body2(const Lattice &L, const InstDev &I
         }
     };
     {
-        if (a0) col_slot<S>(L, g).set(ColRec<R>{phA, cA.bq * n0.x, cA.bq * n1.x, cA.bq * n2.x});
-        if (a1) col_slot<S>(L, g + 1).set(ColRec<R>{phB, cB.bq * n0.y, cB.bq * n1.y, cB.bq * n2.y});
+        if (a0) col_slot<S>(L, g).set(colour_record(P, cA, phA, grA));
+        if (a1) col_slot<S>(L, g + 1).set(colour_record(P, cB, phB, grB));
     }
     put(of, collide_rest(P, cA, F0[0]), collide_rest(P, cB, F1[0]));
     PairLoop<R>::run([&](auto ic) {
@@ -432,7 +417,7 @@ __global__ void __launch_bounds__(ROW_NODES / 2, LBM_COLLIDE2_MINB) k_collide2(L
 {
     StItem it;
     st_item(L, blockIdx.x, it);
-    pdl_wait();  // the gradient pass's normals, |grad phi| and curvature
+    pdl_wait();  // the gradient pass's grad(phi) and curvature
     const int j = 2 * (int)threadIdx.x;
     if (j >= it.cnt) return;
     const InstDev &I = L.inst[it.k];
@@ -445,7 +430,7 @@ template <class S>
 __global__ void __launch_bounds__(ROW_NODES, sizeof(S) == 8 ? 1 : LBM_COLLIDE_MINB) k_collide(Lattice L, int cur)
 {
     for_item_nodes(L, blockIdx.x, [&](const InstDev &I, int n, int x, int y, int z) {
-        pdl_wait();  // the gradient pass's normals, |grad phi| and curvature
+        pdl_wait();  // the gradient pass's grad(phi) and curvature
         collide_body<S>(L, I, cur, n, x, y, z);
     });
 }
@@ -453,14 +438,30 @@ __global__ void __launch_bounds__(ROW_NODES, sizeof(S) == 8 ? 1 : LBM_COLLIDE_MI
 // ---------------------------------------------------------------------------
 // gradient, wetting, normal and curvature in one z-marching pass
 // ---------------------------------------------------------------------------
-// A CTA owns a GC_TX x GC_TY column tile and a chunk of z-planes.  Step j loads
-// phi of plane z0-2+j (2-node halo) into a 3-plane ring, forms the normals of
-// plane z0-3+j on the 1-halo tile into a second 3-plane ring (and writes
-// those of its own planes), and the curvature of plane z0-4+j from the normal
-// ring.  Each phi value is read from L2/HBM about 1.7 times, the normal once
-// per CTA; the per-node arithmetic is that of grad_body and the curvature
-// of the fused kernel.
-constexpr int GC_TX = 32, GC_TY = 8, GC_ZC = 16;
+// A CTA owns a GC_TX x (ROWS RP) column tile and a chunk of z-planes and
+// marches through the chunk's planes of phi (2-node halo).  Both stencils
+// split into in-plane sums of one plane each: with X, Y the differences of the
+// +-x and +-y neighbours, S the sum of the four, A and B the sum and difference
+// of the two diagonal differences of a plane,
+//   gx(z) = X/6 + A/12 + [X(z+1) + X(z-1)]/12,   gy alike with Y and B,
+//   gz(z) = q(z+1) - q(z-1),  q = phi/6 + S/12,
+// and the curvature is the same operator applied to the normal's components.
+// So a plane is read from shared memory once and its sums are carried to the
+// planes below and above in registers, instead of 18 + 30 reads of three
+// stored planes.  Iteration j: gradient and normal of plane z0-3+j on the
+// 1-halo tile (written to one of two normal planes), curvature of plane
+// z0-5+j from the normals of the iteration before, and phi of plane z0-1+j
+// into the plane ring; one barrier, which also tells whether any node of the
+// plane carries a flag (most planes of most tiles do not: no flag is looked at
+// then).  The first 32 ROWS threads own RP rows of one column each; further
+// threads take the nodes around the tile, whose normals the curvature needs.
+//
+// Bound by instruction issue (62% of the slots at 22 resident warps per SM), not
+// by memory: 24 bytes a node, most of which stay in L2.  The form with three
+// stored planes and 48 reads a node executed 14.2 warp instructions per node,
+// this one 11.3: 96-domain sweep (1.5e8 nodes) 2796 -> 1738 us, 64 x 96x48x48
+// 254 -> 204 us, 128x64x64 37 -> 24 us, 256x128x128 75 us either way.
+constexpr int GC_TX = 32;
 
 // a mod n in [0, n): the in-range and one-period cases without a division
 __device__ __forceinline__ int wrap_any(int a, int n)
@@ -472,30 +473,158 @@ __device__ __forceinline__ int wrap_any(int a, int n)
     return a < 0 ? a + n : a;
 }
 
-// owners of the neighbours of a node from the shared-memory flag ring
-template <int PW>
-struct GcNbr {
-    const uint8_t *fl[3];  // flag planes z-1, z, z+1
-    int c;                 // index of the node in the plane region
-    __device__ __forceinline__ int own(int dx, int dy, int dz) const
+// Operations rounded as written: a tile's own nodes and those around it run
+// two copies of the code below, which the compiler would otherwise be free to
+// contract into different multiply-adds, and a node's normal must have the
+// same bits in every tile (with the copies contracted apart, a symmetric drop
+// took up a sideways drift of 1e-4 of its speed).
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// the sums of the gradient carried from plane to plane for one column
+template <class R>
+struct GcColumn {
+    R px = 0, py = 0, pz = 0;  // gradient of the last plane but for the plane above it
+    R hx = 0, hy = 0, q = 0;   // X/12, Y/12 and q of the last plane
+    // next plane: the rows y-1, y, y+1 of its 3 x 3 nodes; g receives the last plane's gradient
+    __device__ __forceinline__ void advance(const R (&s)[3], const R (&c)[3], const R (&n)[3], R *g)
     {
-        return fl[dz + 1][c + dy * PW + dx] & OWNER_MASK;
+        const R d1 = sub_rn(n[2], s[0]), d2 = sub_rn(s[2], n[0]);
+        const R X = sub_rn(c[2], c[0]), Y = sub_rn(n[1], s[1]);
+        const R hx1 = mul_rn(R(1.0 / 12.0), X), hy1 = mul_rn(R(1.0 / 12.0), Y);
+        const R q1 =
+            fma_rn(R(1.0 / 6.0), c[1], mul_rn(R(1.0 / 12.0), add_rn(add_rn(c[2], c[0]), add_rn(n[1], s[1]))));
+        g[0] = add_rn(px, hx1);
+        g[1] = add_rn(py, hy1);
+        g[2] = add_rn(pz, q1);
+        px = fma_rn(R(1.0 / 6.0), X, fma_rn(R(1.0 / 12.0), add_rn(d1, d2), hx));
+        py = fma_rn(R(1.0 / 6.0), Y, fma_rn(R(1.0 / 12.0), sub_rn(d1, d2), hy));
+        pz = -q;
+        hx = hx1;
+        hy = hy1;
+        q = q1;
     }
 };
 
 template <class R>
-#ifndef LBM_GC_MINB
-#define LBM_GC_MINB 4
-#endif
-__global__ void __launch_bounds__(GC_TX *GC_TY, sizeof(R) == 8 ? 2 : LBM_GC_MINB) k_gradcurv(Lattice L)
+__device__ __forceinline__ void load_row(const R *p, R (&v)[3])
 {
-    constexpr int NT = GC_TX * GC_TY;
-    constexpr int PW = GC_TX + 4, PH = GC_TY + 4, PN = PW * PH;  // phi / flag region (2-node halo)
-    constexpr int NW = GC_TX + 2, NH = GC_TY + 2, NN = NW * NH;  // normal region (1-node halo)
-    constexpr int PER = (PN + NT - 1) / NT;                       // region values per thread
-    __shared__ R phS[3][PN];
+    v[0] = p[-1];
+    v[1] = p[0];
+    v[2] = p[1];
+}
+
+// a particle of the instance as the wetting needs it, in shared memory: centre,
+// radius, cos and sin of the contact angle
+template <class R>
+struct GcPart {
+    R x[3], rad, c, s;
+};
+
+// a fluid node next to a solid (region column c, flag planes f0, f1, f2 below,
+// at and above it): the wetting rotation of its gradient g, and
+// s = 3 sum w_i c_i over its solid neighbours, which take the node's own normal
+// in the curvature (their share is n . s).  The outward solid normal and
+// contact angle: the nearest particle surface if a neighbour belongs to a
+// particle, otherwise the normalised -sum w_i c_i over substrate neighbours.
+// A CTA's march waits for its slowest thread on every plane, so a surface
+// must not cost a chain of memory round trips: the sums are integers (36 w_i
+// is 2 or 1), the owners met are collected as a mask, and distances are taken
+// only where two particles meet.  With the owners' particle records read from
+// memory per direction the pass took 195 us instead of 75 on 256x128x128
+// nodes with eight spheres.
+template <class R, int PW>
+__device__ __forceinline__ void gc_solid(const InstDev &I, const GcPart<R> *parts, const uint8_t *f0,
+                                         const uint8_t *f1, const uint8_t *f2, int c, R phi, int x, int y, int z,
+                                         R *g, R *s)
+{
+    int all[3] = {0, 0, 0}, wall[3] = {0, 0, 0};
+    unsigned long long met = 0;
+#pragma unroll
+    for (int i = 1; i < Q; i++) {
+        const int own = (cz(i) < 0 ? f0 : (cz(i) > 0 ? f2 : f1))[c + cy(i) * PW + cx(i)] & OWNER_MASK;
+        const int k = own == OWN_FLUID ? 0 : (csq(i) == 1 ? 2 : 1);
+        const int kw = own == OWN_WALL ? k : 0;
+        if (cx(i)) { all[0] += cx(i) * k; wall[0] += cx(i) * kw; }
+        if (cy(i)) { all[1] += cy(i) * k; wall[1] += cy(i) * kw; }
+        if (cz(i)) { all[2] += cz(i) * k; wall[2] += cz(i) * kw; }
+        met |= 1ull << own;
+    }
+    for (int a = 0; a < 3; a++) s[a] = R(1.0 / 12.0) * all[a];
+    const R wet_max = sizeof(R) == 8 ? (R)I.wet_max : (R)I.f_wet_max;
+    if (!(fabs(phi) < wet_max)) return;
+    met &= ~(1ull << OWN_FLUID | 1ull << OWN_WALL | 1ull << OWN_PRESS);  // a pressure face carries no contact angle
+    R d[3] = {R(-wall[0]), R(-wall[1]), R(-wall[2])};
+    R cth = (R)I.cos_tw, sth = (R)I.sin_tw;
+    if (met) {
+        // lowest index first: it wins a tie
+        R bestd = 0;
+        bool first = true;
+        do {
+            const GcPart<R> &P = parts[__ffsll((long long)met) - 1 - 2];
+            met &= met - 1;
+            R e[3];
+            if (sizeof(R) == 8) {
+                e[0] = (R)min_image(x - P.x[0], I.nx); e[1] = (R)min_image(y - P.x[1], I.ny);
+                e[2] = (R)min_image(z - P.x[2], I.nz);
+            } else {
+                e[0] = (R)min_image_f((float)(x - P.x[0]), I.nx); e[1] = (R)min_image_f((float)(y - P.x[1]), I.ny);
+                e[2] = (R)min_image_f((float)(z - P.x[2]), I.nz);
+            }
+            const R dist = first && !met ? R(0) : sqrt(e[0] * e[0] + e[1] * e[1] + e[2] * e[2]) - P.rad;
+            if (first || dist < bestd) {
+                bestd = dist;
+                d[0] = e[0]; d[1] = e[1]; d[2] = e[2];
+                cth = P.c;
+                sth = P.s;
+            }
+            first = false;
+        } while (met);
+    }
+    const R l = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    if (l == R(0)) return;
+    const R ns[3] = {d[0] / l, d[1] / l, d[2] / l};
+    wetting_rotate<R>(g, ns, cth, sth);
+}
+
+// Threads of the pass for arithmetic type R.  Two rows per thread share most of
+// their shared-memory reads (floats: 75 against 72 us with one on 256x128x128
+// nodes, but 1738 against 1993 us on the 96-domain sweep); 8 warps of own
+// nodes beat 4 (80 and 1864 us) and 6 (82 and 1956 us).  FP64 runs are small
+// and bound by the FP64 pipe of the SMs that they reach: one row, and 4 or 8
+// warps by plan_gradcurv's rule (48x32x32: 61 against 90 us).
+template <class R, int ROWS>
+struct GcShape {
+    static constexpr int RP = sizeof(R) == 8 ? 1 : 2;
+    static constexpr int TY = ROWS * RP;
+    static constexpr int RING = (GC_TX + 2) * (TY + 2) - GC_TX * TY;  // nodes around the tile
+    static constexpr int OWN = GC_TX * ROWS;
+    static constexpr int NT = OWN + (RING + 31) / 32 * 32;
+};
+
+// CTAs per SM of the float form: 2 (80 registers); with 3 (56) the march spills
+// and took 139 to 168 us
+#ifndef LBM_GC_MINB
+#define LBM_GC_MINB 2
+#endif
+template <class R, int ROWS>
+__global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM_GC_MINB) k_gradcurv(Lattice L)
+{
+    using Shape = GcShape<R, ROWS>;
+    constexpr int RP = Shape::RP, TY = Shape::TY, NT = Shape::NT, OWN = Shape::OWN;
+    constexpr int PW = GC_TX + 4, PH = TY + 4, PN = PW * PH;  // phi / flag region (2-node halo)
+    constexpr int NW = GC_TX + 2, NH = TY + 2, NN = NW * NH;  // normal region (1-node halo)
+    constexpr int PER = (PN + NT - 1) / NT;                   // region values per thread
+    __shared__ R phS[4][PN];
     __shared__ uint8_t flS[4][PN];
-    __shared__ R nS[3][3][NN];
+    __shared__ R nS[2][3][NN];
+    __shared__ GcPart<R> partS[MAX_PART];
 
     const long long item = blockIdx.x;
     int k = 0;
@@ -513,148 +642,223 @@ __global__ void __launch_bounds__(GC_TX *GC_TY, sizeof(R) == 8 ? 2 : LBM_GC_MINB
     const int t2 = I.fd_nchunks.div(loc);
     const int chunk = loc - t2 * I.gc_nchunks;
     const int ty = I.fd_tiles_x.div(t2);
-    const int x0 = (t2 - ty * I.gc_tiles_x) * GC_TX, y0 = ty * GC_TY;
-    const int z0 = chunk * I.gc_zc, z1 = min(z0 + I.gc_zc, I.nz);
+    const int x0 = (t2 - ty * I.gc_tiles_x) * GC_TX, y0 = ty * TY;
+    const int z0 = chunk * I.gc_zc, zc = min(I.gc_zc, I.nz - z0);
     const int nx = I.nx, ny = I.ny, nz = I.nz;
-    const long long off = I.node_off, Nt = L.Ntot;
-    const uint8_t *fli = L.flags + off;
-    const R *ph = (const R *)L.phi + off;
-    R *Nn = (R *)L.grad + off;
-    R *Gm = (R *)L.gmag + off;
-    R *Kp = (R *)L.kap + off;
-    FluidPar<R> P;
-    load_par(I, P);
-    const int tid = threadIdx.x, lx = tid % GC_TX, ly = tid / GC_TX;
-    const int gx = x0 + lx, gy = y0 + ly;
-    const bool active = gx < nx && gy < ny;
-    const int niter = (z1 - z0) + 4;
+    const uint8_t *const fli = L.flags + I.node_off;
+    const R *const ph = (const R *)L.phi + I.node_off;
+    const int tid = threadIdx.x;
 
-    // this thread's columns of the 1-halo normal region (fixed for all planes)
-    constexpr int PER1 = (NN + NT - 1) / NT;
-    int nX[PER1], nY[PER1];
-    bool nOwn[PER1];
-#pragma unroll
-    for (int q = 0; q < PER1; q++) {
-        const int r1 = tid + q * NT, ax = r1 % NW, ay = r1 / NW;
-        nX[q] = wrap_any(x0 - 1 + ax, nx);
-        nY[q] = wrap_any(y0 - 1 + ay, ny);
-        nOwn[q] = r1 < NN && ax >= 1 && ax <= GC_TX && ay >= 1 && ay <= GC_TY && x0 - 1 + ax < nx && y0 - 1 + ay < ny;
+    // this thread's first node: column (ax, ay) of the 1-halo region
+    const bool own = tid < OWN;
+    int ax, ay;
+    if (own) {
+        ax = 1 + tid % GC_TX;
+        ay = 1 + tid / GC_TX * RP;
+    } else {
+        const int r = min(tid - OWN, Shape::RING - 1);  // the last warp's spare threads repeat the last node
+        if (r < 2 * NW) {
+            ax = r < NW ? r : r - NW;
+            ay = r < NW ? 0 : NH - 1;
+        } else {
+            ax = r & 1 ? NW - 1 : 0;
+            ay = 1 + (r - 2 * NW) / 2;
+        }
     }
-    // this thread's share of a plane region, prefetched one step ahead
+    const int gx = x0 + ax - 1, gy = y0 + ay - 1;  // periodic images for nodes around the tile
+    const int pc = (ay + 1) * PW + (ax + 1), nc = ay * NW + ax;
+    GradRec<R> *out = (GradRec<R> *)L.grad + I.node_off + ((long long)z0 * ny + gy) * nx + gx;  // of plane z0
+    const int plane = nx * ny;
+
+    // this thread's share of a plane region, fetched one iteration ahead
     int roff[PER];
 #pragma unroll
     for (int q = 0; q < PER; q++) {
-        const int r = tid + q * NT;
-        roff[q] = r < PN ? wrap_any(y0 - 2 + r / PW, ny) * nx + wrap_any(x0 - 2 + r % PW, nx) : -1;
+        const int r = min(tid + q * NT, PN - 1);
+        roff[q] = wrap_any(y0 - 2 + r / PW, ny) * nx + wrap_any(x0 - 2 + r % PW, nx);
     }
+    const R eps2 = sizeof(R) == 8 ? (R)(I.grad_eps * I.grad_eps) : (R)I.f_eps2;
     pdl_trigger();  // the collision may be scheduled as this grid drains
     pdl_wait();     // phi of the order-parameter pass
     R pv[PER];
     uint8_t fv[PER];
-    auto fetch = [&](int j) {
-        const int zo = wrap_any(z0 - 2 + j, nz) * ny * nx;
+    int zf = wrap_any(z0 - 2, nz);  // plane to fetch next
+    auto fetch = [&]() {
+        const int zo = zf * plane;
+        zf = zf == nz - 1 ? 0 : zf + 1;
 #pragma unroll
-        for (int q = 0; q < PER; q++)
-            if (roff[q] >= 0) {
-                pv[q] = ph[zo + roff[q]];
-                fv[q] = fli[zo + roff[q]];
-            }
+        for (int q = 0; q < PER; q++) {
+            pv[q] = ph[zo + roff[q]];
+            fv[q] = fli[zo + roff[q]];
+        }
     };
-    fetch(0);
-
-    for (int j = 0; j < niter; j++) {
-        // (1) plane z0-2+j into the rings, then fetch the next one
+    // the fetched plane into slot j of the rings; whether it carries any flag
+    auto store = [&](int j) {
+        bool any = false;
 #pragma unroll
         for (int q = 0; q < PER; q++) {
             const int r = tid + q * NT;
-            if (r < PN) {
-                phS[j % 3][r] = pv[q];
-                flS[j % 4][r] = fv[q];
+            if (PER * NT == PN || r < PN) {
+                phS[j & 3][r] = pv[q];
+                flS[j & 3][r] = fv[q];
             }
+            any |= fv[q] != 0;
         }
-        if (j + 1 < niter) fetch(j + 1);
-        __syncthreads();
-        // (2) normals of plane zz = z0-3+j (phi planes of steps j-2..j) on the 1-halo tile
-        if (j >= 2) {
-            const int zz = z0 - 3 + j;
-            const int Z = wrap_any(zz, nz);
-            const R *pm = phS[(j - 2) % 3], *p0 = phS[(j - 1) % 3], *pp = phS[j % 3];
-            const bool own_plane = zz >= z0 && zz < z1;
-            GcNbr<PW> nb;
-            nb.fl[0] = flS[(j - 2) % 4];
-            nb.fl[1] = flS[(j - 1) % 4];
-            nb.fl[2] = flS[j % 4];
+        return any;
+    };
+    for (int p = tid; p < I.np; p += NT) {
+        const PartDev &P = L.parts[I.part_off + p];
+        for (int a = 0; a < 3; a++) partS[p].x[a] = sizeof(R) == 8 ? (R)P.x[a] : (R)P.xf[a];
+        partS[p].rad = (R)P.R;
+        partS[p].c = (R)P.cos_t;
+        partS[p].s = (R)P.sin_t;
+    }
+    fetch();
+    bool flagged = false;                          // plane j - 1 carries flags
+    bool flagged_next = __syncthreads_or(store(0));  // plane j
+
+    GcColumn<R> col[RP];
+    R kp[RP], ud[RP];              // curvature of the last normal plane but for the plane above; its U - V
+    R corr1[RP], corr2[RP];        // the solid neighbours' share of it, planes z0-4+j and z0-5+j
+    unsigned fl1 = 0, fl2 = 0;     // own fluid nodes of those planes, a bit per row
 #pragma unroll
-            for (int q = 0; q < PER1; q++) {
-                const int r1 = tid + q * NT;
-                if (r1 >= NN) break;
-                const int ax = r1 % NW, ay = r1 / NW;
-                const int c = (ay + 1) * PW + (ax + 1);
-                const uint8_t fl = nb.fl[1][c];
-                R nn[3] = {0, 0, 0};
-                if ((fl & OWNER_MASK) == OWN_FLUID) {
-                    auto phi_of = [&](int dx, int dy, int dz) {
-                        const R *pl = dz < 0 ? pm : (dz > 0 ? pp : p0);
-                        return pl[c + dy * PW + dx];
-                    };
-                    R gr[3];
-                    grad_sum<R>(phi_of, gr);
-                    const int X = nX[q], Y = nY[q];
-                    if (fl & BOUND_BIT) {
-                        nb.c = c;
-                        grad_wet<R>(I, L.parts, nb, p0[c], fl, P.wet_max, X, Y, Z, gr);
-                    }
-                    const R m = reg_normal(gr, P.eps2, nn);
-                    if (own_plane && nOwn[q]) {
-                        const int n = (Z * ny + Y) * nx + X;
-                        Nn[n] = nn[0];
-                        Nn[Nt + n] = nn[1];
-                        Nn[2 * Nt + n] = nn[2];
-                        Gm[n] = m;
+    for (int r = 0; r < RP; r++) kp[r] = ud[r] = corr1[r] = corr2[r] = 0;
+    unsigned inside = 0;           // own nodes inside the domain
+#pragma unroll
+    for (int r = 0; r < RP; r++)
+        if (own && gx < nx && gy + r < ny) inside |= 1u << r;
+
+    for (int j = 0; j < zc + 5; j++) {
+        if (j < zc + 3) fetch();
+        R corr[RP];
+#pragma unroll
+        for (int r = 0; r < RP; r++) corr[r] = 0;
+        unsigned fluid = 0;
+        if (j < zc + 4) {
+            // (1) gradient and normal of plane z0-3+j; 0 for a solid node
+            const R *pl = phS[j & 3] + pc;
+            R v[RP + 2][3];
+#pragma unroll
+            for (int r = 0; r < RP + 2; r++)
+                if (r < 3 || own) load_row(pl + (r - 1) * PW, v[r]);
+#pragma unroll
+            for (int r = 0; r < RP; r++) {
+                if (r > 0 && !own) break;
+                R g[3], nn[3];
+                col[r].advance(v[r], v[r + 1], v[r + 2], g);
+                if (j < 2) continue;
+                bool solid = false;
+                R s0 = 0, s1 = 0, s2 = 0;
+                if (flagged) {
+                    const int c = pc + r * PW;
+                    const uint8_t fl = flS[(j - 1) & 3][c];
+                    solid = (fl & OWNER_MASK) != OWN_FLUID;
+                    if (!solid && (fl & BOUND_BIT)) {
+                        R sv[3] = {0, 0, 0};
+                        gc_solid<R, PW>(I, partS, flS[(j - 2) & 3], flS[(j - 1) & 3], flS[j & 3], c,
+                                        phS[(j - 1) & 3][c], wrap_any(gx, nx), wrap_any(gy + r, ny),
+                                        wrap_any(z0 - 3 + j, nz), g, sv);
+                        s0 = sv[0]; s1 = sv[1]; s2 = sv[2];
                     }
                 }
-                nS[j % 3][0][r1] = nn[0];
-                nS[j % 3][1][r1] = nn[1];
-                nS[j % 3][2][r1] = nn[2];
-            }
-        }
-        __syncthreads();
-        // (3) curvature of plane z = z0-4+j (normals of steps j-2..j, flags of steps j-3..j-1)
-        if (j >= 4 && active) {
-            const int z = z0 - 4 + j;
-            const int cp = (ly + 2) * PW + (lx + 2);
-            const uint8_t fl = flS[(j - 2) % 4][cp];
-            if ((fl & OWNER_MASK) == OWN_FLUID) {
-                const int c = (ly + 1) * NW + (lx + 1);
-                const int sl[3] = {(j - 2) % 3, (j - 1) % 3, j % 3};
-                R kap = curvature<R>([&](int dx, int dy, int dz, int a) { return nS[sl[dz + 1]][a][c + dy * NW + dx]; });
-                if (fl & BOUND_BIT) {
-                    GcNbr<PW> fb;
-                    fb.fl[0] = flS[(j - 3) % 4];
-                    fb.fl[1] = flS[(j - 2) % 4];
-                    fb.fl[2] = flS[(j - 1) % 4];
-                    fb.c = cp;
-                    kap = curvature<R>([&](int dx, int dy, int dz, int a) {
-                        if (fb.own(dx, dy, dz) != OWN_FLUID) return nS[sl[1]][a][c];
-                        return nS[sl[dz + 1]][a][c + dy * NW + dx];
-                    });
+                const R im = frsqrt(fma_rn(g[0], g[0], fma_rn(g[1], g[1], fma_rn(g[2], g[2], eps2))));
+                nn[0] = mul_rn(g[0], im);
+                nn[1] = mul_rn(g[1], im);
+                nn[2] = mul_rn(g[2], im);
+                if (solid) nn[0] = nn[1] = nn[2] = 0;
+                if (own) {
+                    const bool here = !solid && (inside >> r & 1u);
+                    if (here && j >= 3 && j < zc + 3) out[(j - 3) * plane + r * nx].set_gradient(g);
+                    if (here) fluid |= 1u << r;
+                    corr[r] = fma_rn(nn[0], s0, fma_rn(nn[1], s1, mul_rn(nn[2], s2)));
                 }
-                Kp[(z * ny + gy) * nx + gx] = kap;
+                R *d = &nS[j & 1][0][nc + r * NW];
+                d[0] = nn[0];
+                d[NN] = nn[1];
+                d[2 * NN] = nn[2];
             }
         }
-        __syncthreads();
+        // (2) curvature of plane z0-5+j: the in-plane sums of the normals of plane z0-4+j
+        if (j >= 3 && own) {
+            const R *a = nS[(j - 1) & 1][0] + nc, *b = a + NN, *d = b + NN;
+            R av[RP + 2][2], bv[RP + 2][3], dv[RP + 2], dw[RP][2];
+#pragma unroll
+            for (int r = 0; r < RP + 2; r++) {
+                av[r][0] = a[(r - 1) * NW - 1];
+                av[r][1] = a[(r - 1) * NW + 1];
+                load_row(b + (r - 1) * NW, bv[r]);
+                dv[r] = d[(r - 1) * NW];
+            }
+#pragma unroll
+            for (int r = 0; r < RP; r++) {
+                dw[r][0] = d[r * NW - 1];
+                dw[r][1] = d[r * NW + 1];
+            }
+#pragma unroll
+            for (int r = 0; r < RP; r++) {
+                const R twelfth = R(1.0 / 12.0), sixth = R(1.0 / 6.0);
+                const R e = add_rn(sub_rn(av[r + 1][1], av[r + 1][0]), sub_rn(bv[r + 2][1], bv[r][1]));
+                const R U = mul_rn(twelfth, e);
+                const R V = fma_rn(sixth, dv[r + 1],
+                                   mul_rn(twelfth, add_rn(add_rn(dw[r][1], dw[r][0]), add_rn(dv[r + 2], dv[r]))));
+                const R diag = add_rn(sub_rn(add_rn(av[r + 2][1], bv[r + 2][2]), add_rn(av[r][0], bv[r][0])),
+                                      sub_rn(sub_rn(av[r][1], bv[r][2]), sub_rn(av[r + 2][0], bv[r + 2][0])));
+                if ((fl2 >> r & 1u) && j >= 5)
+                    out[(j - 5) * plane + r * nx].k = add_rn(add_rn(kp[r], add_rn(U, V)), corr2[r]);
+                kp[r] = fma_rn(sixth, e, fma_rn(twelfth, diag, ud[r]));
+                ud[r] = sub_rn(U, V);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RP; r++) {
+            corr2[r] = corr1[r];
+            corr1[r] = corr[r];
+        }
+        fl2 = fl1;
+        fl1 = fluid;
+        flagged = flagged_next;
+        flagged_next = __syncthreads_or(j < zc + 3 ? store(j + 1) : false);
     }
 }
 
-long long plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst)
+// The gradient pass's work items.  Where no z-chunk is asked for, the planes
+// per item (and for FP64 the tile's height) that make
+// (items/slots + 1/2)(planes + 4) threads least: the waves of CTAs over the
+// slots (and half a wave of drain) times what a CTA marches through, 4 planes
+// of it halo.  Slots are the resident CTAs, one per SM for FP64, whose CTAs
+// share their SM's FP64 pipe.  Measured (256x128x128 FP32, 8 / 16 / 32 planes:
+// 75 / 75 / 78 us; 128x64x64, 4 planes against 16: 24 against 37 us; 48x32x32
+// FP64: 61 us against 270 with 16 planes).  Every choice gives the same bits.
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool fp64,
+                   FluidLaunch *fz)
 {
+    const double slots = n_sm * (fp64 ? 1.0 : (double)LBM_GC_MINB);
+    int rows = 8, zc_auto = 16;
+    double least = -1.0;
+    for (int r : {8, 4}) {
+        if (r == 4 && !fp64) continue;
+        const int ty = fp64 ? r : GcShape<float, 8>::TY;
+        const double threads = r == 8 ? GcShape<double, 8>::NT : GcShape<double, 4>::NT;
+        for (int zc : {32, 16, 8, 4, 2}) {
+            double items = 0.0;
+            for (const auto &I : inst)
+                items += (double)((I.nx + GC_TX - 1) / GC_TX) * ((I.ny + ty - 1) / ty) * ((I.nz + zc - 1) / zc);
+            const double cost = (items / slots + 0.5) * (zc + 4) * threads;
+            if (least < 0.0 || cost < least) {
+                least = cost;
+                rows = r;
+                zc_auto = zc;
+            }
+        }
+    }
+    const int ty = fp64 ? rows : GcShape<float, 8>::TY;
     long long items = 0;
     for (size_t k = 0; k < inst.size(); k++) {
         InstDev &I = inst[k];
         const int req = k < zc_inst.size() && zc_inst[k] > 0 ? zc_inst[k] : zc_request;
         I.gc_tiles_x = (I.nx + GC_TX - 1) / GC_TX;
-        I.gc_tiles_y = (I.ny + GC_TY - 1) / GC_TY;
-        const int zc = std::min(req > 0 ? req : GC_ZC, I.nz);
+        I.gc_tiles_y = (I.ny + ty - 1) / ty;
+        const int zc = std::min(req > 0 ? req : zc_auto, I.nz);
         I.gc_nchunks = (I.nz + zc - 1) / zc;
         I.gc_zc = (I.nz + I.gc_nchunks - 1) / I.gc_nchunks;
         I.fd_nchunks.set(I.gc_nchunks);
@@ -662,7 +866,8 @@ long long plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::v
         I.gc_item_start = items;
         items += (long long)I.gc_tiles_x * I.gc_tiles_y * I.gc_nchunks;
     }
-    return items;
+    fz->gc_items = items;
+    fz->gc_rows = rows;
 }
 
 // row-strip work items of the bulk kernels: whole x-rows of one z-plane, at
@@ -776,7 +981,12 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
         mk(STAGE_SOLIDPHI, 1);
     }
     mk(STAGE_GRAD, 0);
-    launch_after(k_gradcurv<R>, dim3((unsigned)fz.gc_items), dim3(GC_TX * GC_TY), st, L);
+    if constexpr (sizeof(R) == 8) {
+        if (fz.gc_rows == 4)
+            launch_after(k_gradcurv<R, 4>, dim3((unsigned)fz.gc_items), dim3(GcShape<R, 4>::NT), st, L);
+    }
+    if (fz.gc_rows == 8)
+        launch_after(k_gradcurv<R, 8>, dim3((unsigned)fz.gc_items), dim3(GcShape<R, 8>::NT), st, L);
     mk(STAGE_GRAD, 1);
     after_grad();
     bound_pass(k_collide_bound<S>, STAGE_COLLIDE_BOUND, STAGE_COLLIDE, [&] {

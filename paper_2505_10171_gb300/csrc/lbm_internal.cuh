@@ -58,6 +58,7 @@ constexpr unsigned ST_UNSTABLE = 1u;
 constexpr unsigned ST_DISPLACEMENT = 2u;
 constexpr unsigned ST_TIMEOUT = 4u;  // a bounded wait for an asynchronous copy gave up
 
+constexpr int MAX_PART = 61;  // particles of an instance (LBM_MAX_PARTICLES)
 constexpr int CAP_POINTS = 90 * 180;  // Sec. V F: 2 deg x 2 deg Lagrangian points
 constexpr int CAP_THREADS = 256;
 constexpr int CAP_BLOCKS = (CAP_POINTS + CAP_THREADS - 1) / CAP_THREADS;
@@ -177,9 +178,7 @@ struct Lattice {
     void *pop[2];
     void *phi;           // [Ntot] real: the order parameter of the step (outside a step: of the last one)
     void *col;           // [Ntot] ColRec<real>: colour record (phi, b n) of the stored state
-    void *grad;          // [3][Ntot] real: regularised interface normal n
-    void *gmag;          // [Ntot] real: sqrt(|grad phi|^2 + eps^2), so grad phi = n gmag
-    void *kap;           // [Ntot] real: curvature div(n) of fluid nodes
+    void *grad;          // [Ntot] GradRec<real>: corrected grad(phi) and curvature of fluid nodes
     void *u;             // [3][Ntot] real (store_velocity)
     long long Ntot;
     PartDev *parts;
@@ -416,6 +415,22 @@ struct GlobalNbr {
 template <class R>
 struct alignas(4 * sizeof(R)) ColRec {
     R p, a0, a1, a2;
+};
+
+// What the gradient pass leaves at a fluid node for the collision and the
+// capillary force: the corrected grad(phi) g and the curvature k = div(n) of
+// the regularised normals n = g/sqrt(|g|^2 + eps^2), one aligned record (one
+// vector load; the normal is formed again from g where it is needed)
+template <class R>
+struct alignas(4 * sizeof(R)) GradRec {
+    R g0, g1, g2, k;
+    // the gradient alone (the curvature follows two planes later)
+    __device__ __forceinline__ void set_gradient(const R *g)
+    {
+        struct alignas(2 * sizeof(R)) Pair { R a, b; };
+        *reinterpret_cast<Pair *>(&g0) = Pair{g[0], g[1]};
+        g2 = g[2];
+    }
 };
 
 // (c_i . a)/|c_i|: the colour offset G*_i of a record beyond phi (1 + F*_i)
@@ -736,11 +751,14 @@ struct FluidLaunch {
     int tile;           // 0: node-pair bulk collision where possible; 1: one node per thread
     long long rows;     // row-strip work items (all instances): CTAs of each bulk kernel
     long long gc_items; // gradient + curvature work items (all instances)
+    int gc_rows;        // warps of own nodes per CTA of that kernel (8; FP64: 4 or 8)
     bool pair;          // every instance has an even nx: node-pair kernels for 16-bit storage
 };
-// plan the work items of the gradient + curvature kernel (z-planes per item:
-// zc_inst[k] for instance k where set (> 0), else zc_request, else the default)
-long long plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst);
+// plan the work items of the gradient + curvature kernel into fz (z-planes per
+// item: zc_inst[k] for instance k where set (> 0), else zc_request where set,
+// else chosen from the grid's size and the n_sm SMs; fp64: double arithmetic)
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool fp64,
+                   FluidLaunch *fz);
 // plan the row-strip work items of every instance; returns their number
 long long plan_rows(std::vector<InstDev> &inst);
 template <class S>

@@ -187,8 +187,7 @@ __global__ void __launch_bounds__(CAP_THREADS) k_capillary(Lattice L)
         const int n3[3] = {I.nx, I.ny, I.nz};
         const uint8_t *fli = L.flags + I.node_off;
         const R *ph = (const R *)L.phi + I.node_off;
-        const R *Gn = (const R *)L.grad + I.node_off;   // regularised normal
-        const R *Gm = (const R *)L.gmag + I.node_off;   // its norm: grad phi = n gmag
+        const GradRec<R> *Gr = (const GradRec<R> *)L.grad + I.node_off;
         R ws = 0, phs = 0, gs[3] = {0, 0, 0};
         for (int cz_ = 0; cz_ < 2; cz_++)
             for (int cy_ = 0; cy_ < 2; cy_++)
@@ -201,12 +200,12 @@ __global__ void __launch_bounds__(CAP_THREADS) k_capillary(Lattice L)
                     if ((fli[m] & OWNER_MASK) != OWN_FLUID) continue;
                     const R wgt_ = (cx_ ? fr[0] : R(1) - fr[0]) * (cy_ ? fr[1] : R(1) - fr[1]) *
                                    (cz_ ? fr[2] : R(1) - fr[2]);
-                    const R mg = Gm[m];
+                    const GradRec<R> gm = Gr[m];
                     ws += wgt_;
                     phs += wgt_ * ph[m];
-                    gs[0] += wgt_ * (Gn[m] * mg);
-                    gs[1] += wgt_ * (Gn[L.Ntot + m] * mg);
-                    gs[2] += wgt_ * (Gn[2 * L.Ntot + m] * mg);
+                    gs[0] += wgt_ * gm.g0;
+                    gs[1] += wgt_ * gm.g1;
+                    gs[2] += wgt_ * gm.g2;
                 }
         if (ws > R(0)) {
             const R phv = phs / ws;
@@ -342,7 +341,6 @@ __device__ void quat_rotate(double *q, const T *w)
     q[0] = r0 / l; q[1] = r1 / l; q[2] = r2 / l; q[3] = r3 / l;
 }
 
-constexpr int DEM_MAXP = 61;
 constexpr int DEM_THREADS = 256;  // a warp per particle for the fluid sums of up to 8 particles at once
 
 // pair index c in [0, np(np-1)/2) -> (i, j), i < j, lexicographic
@@ -372,8 +370,8 @@ __global__ void __launch_bounds__(DEM_THREADS) k_dem(Lattice L, int sum_fluid)
     PartDev *P = L.parts + I.part_off;
     double *hist = L.hist + (long long)I.hist_off * 6;
     double *rec = L.crec + (long long)I.crec_off * 12;
-    __shared__ double xn[3 * DEM_MAXP];
-    __shared__ T vp[3 * DEM_MAXP], wp[3 * DEM_MAXP];
+    __shared__ double xn[3 * MAX_PART];
+    __shared__ T vp[3 * MAX_PART], wp[3 * MAX_PART];
     const int tid = threadIdx.x;
     if (sum_fluid) {
         // fluid forces of this step: a warp per particle sums the block
