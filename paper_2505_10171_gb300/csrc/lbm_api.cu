@@ -75,7 +75,7 @@ struct lbm_ctx {
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_pairs;
     cudaEvent_t ev_open[N_STAGES] = {};
     // launch variant of the fluid update
-    FluidLaunch fz = {0, 0, 0, 8, false};
+    FluidLaunch fz = {0, 0, 0, 0, 8, false};
     int zc_request = 0;        // z-planes per gradient work item, 0: automatic
     std::vector<int> zc_inst;  // per instance (the autotuner's size classes), 0: zc_request
     // drop-speed control: per instance integral (3) and last U_a (3); block partials
@@ -102,6 +102,7 @@ struct lbm_ctx {
 static void plan_launch(lbm_ctx *c)
 {
     plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, c->prec == LBM_FP64, &c->fz);
+    plan_phi(c->inst_h, c->n_sm, c->prec == LBM_FP64, &c->fz);
     c->fz.rows = plan_rows(c->inst_h);
     bool even = true;
     for (const auto &I : c->inst_h) even = even && I.nx % 2 == 0;

@@ -6,7 +6,7 @@
 // divergence (curvature) -> CSF + body force -> MRT with Guo forcing, evaluated
 // in its two-relaxation-time form -> recolouring -> write.
 //
-// Kernels of a step: k_phi (one thread per node over row strips) stores phi;
+// Kernels of a step: k_phi (z-marching tiles) stores phi;
 // the solid-phi fill over the listed static solid nodes and the step's list
 // of particle-surface solid nodes; k_gradcurv (z-marching tiles:
 // gradient, wetting, normal, curvature); k_collide (or k_collide2).  Nodes next
@@ -21,21 +21,10 @@
 // Storage type S in {double, float, __half, __nv_bfloat16}; arithmetic in
 // double for S = double and float otherwise.
 #include <algorithm>
+#include <cmath>
 
 #include "lbm_node.cuh"
 
-// CTAs of 256 threads per SM the single-precision order-parameter and
-// collision kernels are compiled for (register budget 65536 / (256 x this)).
-// The order-parameter pass holds 19 pulled offsets and 19 four-value colour
-// records per node: with FP32 offsets 3 CTAs (85 registers) measured faster
-// than 4 (106 against 115 us per 256x128x128 launch), with 16-bit offsets 4
-// (91 against 125 us)
-#ifndef LBM_PHI_MINB
-#define LBM_PHI_MINB 4
-#endif
-#ifndef LBM_PHI_MINB_F32
-#define LBM_PHI_MINB_F32 3
-#endif
 // CTAs per SM of the boundary passes, which run beside the bulk kernels
 #ifndef LBM_BOUND_MINB
 #define LBM_BOUND_MINB 2
@@ -52,26 +41,6 @@ namespace lbmg {
 // ---------------------------------------------------------------------------
 // bulk kernels over all nodes, list kernels over the nodes next to solids
 // ---------------------------------------------------------------------------
-// order parameter of a fluid node none of whose neighbours is solid; the
-// boundary pass (k_phi_bound) does the others.  Keeping the bounce-back code
-// out of the bulk kernel keeps its loads in flight (with it compiled in, the
-// kernel ran 75% longer).
-template <class S>
-__device__ __forceinline__ void phi_body(const Lattice &L, const InstDev &I, int cur, int n, int x, int y, int z)
-{
-    using R = typename Store<S>::real;
-    const long long g = I.node_off + n;
-    const uint8_t fl = L.flags[g];
-    const Pop<S> in(L.pop[cur], I);
-    const ColourOf<S> C(L, I);
-    Nbr nb;
-    nb.init(x, y, z, I.nx, I.ny, I.nz);
-    R v = phi_fluid<S>(nb, in, C);
-    keep(v);
-    if ((fl & OWNER_MASK) != OWN_FLUID || (fl & BOUND_BIT)) return;
-    ((R *)L.phi)[g] = v;
-}
-
 template <class R>
 __device__ __forceinline__ void solidphi_body(const Lattice &L, const InstDev &I, int n, int x, int y, int z)
 {
@@ -86,12 +55,202 @@ __device__ __forceinline__ void solidphi_body(const Lattice &L, const InstDev &I
     ((R *)L.phi)[g] = solid_fill<R>(nb, phi_of);
 }
 
+// a mod n in [0, n): the in-range and one-period cases without a division
+__device__ __forceinline__ int wrap_any(int a, int n)
+{
+    if (a >= 0 && a < n) return a;
+    if (a < 0 && a >= -n) return a + n;
+    if (a >= n && a < 2 * n) return a - n;
+    a %= n;
+    return a < 0 ? a + n : a;
+}
+
+// place of the in-plane source (x - dx, y - dy), dx or dy 0, among five
+__host__ __device__ constexpr int five(int dx, int dy)
+{
+    return dx < 0 ? 1 : (dx > 0 ? 2 : (dy < 0 ? 3 : (dy > 0 ? 4 : 0)));
+}
+
+// ---------------------------------------------------------------------------
+// order parameter of the fluid nodes none of whose neighbours is solid (the
+// boundary pass k_phi_bound does the others)
+// ---------------------------------------------------------------------------
+// phi = sum_i w_i G_i / (1 + sum_i w_i F_i) of the streamed offsets, the
+// colour offset pulled along direction i rebuilt from its source's record:
+//   G_i = p_s (1 + F_i) + (c_i . a_s)/|c_i|,  s = x - c_i.
+// Each record is wanted by 19 nodes.  A CTA owns a PH_TX x PH_TY column tile and
+// marches through a chunk of z-planes; a plane's records (1-node halo) are
+// staged once in shared memory, and every thread takes from each plane its nine
+// p and the plane's sums of a: with
+//   E = a0(x-1) - a0(x+1) + a1(y-1) - a1(y+1),  V = a2/18 + k (sum of a2 at the
+//   four neighbours),  D the diagonal differences,  k = 1/(36 sqrt 2),
+// the plane adds E/18 + k D to its own nodes' sum, k E + V to those above and
+// k E - V to those below: 26 scalar reads a node instead of 19 16-byte ones.
+// The 19 pulled offsets of the next plane are loaded as soon as this plane's
+// are used, so that they are in flight for a whole iteration.
+// Bound by the latency of those loads (96 bytes a node FP32, 58 of 16-bit
+// offsets; 24 resident warps per SM, half the issue slots used): 64 x 96x48x48
+// FP32 472 -> 284 us (4.8 TB/s), 96-domain FP16 sweep 4297 -> 2692 us,
+// 256x128x128 107 -> 93 us (FP16 92 -> 83: two waves of CTAs and little more),
+// against the form that loaded every record where it was wanted.  Three CTAs
+// per SM (80 registers); two 104 to 119 us, four (64, spilling) 213.
+constexpr int PH_TX = 32, PH_TY = 8;
+#ifndef LBM_PHI_MINB
+#define LBM_PHI_MINB 3
+#endif
+
 template <class S>
-__global__ void __launch_bounds__(ROW_NODES, sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? LBM_PHI_MINB_F32 : LBM_PHI_MINB))
+__global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MINB)
     k_phi(Lattice L, int cur)
 {
+    using R = typename Store<S>::real;
+    constexpr int NT = PH_TX * PH_TY, PW = PH_TX + 2, PN = PW * (PH_TY + 2), PER = (PN + NT - 1) / NT;
+    __shared__ R recS[2][4][PN];
     pdl_trigger();  // the gradient pass may be scheduled as this grid drains
-    for_item_nodes(L, blockIdx.x, [&](const InstDev &I, int n, int x, int y, int z) { phi_body<S>(L, I, cur, n, x, y, z); });
+
+    const long long item = blockIdx.x;
+    int lo = 0, hi = L.n_inst - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (L.inst[mid].ph_item_start <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    const InstDev &I = L.inst[lo];
+    const int loc = (int)(item - I.ph_item_start);
+    const int t2 = I.fd_ph_nchunks.div(loc);
+    const int chunk = loc - t2 * I.ph_nchunks;
+    const int ty = I.fd_ph_tiles_x.div(t2);
+    const int x0 = (t2 - ty * I.ph_tiles_x) * PH_TX, y0 = ty * PH_TY;
+    const int z0 = chunk * I.ph_zc, zc = min(I.ph_zc, I.nz - z0);
+    const int nx = I.nx, ny = I.ny, nz = I.nz, N = I.pstride, plane = nx * ny;
+    const S *const pf = Pop<S>(L.pop[cur], I).f;
+    const ColRec<R> *const rec = (const ColRec<R> *)L.col + I.node_off;
+    const uint8_t *const fli = L.flags + I.node_off;
+    R *const phi = (R *)L.phi + I.node_off;
+    const int tid = threadIdx.x, lx = tid % PH_TX, ly = tid / PH_TX;
+    const int gx = x0 + lx, gy = y0 + ly;
+    const bool inside = gx < nx && gy < ny;
+    const int c = (ly + 1) * PW + lx + 1;
+
+    // in-plane offsets of the sources (x - dx, y - dy)
+    int off[3][3];
+    {
+        const int X[3] = {wrap_any(gx + 1, nx), wrap_any(gx, nx), wrap_any(gx - 1, nx)};
+        const int Y[3] = {wrap_any(gy + 1, ny) * nx, wrap_any(gy, ny) * nx, wrap_any(gy - 1, ny) * nx};
+#pragma unroll
+        for (int b = 0; b < 3; b++)
+#pragma unroll
+            for (int a = 0; a < 3; a++) off[b][a] = Y[b] + X[a];
+    }
+    int roff[PER];
+#pragma unroll
+    for (int q = 0; q < PER; q++) {
+        const int r = min(tid + q * NT, PN - 1);
+        roff[q] = wrap_any(y0 - 1 + r / PW, ny) * nx + wrap_any(x0 - 1 + r % PW, nx);
+    }
+    ColRec<R> rv[PER];
+    int zr = wrap_any(z0 - 1, nz);  // plane whose records are fetched next
+    auto fetch = [&]() {
+        const int zo = zr * plane;
+        zr = zr == nz - 1 ? 0 : zr + 1;
+#pragma unroll
+        for (int q = 0; q < PER; q++) rv[q] = rec[zo + roff[q]];
+    };
+    auto store = [&](int j) {
+#pragma unroll
+        for (int q = 0; q < PER; q++) {
+            const int r = tid + q * NT;
+            if (r < PN) {
+                recS[j & 1][0][r] = rv[q].p;
+                recS[j & 1][1][r] = rv[q].a0;
+                recS[j & 1][2][r] = rv[q].a1;
+                recS[j & 1][3][r] = rv[q].a2;
+            }
+        }
+    };
+    // the pulled offsets and flags of target plane zt, in their stored type
+    S F[Q];
+    uint8_t fl = 0;
+    auto pull = [&](int zt) {
+        const int zo[3] = {(zt == nz - 1 ? 0 : zt + 1) * plane, zt * plane, (zt == 0 ? nz - 1 : zt - 1) * plane};
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            const S *const base = pf + (i * N + zo[cz(i) + 1]);
+            F[i] = pop_load(base + off[cy(i) + 1][cx(i) + 1]);
+        }
+        fl = fli[zt * plane + off[1][1]];
+    };
+    fetch();
+    store(0);
+    pull(z0);
+    __syncthreads();
+
+    const R k18 = R(1.0 / 18.0), kd = R(0.70710678118654752440 / 36.0);
+    // p of the last plane ([y][x], sources of the target as off) and the five of
+    // the plane before that a target above pulls from; sums of a to come
+    R p1[3][3], p2[5];
+    R above = 0, own = 0;  // of the plane after the last: what is below gives; of the last plane: all but its plane above
+#pragma unroll
+    for (int b = 0; b < 3; b++)
+#pragma unroll
+        for (int a = 0; a < 3; a++) p1[b][a] = 0;
+#pragma unroll
+    for (int a = 0; a < 5; a++) p2[a] = 0;
+    for (int j = 0; j < zc + 2; j++) {
+        // plane z0-1+j is staged; the target is plane z0-2+j
+        if (j < zc + 1) fetch();
+        const R *s = recS[j & 1][0] + c;
+        R p0[3][3];
+#pragma unroll
+        for (int b = 0; b < 3; b++)
+#pragma unroll
+            for (int a = 0; a < 3; a++) p0[b][a] = s[(1 - b) * PW + 1 - a];
+        const R *a0 = s + PN, *a1 = a0 + PN, *a2 = a1 + PN;
+        const R E = (a0[-1] - a0[1]) + (a1[-PW] - a1[PW]);
+        const R V = k18 * a2[0] + kd * ((a2[-1] + a2[1]) + (a2[-PW] + a2[PW]));
+        const R D = ((a0[-PW - 1] + a1[-PW - 1]) - (a0[PW + 1] + a1[PW + 1])) +
+                    ((a0[PW - 1] - a1[PW - 1]) - (a0[-PW + 1] - a1[-PW + 1]));
+        if (j >= 2) {
+            const R T = own + (kd * E - V);
+            R f[Q];
+#pragma unroll
+            for (int i = 0; i < Q; i++) f[i] = Store<S>::cvt(F[i]);
+            const int zt = z0 - 2 + j;
+            const bool write = inside && !(fl & (OWNER_MASK | BOUND_BIT));  // fluid, no solid beside it
+            if (j < zc + 1) pull(zt + 1);
+            // p (1 + F) and F summed by weight: rest, axes, diagonals
+            R ga = 0, gd = 0, fa = 0, fd = 0;
+#pragma unroll
+            for (int i = 1; i < Q; i++) {
+                const R p = cz(i) == 0 ? p1[cy(i) + 1][cx(i) + 1]
+                                       : (cz(i) < 0 ? p0[cy(i) + 1][cx(i) + 1] : p2[five(cx(i), cy(i))]);
+                const R g = p + p * f[i];
+                if (csq(i) == 1) {
+                    ga += g;
+                    fa += f[i];
+                } else {
+                    gd += g;
+                    fd += f[i];
+                }
+            }
+            const R num = R(1.0 / 3.0) * (p1[1][1] + p1[1][1] * f[0]) + (k18 * ga + (R(1.0 / 36.0) * gd + T));
+            const R den = R(1) + (R(1.0 / 3.0) * f[0] + (k18 * fa + R(1.0 / 36.0) * fd));
+            if (write) phi[zt * plane + off[1][1]] = num / den;
+        }
+        own = above + (k18 * E + kd * D);
+        above = kd * E + V;
+        p2[0] = p1[1][1];
+        p2[1] = p1[1][0];
+        p2[2] = p1[1][2];
+        p2[3] = p1[0][1];
+        p2[4] = p1[2][1];
+#pragma unroll
+        for (int b = 0; b < 3; b++)
+#pragma unroll
+            for (int a = 0; a < 3; a++) p1[b][a] = p0[b][a];
+        if (j < zc + 1) store(j + 1);
+        __syncthreads();
+    }
 }
 
 // instance of global node g (binary search over the node offsets)
@@ -463,16 +622,6 @@ __global__ void __launch_bounds__(ROW_NODES, sizeof(S) == 8 ? 1 : LBM_COLLIDE_MI
 // 254 -> 204 us, 128x64x64 37 -> 24 us, 256x128x128 75 us either way.
 constexpr int GC_TX = 32;
 
-// a mod n in [0, n): the in-range and one-period cases without a division
-__device__ __forceinline__ int wrap_any(int a, int n)
-{
-    if (a >= 0 && a < n) return a;
-    if (a < 0 && a >= -n) return a + n;
-    if (a >= n && a < 2 * n) return a - n;
-    a %= n;
-    return a < 0 ? a + n : a;
-}
-
 // Operations rounded as written: a tile's own nodes and those around it run
 // two copies of the code below, which the compiler would otherwise be free to
 // contract into different multiply-adds, and a node's normal must have the
@@ -821,14 +970,30 @@ __global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM
     }
 }
 
+// Cost of marching chunks of zc planes (and `halo` planes more) through column
+// tiles of tx x ty nodes over all instances, in plane iterations: the waves of
+// CTAs, counted as full ones (a CTA of the last wave runs as long as any) and
+// as what they hold (an SM with fewer CTAs runs them faster) alike, and half a
+// wave of drain.  Measured against it on 256x128x128 FP32, order parameter by
+// planes per chunk 4, 8, 13, 16, 19, 32, 43: 106, 99, 97, 105, 93, 120, 97 us
+// (cost 111, 100, 95, 104, 94, 124, 105); gradient pass 8, 15, 16, 22, 26,
+// 32, 43: 75, 73, 75, 80, 92, 78, 97 us (94, 83, 84, 98, 106, 84, 100).
+static double march_cost(const std::vector<InstDev> &inst, int tx, int ty, int zc, int halo, double slots)
+{
+    double items = 0.0;
+    for (const auto &I : inst)
+        items += (double)((I.nx + tx - 1) / tx) * ((I.ny + ty - 1) / ty) * ((I.nz + zc - 1) / zc);
+    const double waves = items / slots;
+    return (std::ceil(waves) + waves + 0.5) * (zc + halo);
+}
+constexpr int ZC_MAX = 64;
+
 // The gradient pass's work items.  Where no z-chunk is asked for, the planes
-// per item (and for FP64 the tile's height) that make
-// (items/slots + 1/2)(planes + 4) threads least: the waves of CTAs over the
-// slots (and half a wave of drain) times what a CTA marches through, 4 planes
-// of it halo.  Slots are the resident CTAs, one per SM for FP64, whose CTAs
-// share their SM's FP64 pipe.  Measured (256x128x128 FP32, 8 / 16 / 32 planes:
-// 75 / 75 / 78 us; 128x64x64, 4 planes against 16: 24 against 37 us; 48x32x32
-// FP64: 61 us against 270 with 16 planes).  Every choice gives the same bits.
+// per item (and for FP64 the tile's height, by the threads that march) of the
+// least cost.  Slots are the resident CTAs; one per SM for FP64, whose CTAs
+// share their SM's FP64 pipe.  128x64x64 FP32, 4 planes against 16: 24 against
+// 37 us; 48x32x32 FP64: 61 us against 270 with 16 planes.  Every choice gives
+// the same bits.
 void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool fp64,
                    FluidLaunch *fz)
 {
@@ -839,11 +1004,8 @@ void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector
         if (r == 4 && !fp64) continue;
         const int ty = fp64 ? r : GcShape<float, 8>::TY;
         const double threads = r == 8 ? GcShape<double, 8>::NT : GcShape<double, 4>::NT;
-        for (int zc : {32, 16, 8, 4, 2}) {
-            double items = 0.0;
-            for (const auto &I : inst)
-                items += (double)((I.nx + GC_TX - 1) / GC_TX) * ((I.ny + ty - 1) / ty) * ((I.nz + zc - 1) / zc);
-            const double cost = (items / slots + 0.5) * (zc + 4) * threads;
+        for (int zc = ZC_MAX; zc >= 2; zc--) {
+            const double cost = march_cost(inst, GC_TX, ty, zc, 4, slots) * threads;
             if (least < 0.0 || cost < least) {
                 least = cost;
                 rows = r;
@@ -868,6 +1030,35 @@ void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector
     }
     fz->gc_items = items;
     fz->gc_rows = rows;
+}
+
+// The order-parameter pass's work items, planned alike: one plane of halo
+// staged on each side of a chunk
+void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz)
+{
+    const double slots = n_sm * (fp64 ? 1.0 : (double)LBM_PHI_MINB);
+    int best = 16;
+    double least = -1.0;
+    for (int zc = ZC_MAX; zc >= 2; zc--) {
+        const double cost = march_cost(inst, PH_TX, PH_TY, zc, 2, slots);
+        if (least < 0.0 || cost < least) {
+            least = cost;
+            best = zc;
+        }
+    }
+    long long items = 0;
+    for (auto &I : inst) {
+        I.ph_tiles_x = (I.nx + PH_TX - 1) / PH_TX;
+        const int tiles_y = (I.ny + PH_TY - 1) / PH_TY;
+        const int zc = std::min(best, I.nz);
+        I.ph_nchunks = (I.nz + zc - 1) / zc;
+        I.ph_zc = (I.nz + I.ph_nchunks - 1) / I.ph_nchunks;
+        I.fd_ph_nchunks.set(I.ph_nchunks);
+        I.fd_ph_tiles_x.set(I.ph_tiles_x);
+        I.ph_item_start = items;
+        items += (long long)I.ph_tiles_x * tiles_y * I.ph_nchunks;
+    }
+    fz->ph_items = items;
 }
 
 // row-strip work items of the bulk kernels: whole x-rows of one z-plane, at
@@ -974,7 +1165,9 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
         }
         *launches += 1;
     };
-    bound_pass(k_phi_bound<S>, STAGE_PHI_BOUND, STAGE_PHI, [&] { k_phi<S><<<grid, ROW_NODES, 0, st>>>(L, cur); });
+    bound_pass(k_phi_bound<S>, STAGE_PHI_BOUND, STAGE_PHI, [&] {
+        k_phi<S><<<(unsigned)fz.ph_items, PH_TX * PH_TY, 0, st>>>(L, cur);
+    });
     if (!fill_done) {
         mk(STAGE_SOLIDPHI, 0);
         fill_solid_phi(st);

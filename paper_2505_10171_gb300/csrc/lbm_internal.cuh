@@ -125,6 +125,11 @@ struct InstDev {
     long long gc_item_start;
     int gc_tiles_x, gc_tiles_y, gc_nchunks, gc_zc;
     FastDiv fd_nchunks, fd_tiles_x;  // gc_nchunks, gc_tiles_x
+    // order-parameter work items: ph_tiles_x column tiles along x, ph_nchunks
+    // z-chunks of ph_zc planes
+    long long ph_item_start;
+    int ph_tiles_x, ph_nchunks, ph_zc;
+    FastDiv fd_ph_nchunks, fd_ph_tiles_x;
     // drop-speed control (body force on phase a): component mask, interval,
     // target velocity, PI gains, base force
     int sp_mask, sp_interval;
@@ -232,6 +237,7 @@ struct Store<double> {
     using real = double;
     static __device__ __forceinline__ double ld(const double *p) { return pop_load(p); }
     static __device__ __forceinline__ double lds(const double *p) { return *p; }  // shared memory
+    static __device__ __forceinline__ double cvt(double v) { return v; }
     static __device__ __forceinline__ void st(double *p, double v) { *p = v; }
 };
 template <>
@@ -239,6 +245,7 @@ struct Store<float> {
     using real = float;
     static __device__ __forceinline__ float ld(const float *p) { return pop_load(p); }
     static __device__ __forceinline__ float lds(const float *p) { return *p; }  // shared memory
+    static __device__ __forceinline__ float cvt(float v) { return v; }
     static __device__ __forceinline__ void st(float *p, float v) { *p = v; }
 };
 template <>
@@ -246,6 +253,7 @@ struct Store<__half> {
     using real = float;
     static __device__ __forceinline__ float ld(const __half *p) { return __half2float(pop_load(p)); }
     static __device__ __forceinline__ float lds(const __half *p) { return __half2float(*p); }  // shared memory
+    static __device__ __forceinline__ float cvt(__half v) { return __half2float(v); }
     static __device__ __forceinline__ void st(__half *p, float v) { *p = __float2half_rn(v); }
 };
 template <>
@@ -253,6 +261,7 @@ struct Store<__nv_bfloat16> {
     using real = float;
     static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(pop_load(p)); }
     static __device__ __forceinline__ float lds(const __nv_bfloat16 *p) { return __bfloat162float(*p); }  // shared memory
+    static __device__ __forceinline__ float cvt(__nv_bfloat16 v) { return __bfloat162float(v); }
     static __device__ __forceinline__ void st(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
@@ -563,31 +572,6 @@ __device__ __forceinline__ void gather_all(const InstDev &I, const PartDev *part
     *sG = g;
 }
 
-// order parameter after streaming of a fluid node none of whose neighbours is
-// solid: phi = sum_i w_i G_i / (1 + sum_i w_i F_i) with G_i rebuilt from the
-// source node's colour state
-template <class S, class A>
-__device__ __forceinline__ typename Store<S>::real phi_fluid(const A &nbr, const Pop<S> &in,
-                                                             const ColourOf<S> &C)
-{
-    using R = typename Store<S>::real;
-    R sF = 0, sG = 0;
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        const int s = nbr.idx(-cx(i), -cy(i), -cz(i));
-        const R F = in.F(i, s);
-        const ColRec<R> cs = C.at(s);
-        sF += wgt<R>(i) * F;
-        R g = cs.p * (R(1) + F);
-        if (i) g += col_rec(i, cs);
-        sG += wgt<R>(i) * g;
-    }
-    return sG / (R(1) + sF);
-}
-
-template <class R>
-__device__ __forceinline__ R dsqrt(R v) { return sqrt(v); }
-
 // Sec. V E geometric wetting: rotate g so that -g/|g| makes the angle theta
 // with the outward solid normal ns, keeping |g|; of the two candidates the one
 // closer to the original direction is kept.
@@ -750,6 +734,7 @@ constexpr int FORM_PLAIN = 2;  // the launch form of the fluid update (the value
 struct FluidLaunch {
     int tile;           // 0: node-pair bulk collision where possible; 1: one node per thread
     long long rows;     // row-strip work items (all instances): CTAs of each bulk kernel
+    long long ph_items; // order-parameter work items (all instances)
     long long gc_items; // gradient + curvature work items (all instances)
     int gc_rows;        // warps of own nodes per CTA of that kernel (8; FP64: 4 or 8)
     bool pair;          // every instance has an even nx: node-pair kernels for 16-bit storage
@@ -759,6 +744,8 @@ struct FluidLaunch {
 // else chosen from the grid's size and the n_sm SMs; fp64: double arithmetic)
 void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool fp64,
                    FluidLaunch *fz);
+// plan the work items of the order-parameter kernel into fz
+void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz);
 // plan the row-strip work items of every instance; returns their number
 long long plan_rows(std::vector<InstDev> &inst);
 template <class S>
