@@ -143,6 +143,7 @@ static Lattice make_lattice(const lbm_ctx *c)
     L.static_bfl = c->static_bfl;
     L.n_static_bfl = c->n_static_bfl;
     L.flags = c->flags;
+    L.mark = c->prec == LBM_FP64 ? 8 : (c->prec == LBM_FP32 ? 4 : 0);
     L.pop[0] = c->pop[0];
     L.pop[1] = c->pop[1];
     L.phi = c->phi;
@@ -987,6 +988,7 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
         I.f_eta_a = (float)I.eta_a; I.f_eta_b = (float)I.eta_b;
         I.f_eps2 = (float)(I.grad_eps * I.grad_eps); I.f_wet_max = (float)I.wet_max;
         for (int a = 0; a < 3; a++) { I.f_body_a[a] = (float)I.body_a[a]; I.f_body_b[a] = (float)I.body_b[a]; }
+        for (int a = 0; a < 3; a++) I.f_wall_u[a] = (float)I.wall_u[a];
         I.f_ir0 = (float)(1.0 / I.rho0);
         I.f_h_ia = (float)(0.5 / I.eta_a);
         I.f_h_ib = (float)(0.5 / I.eta_b);
@@ -1355,26 +1357,28 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
         // solid nodes next to non-static ones; mode 1: non-static nodes next to
         // static solids)
         Lattice L = make_lattice(ctx);
-        unsigned long long *cnt = nullptr;
-        CU(cudaMalloc((void **)&cnt, sizeof(unsigned long long)));
+        const long long nb = static_bound_blocks(L);
+        long long *offs = nullptr;  // offsets [nb + 1], then counts [nb]
+        CU(cudaMalloc((void **)&offs, sizeof(long long) * (size_t)(nb + 1) + sizeof(int) * (size_t)nb));
+        int *blocks = (int *)(offs + nb + 1);
         long long **lists[2] = {&ctx->static_list, &ctx->static_bfl};
         long long *counts[2] = {&ctx->n_static, &ctx->n_static_bfl};
-        for (int mode = 0; mode < 2; mode++) {
-            unsigned long long h = 0;
-            CU(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), ctx->stream));
-            launch_static_bound(L, nullptr, cnt, mode, ctx->stream);
-            CU(cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, ctx->stream));
-            CU(cudaStreamSynchronize(ctx->stream));
-            if (h > 0) {
-                CU(cudaMalloc((void **)lists[mode], sizeof(long long) * h));
-                CU(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), ctx->stream));
-                launch_static_bound(L, *lists[mode], cnt, mode, ctx->stream);
-                CU(cudaStreamSynchronize(ctx->stream));
-            }
-            *counts[mode] = (long long)h;
+        cudaError_t e = cudaSuccess;
+        for (int mode = 0; mode < 2 && e == cudaSuccess; mode++) {
+            long long h = 0;
+            launch_static_count(L, blocks, offs, mode, ctx->stream);
+            e = cudaMemcpyAsync(&h, offs + nb, sizeof h, cudaMemcpyDeviceToHost, ctx->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+            if (e == cudaSuccess && h > 0 && !*lists[mode]) e = cudaMalloc((void **)lists[mode], sizeof(long long) * h);
+            if (e == cudaSuccess && h > 0) launch_static_fill(L, offs, *lists[mode], mode, ctx->stream);
+            if (e == cudaSuccess) *counts[mode] = h;
         }
+        if (e == cudaSuccess && L.mark)
+            dispatch(ctx->prec, [&](auto *tag) { launch_mark_solid<std::remove_pointer_t<decltype(tag)>>(L, ctx->stream); });
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // before offs goes
+        cudaFree(offs);
+        CU(e);
         CU(cudaGetLastError());
-        cudaFree(cnt);
         ctx->static_ready = true;
         drop_graph(ctx);
     }

@@ -41,20 +41,6 @@ namespace lbmg {
 // ---------------------------------------------------------------------------
 // bulk kernels over all nodes, list kernels over the nodes next to solids
 // ---------------------------------------------------------------------------
-template <class R>
-__device__ __forceinline__ void solidphi_body(const Lattice &L, const InstDev &I, int n, int x, int y, int z)
-{
-    const long long g = I.node_off + n;
-    const uint8_t fl = L.flags[g];
-    if ((fl & OWNER_MASK) == OWN_FLUID || !(fl & BOUND_BIT)) return;
-    GlobalNbr nb;
-    nb.nb.init(x, y, z, I.nx, I.ny, I.nz);
-    nb.fli = L.flags + I.node_off;
-    const R *ph = (const R *)L.phi + I.node_off;
-    auto phi_of = [&](int dx, int dy, int dz) { return ph[nb.idx(dx, dy, dz)]; };
-    ((R *)L.phi)[g] = solid_fill<R>(nb, phi_of);
-}
-
 // a mod n in [0, n): the in-range and one-period cases without a division
 __device__ __forceinline__ int wrap_any(int a, int n)
 {
@@ -253,6 +239,9 @@ __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MIN
     }
 }
 
+// ---------------------------------------------------------------------------
+// boundary lists
+// ---------------------------------------------------------------------------
 // instance of global node g (binary search over the node offsets)
 __device__ __forceinline__ int inst_of_node(const Lattice &L, long long g)
 {
@@ -265,14 +254,13 @@ __device__ __forceinline__ int inst_of_node(const Lattice &L, long long g)
     return lo;
 }
 
-// static solid nodes with a neighbour that is not static solid: the only
-// static nodes the solid-phi fill can reach.  count pass (list == null) or
-// fill pass; the order of the list does not matter.
-__global__ void k_static_bound(Lattice L, long long *list, unsigned long long *count, int mode)
+// static solid nodes with a neighbour that is not static solid (mode 0), or
+// the other way round (mode 1): whether global node g is one, and its entry
+__device__ __forceinline__ bool static_bound(const Lattice &L, long long g, int mode, long long *entry)
 {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= L.Ntot || own_static(L.flags[g] & OWNER_MASK) != (mode == 0)) return;
-    const InstDev &I = L.inst[inst_of_node(L, g)];
+    if (g >= L.Ntot || own_static(L.flags[g] & OWNER_MASK) != (mode == 0)) return false;
+    const int k = inst_of_node(L, g);
+    const InstDev &I = L.inst[k];
     const int n = (int)(g - I.node_off);
     const int x = n % I.nx, y = (n / I.nx) % I.ny, z = n / (I.nx * I.ny);
     Nbr nb;
@@ -281,29 +269,86 @@ __global__ void k_static_bound(Lattice L, long long *list, unsigned long long *c
     bool hit = false;
 #pragma unroll
     for (int i = 1; i < Q; i++) hit |= own_static(fli[nb.at(cx(i), cy(i), cz(i))] & OWNER_MASK) != (mode == 0);
+    *entry = list_entry(k, n);
+    return hit;
+}
+
+// The lists are in node order: consecutive threads of the passes over them
+// then work on nodes of one row, whose loads share sectors.  (Appended with one
+// atomic per node, 64x64x1024 tube: order-parameter boundary pass 98 us and
+// collision boundary pass 187 us for 300 000 nodes; in order 88 us, and the
+// latter is gone.)
+constexpr int SB_THREADS = 256;
+__global__ void __launch_bounds__(SB_THREADS) k_static_count(Lattice L, int mode, int *blocks)
+{
+    long long e;
+    const int c = __syncthreads_count(static_bound(L, (long long)blockIdx.x * SB_THREADS + threadIdx.x, mode, &e));
+    if (threadIdx.x == 0) blocks[blockIdx.x] = c;
+}
+
+// offs[b] = sum of blocks[0..b), offs[nb] = sum of all: one CTA, a run of
+// consecutive blocks per thread
+__global__ void __launch_bounds__(1024) k_static_scan(const int *blocks, long long nb, long long *offs)
+{
+    __shared__ long long sh[1024];
+    const int t = threadIdx.x;
+    const long long per = (nb + 1023) / 1024, b0 = min(nb, t * per), b1 = min(nb, b0 + per);
+    long long s = 0;
+    for (long long b = b0; b < b1; b++) s += blocks[b];
+    sh[t] = s;
+    __syncthreads();
+    for (int d = 1; d < 1024; d <<= 1) {
+        const long long v = t >= d ? sh[t - d] : 0;
+        __syncthreads();
+        sh[t] += v;
+        __syncthreads();
+    }
+    long long o = sh[t] - s;
+    for (long long b = b0; b < b1; b++) {
+        offs[b] = o;
+        o += blocks[b];
+    }
+    if (t == 1023) offs[nb] = sh[1023];
+}
+
+__global__ void __launch_bounds__(SB_THREADS) k_static_fill(Lattice L, int mode, const long long *offs, long long *list)
+{
+    __shared__ int warps[SB_THREADS / 32];
+    long long e = 0;
+    const bool hit = static_bound(L, (long long)blockIdx.x * SB_THREADS + threadIdx.x, mode, &e);
+    const unsigned m = __ballot_sync(0xffffffffu, hit);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) warps[wid] = __popc(m);
+    __syncthreads();
     if (!hit) return;
-    const unsigned long long k = atomicAdd(count, 1ull);
-    if (list) list[k] = g;
+    long long o = offs[blockIdx.x] + __popc(m & ((1u << lane) - 1u));
+    for (int w = 0; w < wid; w++) o += warps[w];
+    list[o] = e;
 }
 
-// solid-phi fill of the listed static nodes
+long long static_bound_blocks(const Lattice &L) { return (L.Ntot + SB_THREADS - 1) / SB_THREADS; }
+void launch_static_count(const Lattice &L, int *blocks, long long *offs, int mode, cudaStream_t st)
+{
+    const long long nb = static_bound_blocks(L);
+    k_static_count<<<(unsigned)nb, SB_THREADS, 0, st>>>(L, mode, blocks);
+    k_static_scan<<<1, 1024, 0, st>>>(blocks, nb, offs);
+}
+void launch_static_fill(const Lattice &L, const long long *offs, long long *list, int mode, cudaStream_t st)
+{
+    k_static_fill<<<(unsigned)static_bound_blocks(L), SB_THREADS, 0, st>>>(L, mode, offs, list);
+}
+
 template <class R>
-__global__ void k_solidphi_list(Lattice L)
+__global__ void __launch_bounds__(256) k_mark_solid(Lattice L)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.n_static) return;
-    const long long g = L.static_list[i];
-    const InstDev &I = L.inst[inst_of_node(L, g)];
-    const int n = (int)(g - I.node_off);
-    const int x = n % I.nx, y = (n / I.nx) % I.ny, z = n / (I.nx * I.ny);
-    solidphi_body<R>(L, I, n, x, y, z);
+    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < L.Ntot && (L.flags[g] & OWNER_MASK) != OWN_FLUID) set_solid_mark(((GradRec<R> *)L.grad)[g]);
 }
-
-void launch_static_bound(const Lattice &L, long long *list, unsigned long long *count, int mode, cudaStream_t st)
+template <class S>
+void launch_mark_solid(const Lattice &L, cudaStream_t st)
 {
-    k_static_bound<<<(unsigned)((L.Ntot + 255) / 256), 256, 0, st>>>(L, list, count, mode);
+    k_mark_solid<typename Store<S>::real><<<(unsigned)((L.Ntot + 255) / 256), 256, 0, st>>>(L);
 }
-
 
 // the fluid nodes next to a solid inside the particle cubes (cubes of side
 // cap_side around each particle, cap_blocks CTAs each), appended to L.pbl
@@ -325,8 +370,9 @@ __global__ void __launch_bounds__(PART_THREADS) k_bound_list(Lattice L)
     if (t < reg.count()) {
         int x, y, z;
         reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
-        g = I.node_off + ((long long)z * I.ny + y) * I.nx + x;
-        const uint8_t fl = L.flags[g];
+        const int n = (z * I.ny + y) * I.nx + x;
+        g = list_entry(P0.inst, n);
+        const uint8_t fl = L.flags[I.node_off + n];
         fluid = (fl & OWNER_MASK) == OWN_FLUID && (fl & BOUND_BIT);
         solid = (fl & OWNER_MASK) != OWN_FLUID && (fl & BOUND_BIT);
     }
@@ -344,76 +390,93 @@ __global__ void __launch_bounds__(PART_THREADS) k_bound_list(Lattice L)
     append(solid, L.psl, L.psl_n);
 }
 
-// work item t of the boundary passes: the listed particle nodes, then the
-// static list of nodes next to static solids
-__device__ __forceinline__ void bound_item(const Lattice &L, long long npb, long long t, const InstDev **Ip, int *n,
-                                           int *x, int *y, int *z)
+// node of a list entry
+__device__ __forceinline__ const InstDev &list_node(const Lattice &L, long long e, int *n, int *x, int *y, int *z)
 {
-    const long long g = t < npb ? L.pbl[t] : L.static_bfl[t - npb];
-    const InstDev &I = L.inst[inst_of_node(L, g)];
-    *n = (int)(g - I.node_off);
-    *x = *n % I.nx;
-    *y = (*n / I.nx) % I.ny;
-    *z = *n / (I.nx * I.ny);
-    *Ip = &I;
+    const InstDev &I = L.inst[e >> 32];
+    *n = (int)(unsigned)e;
+    const int row = I.fd_nx.div(*n);
+    *x = *n - row * I.nx;
+    *z = I.fd_ny.div(row);
+    *y = row - *z * I.ny;
+    return I;
 }
 
-// the boundary passes: fluid nodes next to a solid, with the bounce-back
-// pull (Sec. V A), grid-stride over the work list; a node listed twice (two
-// cubes, or a cube and the static list) is written twice with the same value
+// The boundary passes: fluid nodes next to a solid, with the bounce-back pull
+// (Sec. V A), grid-stride over the listed particle nodes and the static list
+// of nodes next to walls; a node listed twice (two cubes, or a cube and the
+// static list) is written twice with the same value.
+//
+// The order-parameter pass forms every bounced offset F_i; FP32 and FP64
+// storage keep it in slot i of the solid source itself, which no other node
+// pulls and no kernel reads otherwise, so that the bulk collision pulls these
+// nodes like all others and has no boundary pass.  (16-bit storage would round
+// the offset there; its collision takes these nodes in k_collide_bound.)  The
+// bulk order-parameter pass may load such a slot while it is written: for a
+// node next to a solid, whose value it drops.
 template <class S>
-__device__ __forceinline__ void phi_bound_node(const Lattice &L, int cur, const InstDev *I, int n, int x, int y, int z)
+constexpr bool BOUNCE_IN_SLOTS = sizeof(S) >= 4;
+
+template <class S>
+__device__ __forceinline__ void phi_bound_node(const Lattice &L, int cur, long long e)
 {
     using R = typename Store<S>::real;
-    const long long g = I->node_off + n;
-    const uint8_t fl = L.flags[g];
-    if ((fl & OWNER_MASK) != OWN_FLUID || !(fl & BOUND_BIT)) return;
-    const Pop<S> in(L.pop[cur], *I);
-    const ColourOf<S> C(L, *I);
-    GlobalNbr nb;
-    nb.nb.init(x, y, z, I->nx, I->ny, I->nz);
-    nb.fli = L.flags + I->node_off;
-    R F[Q], sF = 0, sG = 0;
-    gather_all<S>(*I, L.parts, nb, in, &C, n, F, &sG, x, y, z);
+    int n, x, y, z;
+    const InstDev &I = list_node(L, e, &n, &x, &y, &z);
+    const uint8_t *fli = L.flags + I.node_off;
+    const uint8_t fl = fli[n];
+    const Pop<S> in(L.pop[cur], I);
+    const ColourOf<S> C(L, I);
+    Nbr nb;
+    nb.init(x, y, z, I.nx, I.ny, I.nz);
+    int own[Q];
+    R F[Q], sF = 0;
+    gather_links<S>(I, L.parts, fli, nb, in, n, x, y, z, own, F);
+    const R sG = gather_colour<S>(nb, C, n, own, F);
+    if ((fl & OWNER_MASK) != OWN_FLUID || !(fl & BOUND_BIT)) return;  // covered by a particle
 #pragma unroll
     for (int i = 0; i < Q; i++) sF += wgt<R>(i) * F[i];
-    ((R *)L.phi)[g] = sG / (R(1) + sF);
-}
-
-template <class S>
-__global__ void __launch_bounds__(PART_THREADS, LBM_BOUND_MINB) k_phi_bound(Lattice L, int cur)
-{
-    const long long npb = L.pbl_n ? (long long)*L.pbl_n : 0;
-    const long long total = npb + L.n_static_bfl;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const InstDev *I;
-        int n, x, y, z;
-        bound_item(L, npb, t, &I, &n, &x, &y, &z);
-        phi_bound_node<S>(L, cur, I, n, x, y, z);
+    ((R *)L.phi)[I.node_off + n] = sG / (R(1) + sF);
+    if (BOUNCE_IN_SLOTS<S>) {
+#pragma unroll
+        for (int i = 1; i < Q; i++)
+            if (own[i] != OWN_FLUID) in.setF(i, nb.at(-cx(i), -cy(i), -cz(i)), F[i]);
     }
 }
 
 template <class S>
-__device__ __forceinline__ void collide_bound_node(const Lattice &L, int cur, const InstDev *I, int n, int x, int y,
-                                                   int z)
+__global__ void __launch_bounds__(PART_THREADS, sizeof(S) == 8 ? 1 : LBM_BOUND_MINB) k_phi_bound(Lattice L, int cur)
+{
+    const long long npb = L.pbl_n ? (long long)*L.pbl_n : 0;
+    const long long total = npb + L.n_static_bfl;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+         t += (long long)gridDim.x * blockDim.x)
+        phi_bound_node<S>(L, cur, t < npb ? L.pbl[t] : L.static_bfl[t - npb]);
+}
+
+template <class S>
+__device__ __forceinline__ void collide_bound_node(const Lattice &L, int cur, long long e)
 {
     using R = typename Store<S>::real;
-    const long long g = I->node_off + n;
-    const uint8_t fl = L.flags[g];
-    if ((fl & OWNER_MASK) != OWN_FLUID || !(fl & BOUND_BIT)) return;
-    const Pop<S> in(L.pop[cur], *I);
-    const Pop<S> out(L.pop[cur ^ 1], *I);
-    R *U = I->store_u ? (R *)L.u + I->node_off : nullptr;
-    GlobalNbr nb;
-    nb.nb.init(x, y, z, I->nx, I->ny, I->nz);
-    nb.fli = L.flags + I->node_off;
+    int n, x, y, z;
+    const InstDev &I = list_node(L, e, &n, &x, &y, &z);
+    const uint8_t *fli = L.flags + I.node_off;
+    const long long g = I.node_off + n;
+    const uint8_t fl = fli[n];
+    const Pop<S> in(L.pop[cur], I);
+    const Pop<S> out(L.pop[cur ^ 1], I);
+    const GradRec<R> gr = ((const GradRec<R> *)L.grad)[g];
+    const R phi = ((const R *)L.phi)[g];
+    R *U = I.store_u ? (R *)L.u + I.node_off : nullptr;
+    Nbr nb;
+    nb.init(x, y, z, I.nx, I.ny, I.nz);
+    int own[Q];
     R F[Q];
-    gather_all<S>(*I, L.parts, nb, in, (const ColourOf<S> *)nullptr, n, F, (R *)nullptr, x, y, z);
+    gather_links<S>(I, L.parts, fli, nb, in, n, x, y, z, own, F);
+    if ((fl & OWNER_MASK) != OWN_FLUID || !(fl & BOUND_BIT)) return;
     FluidPar<R> P;
-    load_par(*I, P);
-    collide_store_phi<S>(P, F, ((const R *)L.phi)[g], ((const GradRec<R> *)L.grad)[g], out, n, col_slot<S>(L, g), U,
-                         L.Ntot, L.status);
+    load_par(I, P);
+    collide_store_phi<S>(P, F, phi, gr, out, n, col_slot<S>(L, g), U, L.Ntot, L.status);
 }
 
 template <class S>
@@ -422,25 +485,43 @@ __global__ void __launch_bounds__(PART_THREADS, LBM_BOUND_MINB) k_collide_bound(
     const long long npb = L.pbl_n ? (long long)*L.pbl_n : 0;
     const long long total = npb + L.n_static_bfl;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const InstDev *I;
-        int n, x, y, z;
-        bound_item(L, npb, t, &I, &n, &x, &y, &z);
-        collide_bound_node<S>(L, cur, I, n, x, y, z);
-    }
+         t += (long long)gridDim.x * blockDim.x)
+        collide_bound_node<S>(L, cur, t < npb ? L.pbl[t] : L.static_bfl[t - npb]);
 }
 
-// solid-phi fill of the listed particle-surface solid nodes, grid-stride
+// phi of the solid nodes next to fluid, the listed static ones and the step's
+// list of particle-surface ones: the w-weighted mean over their fluid
+// neighbours
 template <class R>
-__global__ void __launch_bounds__(PART_THREADS) k_solidphi_plist(Lattice L)
+__global__ void __launch_bounds__(PART_THREADS) k_solidphi(Lattice L)
 {
-    const long long nps = (long long)*L.psl_n;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < nps;
+    const long long nps = L.psl_n ? (long long)*L.psl_n : 0;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < nps + L.n_static;
          t += (long long)gridDim.x * blockDim.x) {
-        const long long g = L.psl[t];
-        const InstDev &I = L.inst[inst_of_node(L, g)];
-        const int n = (int)(g - I.node_off);
-        solidphi_body<R>(L, I, n, n % I.nx, (n / I.nx) % I.ny, n / (I.nx * I.ny));
+        int n, x, y, z;
+        const InstDev &I = list_node(L, t < nps ? L.psl[t] : L.static_list[t - nps], &n, &x, &y, &z);
+        const uint8_t *fli = L.flags + I.node_off;
+        R *ph = (R *)L.phi + I.node_off;
+        Nbr nb;
+        nb.init(x, y, z, I.nx, I.ny, I.nz);
+        const uint8_t fl = fli[n];
+        int own[Q];
+        R p[Q];
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            const int s = nb.at(cx(i), cy(i), cz(i));
+            own[i] = fli[s];
+            p[i] = ph[s];
+        }
+        if ((fl & OWNER_MASK) == OWN_FLUID || !(fl & BOUND_BIT)) continue;
+        R sw = 0, sp = 0;
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            if ((own[i] & OWNER_MASK) != OWN_FLUID) continue;
+            sw += wgt<R>(i);
+            sp += wgt<R>(i) * p[i];
+        }
+        ph[n] = sw > R(0) ? sp / sw : R(0);
     }
 }
 
@@ -451,8 +532,8 @@ __device__ __forceinline__ void collide_body(const Lattice &L, const InstDev &I,
     const long long g = I.node_off + n;
     const Pop<S> in(L.pop[cur], I);
     const Pop<S> out(L.pop[cur ^ 1], I);
-    // every load of an interior fluid node is issued before the flag is tested
-    const uint8_t fl = L.flags[g];
+    // every load is issued before the node's kind is tested
+    const uint8_t fl = BOUNCE_IN_SLOTS<S> ? 0 : L.flags[g];
     const GradRec<R> gr = ((const GradRec<R> *)L.grad)[g];
     const R phi = ((const R *)L.phi)[g];
     Nbr nb;
@@ -463,11 +544,11 @@ __device__ __forceinline__ void collide_body(const Lattice &L, const InstDev &I,
 #pragma unroll
     for (int i = 0; i < Q; i++) keep(F[i]);
     R *U = I.store_u ? (R *)L.u + I.node_off : nullptr;
-    if ((fl & OWNER_MASK) != OWN_FLUID) {
+    if (BOUNCE_IN_SLOTS<S> ? solid_mark(gr) : (fl & OWNER_MASK) != OWN_FLUID) {
         if (U) { U[n] = 0; U[L.Ntot + n] = 0; U[2 * L.Ntot + n] = 0; }
         return;
     }
-    // nodes next to a solid belong to the boundary pass k_collide_bound
+    // 16-bit storage: nodes next to a solid belong to the boundary pass
     if (fl & BOUND_BIT) return;
     FluidPar<R> P;
     load_par(I, P);
@@ -1084,6 +1165,7 @@ long long plan_rows(std::vector<InstDev> &inst)
         I.fd_plane.set(I.st_ygroups * I.st_nseg);
         I.fd_nseg.set(I.st_nseg);
         I.fd_nx.set(I.nx);
+        I.fd_ny.set(I.ny);
         I.st_item_start = total;
         total += (long long)I.nz * I.st_ygroups * I.st_nseg;
     }
@@ -1131,41 +1213,42 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     // pass writes, so beside the bulk kernel it follows that pass on the side lane
     bool fill_done = false;
     auto fill_solid_phi = [&](cudaStream_t s) {
-        if (L.n_static > 0) {
-            k_solidphi_list<R><<<(unsigned)((L.n_static + 255) / 256), 256, 0, s>>>(L);
-            *launches += 1;
-        }
-        if (L.n_parts > 0) {
-            k_solidphi_plist<R><<<(unsigned)std::max(L.bound_ctas / 2, 1), PART_THREADS, 0, s>>>(L);
-            *launches += 1;
-        }
         fill_done = true;
+        if (L.n_static == 0 && L.n_parts == 0) return;
+        const long long ctas = (L.n_static + PART_THREADS - 1) / PART_THREADS + (L.n_parts ? L.bound_ctas / 2 : 0);
+        k_solidphi<R><<<(unsigned)std::max(std::min(ctas, 8ll * L.bound_ctas), 1ll), PART_THREADS, 0, s>>>(L);
+        *launches += 1;
     };
     // boundary pass beside (side lane) or after the bulk kernel; profiling
     // (no side lane) times the two separately
-    auto bound_pass = [&](auto kernel, int bstage, int stage, auto &&bulk) {
+    auto bound_pass = [&](auto kernel, bool needed, int bstage, int stage, auto &&bulk) {
         if (lane.side) {
-            cudaEventRecord(lane.a, st);
-            cudaStreamWaitEvent(lane.side, lane.a, 0);
-            if (stage == STAGE_PHI) list_bound(lane.side);
-            kernel<<<bgrid, PART_THREADS, 0, lane.side>>>(L, cur);
-            if (stage == STAGE_PHI) fill_solid_phi(lane.side);
-            cudaEventRecord(lane.b, lane.side);
+            if (needed) {
+                cudaEventRecord(lane.a, st);
+                cudaStreamWaitEvent(lane.side, lane.a, 0);
+                if (stage == STAGE_PHI) list_bound(lane.side);
+                kernel<<<bgrid, PART_THREADS, 0, lane.side>>>(L, cur);
+                if (stage == STAGE_PHI) fill_solid_phi(lane.side);
+                cudaEventRecord(lane.b, lane.side);
+            }
             if (stage == STAGE_COLLIDE) lane.after_collide_bound();
             bulk();
-            cudaStreamWaitEvent(st, lane.b, 0);
+            if (needed) cudaStreamWaitEvent(st, lane.b, 0);
         } else {
             mk(stage, 0);
             bulk();
             mk(stage, 1);
-            mk(bstage, 0);
-            if (stage == STAGE_PHI) list_bound(st);
-            kernel<<<bgrid, PART_THREADS, 0, st>>>(L, cur);
-            mk(bstage, 1);
+            if (needed) {
+                mk(bstage, 0);
+                if (stage == STAGE_PHI) list_bound(st);
+                kernel<<<bgrid, PART_THREADS, 0, st>>>(L, cur);
+                mk(bstage, 1);
+            }
         }
-        *launches += 1;
+        if (needed) *launches += 1;
     };
-    bound_pass(k_phi_bound<S>, STAGE_PHI_BOUND, STAGE_PHI, [&] {
+    const bool any_bound = L.n_parts > 0 || L.n_static_bfl > 0;
+    bound_pass(k_phi_bound<S>, any_bound, STAGE_PHI_BOUND, STAGE_PHI, [&] {
         k_phi<S><<<(unsigned)fz.ph_items, PH_TX * PH_TY, 0, st>>>(L, cur);
     });
     if (!fill_done) {
@@ -1182,20 +1265,23 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
         launch_after(k_gradcurv<R, 8>, dim3((unsigned)fz.gc_items), dim3(GcShape<R, 8>::NT), st, L);
     mk(STAGE_GRAD, 1);
     after_grad();
-    bound_pass(k_collide_bound<S>, STAGE_COLLIDE_BOUND, STAGE_COLLIDE, [&] {
-        if constexpr (sizeof(S) == 2) {
-            if (pair) {
-                launch_after(k_collide2<S>, grid, dim3(ROW_NODES / 2), st, L, cur);
-                return;
-            }
-        }
+    if constexpr (BOUNCE_IN_SLOTS<S>) {
+        if (lane.side) lane.after_collide_bound();
+        mk(STAGE_COLLIDE, 0);
         launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
-    });
+        mk(STAGE_COLLIDE, 1);
+    } else {
+        bound_pass(k_collide_bound<S>, any_bound, STAGE_COLLIDE_BOUND, STAGE_COLLIDE, [&] {
+            if (pair) launch_after(k_collide2<S>, grid, dim3(ROW_NODES / 2), st, L, cur);
+            else launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
+        });
+    }
     *launches += 3;
 }
 
 
 #define INST(S)                                                                                                   \
+    template void launch_mark_solid<S>(const Lattice &, cudaStream_t);                                             \
     template void launch_fluid_step<S>(const Lattice &, int, cudaStream_t, long long *, const Marker &,            \
                                        const FluidLaunch &, const Hook &, const SideLane &);
 INST(double)

@@ -112,12 +112,13 @@ struct InstDev {
     float f_rho0, f_sigma, f_beta, f_eta_a, f_eta_b, f_eps2, f_wet_max;
     float f_body_a[3], f_body_b[3];
     float f_ir0, f_h_ia, f_h_ib;
+    float f_wall_u[3];
     // row-strip work items of the bulk kernels: st_rows whole x-rows of one z-plane per item
     // (st_nseg = 1, st_seg = nx), or one row cut into st_nseg segments of at
     // most st_seg nodes; st_ygroups items cover the y rows of a plane
     long long st_item_start;
     int st_rows, st_seg, st_nseg, st_ygroups;
-    FastDiv fd_plane, fd_nseg, fd_nx;  // st_ygroups st_nseg, st_nseg, nx
+    FastDiv fd_plane, fd_nseg, fd_nx, fd_ny;  // st_ygroups st_nseg, st_nseg, nx, ny
     // surrogate inputs: shell gap, velocity and radius scales
     double sh_gap, sh_uref, sh_rref, sh_box;
     // gradient + curvature work items: gc_tiles_x * gc_tiles_y column tiles x
@@ -175,11 +176,13 @@ struct Lattice {
     int n_inst;
     long long n_items;   // row-strip work items of all instances
     int buoyancy;        // some instance has a nonzero buoyancy_a: the immersed fractions are summed
-    const long long *static_list;  // static solid nodes next to non-static ones (global node index)
+    // boundary lists: entries of list_entry, the static ones in node order
+    const long long *static_list;  // static solid nodes next to non-static ones
     long long n_static;
     const long long *static_bfl;   // non-static nodes next to static solid ones
     long long n_static_bfl;
     uint8_t *flags;
+    int mark;            // bytes of a real where solid nodes' gradient records are marked, 0: 16-bit storage
     void *pop[2];
     void *phi;           // [Ntot] real: the order parameter of the step (outside a step: of the last one)
     void *col;           // [Ntot] ColRec<real>: colour record (phi, b n) of the stored state
@@ -192,7 +195,7 @@ struct Lattice {
     int geom_blocks;     // blocks per particle of the geometry kernels
     int geom_side;       // side of the cube the geometry kernels cover
     int cap_side;        // side of the cube of phi around a particle for the capillary force
-    long long *pbl;              // fluid nodes next to a solid inside the particle cubes (global index), this step
+    long long *pbl;              // fluid nodes next to a solid inside the particle cubes, this step
     unsigned long long *pbl_n;   // their number
     long long *psl;              // solid nodes next to fluid inside the particle cubes, this step
     unsigned long long *psl_n;   // their number
@@ -327,6 +330,13 @@ __device__ __forceinline__ float min_image_f(float d, int n)
     return d >= h ? d - n : (d < -h ? d + n : d);
 }
 
+template <class R>
+__device__ __forceinline__ R min_image_r(R d, int n)
+{
+    const R h = R(0.5) * n;
+    return d >= h ? d - n : (d < -h ? d + n : d);
+}
+
 // periodic neighbourhood of one node: x coordinates and row/plane offsets of
 // x-1..x+1, y-1..y+1, z-1..z+1 (instance-local 32-bit node indices; every
 // instance has fewer than 2^31/38 nodes)
@@ -349,31 +359,6 @@ __device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float frcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double frsqrt(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
-
-// velocity of the solid owning a node at the point xw (Sec. V A)
-template <class R>
-__device__ __forceinline__ void surface_velocity(const InstDev &I, const PartDev *parts, int owner, R xw, R yw, R zw,
-                                                 R *u)
-{
-    // in R: double in the FP64 mode, float (with the float particle centres)
-    // otherwise; the link midpoints are half-integers, exact in either
-    if (owner == OWN_WALL) {
-        u[0] = (R)I.wall_u[0]; u[1] = (R)I.wall_u[1]; u[2] = (R)I.wall_u[2];
-        return;
-    }
-    const PartDev &P = parts[I.part_off + owner - 2];
-    R d0, d1, d2;
-    if (sizeof(R) == 8) {
-        d0 = (R)min_image(xw - P.x[0], I.nx); d1 = (R)min_image(yw - P.x[1], I.ny); d2 = (R)min_image(zw - P.x[2], I.nz);
-    } else {
-        d0 = (R)min_image_f((float)xw - P.xf[0], I.nx); d1 = (R)min_image_f((float)yw - P.xf[1], I.ny);
-        d2 = (R)min_image_f((float)zw - P.xf[2], I.nz);
-    }
-    const R w0 = (R)P.w[0], w1 = (R)P.w[1], w2 = (R)P.w[2];
-    u[0] = (R)P.v[0] + (w1 * d2 - w2 * d1);
-    u[1] = (R)P.v[1] + (w2 * d0 - w0 * d2);
-    u[2] = (R)P.v[2] + (w0 * d1 - w1 * d0);
-}
 
 // cube of side `side` (clamped to the domain) centred on a particle's node
 struct Region {
@@ -408,15 +393,6 @@ struct Region {
     }
 };
 
-// neighbourhood of a node in global memory: node index and owner of the node
-// at offset (dx, dy, dz), periodic
-struct GlobalNbr {
-    Nbr nb;
-    const uint8_t *fli;  // flags of the instance
-    __device__ __forceinline__ int idx(int dx, int dy, int dz) const { return nb.at(dx, dy, dz); }
-    __device__ __forceinline__ int own(int dx, int dy, int dz) const { return fli[nb.at(dx, dy, dz)] & OWNER_MASK; }
-};
-
 // The colour record of a node of the stored state (see the top of this
 // file): the order parameter phi of the collision that produced it and
 // a = b n, one 16-byte (FP64: 32-byte) aligned record, so that a pulled source
@@ -441,6 +417,21 @@ struct alignas(4 * sizeof(R)) GradRec {
         g2 = g[2];
     }
 };
+
+// The curvature slot of a node that was solid in the step's gradient pass: a
+// NaN of its own (arithmetic makes the canonical one), so that the FP32 and
+// FP64 collision knows its nodes without their flags, which the owner update
+// beside it may be changing.  Written when the solid map is built or changed.
+__device__ __forceinline__ void set_solid_mark(GradRec<float> &r) { r.k = __int_as_float(0x7fc0dead); }
+__device__ __forceinline__ void set_solid_mark(GradRec<double> &r) { r.k = __longlong_as_double(0x7ff8dead00000000ll); }
+__device__ __forceinline__ bool solid_mark(const GradRec<float> &r) { return __float_as_int(r.k) == 0x7fc0dead; }
+__device__ __forceinline__ bool solid_mark(const GradRec<double> &r)
+{
+    return __double_as_longlong(r.k) == 0x7ff8dead00000000ll;
+}
+
+// entry of a boundary list: instance and instance-local node
+__device__ __forceinline__ long long list_entry(int inst, int n) { return (long long)inst << 32 | (unsigned)n; }
 
 // (c_i . a)/|c_i|: the colour offset G*_i of a record beyond phi (1 + F*_i)
 template <class R>
@@ -495,81 +486,125 @@ __device__ __forceinline__ ColSlotOf<S> col_slot(const Lattice &L, long long g)
     return ColSlotOf<S>{(ColRec<typename Store<S>::real> *)L.col + g};
 }
 
-// Pull streaming (Sec. IV) into fluid node n, with the Sec. V A halfway
-// bounce-back where the source node is solid:
+// Pull streaming (Sec. IV) into fluid node n next to a solid, with the Sec. V A
+// halfway bounce-back where the source node is solid:
 //   f_i(x) = f*_ibar(x) + 6 w_i rho^{a,b}(x) c_i.u_w,
 // rho^{a,b}(x) of the node's own pre-streaming state, u_w at the link midpoint.
-// Every flag and population load is issued before any is used (one dependent
-// round trip instead of one per link).  F receives the 19 total offsets.
 // A source on a pressure face (Sec. V D) gives the anti-bounce-back value
 //   f_i = -f*_ibar(x) + 2 w_i rho_w [1 + (c_i.u_w)^2/(2 cs^4) - u_w^2/(2 cs^2)],
 // rho_w the face's density (inlet below, outlet above), u_w = j*/rho* of the
-// node's own post-collision state; the colour split of rho_w follows that
-// state's phi, so the colour offset is phi(x)(1 + F_i) + (c_i . a(x))/|c_i|.
-// With C set, *sG receives sum_i w_i G_i of the streamed colour offsets:
-// G_i(x) = G*_i(x - c_i) from a fluid source; from a solid one
-// G*_ibar(x) + 6 (rho^a - rho^b)(x)/rho0 c_i.u_w, and since
-// (rho^a - rho^b)(x) = phi(x) rho(x) that is phi(x)(1 + F_i(x)) - (c_i . a(x))/|c_i|.
-template <class S, class A>
-__device__ __forceinline__ void gather_all(const InstDev &I, const PartDev *parts, const A &nbr,
-                                           const Pop<S> &in, const ColourOf<S> *C, int n,
-                                           typename Store<S>::real *F, typename Store<S>::real *sG, int x, int y,
-                                           int z)
+// node's own post-collision state.  own[i] and F[i] receive the owner of
+// direction i's source and the streamed total offset.
+// Every flag and population load is issued before any is used, and a
+// particle's state is read once per particle met (mostly one), not per link:
+// a chain of round trips per link is what these passes would wait on.
+template <class S>
+__device__ __forceinline__ void gather_links(const InstDev &I, const PartDev *parts, const uint8_t *fli, const Nbr &nb,
+                                             const Pop<S> &in, int n, int x, int y, int z, int (&own)[Q],
+                                             typename Store<S>::real (&F)[Q])
 {
     using R = typename Store<S>::real;
-    int own[Q];
-    R pF[Q], oF[Q];
+    R oF[Q];
 #pragma unroll
     for (int i = 0; i < Q; i++) {
-        const int s = nbr.idx(-cx(i), -cy(i), -cz(i));
-        own[i] = nbr.own(-cx(i), -cy(i), -cz(i));
-        pF[i] = in.F(i, s);
+        const int s = nb.at(-cx(i), -cy(i), -cz(i));
+        own[i] = fli[s];
+        F[i] = in.F(i, s);
         oF[i] = in.F(i, n);
     }
-    R sF = 0, jw[3] = {0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < Q; j++) {
-        sF += wgt<R>(j) * oF[j];
-        if (cx(j)) jw[0] += wgt<R>(j) * cx(j) * oF[j];
-        if (cy(j)) jw[1] += wgt<R>(j) * cy(j) * oF[j];
-        if (cz(j)) jw[2] += wgt<R>(j) * cz(j) * oF[j];
-    }
-    const R rr = R(1) + sF;
+    R sF = 0;
+    unsigned long long met = 0;
 #pragma unroll
     for (int i = 0; i < Q; i++) {
-        if (own[i] == OWN_FLUID) {
-            F[i] = pF[i];
-            continue;
+        sF += wgt<R>(i) * oF[i];
+        own[i] &= OWNER_MASK;
+        met |= 1ull << own[i];
+    }
+    const R rr = R(1) + sF;
+    if (met >> OWN_WALL & 1) {
+        R uw[3];
+        for (int a = 0; a < 3; a++) uw[a] = sizeof(R) == 8 ? (R)I.wall_u[a] : (R)I.f_wall_u[a];
+#pragma unroll
+        for (int i = 1; i < Q; i++)
+            if (own[i] == OWN_WALL)
+                F[i] = oF[opp(i)] + R(6) * rr * (cx(i) * uw[0] + cy(i) * uw[1] + cz(i) * uw[2]);
+    }
+    if (met >> OWN_PRESS & 1) {
+        R j[3] = {0, 0, 0};
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            if (cx(i)) j[0] += wgt<R>(i) * cx(i) * oF[i];
+            if (cy(i)) j[1] += wgt<R>(i) * cy(i) * oF[i];
+            if (cz(i)) j[2] += wgt<R>(i) * cz(i) * oF[i];
         }
-        if (own[i] == OWN_PRESS) {
-            const R irr = R(1) / rr;
-            const R u0 = jw[0] * irr, u1 = jw[1] * irr, u2 = jw[2] * irr;
+        const R irr = R(1) / rr;
+        const R u0 = j[0] * irr, u1 = j[1] * irr, u2 = j[2] * irr;
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            if (own[i] != OWN_PRESS) continue;
             const R cu = cx(i) * u0 + cy(i) * u1 + cz(i) * u2;
             const R rw = sizeof(R) == 8 ? (R)(cz(i) > 0 ? I.rin : I.rout) : (R)(cz(i) > 0 ? I.f_rin : I.f_rout);
             F[i] = R(-2) - oF[opp(i)] + R(2) * rw * (R(1) + R(4.5) * cu * cu - R(1.5) * (u0 * u0 + u1 * u1 + u2 * u2));
-            continue;
         }
-        R uw[3];
-        surface_velocity<R>(I, parts, own[i], x - R(0.5) * cx(i), y - R(0.5) * cy(i), z - R(0.5) * cz(i), uw);
-        const R cu = cx(i) * uw[0] + cy(i) * uw[1] + cz(i) * uw[2];
-        F[i] = oF[opp(i)] + R(6) * rr * cu;
     }
-    if (!C) return;
-    const ColRec<R> cn = C->at(n);
-    R g = 0;
+    met &= ~(1ull << OWN_FLUID | 1ull << OWN_WALL | 1ull << OWN_PRESS);
+    while (met) {
+        const int o = __ffsll((long long)met) - 1;
+        met &= met - 1;
+        const PartDev &P = parts[I.part_off + o - 2];
+        R c[3], v[3], w[3];
+        for (int a = 0; a < 3; a++) {
+            c[a] = sizeof(R) == 8 ? (R)P.x[a] : (R)P.xf[a];
+            v[a] = (R)P.v[a];
+            w[a] = (R)P.w[a];
+        }
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        R gi;
-        if (own[i] == OWN_FLUID) {
-            gi = C->G(i, nbr.idx(-cx(i), -cy(i), -cz(i)), F[i]);
-        } else if (own[i] == OWN_PRESS) {
-            gi = cn.p * (R(1) + F[i]) + col_rec(i, cn);
-        } else {
-            gi = cn.p * (R(1) + F[i]) - col_rec(i, cn);
+        for (int i = 1; i < Q; i++) {
+            if (own[i] != o) continue;
+            // u_w = v + w x (link midpoint - centre), in R: the midpoints are half-integers, exact in either
+            const R d0 = min_image_r<R>((x - R(0.5) * cx(i)) - c[0], I.nx), d1 = min_image_r<R>((y - R(0.5) * cy(i)) - c[1], I.ny),
+                    d2 = min_image_r<R>((z - R(0.5) * cz(i)) - c[2], I.nz);
+            const R u0 = v[0] + (w[1] * d2 - w[2] * d1), u1 = v[1] + (w[2] * d0 - w[0] * d2),
+                    u2 = v[2] + (w[0] * d1 - w[1] * d0);
+            F[i] = oF[opp(i)] + R(6) * rr * (cx(i) * u0 + cy(i) * u1 + cz(i) * u2);
         }
-        g += wgt<R>(i) * gi;
     }
-    *sG = g;
+}
+
+// sum_i w_i G_i of the streamed colour offsets of that node:
+// G_i(x) = G*_i(x - c_i) from a fluid source; from a solid one
+// G*_ibar(x) + 6 (rho^a - rho^b)(x)/rho0 c_i.u_w, and since
+// (rho^a - rho^b)(x) = phi(x) rho(x) that is phi(x)(1 + F_i(x)) - (c_i . a(x))/|c_i|;
+// from a pressure face, whose colour split follows the node's own state,
+// phi(x)(1 + F_i) + (c_i . a(x))/|c_i|.  The sources' records are read in three
+// batches, whatever their owner (a solid node's record is not used).
+template <class S>
+__device__ __forceinline__ typename Store<S>::real gather_colour(const Nbr &nb, const ColourOf<S> &C, int n,
+                                                                 const int (&own)[Q],
+                                                                 const typename Store<S>::real (&F)[Q])
+{
+    using R = typename Store<S>::real;
+    const ColRec<R> cn = C.at(n);
+    R g = wgt<R>(0) * (cn.p * (R(1) + F[0]));
+#pragma unroll
+    for (int b = 0; b < 3; b++) {
+        ColRec<R> r[6];
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            const int i = 1 + 6 * b + k;
+            r[k] = C.at(nb.at(-cx(i), -cy(i), -cz(i)));
+        }
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            const int i = 1 + 6 * b + k;
+            const bool fluid = own[i] == OWN_FLUID;
+            const ColRec<R> s = {fluid ? r[k].p : cn.p, fluid ? r[k].a0 : cn.a0, fluid ? r[k].a1 : cn.a1,
+                                 fluid ? r[k].a2 : cn.a2};
+            const R t = col_rec(i, s);
+            g += wgt<R>(i) * (s.p * (R(1) + F[i]) + (fluid || own[i] == OWN_PRESS ? t : -t));
+        }
+    }
+    return g;
 }
 
 // Sec. V E geometric wetting: rotate g so that -g/|g| makes the angle theta
@@ -819,10 +854,16 @@ template <class S>
 void launch_mass_sums(const Lattice &L, int cur, int inst, long long N, double *partial, int nblk, double *out,
                       cudaStream_t st);
 void launch_boundary_full(const Lattice &L, int inst, long long N, cudaStream_t st);
-// count (list == null) or fill a static boundary list: mode 0 static solid
-// nodes with a non-static neighbour, mode 1 non-static nodes with a static
-// solid neighbour
-void launch_static_bound(const Lattice &L, long long *list, unsigned long long *count, int mode, cudaStream_t st);
+// a static boundary list, in node order: mode 0 static solid nodes with a
+// non-static neighbour, mode 1 non-static nodes with a static solid
+// neighbour.  Count: blocks[b] entries of block b (static_bound_blocks of
+// them), then offs[b] entries before it, offs[nblocks] all; fill after that.
+long long static_bound_blocks(const Lattice &L);
+void launch_static_count(const Lattice &L, int *blocks, long long *offs, int mode, cudaStream_t st);
+void launch_static_fill(const Lattice &L, const long long *offs, long long *list, int mode, cudaStream_t st);
+// solid marks of every node's gradient record (FP32 and FP64 storage)
+template <class S>
+void launch_mark_solid(const Lattice &L, cudaStream_t st);
 void launch_mark_particles(const Lattice &L, cudaStream_t st);
 
 }  // namespace lbmg

@@ -1,7 +1,6 @@
 // Per-node device functions of the fluid update (Sec. IV, V E of arXiv
 // 2505.10171), shared by the kernels so that all run the same arithmetic:
-// solid-node phi, collision + recolouring + write,
-// colour record.
+// collision + recolouring + write, colour record.
 #pragma once
 
 #include <type_traits>
@@ -12,21 +11,6 @@ namespace lbmg {
 // ---------------------------------------------------------------------------
 // per-node device functions
 // ---------------------------------------------------------------------------
-
-// phi of a solid node: w-weighted mean over its fluid neighbours; phi_of(dx,
-// dy, dz) returns the order parameter of the neighbour
-template <class R, class A, class PhiF>
-__device__ __forceinline__ R solid_fill(const A &nbr, const PhiF &phi_of)
-{
-    R sw = 0, sp = 0;
-#pragma unroll
-    for (int i = 1; i < Q; i++) {
-        if (nbr.own(cx(i), cy(i), cz(i)) != OWN_FLUID) continue;
-        sw += wgt<R>(i);
-        sp += wgt<R>(i) * phi_of(cx(i), cy(i), cz(i));
-    }
-    return sw > R(0) ? sp / sw : R(0);
-}
 
 // the node's state before the per-direction updates of the collision
 template <class R>

@@ -48,13 +48,6 @@ __device__ __forceinline__ void block_sum6(T *v, double *out) { block_sum<6>(v, 
 __device__ __forceinline__ void centre(const PartDev &P, double *c) { c[0] = P.x[0]; c[1] = P.x[1]; c[2] = P.x[2]; }
 __device__ __forceinline__ void centre(const PartDev &P, float *c) { c[0] = P.xf[0]; c[1] = P.xf[1]; c[2] = P.xf[2]; }
 
-template <class R>
-__device__ __forceinline__ R min_image_r(R d, int n)
-{
-    const R h = R(0.5) * n;
-    return d >= h ? d - n : (d < -h ? d + n : d);
-}
-
 // Sec. V B momentum exchange (Wen 2014, Galilean invariant): per link from a
 // fluid node x into particle p, force on p = (c_out - u_w) f_out - (c_in - u_w) f_in
 // with f_out = f*_ibar(x) leaving towards the solid and f_in = f_i(x) bounced
@@ -600,6 +593,12 @@ __global__ void __launch_bounds__(PART_THREADS) k_geom_bound(Lattice L, int side
         int x, y, z;
         reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
         set_boundary(L, I, x, y, z);
+        // the solid mark of a covered node's gradient record (see set_solid_mark)
+        const long long g = I.node_off + ((long long)z * I.ny + y) * I.nx + x;
+        if ((L.flags[g] & OWNER_MASK) != OWN_FLUID) {
+            if (L.mark == 8) set_solid_mark(((GradRec<double> *)L.grad)[g]);
+            else if (L.mark == 4) set_solid_mark(((GradRec<float> *)L.grad)[g]);
+        }
     }
 }
 
