@@ -36,13 +36,16 @@ struct lbm_ctx {
     std::vector<PartDev> parts_h;
     PartDev *parts_d = nullptr;
     double *mem_part = nullptr, *cap_part = nullptr, *hist = nullptr;
-    long long *pbl = nullptr, *psl = nullptr;  // lists of particle-adjacent fluid / solid nodes
-    unsigned long long *pbl_n = nullptr, *psl_n = nullptr;
+    // per-step lists: particle-adjacent fluid / solid nodes, uncovered / covered
+    // nodes (one allocation), and their lengths
+    long long *lists = nullptr;
+    long long list_cap = 0;  // entries of each
+    unsigned long long *list_n = nullptr;
     int n_sm = 1;
-    double *cap_pts = nullptr;  // Lagrangian surface-point table
+    double *cap_pts = nullptr;  // Lagrangian surface-point table, then in single precision
     double *crec = nullptr;     // DEM contact records
     unsigned *status = nullptr;
-    int mem_blocks = 1, geom_blocks = 1, geom_side = 1, cap_side = 1, cap_blocks = 1;
+    int mem_blocks = 1, mem_side = 1, geom_blocks = 1, geom_side = 1;
     int cur = 0;
     long long steps = 0;
     bool stepped = false;
@@ -154,21 +157,25 @@ static Lattice make_lattice(const lbm_ctx *c)
     L.parts = c->parts_d;
     L.n_parts = (int)c->parts_h.size();
     L.mem_blocks = c->mem_blocks;
+    L.mem_side = c->mem_side;
     L.geom_blocks = c->geom_blocks;
     L.geom_side = c->geom_side;
-    L.cap_side = c->cap_side;
-    L.pbl = c->pbl;
-    L.pbl_n = c->pbl_n;
-    L.psl = c->psl;
-    L.psl_n = c->psl_n;
+    L.pbl = c->lists;
+    L.psl = c->lists + c->list_cap;
+    L.fresh = c->lists + 2 * c->list_cap;
+    L.covered = c->lists + 3 * c->list_cap;
+    L.list_n = c->list_n;
 #ifndef LBM_BOUND_CTAS_PER_SM
-#define LBM_BOUND_CTAS_PER_SM 2
+#define LBM_BOUND_CTAS_PER_SM 8
 #endif
     L.bound_ctas = LBM_BOUND_CTAS_PER_SM * c->n_sm;
-    L.cap_blocks = c->cap_blocks;
     L.mem_part = c->mem_part;
     L.cap_part = c->cap_part;
     L.cap_pts = c->cap_pts;
+    L.cap_pts_f = (const float *)(c->cap_pts + 4 * CAP_POINTS);
+    L.ring = c->ring;
+    L.ring_slots = c->ring_slots;
+    L.ring_ctr = c->ring ? c->ring_ctr : nullptr;
     L.hist = c->hist;
     L.crec = c->crec;
     L.status = c->status;
@@ -584,8 +591,6 @@ static void profile_mark(void *self, int stage, int after)
     else c->ev_pairs.push_back({stage, {c->ev_open[stage], e}});
 }
 
-static void enqueue_ring(const lbm_ctx *c, cudaStream_t st, long long *launches);
-
 // the device address of a caller buffer this context's device can write:
 // page-locked host memory (mapped under unified addressing), managed memory,
 // or device memory of this device; null otherwise (pageable host memory,
@@ -604,6 +609,16 @@ static void *device_addressable(const void *p)
     return nullptr;
 }
 
+// One step.  Main stream: order parameter, gradient, collision, refill.  Side
+// stream, beside them: the boundary passes; the contacts and the momentum
+// exchange (they need only the state before the step); once the gradients are
+// there the capillary force, the DEM and the new owners.  The FP32 and FP64
+// collision reads no flags, so the boundary bits and lists follow there too;
+// 16-bit storage's does (its boundary bits), so there they wait for it, as the
+// DEM waits for the collision's boundary pass, which reads the particles.  The
+// refill needs the collision's output.  With the surrogate the forces need the
+// collision's velocity, and all that follows stays in the main stream.
+// Profiling keeps one stream (per-kernel events).
 static void enqueue_step(lbm_ctx *c, long long *launches)
 {
     Lattice L = make_lattice(c);
@@ -616,74 +631,60 @@ static void enqueue_step(lbm_ctx *c, long long *launches)
     dispatch(c->prec, [&](auto *tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
         const bool sur = c->force_model == LBM_FORCE_SURROGATE;
-        // resolved forces beside the fluid kernels: the momentum exchange reads
-        // only the step's input populations (the fluid kernels write the other
-        // buffer), the capillary force only phi, n and |grad phi| once the
-        // gradient pass is done.  Profiling keeps one stream (per-kernel events).
-        const bool fork = !sur && !c->profile && L.n_parts > 0;
-        bool owner_done = false;  // owners updated on the side stream
+        const bool fork = !c->profile && (L.n_parts > 0 || L.n_static_bfl > 0);
+        constexpr bool early = sizeof(S) >= 4;  // boundary bits and lists beside the collision
+        struct Ctx2 {
+            lbm_ctx *c;
+            const Lattice *L;
+            long long *launches;
+            const Marker *mk;
+            int cur;
+            bool sur;
+        } h2 = {c, &L, launches, &mk, cur, sur};
+        SideLane lane;
         if (fork) {
-            cudaEventRecord(c->ev_fork, c->stream);
-            cudaStreamWaitEvent(c->side, c->ev_fork, 0);
-            launch_momentum_exchange<S>(L, cur, c->side, launches, mk);
-            struct Ctx2 {
-                lbm_ctx *c;
-                const Lattice *L;
-                long long *launches;
-                const Marker *mk;
-            } h2 = {c, &L, launches, &mk};
-            Hook hook;
-            hook.self = &h2;
-            hook.fn = [](void *p) {
-                Ctx2 *q = (Ctx2 *)p;
-                cudaEventRecord(q->c->ev_grad, q->c->stream);
-                cudaStreamWaitEvent(q->c->side, q->c->ev_grad, 0);
-                launch_capillary<S>(*q->L, q->c->side, q->launches, *q->mk);
-                cudaEventRecord(q->c->ev_join, q->c->side);
-            };
-            // the DEM needs the fluid forces of the step and must see the
-            // particle state the collision's boundary pass reads: it follows
-            // that pass on the side stream, beside the bulk collision
-            SideLane lane;
             lane.side = c->side;
             lane.a = c->ev_a;
             lane.b = c->ev_b;
-            lane.after_collide_bound.self = &h2;
+            lane.after_phi_bound.self = lane.after_grad.self = lane.after_collide_bound.self = &h2;
+            lane.after_phi_bound.fn = [](void *p) {
+                Ctx2 *q = (Ctx2 *)p;
+                launch_contacts<S>(*q->L, q->c->side, q->launches, *q->mk);
+                if (!q->sur) launch_momentum_exchange<S>(*q->L, q->cur, q->c->side, q->launches, *q->mk);
+            };
+            lane.after_grad.fn = [](void *p) {
+                Ctx2 *q = (Ctx2 *)p;
+                if (q->sur || q->L->n_parts == 0) return;
+                cudaEventRecord(q->c->ev_grad, q->c->stream);
+                cudaStreamWaitEvent(q->c->side, q->c->ev_grad, 0);
+                launch_capillary<S>(*q->L, q->c->side, q->launches, *q->mk);
+            };
             lane.after_collide_bound.fn = [](void *p) {
                 Ctx2 *q = (Ctx2 *)p;
-                launch_dem<S>(*q->L, q->c->side, q->launches, *q->mk, true);
-                enqueue_ring(q->c, q->c->side, q->launches);
-                // the new owners beside the bulk collision: the nodes whose
-                // owner changes are solid or next to a solid before and after,
-                // which the bulk collision skips either way; with a stored
-                // velocity it would zero that of newly covered nodes, so then
-                // the owners follow the collision
-                if (!q->c->u) launch_geom_owner(*q->L, q->c->side, q->launches, *q->mk);
+                if (!q->sur) {
+                    launch_dem<S>(*q->L, q->c->side, q->launches, *q->mk, true);
+                    // (16-bit storage: the collision would zero the stored
+                    // velocity of newly covered nodes, so then they follow it)
+                    if (early || !q->c->u) launch_geom_owner(*q->L, q->c->side, q->launches, *q->mk);
+                    if (early) launch_geom_surface(*q->L, q->c->side, q->launches, *q->mk);
+                }
                 cudaEventRecord(q->c->ev_join, q->c->side);
             };
-            owner_done = !c->u;
-            launch_fluid_step<S>(L, cur, c->stream, launches, mk, c->fz, hook, lane);
-            cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-        } else {
-            launch_fluid_step<S>(L, cur, c->stream, launches, mk, c->fz);
-            if (sur) launch_surrogate_forces<S>(L, c->mlp, c->feat, c->stream, launches, mk);
-            else launch_particle_forces<S>(L, cur, c->stream, launches, mk);
-            launch_dem<S>(L, c->stream, launches, mk, !sur);
-            enqueue_ring(c, c->stream, launches);
         }
-        // geometry: owners first; then boundary bits (side stream) beside the
-        // refill of uncovered nodes (they touch disjoint data)
-        if (!c->profile && L.n_parts > 0) {
-            if (!owner_done) launch_geom_owner(L, c->stream, launches, mk);
-            cudaEventRecord(c->ev_fork, c->stream);
-            cudaStreamWaitEvent(c->side, c->ev_fork, 0);
-            launch_geom_bound(L, c->side, launches, mk);
-            cudaEventRecord(c->ev_join, c->side);
-            launch_refill<S>(L, cur ^ 1, c->stream, launches, mk);
-            cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-        } else {
-            launch_geometry<S>(L, cur ^ 1, c->stream, launches, mk);
+        // without a side lane the contacts go first: nothing of the step moves a particle before the DEM
+        if (!fork) launch_contacts<S>(L, c->stream, launches, mk);
+        launch_fluid_step<S>(L, cur, c->stream, launches, mk, c->fz, lane);
+        if (fork) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+        if (sur) {
+            launch_surrogate_forces<S>(L, c->mlp, c->feat, c->stream, launches, mk);
+        } else if (!fork) {
+            launch_momentum_exchange<S>(L, cur, c->stream, launches, mk);
+            launch_capillary<S>(L, c->stream, launches, mk);
         }
+        if (sur || !fork) launch_dem<S>(L, c->stream, launches, mk, !sur);
+        if (sur || !fork || !(early || !c->u)) launch_geom_owner(L, c->stream, launches, mk);
+        if (sur || !fork || !early) launch_geom_surface(L, c->stream, launches, mk);
+        launch_refill<S>(L, cur ^ 1, c->stream, launches, mk);
     });
     c->cur ^= 1;
 }
@@ -769,6 +770,31 @@ static lbm_status validate(lbm_ctx *ctx, const lbm_params &p, int k)
     return LBM_OK;
 }
 
+// Sec. V F surface points alpha_j = (j + 1/2) 2 deg, varphi_k = k 2 deg: unit
+// normal and sin(alpha), in double precision, then in single; the same for
+// every context, evaluated once
+static const std::vector<double> &surface_points()
+{
+    static const std::vector<double> table = [] {
+        std::vector<double> t(6 * (size_t)CAP_POINTS);
+        float *f = reinterpret_cast<float *>(t.data() + 4 * (size_t)CAP_POINTS);
+        const double da = 2.0 * M_PI / 180.0;
+        for (int j = 0; j < 90; j++)
+            for (int k = 0; k < 180; k++) {
+                const double al = (j + 0.5) * da, vp = k * da;
+                const double v[4] = {std::sin(al) * std::cos(vp), std::sin(al) * std::sin(vp), std::cos(al),
+                                     std::sin(al)};
+                for (int a = 0; a < 4; a++) {
+                    const size_t i = 4 * (size_t)(j * 180 + k) + a;
+                    t[i] = v[a];
+                    f[i] = (float)v[a];
+                }
+            }
+        return t;
+    }();
+    return table;
+}
+
 static const char *status_text(unsigned s)
 {
     if (s & ST_UNSTABLE) return "device: non-finite or non-positive density (unstable run)";
@@ -798,46 +824,11 @@ static void drop_graph(lbm_ctx *c)
 }
 
 // the records of lbm_particle_forces, packed on the device (one thread per
-// particle of the instance)
-__device__ __forceinline__ void pack_record(const PartDev &q, double *o)
-{
-    for (int a = 0; a < 3; a++) {
-        o[a] = q.Feta[a]; o[3 + a] = q.Teta[a];
-        o[6 + a] = q.Fsig[a]; o[9 + a] = q.Tsig[a];
-        o[12 + a] = q.Fc[a]; o[15 + a] = q.Tc[a];
-        o[18 + a] = q.x[a]; o[21 + a] = q.v[a]; o[24 + a] = q.w[a];
-    }
-    for (int a = 0; a < 4; a++) o[27 + a] = q.q[a];
-    o[31] = q.m;
-    o[32] = q.sub;
-    for (int a = 0; a < 3; a++) o[33 + a] = q.Fb[a];
-}
-
+// entry)
 __global__ void k_pack_records(const PartDev *parts, int np, double *out)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    pack_record(parts[p], out + (size_t)LBM_PARTICLE_RECORD * p);
-}
-
-// the records of every particle of the context into slot (*ctr mod slots) of
-// the record ring, then *ctr + 1 (one CTA)
-__global__ void k_pack_ring(const PartDev *parts, int np, double *ring, int slots, long long *ctr)
-{
-    const long long k = *ctr;
-    double *slot = ring + (size_t)(k % slots) * LBM_PARTICLE_RECORD * np;
-    for (int p = threadIdx.x; p < np; p += blockDim.x) pack_record(parts[p], slot + (size_t)LBM_PARTICLE_RECORD * p);
-    __syncthreads();
-    if (threadIdx.x == 0) *ctr = k + 1;
-}
-
-// the step's particle records into the record ring, if one is set; the
-// particle state is final once the DEM has run
-static void enqueue_ring(const lbm_ctx *c, cudaStream_t st, long long *launches)
-{
-    if (!c->ring || c->parts_h.empty()) return;
-    k_pack_ring<<<1, 64, 0, st>>>(c->parts_d, (int)c->parts_h.size(), c->ring, c->ring_slots, c->ring_ctr);
-    *launches += 1;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < np * RECORD) out[k] = record_entry(parts[k / RECORD], k % RECORD);
 }
 
 // ---------------------------------------------------------------------------
@@ -865,10 +856,8 @@ void lbm_destroy(lbm_ctx *ctx)
     cudaFree(ctx->speed_d);
     cudaFree(ctx->rec_d);
     cudaFree(ctx->ring_ctr);
-    cudaFree(ctx->pbl);
-    cudaFree(ctx->pbl_n);
-    cudaFree(ctx->psl);
-    cudaFree(ctx->psl_n);
+    cudaFree(ctx->lists);
+    cudaFree(ctx->list_n);
     cudaFree(ctx->speed_part);
     mlp_free(ctx->mlp);
     cudaFree(ctx->feat);
@@ -989,6 +978,7 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
         I.f_eps2 = (float)(I.grad_eps * I.grad_eps); I.f_wet_max = (float)I.wet_max;
         for (int a = 0; a < 3; a++) { I.f_body_a[a] = (float)I.body_a[a]; I.f_body_b[a] = (float)I.body_b[a]; }
         for (int a = 0; a < 3; a++) I.f_wall_u[a] = (float)I.wall_u[a];
+        I.f_cap = (float)(I.cap_norm * I.sigma);
         I.f_ir0 = (float)(1.0 / I.rho0);
         I.f_h_ia = (float)(0.5 / I.eta_a);
         I.f_h_ib = (float)(0.5 / I.eta_b);
@@ -1053,20 +1043,8 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
         lbm_destroy(ctx);
         return st;
     }
-    // Sec. V F surface points alpha_j = (j + 1/2) 2 deg, varphi_k = k 2 deg:
-    // unit normal and sin(alpha), evaluated once on the host
     {
-        std::vector<double> tab(4 * (size_t)CAP_POINTS);
-        const double da = 2.0 * M_PI / 180.0;
-        for (int j = 0; j < 90; j++)
-            for (int k = 0; k < 180; k++) {
-                const double al = (j + 0.5) * da, vp = k * da;
-                double *t = &tab[4 * (size_t)(j * 180 + k)];
-                t[0] = std::sin(al) * std::cos(vp);
-                t[1] = std::sin(al) * std::sin(vp);
-                t[2] = std::cos(al);
-                t[3] = std::sin(al);
-            }
+        const std::vector<double> &tab = surface_points();
         if ((st = alloc((void **)&ctx->cap_pts, sizeof(double) * tab.size()))) {
             lbm_destroy(ctx);
             return st;
@@ -1241,6 +1219,7 @@ lbm_status lbm_add_particles(lbm_ctx *ctx, int inst, int n, const lbm_particle *
         }
         d.q[0] = 1.0;
         d.R = q.R_p;
+        d.Rf = (float)q.R_p;
         d.Rc = q.R_p + p.delta_R;
         d.m = q.rho_p * 4.0 / 3.0 * M_PI * q.R_p * q.R_p * q.R_p;
         d.I = 0.4 * d.m * q.R_p * q.R_p;
@@ -1301,23 +1280,27 @@ lbm_status lbm_add_particles(lbm_ctx *ctx, int inst, int n, const lbm_particle *
     double Rmax = 0.0;
     for (auto &q : all) Rmax = std::max(Rmax, q.R);
     int mem_side = 2 * (int)std::ceil(Rmax) + 5;
-    for (auto &q : all) q.mem_side = mem_side;
+    ctx->mem_side = mem_side;
     ctx->parts_h = all;
-    ctx->mem_blocks = (int)(((long long)mem_side * mem_side * mem_side + PART_THREADS - 1) / PART_THREADS);
+    ctx->mem_blocks = (int)(((long long)mem_side * mem_side * mem_side + MEM_THREADS - 1) / MEM_THREADS);
     ctx->geom_side = 2 * (int)std::ceil(Rmax) + 4 * GEOM_MARGIN + 3;
-    ctx->cap_side = 2 * (int)std::ceil(Rmax) + 11;
-    ctx->cap_blocks = (int)(((long long)ctx->cap_side * ctx->cap_side * ctx->cap_side + PART_THREADS - 1) / PART_THREADS);
     long long gs3 = (long long)(ctx->geom_side + 2) * (ctx->geom_side + 2) * (ctx->geom_side + 2);
-    ctx->geom_blocks = (int)std::min<long long>((gs3 + PART_THREADS - 1) / PART_THREADS, 256);
+    // CTAs per particle of the geometry kernels: a node per thread until the GPU
+    // is full (8 CTAs per SM), then up to 16, since a CTA's start (particle and
+    // instance records, two round trips) costs more than its nodes
+    {
+        const long long per_node = (gs3 + PART_THREADS - 1) / PART_THREADS;
+        const long long fill = 8ll * ctx->n_sm / std::max<long long>((long long)all.size(), 1);
+        ctx->geom_blocks = (int)std::max<long long>(1, std::min(per_node, std::max(fill, (per_node + 15) / 16)));
+    }
     const size_t np = all.size();
     CU(cudaStreamSynchronize(ctx->stream));
     cudaFree(ctx->parts_d);
     cudaFree(ctx->rec_d);
     ctx->rec_d = nullptr;
     ctx->ring = nullptr;  // a ring slot holds every particle: set it again
-    cudaFree(ctx->pbl);
-    cudaFree(ctx->psl);
-    ctx->pbl = ctx->psl = nullptr;
+    cudaFree(ctx->lists);
+    ctx->lists = nullptr;
     cudaFree(ctx->mem_part);
     cudaFree(ctx->cap_part);
     cudaFree(ctx->hist);
@@ -1325,11 +1308,11 @@ lbm_status lbm_add_particles(lbm_ctx *ctx, int inst, int n, const lbm_particle *
     ctx->parts_d = nullptr;
     ctx->mem_part = ctx->cap_part = ctx->hist = ctx->crec = nullptr;
     CU(cudaMalloc((void **)&ctx->parts_d, sizeof(PartDev) * np));
-    // every node of every particle's cube can be listed once per cube
-    CU(cudaMalloc((void **)&ctx->pbl, sizeof(long long) * np * (size_t)ctx->cap_blocks * PART_THREADS));
-    CU(cudaMalloc((void **)&ctx->psl, sizeof(long long) * np * (size_t)ctx->cap_blocks * PART_THREADS));
-    if (!ctx->pbl_n) CU(cudaMalloc((void **)&ctx->pbl_n, sizeof(unsigned long long)));
-    if (!ctx->psl_n) CU(cudaMalloc((void **)&ctx->psl_n, sizeof(unsigned long long)));
+    // the nodes of a particle and within one link of it lie in a cube of this side
+    const long long ls = 2 * (long long)std::ceil(Rmax) + 5;
+    ctx->list_cap = (long long)np * ls * ls * ls;
+    CU(cudaMalloc((void **)&ctx->lists, sizeof(long long) * 4 * (size_t)ctx->list_cap));
+    if (!ctx->list_n) CU(cudaMalloc((void **)&ctx->list_n, sizeof(unsigned long long) * 4));
     CU(cudaMalloc((void **)&ctx->mem_part, sizeof(double) * MEM_PART * np * ctx->mem_blocks));
     CU(cudaMalloc((void **)&ctx->cap_part, sizeof(double) * CAP_PART * np * CAP_BLOCKS));
     CU(cudaMalloc((void **)&ctx->hist, sizeof(double) * 6 * std::max(hist, 1)));
@@ -1375,6 +1358,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
         }
         if (e == cudaSuccess && L.mark)
             dispatch(ctx->prec, [&](auto *tag) { launch_mark_solid<std::remove_pointer_t<decltype(tag)>>(L, ctx->stream); });
+        if (e == cudaSuccess) launch_first_lists(L, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // before offs goes
         cudaFree(offs);
         CU(e);
@@ -1562,12 +1546,12 @@ lbm_status lbm_particle_forces_async(lbm_ctx *ctx, int inst, double *out)
     // addressing maps, or device / managed memory) is written by the packing
     // kernel itself: no separate copy in the stream
     if (void *d = device_addressable(out)) {
-        k_pack_records<<<(I.np + 63) / 64, 64, 0, ctx->stream>>>(ctx->parts_d + I.part_off, I.np, (double *)d);
+        k_pack_records<<<(I.np * RECORD + 127) / 128, 128, 0, ctx->stream>>>(ctx->parts_d + I.part_off, I.np, (double *)d);
         CU(cudaGetLastError());
         return LBM_OK;
     }
     double *dst = ctx->rec_d + (size_t)LBM_PARTICLE_RECORD * I.part_off;
-    k_pack_records<<<(I.np + 63) / 64, 64, 0, ctx->stream>>>(ctx->parts_d + I.part_off, I.np, dst);
+    k_pack_records<<<(I.np * RECORD + 127) / 128, 128, 0, ctx->stream>>>(ctx->parts_d + I.part_off, I.np, dst);
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(out, dst, sizeof(double) * LBM_PARTICLE_RECORD * I.np, cudaMemcpyDeviceToHost,
                        ctx->stream));

@@ -25,7 +25,10 @@
 
 #include "lbm_node.cuh"
 
-// CTAs per SM of the boundary passes, which run beside the bulk kernels
+// Boundary passes, which run beside the bulk kernels: CTAs of 64 threads, so
+// that a short list reaches many SMs (FP64: as many FP64 pipes), 4 times this
+// many per SM
+constexpr int BOUND_THREADS = 64;
 #ifndef LBM_BOUND_MINB
 #define LBM_BOUND_MINB 2
 #endif
@@ -350,46 +353,6 @@ void launch_mark_solid(const Lattice &L, cudaStream_t st)
     k_mark_solid<typename Store<S>::real><<<(unsigned)((L.Ntot + 255) / 256), 256, 0, st>>>(L);
 }
 
-// the fluid nodes next to a solid inside the particle cubes (cubes of side
-// cap_side around each particle, cap_blocks CTAs each), appended to L.pbl
-// with one atomic per warp: the particle part of the boundary passes' work
-// list, rebuilt at the start of every step (the flags do not change within
-// a step); likewise the solid nodes next to fluid, for the solid-phi fill,
-// to L.psl.  Order within a list does not matter; a node in two cubes is
-// listed twice and written twice with the same value.
-__global__ void __launch_bounds__(PART_THREADS) k_bound_list(Lattice L)
-{
-    const long long b = blockIdx.x;
-    const long long t = (b % L.cap_blocks) * blockDim.x + threadIdx.x;
-    const PartDev &P0 = L.parts[b / L.cap_blocks];
-    const InstDev &I = L.inst[P0.inst];
-    Region reg;
-    reg.init(P0.x, L.cap_side, I.nx, I.ny, I.nz);
-    bool fluid = false, solid = false;
-    long long g = 0;
-    if (t < reg.count()) {
-        int x, y, z;
-        reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
-        const int n = (z * I.ny + y) * I.nx + x;
-        g = list_entry(P0.inst, n);
-        const uint8_t fl = L.flags[I.node_off + n];
-        fluid = (fl & OWNER_MASK) == OWN_FLUID && (fl & BOUND_BIT);
-        solid = (fl & OWNER_MASK) != OWN_FLUID && (fl & BOUND_BIT);
-    }
-    const int lane = threadIdx.x & 31;
-    auto append = [&](bool take, long long *list, unsigned long long *count) {
-        const unsigned m = __ballot_sync(0xffffffffu, take);
-        if (!m) return;
-        const int leader = __ffs(m) - 1;
-        unsigned long long base = 0;
-        if (lane == leader) base = atomicAdd(count, (unsigned long long)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (take) list[base + __popc(m & ((1u << lane) - 1u))] = g;
-    };
-    append(fluid, L.pbl, L.pbl_n);
-    append(solid, L.psl, L.psl_n);
-}
-
 // node of a list entry
 __device__ __forceinline__ const InstDev &list_node(const Lattice &L, long long e, int *n, int *x, int *y, int *z)
 {
@@ -445,9 +408,9 @@ __device__ __forceinline__ void phi_bound_node(const Lattice &L, int cur, long l
 }
 
 template <class S>
-__global__ void __launch_bounds__(PART_THREADS, sizeof(S) == 8 ? 1 : LBM_BOUND_MINB) k_phi_bound(Lattice L, int cur)
+__global__ void __launch_bounds__(BOUND_THREADS, sizeof(S) == 8 ? 4 : 4 * LBM_BOUND_MINB) k_phi_bound(Lattice L, int cur)
 {
-    const long long npb = L.pbl_n ? (long long)*L.pbl_n : 0;
+    const long long npb = L.n_parts ? (long long)L.list_n[LIST_FLUID] : 0;
     const long long total = npb + L.n_static_bfl;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
          t += (long long)gridDim.x * blockDim.x)
@@ -480,9 +443,9 @@ __device__ __forceinline__ void collide_bound_node(const Lattice &L, int cur, lo
 }
 
 template <class S>
-__global__ void __launch_bounds__(PART_THREADS, LBM_BOUND_MINB) k_collide_bound(Lattice L, int cur)
+__global__ void __launch_bounds__(BOUND_THREADS, 4 * LBM_BOUND_MINB) k_collide_bound(Lattice L, int cur)
 {
-    const long long npb = L.pbl_n ? (long long)*L.pbl_n : 0;
+    const long long npb = L.n_parts ? (long long)L.list_n[LIST_FLUID] : 0;
     const long long total = npb + L.n_static_bfl;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
          t += (long long)gridDim.x * blockDim.x)
@@ -495,7 +458,7 @@ __global__ void __launch_bounds__(PART_THREADS, LBM_BOUND_MINB) k_collide_bound(
 template <class R>
 __global__ void __launch_bounds__(PART_THREADS) k_solidphi(Lattice L)
 {
-    const long long nps = L.psl_n ? (long long)*L.psl_n : 0;
+    const long long nps = L.n_parts ? (long long)L.list_n[LIST_SOLID] : 0;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < nps + L.n_static;
          t += (long long)gridDim.x * blockDim.x) {
         int n, x, y, z;
@@ -1192,7 +1155,7 @@ static void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream
 
 template <class S>
 void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk,
-                       const FluidLaunch &fz, const Hook &after_grad, const SideLane &lane)
+                       const FluidLaunch &fz, const SideLane &lane)
 {
     using R = typename Store<S>::real;
     const dim3 grid((unsigned)fz.rows);  // one CTA per row-strip work item
@@ -1200,62 +1163,40 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     // boundary passes: grid-stride over the listed particle nodes and the
     // static list of nodes next to walls
     const dim3 bgrid((unsigned)std::max(L.bound_ctas, 1));
-    auto list_bound = [&](cudaStream_t s) {
-        if (L.n_parts == 0) return;
-        cudaMemsetAsync(L.pbl_n, 0, sizeof(unsigned long long), s);
-        cudaMemsetAsync(L.psl_n, 0, sizeof(unsigned long long), s);
-        k_bound_list<<<(unsigned)((long long)L.n_parts * L.cap_blocks), PART_THREADS, 0, s>>>(L);
-        *launches += 1;
-    };
-    // phi of solid nodes next to fluid: the listed static nodes and the
-    // particle-surface solid nodes the step's list scan found in the cubes.
-    // It reads phi only at fluid nodes next to a solid, which the boundary
-    // pass writes, so beside the bulk kernel it follows that pass on the side lane
-    bool fill_done = false;
-    auto fill_solid_phi = [&](cudaStream_t s) {
-        fill_done = true;
-        if (L.n_static == 0 && L.n_parts == 0) return;
-        const long long ctas = (L.n_static + PART_THREADS - 1) / PART_THREADS + (L.n_parts ? L.bound_ctas / 2 : 0);
-        k_solidphi<R><<<(unsigned)std::max(std::min(ctas, 8ll * L.bound_ctas), 1ll), PART_THREADS, 0, s>>>(L);
-        *launches += 1;
-    };
-    // boundary pass beside (side lane) or after the bulk kernel; profiling
-    // (no side lane) times the two separately
-    auto bound_pass = [&](auto kernel, bool needed, int bstage, int stage, auto &&bulk) {
-        if (lane.side) {
-            if (needed) {
-                cudaEventRecord(lane.a, st);
-                cudaStreamWaitEvent(lane.side, lane.a, 0);
-                if (stage == STAGE_PHI) list_bound(lane.side);
-                kernel<<<bgrid, PART_THREADS, 0, lane.side>>>(L, cur);
-                if (stage == STAGE_PHI) fill_solid_phi(lane.side);
-                cudaEventRecord(lane.b, lane.side);
-            }
-            if (stage == STAGE_COLLIDE) lane.after_collide_bound();
-            bulk();
-            if (needed) cudaStreamWaitEvent(st, lane.b, 0);
-        } else {
-            mk(stage, 0);
-            bulk();
-            mk(stage, 1);
-            if (needed) {
-                mk(bstage, 0);
-                if (stage == STAGE_PHI) list_bound(st);
-                kernel<<<bgrid, PART_THREADS, 0, st>>>(L, cur);
-                mk(bstage, 1);
-            }
-        }
-        if (needed) *launches += 1;
-    };
     const bool any_bound = L.n_parts > 0 || L.n_static_bfl > 0;
-    bound_pass(k_phi_bound<S>, any_bound, STAGE_PHI_BOUND, STAGE_PHI, [&] {
-        k_phi<S><<<(unsigned)fz.ph_items, PH_TX * PH_TY, 0, st>>>(L, cur);
-    });
-    if (!fill_done) {
+    // phi of solid nodes next to fluid reads phi only at fluid nodes next to a
+    // solid, which the boundary pass writes, so it follows that pass beside the
+    // bulk kernel
+    auto fill_solid_phi = [&](cudaStream_t s) {
+        if (L.n_static == 0 && L.n_parts == 0) return;
+        const long long ctas = (L.n_static + PART_THREADS - 1) / PART_THREADS + (L.n_parts ? L.bound_ctas / 8 : 0);
         mk(STAGE_SOLIDPHI, 0);
-        fill_solid_phi(st);
+        k_solidphi<R><<<(unsigned)std::max(std::min(ctas, 8ll * L.bound_ctas), 1ll), PART_THREADS, 0, s>>>(L);
         mk(STAGE_SOLIDPHI, 1);
-    }
+        *launches += 1;
+    };
+    // a boundary pass beside the bulk kernels (side lane), from here in the
+    // main stream on; profiling (no side lane) times it alone
+    auto bound_pass = [&](auto kernel, int stage) {
+        if (!any_bound) return;
+        cudaStream_t s = lane.side ? lane.side : st;
+        if (lane.side) {
+            cudaEventRecord(lane.a, st);
+            cudaStreamWaitEvent(lane.side, lane.a, 0);
+        }
+        mk(stage, 0);
+        kernel<<<bgrid, BOUND_THREADS, 0, s>>>(L, cur);
+        mk(stage, 1);
+        *launches += 1;
+    };
+    bound_pass(k_phi_bound<S>, STAGE_PHI_BOUND);
+    fill_solid_phi(lane.side && any_bound ? lane.side : st);
+    if (lane.side && any_bound) cudaEventRecord(lane.b, lane.side);
+    lane.after_phi_bound();
+    mk(STAGE_PHI, 0);
+    k_phi<S><<<(unsigned)fz.ph_items, PH_TX * PH_TY, 0, st>>>(L, cur);
+    mk(STAGE_PHI, 1);
+    if (lane.side && any_bound) cudaStreamWaitEvent(st, lane.b, 0);
     mk(STAGE_GRAD, 0);
     if constexpr (sizeof(R) == 8) {
         if (fz.gc_rows == 4)
@@ -1264,17 +1205,21 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     if (fz.gc_rows == 8)
         launch_after(k_gradcurv<R, 8>, dim3((unsigned)fz.gc_items), dim3(GcShape<R, 8>::NT), st, L);
     mk(STAGE_GRAD, 1);
-    after_grad();
+    lane.after_grad();
     if constexpr (BOUNCE_IN_SLOTS<S>) {
-        if (lane.side) lane.after_collide_bound();
+        lane.after_collide_bound();
         mk(STAGE_COLLIDE, 0);
         launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
         mk(STAGE_COLLIDE, 1);
     } else {
-        bound_pass(k_collide_bound<S>, any_bound, STAGE_COLLIDE_BOUND, STAGE_COLLIDE, [&] {
-            if (pair) launch_after(k_collide2<S>, grid, dim3(ROW_NODES / 2), st, L, cur);
-            else launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
-        });
+        bound_pass(k_collide_bound<S>, STAGE_COLLIDE_BOUND);
+        if (lane.side && any_bound) cudaEventRecord(lane.b, lane.side);
+        lane.after_collide_bound();
+        mk(STAGE_COLLIDE, 0);
+        if (pair) launch_after(k_collide2<S>, grid, dim3(ROW_NODES / 2), st, L, cur);
+        else launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
+        mk(STAGE_COLLIDE, 1);
+        if (lane.side && any_bound) cudaStreamWaitEvent(st, lane.b, 0);
     }
     *launches += 3;
 }
@@ -1283,7 +1228,7 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
 #define INST(S)                                                                                                   \
     template void launch_mark_solid<S>(const Lattice &, cudaStream_t);                                             \
     template void launch_fluid_step<S>(const Lattice &, int, cudaStream_t, long long *, const Marker &,            \
-                                       const FluidLaunch &, const Hook &, const SideLane &);
+                                       const FluidLaunch &, const SideLane &);
 INST(double)
 INST(float)
 INST(__half)

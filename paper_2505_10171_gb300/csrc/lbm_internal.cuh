@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <vector>
@@ -64,6 +65,12 @@ constexpr int CAP_THREADS = 256;
 constexpr int CAP_BLOCKS = (CAP_POINTS + CAP_THREADS - 1) / CAP_THREADS;
 constexpr int CAP_PART = 8;  // per block: F_sig, T_sig, sum s dA, sum dA
 constexpr int PART_THREADS = 256;
+// the momentum exchange in small CTAs: its links are arithmetic-heavy (FP64
+// storage: FP64-bound) and few, so they are spread over the SMs
+constexpr int MEM_THREADS = 64;
+constexpr int RECORD = 36;  // doubles of a particle record (LBM_PARTICLE_RECORD)
+// lists rebuilt each step and their counters
+enum ListId { LIST_FLUID = 0, LIST_SOLID, LIST_FRESH, LIST_COVERED };
 // doubles per block partial of the momentum exchange: force and torque of the
 // small part, then the integer sums K and 2M of the rest part
 constexpr int MEM_PART = 12;
@@ -113,6 +120,7 @@ struct InstDev {
     float f_body_a[3], f_body_b[3];
     float f_ir0, f_h_ia, f_h_ib;
     float f_wall_u[3];
+    float f_cap;  // cap_norm sigma
     // row-strip work items of the bulk kernels: st_rows whole x-rows of one z-plane per item
     // (st_nseg = 1, st_seg = nx), or one row cut into st_nseg segments of at
     // most st_seg nodes; st_ygroups items cover the y rows of a plane
@@ -166,9 +174,11 @@ struct PartDev {
     double Fp[3], Tp[3];
     double Feta[3], Teta[3], Fsig[3], Tsig[3], Fc[3], Tc[3];
     double sub, Fb[3];    // immersed volume fraction in phase a, buoyancy
+    double xn[3];         // predicted position of the step
     float xf[3], xfo[3];  // single-precision copies of x and x_old
     float R2lo, R2hi;     // |x - x_p|^2 below / above these is inside / outside for sure
-    int kin, inst, local, mem_side;
+    float Rf;             // R in single precision
+    int kin, inst, local;
 };
 
 struct Lattice {
@@ -192,18 +202,25 @@ struct Lattice {
     PartDev *parts;
     int n_parts;
     int mem_blocks;      // blocks per particle of the momentum-exchange kernel
+    int mem_side;        // side of the cube it covers
     int geom_blocks;     // blocks per particle of the geometry kernels
     int geom_side;       // side of the cube the geometry kernels cover
-    int cap_side;        // side of the cube of phi around a particle for the capillary force
-    long long *pbl;              // fluid nodes next to a solid inside the particle cubes, this step
-    unsigned long long *pbl_n;   // their number
-    long long *psl;              // solid nodes next to fluid inside the particle cubes, this step
-    unsigned long long *psl_n;   // their number
+    // lists of list_entry that the geometry kernels of the step before (for the
+    // first step launch_first_lists) have filled, and their lengths by ListId: fluid
+    // nodes next to a particle, particle nodes next to fluid, uncovered and
+    // covered nodes
+    long long *pbl, *psl, *fresh, *covered;
+    unsigned long long *list_n;
     int bound_ctas;              // CTAs of the grid-stride boundary passes
-    int cap_blocks;      // blocks per particle covering that cube
     double *mem_part;    // [n_parts][mem_blocks][MEM_PART]
     double *cap_part;    // [n_parts][CAP_BLOCKS][CAP_PART]
     const double *cap_pts;  // [CAP_POINTS][4]: unit normal (3) and sin(alpha) of each surface point
+    const float *cap_pts_f; // the same in single precision
+    // record ring (null: none): every step's records go to slot (*ring_ctr - 1) mod
+    // ring_slots, ring_ctr counting the steps begun
+    double *ring;
+    int ring_slots;
+    long long *ring_ctr;
     double *hist;        // contact springs: per instance np*(np+1) records of 6
     double *crec;        // DEM contact forces: per instance np + np(np-1)/2 records of 12
     unsigned *status;
@@ -363,25 +380,30 @@ __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
 // cube of side `side` (clamped to the domain) centred on a particle's node
 struct Region {
     int lo[3], sz[3];
-    __device__ __forceinline__ void init(const double *xc, int side, int nx, int ny, int nz)
+    // (from the single-precision centre, which may round up to the next node: the
+    // sides leave room for that, and FP64 here would bind the kernels that run
+    // one thread per node of the cube)
+    __device__ __forceinline__ void init(const float *xc, int side, int nx, int ny, int nz)
     {
         const int n[3] = {nx, ny, nz};
         for (int a = 0; a < 3; a++) {
             int s = side < n[a] ? side : n[a];
             sz[a] = s;
-            int lo_ = (int)floor(xc[a]) - (s - 1) / 2;
+            int lo_ = (int)floorf(xc[a]) - (s - 1) / 2;
             lo[a] = s == n[a] ? 0 : lo_;
         }
     }
     __device__ __forceinline__ long long count() const { return (long long)sz[0] * sz[1] * sz[2]; }
     // node t of the cube (t < count < 2^31); lo + i lies in (-n, 2n), so one
     // conditional wrap per axis suffices
-    __device__ __forceinline__ void coord(long long t, int nx, int ny, int nz, int *x, int *y, int *z) const
+    // (fd divides by the side asked for, the size of every axis that it fits)
+    __device__ __forceinline__ void coord(long long t, const FastDiv &fd, int nx, int ny, int nz, int *x, int *y,
+                                          int *z) const
     {
         const int tt = (int)t;
-        const int ij = tt / sz[0];
+        const int ij = sz[0] == (int)fd.d ? fd.div(tt) : tt / sz[0];
         const int i = tt - ij * sz[0];
-        const int k = ij / sz[1];
+        const int k = sz[1] == (int)fd.d ? fd.div(ij) : ij / sz[1];
         const int j = ij - k * sz[1];
         int a = lo[0] + i, b = lo[1] + j, c = lo[2] + k;
         a += a < 0 ? nx : (a >= nx ? -nx : 0);
@@ -428,6 +450,18 @@ __device__ __forceinline__ bool solid_mark(const GradRec<float> &r) { return __f
 __device__ __forceinline__ bool solid_mark(const GradRec<double> &r)
 {
     return __double_as_longlong(r.k) == 0x7ff8dead00000000ll;
+}
+
+// entry a of a particle's record (the layout of lbm_particle_forces)
+__device__ __forceinline__ double record_entry(const PartDev &q, int a)
+{
+    static_assert(offsetof(PartDev, Tc) == offsetof(PartDev, Feta) + 15 * sizeof(double) &&
+                      offsetof(PartDev, q) == offsetof(PartDev, x) + 9 * sizeof(double) &&
+                      offsetof(PartDev, Fb) == offsetof(PartDev, sub) + sizeof(double),
+                  "the record's parts are contiguous");
+    if (a < 18) return (&q.Feta[0])[a];  // F_eta, T_eta, F_sig, T_sig, F_c, T_c
+    if (a < 31) return (&q.x[0])[a - 18];  // x, v, w, q
+    return a == 31 ? q.m : (&q.sub)[a - 32];  // sub, F_b
 }
 
 // entry of a boundary list: instance and instance-local node
@@ -732,7 +766,7 @@ __device__ __forceinline__ void for_item_nodes(const Lattice &L, long long item,
 enum Stage {
     STAGE_PHI = 0, STAGE_SOLIDPHI, STAGE_GRAD, STAGE_COLLIDE, STAGE_MEM, STAGE_CAPILLARY, STAGE_DEM,
     STAGE_GEOM_OWNER, STAGE_GEOM_BOUND, STAGE_REFILL, STAGE_FUSED, STAGE_REGION, STAGE_CURV, STAGE_SURROGATE,
-    STAGE_PHI_BOUND, STAGE_COLLIDE_BOUND, N_STAGES
+    STAGE_PHI_BOUND, STAGE_COLLIDE_BOUND, STAGE_CONTACTS, N_STAGES
 };
 
 // optional per-kernel marker: called right before and right after each launch
@@ -745,8 +779,7 @@ struct Marker {
     }
 };
 
-// host-side hook run by the fluid launcher once grad(phi), the normals and
-// the curvature of the step are final
+// host-side hook of the fluid launcher
 struct Hook {
     void (*fn)(void *self) = nullptr;
     void *self = nullptr;
@@ -756,12 +789,14 @@ struct Hook {
     }
 };
 
-// a second stream with two events: the plain form runs its boundary passes
-// there, beside the bulk kernels (they write disjoint nodes)
+// a second stream with two events: the boundary passes run there, beside the
+// bulk kernels (they write disjoint nodes), and what the hooks enqueue
 struct SideLane {
     cudaStream_t side = nullptr;
     cudaEvent_t a = nullptr, b = nullptr;
-    Hook after_collide_bound;  // more side-stream work after the collision's boundary pass
+    Hook after_phi_bound;      // after the order parameter's boundary pass and the solid-phi fill
+    Hook after_grad;           // once grad(phi) and the curvature of the step are final
+    Hook after_collide_bound;  // after the collision's boundary pass (16-bit storage)
 };
 
 // host-side kernel launchers (defined in the .cu files)
@@ -785,27 +820,26 @@ void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz);
 long long plan_rows(std::vector<InstDev> &inst);
 template <class S>
 void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk,
-                       const FluidLaunch &fz, const Hook &after_grad = Hook(), const SideLane &lane = SideLane());
+                       const FluidLaunch &fz, const SideLane &lane = SideLane());
+// Verlet prediction and contact forces (from the state before the step)
 template <class S>
-void launch_particle_forces(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk);
-// the two halves of it: momentum exchange (needs only the step's input
-// populations) and capillary force (needs the step's phi and normals)
+void launch_contacts(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk);
+// momentum exchange (needs only the step's input populations) and capillary
+// force (needs the step's phi and gradients)
 template <class S>
 void launch_momentum_exchange(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk);
 template <class S>
 void launch_capillary(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk);
-template <class S>
-void launch_geometry(const Lattice &L, int nxt, cudaStream_t st, long long *launches, const Marker &mk);
-// its three parts: owners and fresh bits (first), then boundary bits and the
-// refill of fresh nodes, which touch disjoint data and may run concurrently
-void launch_geom_owner(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk);
-void launch_geom_bound(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk);
-template <class S>
-void launch_refill(const Lattice &L, int nxt, cudaStream_t st, long long *launches, const Marker &mk);
 // sum_fluid: gather the momentum-exchange and capillary partial sums first
 // (false when the surrogate has written the fluid forces)
 template <class S>
 void launch_dem(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk, bool sum_fluid);
+// geometry: owners and fresh bits, then boundary bits and lists, and the
+// refill of fresh nodes (after the collision)
+void launch_geom_owner(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk);
+void launch_geom_surface(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk);
+template <class S>
+void launch_refill(const Lattice &L, int nxt, cudaStream_t st, long long *launches, const Marker &mk);
 
 // ---------------------------------------------------------------------------
 // learned force surrogate (lbm_mlp.cu)
@@ -865,5 +899,7 @@ void launch_static_fill(const Lattice &L, const long long *offs, long long *list
 template <class S>
 void launch_mark_solid(const Lattice &L, cudaStream_t st);
 void launch_mark_particles(const Lattice &L, cudaStream_t st);
+// the first step's particle lists
+void launch_first_lists(const Lattice &L, cudaStream_t st);
 
 }  // namespace lbmg

@@ -1,48 +1,67 @@
 // Particle kernels of one coupled time step (Sec. III and V of arXiv 2505.10171):
-//   k_mem        momentum-exchange force and torque per particle (Sec. V B)
-//   k_capillary  capillary force and torque from the Lagrangian surface points
-//                (Sec. V F)
-//   k_dem        fixed-order sums of the per-block partials of both, then
-//                contacts (normal spring-dashpot, Luding sliding and rolling
-//                friction) and velocity-Verlet update (Sec. III): one warp per
-//                particle for the sums, one thread per contact, then one per
-//                particle; positions and velocities FP64, contact arithmetic
-//                FP64 in the FP64 mode and FP32 otherwise
-//   k_geom_*     solid map update and refilling of uncovered nodes (Sec. V C)
+//   k_contacts     velocity-Verlet prediction and contact forces (normal
+//                  spring-dashpot, Luding sliding and rolling friction, Sec. III):
+//                  they need the previous step's forces only, so they run early
+//   k_mem          momentum-exchange force and torque per particle (Sec. V B)
+//   k_capillary    capillary force and torque from the Lagrangian surface points
+//                  (Sec. V F)
+//   k_dem          fixed-order sums of the per-block partials of both, the
+//                  velocity-Verlet correction (Sec. III) and the step's record:
+//                  one warp per particle
+//   k_geom_owner, k_geom_surface, k_refill
+//                  solid map update with the next step's boundary lists, and
+//                  refilling of uncovered nodes (Sec. V C)
 // Per-link and per-point arithmetic runs in the storage precision's arithmetic
-// type (double for FP64 storage, float otherwise); every sum over links,
-// points or contacts is FP64 with a fixed order (warp shuffle, block tree,
-// fixed block order), so results are reproducible run to run.  GB300 executes
-// double precision at a small fraction of the single-precision rate, so the
-// FP64 work is kept to the sums and the DEM.
+// type (double for FP64 storage, float otherwise); positions, velocities and
+// every sum over links, points or contacts are FP64 with a fixed order (warp
+// exchange, then blocks), so results are reproducible run to run.  An FP64
+// warp instruction holds its SM's FP64 pipe for about 16 cycles, so these
+// kernels count them: sums of K values over a warp exchange halves (K + 4
+// additions, not 5 K), and the work is spread over SMs in small CTAs.
 #include "lbm_internal.cuh"
 
 namespace lbmg {
 
-// deterministic block sum of 6 doubles; thread 0 writes them to out
+// Sums of K values (a power of two, 2 to 16) over the 32 lanes by exchanging
+// halves: at each of the first log2 K steps a lane keeps half of its values and
+// adds its partner's copies of them, so that K - 1 additions (and one per step
+// left) do the work of 5 K.  The sum of value a is left in v[0] of lane
+// a 32/K (and of the lanes above it up to the next one's).
 template <int K, class T>
-__device__ __forceinline__ void block_sum(T *v, double *out)
+__device__ __forceinline__ void warp_sums(T *v)
 {
-    __shared__ T sm[PART_THREADS / 32][K];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-    for (int a = 0; a < K; a++)
-        for (int o = 16; o > 0; o >>= 1) v[a] += __shfl_down_sync(0xffffffffu, v[a], o);
-    if (lane == 0)
-        for (int a = 0; a < K; a++) sm[wid][a] = v[a];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int a = 0; a < K; a++) {
-            T s = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += sm[w][a];
-            out[a] = (double)s;
+    for (int h = K / 2; h >= 1; h >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int a = 0; a < h; a++) {
+            const T keep = up ? v[a + h] : v[a], give = up ? v[a] : v[a + h];
+            v[a] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
+        o >>= 1;
     }
-    __syncthreads();  // sm is reused by a second call
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
 }
 
-template <class T>
-__device__ __forceinline__ void block_sum6(T *v, double *out) { block_sum<6>(v, out); }
+// sums of K values over a CTA of NT threads, warps in order; thread a < n
+// writes sum a to out
+template <int K, int NT, class T>
+__device__ __forceinline__ void block_sums(T *v, int n, double *out)
+{
+    __shared__ T sm[NT / 32][K];
+    warp_sums<K>(v);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane % (32 / K) == 0) sm[wid][lane / (32 / K)] = v[0];
+    __syncthreads();
+    if ((int)threadIdx.x < n) {
+        T s = sm[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < NT / 32; w++) s += sm[w][threadIdx.x];
+        out[threadIdx.x] = (double)s;
+    }
+}
 
 // particle centre in the arithmetic type R (single-precision copy for float)
 __device__ __forceinline__ void centre(const PartDev &P, double *c) { c[0] = P.x[0]; c[1] = P.x[1]; c[2] = P.x[2]; }
@@ -63,87 +82,97 @@ __device__ __forceinline__ void centre(const PartDev &P, float *c) { c[0] = P.xf
 // x_p - xr, its force is -(rho0/18) K and its torque -(rho0/18) (M - delta x K)
 // with K = sum k c and M = sum k d x c. The block partials hold the small
 // part's force and torque, K and 2M; the DEM kernel assembles them in FP64.
+//
+// A node's flags and populations are loaded together, whatever its links.
 template <class S>
-__global__ void __launch_bounds__(PART_THREADS) k_mem(Lattice L, int cur)
+__global__ void __launch_bounds__(MEM_THREADS) k_mem(Lattice L, int cur, FastDiv fd)
 {
     using R = typename Store<S>::real;
     const int p = blockIdx.y;
     const PartDev &P = L.parts[p];
     const InstDev &I = L.inst[P.inst];
     Region reg;
-    reg.init(P.x, P.mem_side, I.nx, I.ny, I.nz);
+    reg.init(P.xf, (int)fd.d, I.nx, I.ny, I.nz);
     R acc[6] = {0, 0, 0, 0, 0, 0};
     int kin[6] = {0, 0, 0, 0, 0, 0};  // K, then 2M
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    bool links = false;
+    int x = 0, y = 0, z = 0, n = 0;
+    const uint8_t *fli = L.flags + I.node_off;
     if (t < reg.count()) {
-        int x, y, z;
-        reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
-        const int n = (z * I.ny + y) * I.nx + x;
-        const uint8_t *fli = L.flags + I.node_off;
+        reg.coord(t, fd, I.nx, I.ny, I.nz, &x, &y, &z);
+        n = (z * I.ny + y) * I.nx + x;
         const uint8_t fl = fli[n];
-        if ((fl & OWNER_MASK) == OWN_FLUID && (fl & BOUND_BIT)) {
-            const Pop<S> in(L.pop[cur], I);
-            Nbr nb;
-            nb.init(x, y, z, I.nx, I.ny, I.nz);
-            const int mine = 2 + P.local;
-            // twice the node's offset from xr, minimum image (|.| < n)
-            const int xr[3] = {(int)floor(P.x[0]), (int)floor(P.x[1]), (int)floor(P.x[2])};
-            const int per[3] = {I.nx, I.ny, I.nz};
-            const int pos[3] = {x, y, z};
-            int D0[3];
-            for (int a = 0; a < 3; a++) {
-                int d = 2 * (pos[a] - xr[a]);
-                d += d >= per[a] ? -2 * per[a] : (d < -per[a] ? 2 * per[a] : 0);
-                D0[a] = d;
-            }
-            R rr = -1;
-            R c[3], v[3], w[3];
-            centre(P, c);
-            for (int a = 0; a < 3; a++) { v[a] = (R)P.v[a]; w[a] = (R)P.w[a]; }
-            const R r0 = (R)I.rho0;
-            for (int i = 1; i < Q; i++) {
-                if ((fli[nb.at(-cx(i), -cy(i), -cz(i))] & OWNER_MASK) != mine) continue;
-                if (rr < R(0)) {
-                    R sF = 0;
-                    for (int j = 0; j < Q; j++) sF += wgt<R>(j) * in.F(j, n);
-                    rr = R(1) + sF;
-                }
-                const int ci[3] = {cx(i), cy(i), cz(i)};
-                const R lev[3] = {min_image_r<R>(x - R(0.5) * ci[0] - c[0], I.nx),
-                                  min_image_r<R>(y - R(0.5) * ci[1] - c[1], I.ny),
-                                  min_image_r<R>(z - R(0.5) * ci[2] - c[2], I.nz)};
-                const R uw[3] = {v[0] + (w[1] * lev[2] - w[2] * lev[1]), v[1] + (w[2] * lev[0] - w[0] * lev[2]),
-                                 v[2] + (w[0] * lev[1] - w[1] * lev[0])};
-                const R wt = wgt<R>(i) * r0;
-                const R Fo = in.F(opp(i), n);
-                const R cu = ci[0] * uw[0] + ci[1] * uw[1] + ci[2] * uw[2];
-                const R e = R(6) * rr * cu;
-                const R q = R(2) * Fo + e;
-                R dp[3];
-                for (int a = 0; a < 3; a++) dp[a] = wt * (uw[a] * e - ci[a] * q);
-                acc[0] += dp[0];
-                acc[1] += dp[1];
-                acc[2] += dp[2];
-                acc[3] += lev[1] * dp[2] - lev[2] * dp[1];
-                acc[4] += lev[2] * dp[0] - lev[0] * dp[2];
-                acc[5] += lev[0] * dp[1] - lev[1] * dp[0];
-                // rest part: k c and k (2d) x c, 2d = D0 - c
-                const int k = csq(i) == 1 ? 2 : 1;
-                const int D[3] = {D0[0] - ci[0], D0[1] - ci[1], D0[2] - ci[2]};
-                kin[0] += k * ci[0];
-                kin[1] += k * ci[1];
-                kin[2] += k * ci[2];
-                kin[3] += k * (D[1] * ci[2] - D[2] * ci[1]);
-                kin[4] += k * (D[2] * ci[0] - D[0] * ci[2]);
-                kin[5] += k * (D[0] * ci[1] - D[1] * ci[0]);
-            }
+        links = (fl & OWNER_MASK) == OWN_FLUID && (fl & BOUND_BIT);
+    }
+    if (links) {
+        const Pop<S> in(L.pop[cur], I);
+        Nbr nb;
+        nb.init(x, y, z, I.nx, I.ny, I.nz);
+        const int mine = 2 + P.local;
+        int own[Q];
+        R F[Q];
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            own[i] = fli[nb.at(-cx(i), -cy(i), -cz(i))];
+            F[i] = in.F(i, n);
+        }
+        R c[3], v[3], w[3];
+        centre(P, c);
+        for (int a = 0; a < 3; a++) { v[a] = (R)P.v[a]; w[a] = (R)P.w[a]; }
+        // twice the node's offset from xr, minimum image (|.| < n)
+        const int per[3] = {I.nx, I.ny, I.nz};
+        const int pos[3] = {x, y, z};
+        int D0[3];
+        for (int a = 0; a < 3; a++) {
+            int d = 2 * (pos[a] - (int)floor(P.x[a]));
+            d += d >= per[a] ? -2 * per[a] : (d < -per[a] ? 2 * per[a] : 0);
+            D0[a] = d;
+        }
+        const R r0 = sizeof(R) == 8 ? (R)I.rho0 : (R)I.f_rho0;
+        R rr = 1;
+#pragma unroll
+        for (int i = 0; i < Q; i++) rr += wgt<R>(i) * F[i];
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            if ((own[i] & OWNER_MASK) != mine) continue;
+            const R lev[3] = {min_image_r<R>((x - R(0.5) * cx(i)) - c[0], I.nx),
+                              min_image_r<R>((y - R(0.5) * cy(i)) - c[1], I.ny),
+                              min_image_r<R>((z - R(0.5) * cz(i)) - c[2], I.nz)};
+            const R uw[3] = {v[0] + (w[1] * lev[2] - w[2] * lev[1]), v[1] + (w[2] * lev[0] - w[0] * lev[2]),
+                             v[2] + (w[0] * lev[1] - w[1] * lev[0])};
+            const R wt = wgt<R>(i) * r0;
+            const R e = R(6) * rr * (cx(i) * uw[0] + cy(i) * uw[1] + cz(i) * uw[2]);
+            const R q = R(2) * F[opp(i)] + e;
+            const R dp[3] = {wt * (uw[0] * e - cx(i) * q), wt * (uw[1] * e - cy(i) * q), wt * (uw[2] * e - cz(i) * q)};
+            acc[0] += dp[0];
+            acc[1] += dp[1];
+            acc[2] += dp[2];
+            acc[3] += lev[1] * dp[2] - lev[2] * dp[1];
+            acc[4] += lev[2] * dp[0] - lev[0] * dp[2];
+            acc[5] += lev[0] * dp[1] - lev[1] * dp[0];
+            // rest part: k c and k (2d) x c, 2d = D0 - c
+            const int k = csq(i) == 1 ? 2 : 1;
+            const int E[3] = {D0[0] - cx(i), D0[1] - cy(i), D0[2] - cz(i)};
+            kin[0] += k * cx(i);
+            kin[1] += k * cy(i);
+            kin[2] += k * cz(i);
+            kin[3] += k * (E[1] * cz(i) - E[2] * cy(i));
+            kin[4] += k * (E[2] * cx(i) - E[0] * cz(i));
+            kin[5] += k * (E[0] * cy(i) - E[1] * cx(i));
         }
     }
     double *out = L.mem_part + ((long long)p * L.mem_blocks + blockIdx.x) * MEM_PART;
-    double accd[6];
-    for (int a = 0; a < 6; a++) accd[a] = (double)acc[a];
-    block_sum6(accd, out);
-    block_sum6(kin, out + 6);
+    if (!__syncthreads_or(links)) {  // most blocks of the cube: nothing to add
+        if (threadIdx.x < MEM_PART) out[threadIdx.x] = 0.0;
+        return;
+    }
+    double accd[8];
+    for (int a = 0; a < 8; a++) accd[a] = a < 6 ? (double)acc[a] : 0.0;
+    block_sums<8, MEM_THREADS>(accd, 6, out);
+    int kin8[8];
+    for (int a = 0; a < 8; a++) kin8[a] = a < 6 ? kin[a] : 0;
+    block_sums<8, MEM_THREADS>(kin8, 6, out + 6);
 }
 
 // Sec. V F: dF = C sigma (1 - phi^2) dA (n x n_s) x n at the points
@@ -152,83 +181,102 @@ __global__ void __launch_bounds__(PART_THREADS) k_mem(Lattice L, int cur)
 // torque R_p n_s x dF.  With BUOY also the phase-a share of the surface for
 // the buoyancy (reading c28): s = (1 + phi)/2 clipped to [0, 1] and dA, summed
 // over the points with a fluid corner.
+//
+// The eight corners' flags, phi and gradients are loaded together, solid or not.
+__device__ __forceinline__ void surface_point(const Lattice &L, int pt, float *t)
+{
+    const float4 v = reinterpret_cast<const float4 *>(L.cap_pts_f)[pt];
+    t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+}
+__device__ __forceinline__ void surface_point(const Lattice &L, int pt, double *t)
+{
+    for (int a = 0; a < 4; a++) t[a] = L.cap_pts[4 * pt + a];
+}
+
 template <class R, bool BUOY>
 __global__ void __launch_bounds__(CAP_THREADS) k_capillary(Lattice L)
 {
     const int p = blockIdx.y;
     const PartDev &P = L.parts[p];
     const InstDev &I = L.inst[P.inst];
-    double acc[CAP_PART] = {0, 0, 0, 0, 0, 0, 0, 0};
+    R acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const int pt = blockIdx.x * blockDim.x + threadIdx.x;
     if (pt < CAP_POINTS) {
-        const double *tp = L.cap_pts + 4 * pt;
-        const R ns[3] = {(R)tp[0], (R)tp[1], (R)tp[2]};
-        const R sa = (R)tp[3];
+        R tp[4];
+        surface_point(L, pt, tp);
+        const R ns[3] = {tp[0], tp[1], tp[2]};
+        const R sa = tp[3];
         const R da = R(2.0 * M_PI / 180.0);
         R c[3];
         centre(P, c);
-        const R Rp = (R)P.R;
+        const R Rp = sizeof(R) == 8 ? (R)P.R : (R)P.Rf;
         const R xi[3] = {c[0] + Rp * ns[0], c[1] + Rp * ns[1], c[2] + Rp * ns[2]};
         const R dA = Rp * Rp * sa * da * da;
-        int b[3];
+        int lo[3], hi[3];
         R fr[3];
+        const int n3[3] = {I.nx, I.ny, I.nz};
         for (int a = 0; a < 3; a++) {
             const R fl = floor(xi[a]);
-            b[a] = (int)fl;
             fr[a] = xi[a] - fl;
+            const int b = (int)fl;
+            lo[a] = b < 0 ? b + n3[a] : (b >= n3[a] ? b - n3[a] : b);
+            hi[a] = b + 1 < 0 ? b + 1 + n3[a] : (b + 1 >= n3[a] ? b + 1 - n3[a] : b + 1);
         }
-        const int n3[3] = {I.nx, I.ny, I.nz};
         const uint8_t *fli = L.flags + I.node_off;
         const R *ph = (const R *)L.phi + I.node_off;
         const GradRec<R> *Gr = (const GradRec<R> *)L.grad + I.node_off;
+        uint8_t fl[8];
+        R pc[8];
+        GradRec<R> gc[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const int X = k & 1 ? hi[0] : lo[0], Y = k & 2 ? hi[1] : lo[1], Z = k & 4 ? hi[2] : lo[2];
+            const int m = (Z * I.ny + Y) * I.nx + X;
+            fl[k] = fli[m];
+            pc[k] = ph[m];
+            gc[k] = Gr[m];
+        }
         R ws = 0, phs = 0, gs[3] = {0, 0, 0};
-        for (int cz_ = 0; cz_ < 2; cz_++)
-            for (int cy_ = 0; cy_ < 2; cy_++)
-                for (int cx_ = 0; cx_ < 2; cx_++) {
-                    int X = b[0] + cx_, Y = b[1] + cy_, Z = b[2] + cz_;
-                    X = X < 0 ? X + n3[0] : (X >= n3[0] ? X - n3[0] : X);
-                    Y = Y < 0 ? Y + n3[1] : (Y >= n3[1] ? Y - n3[1] : Y);
-                    Z = Z < 0 ? Z + n3[2] : (Z >= n3[2] ? Z - n3[2] : Z);
-                    const long long m = ((long long)Z * I.ny + Y) * I.nx + X;
-                    if ((fli[m] & OWNER_MASK) != OWN_FLUID) continue;
-                    const R wgt_ = (cx_ ? fr[0] : R(1) - fr[0]) * (cy_ ? fr[1] : R(1) - fr[1]) *
-                                   (cz_ ? fr[2] : R(1) - fr[2]);
-                    const GradRec<R> gm = Gr[m];
-                    ws += wgt_;
-                    phs += wgt_ * ph[m];
-                    gs[0] += wgt_ * gm.g0;
-                    gs[1] += wgt_ * gm.g1;
-                    gs[2] += wgt_ * gm.g2;
-                }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            if ((fl[k] & OWNER_MASK) != OWN_FLUID) continue;
+            const R wgt_ = (k & 1 ? fr[0] : R(1) - fr[0]) * (k & 2 ? fr[1] : R(1) - fr[1]) * (k & 4 ? fr[2] : R(1) - fr[2]);
+            ws += wgt_;
+            phs += wgt_ * pc[k];
+            gs[0] += wgt_ * gc[k].g0;
+            gs[1] += wgt_ * gc[k].g1;
+            gs[2] += wgt_ * gc[k].g2;
+        }
         if (ws > R(0)) {
             const R phv = phs / ws;
             if (BUOY) {
-                const R sa = fmin(fmax(R(0.5) * (R(1) + phv), R(0)), R(1));
-                acc[6] = (double)(sa * dA);
-                acc[7] = (double)dA;
+                acc[6] = fmin(fmax(R(0.5) * (R(1) + phv), R(0)), R(1)) * dA;
+                acc[7] = dA;
             }
             const R g0 = gs[0] / ws, g1 = gs[1] / ws, g2 = gs[2] / ws;
             if (fabs(phv) < R(1)) {
-                const R eps2 = (R)(I.grad_eps * I.grad_eps);
+                const R eps2 = sizeof(R) == 8 ? (R)(I.grad_eps * I.grad_eps) : (R)I.f_eps2;
                 const R gr = sqrt(g0 * g0 + g1 * g1 + g2 * g2 + eps2);
                 const R nn[3] = {g0 / gr, g1 / gr, g2 / gr};
                 const R c0 = nn[1] * ns[2] - nn[2] * ns[1], c1 = nn[2] * ns[0] - nn[0] * ns[2],
                         c2 = nn[0] * ns[1] - nn[1] * ns[0];
                 const R mv[3] = {c1 * nn[2] - c2 * nn[1], c2 * nn[0] - c0 * nn[2], c0 * nn[1] - c1 * nn[0]};
-                const R coef = (R)(I.cap_norm * I.sigma) * (R(1) - phv * phv) * dA;
+                const R coef = (sizeof(R) == 8 ? (R)(I.cap_norm * I.sigma) : (R)I.f_cap) * (R(1) - phv * phv) * dA;
                 R dF[3];
                 for (int a = 0; a < 3; a++) dF[a] = coef * mv[a];
                 const R r[3] = {Rp * ns[0], Rp * ns[1], Rp * ns[2]};
-                acc[0] = (double)dF[0];
-                acc[1] = (double)dF[1];
-                acc[2] = (double)dF[2];
-                acc[3] = (double)(r[1] * dF[2] - r[2] * dF[1]);
-                acc[4] = (double)(r[2] * dF[0] - r[0] * dF[2]);
-                acc[5] = (double)(r[0] * dF[1] - r[1] * dF[0]);
+                acc[0] = dF[0];
+                acc[1] = dF[1];
+                acc[2] = dF[2];
+                acc[3] = r[1] * dF[2] - r[2] * dF[1];
+                acc[4] = r[2] * dF[0] - r[0] * dF[2];
+                acc[5] = r[0] * dF[1] - r[1] * dF[0];
             }
         }
     }
-    block_sum<BUOY ? 8 : 6>(acc, L.cap_part + ((long long)p * CAP_BLOCKS + blockIdx.x) * CAP_PART);
+    double accd[8];
+    for (int a = 0; a < 8; a++) accd[a] = a < (BUOY ? 8 : 6) ? (double)acc[a] : 0.0;
+    block_sums<8, CAP_THREADS>(accd, BUOY ? 8 : 6, L.cap_part + ((long long)p * CAP_BLOCKS + blockIdx.x) * CAP_PART);
 }
 
 
@@ -334,8 +382,6 @@ __device__ void quat_rotate(double *q, const T *w)
     q[0] = r0 / l; q[1] = r1 / l; q[2] = r2 / l; q[3] = r3 / l;
 }
 
-constexpr int DEM_THREADS = 256;  // a warp per particle for the fluid sums of up to 8 particles at once
-
 // pair index c in [0, np(np-1)/2) -> (i, j), i < j, lexicographic
 __device__ __forceinline__ void pair_of(int c, int np, int *i, int *j)
 {
@@ -350,87 +396,34 @@ __device__ __forceinline__ void pair_of(int c, int np, int *i, int *j)
 
 __device__ __forceinline__ int pair_index(int i, int j, int np) { return i * np - i * (i + 1) / 2 + (j - i - 1); }
 
-// one block per instance.  Velocity-Verlet predictor per particle; contact
-// forces one thread per contact (substrate contacts, then pairs), kept per
-// contact; corrector per particle, adding its contacts in a fixed order
-// (substrate, then partners in increasing index).
-template <class T, bool BUOY>
-__global__ void __launch_bounds__(DEM_THREADS) k_dem(Lattice L, int sum_fluid)
+// Velocity-Verlet prediction per particle (kept in its xn) and contact forces,
+// one thread per contact (substrate contacts, then pairs), kept per contact; one
+// block per instance.  All of it follows from the particles' state and the
+// previous step's forces, so it runs early in the step, beside the fluid
+// kernels.  Block 0 counts the step for the record ring.
+constexpr int CONTACT_THREADS = 128;
+template <class T>
+__global__ void __launch_bounds__(CONTACT_THREADS) k_contacts(Lattice L)
 {
     const InstDev &I = L.inst[blockIdx.x];
     const int np = I.np;
+    const int tid = threadIdx.x;
+    if (L.ring_ctr && blockIdx.x == 0 && tid == 0) *L.ring_ctr += 1;
     if (np == 0) return;
     PartDev *P = L.parts + I.part_off;
     double *hist = L.hist + (long long)I.hist_off * 6;
     double *rec = L.crec + (long long)I.crec_off * 12;
     __shared__ double xn[3 * MAX_PART];
     __shared__ T vp[3 * MAX_PART], wp[3 * MAX_PART];
-    const int tid = threadIdx.x;
-    if (sum_fluid) {
-        // fluid forces of this step: a warp per particle sums the block
-        // partials of the momentum-exchange and capillary kernels, lanes over
-        // a fixed block stride, then a fixed shuffle tree (deterministic)
-        const int lane = tid & 31, wid = tid >> 5;
-        for (int p = wid; p < np; p += DEM_THREADS / 32) {
-            const long long pg = I.part_off + p;
-            constexpr int NC = BUOY ? CAP_PART : 6;  // capillary partials used
-            double s[12 + NC];
-            for (int a = 0; a < 12 + NC; a++) s[a] = 0.0;
-            for (int b = lane; b < L.mem_blocks; b += 32)
-                for (int a = 0; a < MEM_PART; a++) s[a] += L.mem_part[(pg * L.mem_blocks + b) * MEM_PART + a];
-            for (int b = lane; b < CAP_BLOCKS; b += 32)
-                for (int a = 0; a < NC; a++) s[12 + a] += L.cap_part[(pg * CAP_BLOCKS + b) * CAP_PART + a];
-            for (int o = 16; o > 0; o >>= 1)
-                for (int a = 0; a < 12 + NC; a++) s[a] += __shfl_down_sync(0xffffffffu, s[a], o);
-            if (lane == 0) {
-                // momentum exchange: small part plus the exact rest part
-                // -(rho0/18) K, -(rho0/18) (M - delta x K), M = (2M)/2
-                const double g = -I.rho0 / 18.0;
-                double dl[3], K[3], M[3];
-                for (int a = 0; a < 3; a++) {
-                    dl[a] = P[p].x[a] - floor(P[p].x[a]);
-                    K[a] = s[6 + a];
-                    M[a] = 0.5 * s[9 + a];
-                }
-                const double dK[3] = {dl[1] * K[2] - dl[2] * K[1], dl[2] * K[0] - dl[0] * K[2],
-                                      dl[0] * K[1] - dl[1] * K[0]};
-                for (int a = 0; a < 3; a++) {
-                    P[p].Feta[a] = s[a] + g * K[a];
-                    P[p].Teta[a] = s[3 + a] + g * (M[a] - dK[a]);
-                    P[p].Fsig[a] = s[12 + a];
-                    P[p].Tsig[a] = s[15 + a];
-                }
-                // buoyancy (reading c28): a flat interface at height h = (2a - 1) R
-                // above the centre leaves the volume fraction (1 + t)^2 (2 - t)/4,
-                // t = h/R, of the sphere below it (a spherical zone's area is
-                // proportional to its height)
-                if constexpr (BUOY) {
-                    double sub = 0.0;
-                    if (s[19] > 0.0) {
-                        const double t = 2.0 * (s[18] / s[19]) - 1.0;
-                        sub = (1.0 + t) * (1.0 + t) * (2.0 - t) / 4.0;
-                    }
-                    const double vol = 4.0 / 3.0 * M_PI * P[p].R * P[p].R * P[p].R;
-                    P[p].sub = sub;
-                    for (int a = 0; a < 3; a++) P[p].Fb[a] = vol * sub * I.buoy[a];
-                }
-            }
-        }
-        __syncthreads();
+    for (int k = tid; k < 3 * np; k += blockDim.x) {
+        const int p = k / 3, a = k - 3 * p;
+        const PartDev &q = P[p];
+        const double acc = q.kin ? 0.0 : q.Fp[a] * q.inv_m, alp = q.kin ? 0.0 : q.Tp[a] * q.inv_I;
+        xn[k] = q.x[a] + q.v[a] + 0.5 * acc;
+        vp[k] = (T)(q.v[a] + acc);
+        wp[k] = (T)(q.w[a] + alp);
+        P[p].xn[a] = xn[k];
     }
-    for (int p = tid; p < np; p += blockDim.x)
-        for (int a = 0; a < 3; a++) {
-            if (P[p].kin) {
-                xn[3 * p + a] = P[p].x[a] + P[p].v[a];
-                vp[3 * p + a] = (T)P[p].v[a];
-                wp[3 * p + a] = (T)P[p].w[a];
-            } else {
-                const double acc = P[p].Fp[a] * P[p].inv_m, alp = P[p].Tp[a] * P[p].inv_I;
-                xn[3 * p + a] = P[p].x[a] + P[p].v[a] + 0.5 * acc;
-                vp[3 * p + a] = (T)(P[p].v[a] + acc);
-                wp[3 * p + a] = (T)(P[p].w[a] + alp);
-            }
-        }
     __syncthreads();
     const int npair = np * (np - 1) / 2;
     for (int c = tid; c < np + npair; c += blockDim.x) {
@@ -470,50 +463,117 @@ __global__ void __launch_bounds__(DEM_THREADS) k_dem(Lattice L, int sum_fluid)
         for (int a = 0; a < 6; a++) hs[a] = touch ? (double)xi[a] : 0.0;
         for (int a = 0; a < 12; a++) r[a] = (double)rt[a];
     }
-    __syncthreads();
-    for (int p = tid; p < np; p += blockDim.x) {
-        double Fc[3] = {0, 0, 0}, Tc[3] = {0, 0, 0};
-        const double *r = rec + 12 * p;
-        for (int a = 0; a < 3; a++) { Fc[a] += r[a]; Tc[a] += r[3 + a]; }
+}
+
+// The step of a particle, by one warp: the fluid forces from the block partials
+// of the momentum-exchange and capillary kernels (lanes over a fixed block
+// stride, then warp_sums; sum_fluid 0: the surrogate has set them), contacts
+// added in a fixed order (substrate, then partners in increasing index), the
+// velocity-Verlet correction with lane a and 3 + a on axis a, and the record
+// in the record ring.  It also empties the boundary and refill lists that the
+// geometry kernels after it fill.  One warp a CTA: the particles' FP64 chains
+// run on as many SMs (a CTA of 8 warps per instance, contacts included, took
+// 28 us for 8 particles and 17 for one; now 14, and 6 for the contacts).
+template <class T, bool BUOY>
+__global__ void __launch_bounds__(32) k_dem(Lattice L, int sum_fluid)
+{
+    const int pg = blockIdx.x, lane = threadIdx.x;
+    if (pg == 0 && lane < 4) L.list_n[lane] = 0;
+    PartDev &P = L.parts[pg];
+    const InstDev &I = L.inst[P.inst];
+    const int np = I.np, p = P.local;
+    const double *rec = L.crec + (long long)I.crec_off * 12;
+    __shared__ double s[20], now[6];
+    if (sum_fluid) {
+        double m[16], c[8];
+        for (int a = 0; a < 16; a++) m[a] = 0.0;
+        for (int a = 0; a < 8; a++) c[a] = 0.0;
+        constexpr int NC = BUOY ? 8 : 6;  // capillary partials used
+        for (int b = lane; b < CAP_BLOCKS; b += 32)
+            for (int a = 0; a < NC; a++) c[a] += L.cap_part[((long long)pg * CAP_BLOCKS + b) * CAP_PART + a];
+        for (int b = lane; b < L.mem_blocks; b += 32)
+            for (int a = 0; a < MEM_PART; a++) m[a] += L.mem_part[((long long)pg * L.mem_blocks + b) * MEM_PART + a];
+        warp_sums<16>(m);
+        warp_sums<8>(c);
+        if (lane % 2 == 0 && lane / 2 < 12) s[lane / 2] = m[0];
+        if (lane % 4 == 0) s[12 + lane / 4] = c[0];
+        __syncwarp();
+        if (lane < 3) {
+            // momentum exchange: small part plus the exact rest part
+            // -(rho0/18) K, -(rho0/18) (M - delta x K), M = (2M)/2
+            const double g = -I.rho0 / 18.0;
+            const int a1 = lane == 2 ? 0 : lane + 1, a2 = lane == 0 ? 2 : lane - 1;
+            const double d1 = P.x[a1] - floor(P.x[a1]), d2 = P.x[a2] - floor(P.x[a2]);
+            P.Feta[lane] = s[lane] + g * s[6 + lane];
+            P.Teta[lane] = s[3 + lane] + g * (0.5 * s[9 + lane] - (d1 * s[6 + a2] - d2 * s[6 + a1]));
+            P.Fsig[lane] = s[12 + lane];
+            P.Tsig[lane] = s[15 + lane];
+            // buoyancy (reading c28): a flat interface at height h = (2a - 1) R
+            // above the centre leaves the volume fraction (1 + t)^2 (2 - t)/4,
+            // t = h/R, of the sphere below it (a spherical zone's area is
+            // proportional to its height)
+            if constexpr (BUOY) {
+                double sub = 0.0;
+                if (s[19] > 0.0) {
+                    const double t = 2.0 * (s[18] / s[19]) - 1.0;
+                    sub = (1.0 + t) * (1.0 + t) * (2.0 - t) / 4.0;
+                }
+                if (lane == 0) P.sub = sub;
+                P.Fb[lane] = 4.0 / 3.0 * M_PI * P.R * P.R * P.R * sub * I.buoy[lane];
+            }
+        }
+        __syncwarp();
+    }
+    // contacts: lanes 0..2 the force, 3..5 the torque
+    double contact = 0.0, total = 0.0, wold = 0.0;
+    if (lane < 6) {
+        contact = rec[12 * p + lane];
+#pragma unroll 4
         for (int q = 0; q < np; q++) {
             if (q == p) continue;
-            const double *rp = rec + 12 * (np + (q < p ? pair_index(q, p, np) : pair_index(p, q, np)));
-            const int off = q < p ? 6 : 0;  // p is the second member of (q, p)
-            for (int a = 0; a < 3; a++) { Fc[a] += rp[off + a]; Tc[a] += rp[off + 3 + a]; }
+            // p is the second member of (q, p), q < p
+            contact += rec[12 * (np + (q < p ? pair_index(q, p, np) : pair_index(p, q, np))) + (q < p ? 6 : 0) + lane];
         }
-        PartDev &Q_ = P[p];
-        double F[3], Tq[3], wold[3];
-        for (int a = 0; a < 3; a++) {
-            Q_.Fc[a] = Fc[a];
-            Q_.Tc[a] = Tc[a];
-            F[a] = Fc[a] + I.g_part[a] + Q_.Feta[a] + Q_.Fsig[a] + Q_.Fb[a];
-            Tq[a] = Tc[a] + Q_.Teta[a] + Q_.Tsig[a];
-            wold[a] = Q_.w[a];
-            Q_.x_old[a] = Q_.x[a];
-            Q_.xfo[a] = Q_.xf[a];
+        if (lane < 3) {
+            P.Fc[lane] = contact;
+            total = contact + I.g_part[lane] + P.Feta[lane] + P.Fsig[lane] + P.Fb[lane];
+            if (!P.kin) P.v[lane] += 0.5 * (P.Fp[lane] + total) * P.inv_m;
+            P.Fp[lane] = total;
+        } else {
+            const int a = lane - 3;
+            P.Tc[a] = contact;
+            total = contact + P.Teta[a] + P.Tsig[a];
+            wold = P.w[a];
+            if (!P.kin) P.w[a] += 0.5 * (P.Tp[a] + total) * P.inv_I;
+            P.Tp[a] = total;
+            now[a] = 0.5 * (wold + P.w[a]);
         }
-        if (!Q_.kin)
-            for (int a = 0; a < 3; a++) {
-                Q_.v[a] += 0.5 * (Q_.Fp[a] + F[a]) * Q_.inv_m;
-                Q_.w[a] += 0.5 * (Q_.Tp[a] + Tq[a]) * Q_.inv_I;
-            }
-        const T wm[3] = {(T)(0.5 * (wold[0] + Q_.w[0])), (T)(0.5 * (wold[1] + Q_.w[1])),
-                         (T)(0.5 * (wold[2] + Q_.w[2]))};
-        quat_rotate<T>(Q_.q, wm);
-        // the geometry kernels assume a move below the margin: a larger or
-        // non-finite one sets the status and leaves the particle where it was
-        // (the run is reported unstable), so that nothing indexes with it
-        bool ok = true;
-        for (int a = 0; a < 3; a++) ok = ok && fabs(xn[3 * p + a] - Q_.x[a]) < GEOM_MARGIN - 1;
+    }
+    // the geometry kernels assume a move below the margin: a larger or
+    // non-finite one sets the status and leaves the particle where it was
+    // (the run is reported unstable), so that nothing indexes with it
+    const bool near = lane >= 3 || fabs(P.xn[lane] - P.x[lane]) < GEOM_MARGIN - 1;
+    const bool ok = __all_sync(0xffffffffu, near);
+    if (lane < 3) {
+        const int per = lane == 0 ? I.nx : (lane == 1 ? I.ny : I.nz);
+        const double x0 = P.x[lane], xn = P.xn[lane];
+        P.x_old[lane] = x0;
+        P.xfo[lane] = P.xf[lane];
+        // periodic domain: positions kept in [0, n)
+        const double x1 = ok ? xn - per * floor(xn / per) : x0;
+        P.x[lane] = x1;
+        P.xf[lane] = (float)x1;
+    }
+    __syncwarp();
+    if (lane == 0) {
         if (!ok) atomicOr(L.status, ST_DISPLACEMENT);
-        const int per[3] = {I.nx, I.ny, I.nz};
-        for (int a = 0; a < 3; a++) {
-            // periodic domain: positions kept in [0, n)
-            if (ok) Q_.x[a] = xn[3 * p + a] - per[a] * floor(xn[3 * p + a] / per[a]);
-            Q_.xf[a] = (float)Q_.x[a];
-            Q_.Fp[a] = F[a];
-            Q_.Tp[a] = Tq[a];
-        }
+        const T wm[3] = {(T)now[0], (T)now[1], (T)now[2]};
+        quat_rotate<T>(P.q, wm);
+    }
+    __syncwarp();
+    if (L.ring) {
+        double *slot = L.ring + ((size_t)((*L.ring_ctr - 1) % L.ring_slots) * L.n_parts + pg) * RECORD;
+        for (int a = lane; a < RECORD; a += 32) slot[a] = record_entry(P, a);
     }
 }
 
@@ -541,64 +601,139 @@ __device__ __forceinline__ int particle_owner(const InstDev &I, const PartDev *p
     return OWN_FLUID;
 }
 
-// new owner and fresh bit inside a particle's region (pure function of the
-// particle positions, so overlapping regions write identical bytes)
-__global__ void __launch_bounds__(PART_THREADS) k_geom_owner(Lattice L, int side)
+// is node (x, y, z) inside particle P at its current (which 0) or previous position
+__device__ __forceinline__ bool inside_particle(const InstDev &I, const PartDev &P, int x, int y, int z, int which)
+{
+    const float *cf = which ? P.xfo : P.xf;
+    const float e0 = min_image_r<float>((float)x - cf[0], I.nx);
+    const float e1 = min_image_r<float>((float)y - cf[1], I.ny);
+    const float e2 = min_image_r<float>((float)z - cf[2], I.nz);
+    const float d2 = e0 * e0 + e1 * e1 + e2 * e2;
+    if (d2 > P.R2hi) return false;
+    if (d2 < P.R2lo) return true;
+    const double *c = which ? P.x_old : P.x;
+    const double d0 = min_image(x - c[0], I.nx), d1 = min_image(y - c[1], I.ny), dd = min_image(z - c[2], I.nz);
+    return d0 * d0 + d1 * d1 + dd * dd < P.R * P.R;
+}
+
+// New owner and fresh bit inside a particle's region (a pure function of the
+// particle positions, so overlapping regions write identical bytes).  Only a
+// node inside the region's own particle, now or before, or left fresh by the
+// step before can change here: the others cost two distances (with all
+// particles' distances taken for every node, 512 spheres R = 3 took 126 us,
+// now 44).  Uncovered and newly covered nodes are listed once, for the refill.
+__global__ void __launch_bounds__(PART_THREADS) k_geom_owner(Lattice L, FastDiv fd)
 {
     const PartDev &P = L.parts[blockIdx.y];
     const InstDev &I = L.inst[P.inst];
     Region reg;
-    reg.init(P.x, side, I.nx, I.ny, I.nz);
+    reg.init(P.xf, (int)fd.d, I.nx, I.ny, I.nz);
+    const int mine = 2 + P.local;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < reg.count();
          t += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
-        reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
-        const long long g = I.node_off + ((long long)z * I.ny + y) * I.nx + x;
-        const uint8_t old = L.flags[g];
+        reg.coord(t, fd, I.nx, I.ny, I.nz, &x, &y, &z);
+        const int n = (z * I.ny + y) * I.nx + x;
+        uint8_t *fl = L.flags + I.node_off + n;
+        const uint8_t old = *fl;
         if (own_static(old & OWNER_MASK)) continue;
+        if (!(old & FRESH_BIT) && !inside_particle(I, P, x, y, z, 0) && !inside_particle(I, P, x, y, z, 1)) continue;
         const int own = particle_owner(I, L.parts, x, y, z, 0);
         const int prev = particle_owner(I, L.parts, x, y, z, 1);
         uint8_t f = (uint8_t)own;
-        if (own == OWN_FLUID && prev != OWN_FLUID) f |= FRESH_BIT;
-        L.flags[g] = (uint8_t)(f | (old & BOUND_BIT));
+        if (own == OWN_FLUID && prev != OWN_FLUID) {
+            f |= FRESH_BIT;
+            if (prev == mine) L.fresh[atomicAdd(L.list_n + LIST_FRESH, 1ull)] = list_entry(P.inst, n);
+        }
+        if (own == mine && prev == OWN_FLUID) L.covered[atomicAdd(L.list_n + LIST_COVERED, 1ull)] = list_entry(P.inst, n);
+        *fl = (uint8_t)(f | (old & BOUND_BIT));
     }
 }
 
-// boundary bit: fluid with a solid neighbour, or solid with a fluid neighbour
-__device__ __forceinline__ void set_boundary(const Lattice &L, const InstDev &I, int x, int y, int z)
+// boundary bit: fluid with a solid neighbour, or solid with a fluid neighbour.
+// *mine: some neighbour is owned by `owner`; returns the flags.
+__device__ __forceinline__ uint8_t set_boundary(const Lattice &L, const InstDev &I, int x, int y, int z, int owner,
+                                                bool *mine)
 {
     const uint8_t *fli = L.flags + I.node_off;
     const int n = (z * I.ny + y) * I.nx + x;
-    const uint8_t f = fli[n];
-    const bool fluid = (f & OWNER_MASK) == OWN_FLUID;
     Nbr nb;
     nb.init(x, y, z, I.nx, I.ny, I.nz);
-    bool b = false;
+    uint8_t o[Q];
+    o[0] = fli[n];
+#pragma unroll
+    for (int i = 1; i < Q; i++) o[i] = fli[nb.at(cx(i), cy(i), cz(i))];
+    const bool fluid = (o[0] & OWNER_MASK) == OWN_FLUID;
+    bool b = false, m = false;
 #pragma unroll
     for (int i = 1; i < Q; i++) {
-        bool nf = (fli[nb.at(cx(i), cy(i), cz(i))] & OWNER_MASK) == OWN_FLUID;
-        b |= (nf != fluid);
+        const int ow = o[i] & OWNER_MASK;
+        b |= (ow == OWN_FLUID) != fluid;
+        m |= ow == owner;
     }
-    L.flags[I.node_off + n] = (uint8_t)((f & ~BOUND_BIT) | (b ? BOUND_BIT : 0));
+    const uint8_t f = (uint8_t)((o[0] & ~BOUND_BIT) | (b ? BOUND_BIT : 0));
+    if (f != o[0]) L.flags[I.node_off + n] = f;
+    *mine = m;
+    return f;
 }
 
-__global__ void __launch_bounds__(PART_THREADS) k_geom_bound(Lattice L, int side)
+// Boundary bits around the particles, and the next step's lists: the fluid
+// nodes next to a particle (L.pbl, for the boundary passes) and the particles'
+// solid nodes next to fluid (L.psl, for the solid-phi fill), appended with one
+// atomic per warp; order within a list does not matter, a node next to two
+// particles is listed twice and written twice with the same value.  A bit can
+// change only within one link of a node whose owner changed, i.e. within
+// the particle's last displacement and one link of its surface: the other
+// nodes of the cube cost a distance (all: the bits of every node and no lists,
+// when particles are added).  512 spheres R = 3: 80 us with 18 flags read for every node,
+// now 43.
+__global__ void __launch_bounds__(PART_THREADS) k_geom_surface(Lattice L, FastDiv fd, int all)
 {
     const PartDev &P = L.parts[blockIdx.y];
     const InstDev &I = L.inst[P.inst];
     Region reg;
-    reg.init(P.x, side, I.nx, I.ny, I.nz);
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < reg.count();
-         t += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
-        set_boundary(L, I, x, y, z);
-        // the solid mark of a covered node's gradient record (see set_solid_mark)
-        const long long g = I.node_off + ((long long)z * I.ny + y) * I.nx + x;
-        if ((L.flags[g] & OWNER_MASK) != OWN_FLUID) {
-            if (L.mark == 8) set_solid_mark(((GradRec<double> *)L.grad)[g]);
-            else if (L.mark == 4) set_solid_mark(((GradRec<float> *)L.grad)[g]);
+    reg.init(P.xf, (int)fd.d, I.nx, I.ny, I.nz);
+    const int mine = 2 + P.local;
+    const float m0 = min_image_r<float>(P.xf[0] - P.xfo[0], I.nx), m1 = min_image_r<float>(P.xf[1] - P.xfo[1], I.ny),
+                m2 = min_image_r<float>(P.xf[2] - P.xfo[2], I.nz);
+    // one link is at most sqrt 2; 0.1 covers the single-precision distance
+    const float reach = sqrtf(m0 * m0 + m1 * m1 + m2 * m2) + 1.52f;
+    const float lo = fmaxf(P.Rf - reach, 0.0f), hi = P.Rf + reach, lo2 = P.Rf > reach ? lo * lo : -1.0f, hi2 = hi * hi;
+    const long long count = reg.count();
+    const int lane = threadIdx.x & 31;
+    auto append = [&](bool take, long long e, long long *list, unsigned long long *n) {
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        if (!m) return;
+        const int leader = __ffs(m) - 1;
+        unsigned long long base = 0;
+        if (lane == leader) base = atomicAdd(n, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (take) list[base + __popc(m & ((1u << lane) - 1u))] = e;
+    };
+    // warp-uniform trip count: every lane takes part in the ballots
+    for (long long t0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < count;
+         t0 += (long long)gridDim.x * blockDim.x) {
+        const long long t = t0 + lane;
+        bool fluid = false, solid = false;
+        long long e = 0;
+        if (t < count) {
+            int x, y, z;
+            reg.coord(t, fd, I.nx, I.ny, I.nz, &x, &y, &z);
+            const float e0 = min_image_r<float>((float)x - P.xf[0], I.nx), e1 = min_image_r<float>((float)y - P.xf[1], I.ny),
+                        e2 = min_image_r<float>((float)z - P.xf[2], I.nz);
+            const float d2 = e0 * e0 + e1 * e1 + e2 * e2;
+            if (all || (d2 >= lo2 && d2 <= hi2)) {
+                bool next;
+                const uint8_t f = set_boundary(L, I, x, y, z, mine, &next);
+                const int own = f & OWNER_MASK;
+                fluid = own == OWN_FLUID && next;
+                solid = own == mine && (f & BOUND_BIT);
+                e = list_entry(P.inst, (z * I.ny + y) * I.nx + x);
+            }
         }
+        if (all) continue;
+        append(fluid, e, L.pbl, L.list_n + LIST_FLUID);
+        append(solid, e, L.psl, L.list_n + LIST_SOLID);
     }
 }
 
@@ -608,7 +743,8 @@ __global__ void k_boundary_full(Lattice L, int inst)
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < I.N;
          n += (long long)gridDim.x * blockDim.x) {
         int x = (int)(n % I.nx), y = (int)((n / I.nx) % I.ny), z = (int)(n / ((long long)I.nx * I.ny));
-        set_boundary(L, I, x, y, z);
+        bool next;
+        set_boundary(L, I, x, y, z, -1, &next);
     }
 }
 
@@ -623,10 +759,10 @@ __global__ void k_boundary_full(Lattice L, int inst)
 // are phi (1 + F_i) exactly.  A neighbour's rho^a - rho^b is phi rho (its
 // colour offsets sum to phi (1 + sum w F)).
 //
-// Few nodes are uncovered per step (about the swept surface area), so the
-// kernel is a scan of the flags plus, per fresh node, one warp working on it:
-// lane i-1 takes neighbour i and issues its 19 population loads at once, the
-// sums meet in a shuffle reduction and lane i writes direction i.
+// Few nodes are uncovered per step (about the swept surface area): one warp
+// works on each listed one, lane i-1 takes neighbour i and issues its 19
+// population loads at once, the sums meet in a shuffle reduction and lane i
+// writes direction i.  The nodes newly covered get their solid mark.
 template <class R>
 __device__ __forceinline__ R warp_sum(R v)
 {
@@ -690,51 +826,40 @@ __device__ void refill_node(const InstDev &I, const PartDev *parts, const Pop<S>
     }
 }
 
+constexpr int REFILL_THREADS = 128, REFILL_CTAS = 64;
 template <class S>
-__global__ void __launch_bounds__(PART_THREADS) k_refill(Lattice L, int nxt, int side)
+__global__ void __launch_bounds__(REFILL_THREADS) k_refill(Lattice L, int nxt)
 {
     using R = typename Store<S>::real;
-    const PartDev &P0 = L.parts[blockIdx.y];
-    const InstDev &I = L.inst[P0.inst];
-    Region reg;
-    reg.init(P0.x, side, I.nx, I.ny, I.nz);
-    const Pop<S> pop(L.pop[nxt], I);
-    const uint8_t *fli = L.flags + I.node_off;
+    const long long nf = (long long)L.list_n[LIST_FRESH], nc = (long long)L.list_n[LIST_COVERED];
     const int lane = threadIdx.x & 31;
-    const long long count = reg.count();
-    // warp-uniform trip count: every lane takes part in the ballots
-    for (long long t0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < count;
-         t0 += (long long)gridDim.x * blockDim.x) {
-        const long long t = t0 + lane;
-        int x = 0, y = 0, z = 0;
-        bool fresh = false;
-        if (t < count) {
-            reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
-            fresh = (fli[(z * I.ny + y) * I.nx + x] & FRESH_BIT) != 0;
-        }
-        unsigned todo = __ballot_sync(0xffffffffu, fresh);
-        while (todo) {
-            const int src = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int X = __shfl_sync(0xffffffffu, x, src), Y = __shfl_sync(0xffffffffu, y, src),
-                      Z = __shfl_sync(0xffffffffu, z, src);
-            refill_node<S>(I, L.parts, pop, (R *)L.phi + I.node_off, col_slot<S>(L, I.node_off), fli, X, Y, Z,
-                           lane);
-        }
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for (long long k = warp; k < nf; k += (long long)gridDim.x * (REFILL_THREADS / 32)) {
+        const long long e = L.fresh[k];
+        const InstDev &I = L.inst[e >> 32];
+        const int n = (int)(unsigned)e, row = n / I.nx, z = row / I.ny;
+        refill_node<S>(I, L.parts, Pop<S>(L.pop[nxt], I), (R *)L.phi + I.node_off, col_slot<S>(L, I.node_off),
+                       L.flags + I.node_off, n - row * I.nx, row - z * I.ny, z, lane);
     }
+    if (sizeof(S) >= 4)
+        for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nc;
+             k += (long long)gridDim.x * blockDim.x) {
+            const long long e = L.covered[k];
+            set_solid_mark(((GradRec<R> *)L.grad)[L.inst[e >> 32].node_off + (unsigned)e]);
+        }
 }
 
 // initial particle marking: owner at the current positions, no fresh nodes
-__global__ void __launch_bounds__(PART_THREADS) k_mark(Lattice L, int side)
+__global__ void __launch_bounds__(PART_THREADS) k_mark(Lattice L, FastDiv fd)
 {
     const PartDev &P = L.parts[blockIdx.y];
     const InstDev &I = L.inst[P.inst];
     Region reg;
-    reg.init(P.x, side, I.nx, I.ny, I.nz);
+    reg.init(P.xf, (int)fd.d, I.nx, I.ny, I.nz);
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < reg.count();
          t += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
-        reg.coord(t, I.nx, I.ny, I.nz, &x, &y, &z);
+        reg.coord(t, fd, I.nx, I.ny, I.nz, &x, &y, &z);
         const long long g = I.node_off + ((long long)z * I.ny + y) * I.nx + x;
         const uint8_t old = L.flags[g];
         if (own_static(old & OWNER_MASK)) continue;
@@ -743,12 +868,19 @@ __global__ void __launch_bounds__(PART_THREADS) k_mark(Lattice L, int side)
 }
 
 // ---------------------------------------------------------------------------
+static FastDiv divide_by(int side)
+{
+    FastDiv fd;
+    fd.set((unsigned)side);
+    return fd;
+}
+
 template <class S>
 void launch_momentum_exchange(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk)
 {
     if (L.n_parts == 0) return;
     mk(STAGE_MEM, 0);
-    k_mem<S><<<dim3(L.mem_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, cur);
+    k_mem<S><<<dim3(L.mem_blocks, L.n_parts), MEM_THREADS, 0, st>>>(L, cur, divide_by(L.mem_side));
     mk(STAGE_MEM, 1);
     *launches += 1;
 }
@@ -768,10 +900,13 @@ void launch_capillary(const Lattice &L, cudaStream_t st, long long *launches, co
 }
 
 template <class S>
-void launch_particle_forces(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk)
+void launch_contacts(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk)
 {
-    launch_momentum_exchange<S>(L, cur, st, launches, mk);
-    launch_capillary<S>(L, st, launches, mk);
+    if (L.n_parts == 0) return;
+    mk(STAGE_CONTACTS, 0);
+    k_contacts<typename Store<S>::real><<<L.n_inst, CONTACT_THREADS, 0, st>>>(L);
+    mk(STAGE_CONTACTS, 1);
+    *launches += 1;
 }
 
 template <class S>
@@ -781,9 +916,9 @@ void launch_dem(const Lattice &L, cudaStream_t st, long long *launches, const Ma
     if (L.n_parts == 0) return;
     mk(STAGE_DEM, 0);
     if (L.buoyancy)
-        k_dem<R, true><<<L.n_inst, DEM_THREADS, 0, st>>>(L, sum_fluid ? 1 : 0);
+        k_dem<R, true><<<L.n_parts, 32, 0, st>>>(L, sum_fluid ? 1 : 0);
     else
-        k_dem<R, false><<<L.n_inst, DEM_THREADS, 0, st>>>(L, sum_fluid ? 1 : 0);
+        k_dem<R, false><<<L.n_parts, 32, 0, st>>>(L, sum_fluid ? 1 : 0);
     mk(STAGE_DEM, 1);
     *launches += 1;
 }
@@ -791,19 +926,19 @@ void launch_dem(const Lattice &L, cudaStream_t st, long long *launches, const Ma
 void launch_geom_owner(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk)
 {
     if (L.n_parts == 0) return;
-    // region sides: owner/refill cover the solid of the last two positions,
-    // the boundary pass one more node around
+    // region sides: the owner update covers the solid of the last two positions,
+    // the surface pass one more node around
     mk(STAGE_GEOM_OWNER, 0);
-    k_geom_owner<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, L.geom_side);
+    k_geom_owner<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, divide_by(L.geom_side));
     mk(STAGE_GEOM_OWNER, 1);
     *launches += 1;
 }
 
-void launch_geom_bound(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk)
+void launch_geom_surface(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk)
 {
     if (L.n_parts == 0) return;
     mk(STAGE_GEOM_BOUND, 0);
-    k_geom_bound<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, L.geom_side + 2);
+    k_geom_surface<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, divide_by(L.geom_side + 2), 0);
     mk(STAGE_GEOM_BOUND, 1);
     *launches += 1;
 }
@@ -813,25 +948,23 @@ void launch_refill(const Lattice &L, int nxt, cudaStream_t st, long long *launch
 {
     if (L.n_parts == 0) return;
     mk(STAGE_REFILL, 0);
-    k_refill<S><<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, nxt, L.geom_side);
+    k_refill<S><<<REFILL_CTAS, REFILL_THREADS, 0, st>>>(L, nxt);
     mk(STAGE_REFILL, 1);
     *launches += 1;
-}
-
-template <class S>
-void launch_geometry(const Lattice &L, int nxt, cudaStream_t st, long long *launches, const Marker &mk)
-{
-    launch_geom_owner(L, st, launches, mk);
-    launch_geom_bound(L, st, launches, mk);
-    launch_refill<S>(L, nxt, st, launches, mk);
 }
 
 void launch_mark_particles(const Lattice &L, cudaStream_t st)
 {
     if (L.n_parts == 0) return;
-    const int side = L.geom_side;
-    k_mark<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, side);
-    k_geom_bound<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, side + 2);
+    k_mark<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, divide_by(L.geom_side));
+    k_geom_surface<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, divide_by(L.geom_side + 2), 1);
+}
+
+void launch_first_lists(const Lattice &L, cudaStream_t st)
+{
+    if (L.n_parts == 0) return;
+    cudaMemsetAsync(L.list_n, 0, 4 * sizeof(unsigned long long), st);
+    k_geom_surface<<<dim3(L.geom_blocks, L.n_parts), PART_THREADS, 0, st>>>(L, divide_by(L.geom_side + 2), 0);
 }
 
 void launch_boundary_full(const Lattice &L, int inst, long long N, cudaStream_t st)
@@ -842,10 +975,9 @@ void launch_boundary_full(const Lattice &L, int inst, long long N, cudaStream_t 
 }
 
 #define INST(S)                                                                                             \
-    template void launch_particle_forces<S>(const Lattice &, int, cudaStream_t, long long *, const Marker &); \
     template void launch_momentum_exchange<S>(const Lattice &, int, cudaStream_t, long long *, const Marker &); \
     template void launch_capillary<S>(const Lattice &, cudaStream_t, long long *, const Marker &);           \
-    template void launch_geometry<S>(const Lattice &, int, cudaStream_t, long long *, const Marker &);     \
+    template void launch_contacts<S>(const Lattice &, cudaStream_t, long long *, const Marker &);            \
     template void launch_dem<S>(const Lattice &, cudaStream_t, long long *, const Marker &, bool);       \
     template void launch_refill<S>(const Lattice &, int, cudaStream_t, long long *, const Marker &);
 INST(double)

@@ -90,7 +90,7 @@ FORCE_RESOLVED, FORCE_SURROGATE = 0, 1
 FAULT_NONE, FAULT_GEMM_NO_COMMIT = 0, 1
 STAGES = ["phi", "solid_phi", "grad_wetting", "collide", "momentum_exchange", "capillary", "dem", "geom_owner",
           "geom_boundary", "refill", "fused", "particle_region", "curvature", "surrogate", "phi_boundary",
-          "collide_boundary"]
+          "collide_boundary", "contacts"]
 # the launch form of lbm_set_fluid_kernel
 FORM_PLAIN = 2
 
