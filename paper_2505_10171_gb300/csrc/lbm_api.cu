@@ -1829,8 +1829,7 @@ lbm_status lbm_surrogate_predict(lbm_ctx *ctx, const float *X, size_t n, float *
         float *Xd = nullptr, *Yd = nullptr;
         lbm_status s = upload_xy(ctx, X + r0 * MLP_NIN, nullptr, nb, &Xd, &Yd);
         if (s != LBM_OK) return s;
-        mlp_stage(ctx->mlp, Xd, nullptr, nullptr, 0, nb, ctx->stream);
-        CU(mlp_forward(ctx->mlp, nb, ctx->status, ctx->stream));
+        CU(mlp_forward(ctx->mlp, Xd, nb, ctx->status, ctx->stream));
         CU(cudaGetLastError());
         CU(cudaMemcpy2DAsync(Y + r0 * MLP_NOUT, sizeof(float) * MLP_NOUT, ctx->mlp.Y, sizeof(float) * 16,
                              sizeof(float) * MLP_NOUT, nb, cudaMemcpyDeviceToHost, ctx->stream));
@@ -1848,9 +1847,7 @@ lbm_status lbm_surrogate_gradient(lbm_ctx *ctx, const float *X, const float *Y, 
     float *Xd = nullptr, *Yd = nullptr;
     lbm_status s = upload_xy(ctx, X, Y, n, &Xd, &Yd);
     if (s != LBM_OK) return s;
-    mlp_stage(ctx->mlp, Xd, Yd, nullptr, 0, (int)n, ctx->stream);
-    CU(mlp_forward(ctx->mlp, (int)n, ctx->status, ctx->stream));
-    CU(mlp_backward(ctx->mlp, (int)n, nullptr, ctx->status, ctx->stream));
+    CU(mlp_gradient(ctx->mlp, Xd, Yd, nullptr, 0, (int)n, nullptr, ctx->status, ctx->stream));
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(grad, ctx->mlp.grad, sizeof(float) * MLP_NPARAM, cudaMemcpyDeviceToHost, ctx->stream));
     double l = 0.0;
@@ -1907,9 +1904,8 @@ lbm_status lbm_surrogate_train(lbm_ctx *ctx, const float *X, const float *Y, siz
         for (size_t b = 0; b < nb; b++) {
             const long long r0 = (long long)(b * batch);
             const int sz = (int)std::min<size_t>(batch, n - r0);
-            mlp_stage(ctx->mlp, ctx->trX, ctx->trY, ctx->perm, r0, sz, ctx->stream);
-            CU(mlp_forward(ctx->mlp, sz, ctx->status, ctx->stream));
-            CU(mlp_backward(ctx->mlp, sz, ctx->mlp.loss + 1, ctx->status, ctx->stream));
+            CU(mlp_gradient(ctx->mlp, ctx->trX, ctx->trY, ctx->perm, r0, sz, ctx->mlp.loss + 1, ctx->status,
+                            ctx->stream));
             mlp_adam(ctx->mlp, lr, ctx->stream);
         }
         CU(cudaGetLastError());

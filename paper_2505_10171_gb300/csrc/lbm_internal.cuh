@@ -858,7 +858,7 @@ struct Mlp {
     float *theta = nullptr, *grad = nullptr, *adam_m = nullptr, *adam_v = nullptr;  // [MLP_NPARAM]
     __nv_bfloat16 *W1b = nullptr, *W2b = nullptr, *W3b = nullptr;                   // BF16 operand copies
     __nv_bfloat16 *X = nullptr, *H1 = nullptr, *H2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dYb = nullptr;
-    float *Y = nullptr, *dY = nullptr, *T = nullptr;  // [cap][16], [cap][16], [cap][6]
+    float *Y = nullptr, *dY = nullptr;                // [cap][16]
     double *loss_part = nullptr, *loss = nullptr;     // loss[0]: last batch, loss[1]: accumulator
     int cap = 0;
     long long t = 0;  // Adam steps taken
@@ -867,11 +867,12 @@ struct Mlp {
 cudaError_t mlp_alloc(Mlp &m, int cap);
 void mlp_free(Mlp &m);
 void mlp_refresh(const Mlp &m, cudaStream_t st);
-// rows idx[row0 + r] (or row0 + r) of fp32 features [*][387] (and targets [*][6]) into the batch buffers
-void mlp_stage(const Mlp &m, const float *X, const float *Y, const long long *idx, long long row0, int n,
-               cudaStream_t st);
-cudaError_t mlp_forward(const Mlp &m, int n, unsigned *status, cudaStream_t st);
-cudaError_t mlp_backward(const Mlp &m, int n, double *acc, unsigned *status, cudaStream_t st);
+// outputs m.Y [n][16] (6 used) for device inputs X [n][387]
+cudaError_t mlp_forward(const Mlp &m, const float *X, int n, unsigned *status, cudaStream_t st);
+// loss and gradient of the rows idx[row0 + r] (or row0 + r), r < n, of X [*][387]
+// and T [*][6]; the loss is added to *acc where given
+cudaError_t mlp_gradient(const Mlp &m, const float *X, const float *T, const long long *idx, long long row0, int n,
+                         double *acc, unsigned *status, cudaStream_t st);
 void mlp_adam(Mlp &m, double lr, cudaStream_t st);
 template <class S>
 void launch_shell_features(const Lattice &L, int p0, int np, float *feat, cudaStream_t st);

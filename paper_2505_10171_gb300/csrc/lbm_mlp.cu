@@ -5,19 +5,26 @@
 // fifth-generation tensor cores: tcgen05.mma with the accumulator in tensor
 // memory, operands staged in shared memory, FP32 master weights, Adam.
 //
-// GEMM: C[m][n] = sum_k A(m,k) B(n,k), A(m,k) = A[m sam + k sak],
-// B(n,k) = B[n sbn + k sbk] (bf16; zero outside the valid extents), one CTA of
-// 128 threads per 128-row by BN-column tile.  Per 64-wide chunk of k the CTA
-// writes A (128 x 64) and B (BN x 64) into shared memory in the canonical
-// K-major layout without swizzle (8-row x 16-byte core matrices: along k
-// LBO apart, along rows 128 bytes apart), with 16-byte loads where the operand
-// is contiguous along k or along its rows; thread 0 issues four
-// tcgen05.mma.kind::f16 (K = 16 each) and commits them to the stage's
-// mbarrier.  Two stages: the chunk after is staged while the tensor core
-// works on the one before, and a stage is refilled only once the commit of the
-// chunk that read it has arrived (bounded waits).  The epilogue reads the FP32
-// accumulator with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31 = tile rows)
-// and applies bias, tanh or the tanh derivative.
+// The products are small (0.14 GFLOP forward for 1000 rows), so what they cost
+// is latency: launches, round trips to memory, and barriers.  Two kernels:
+//   k_mlp_rows   a CTA takes 128 rows through the whole network: inputs gathered
+//                and rounded to BF16 on the way into shared memory, the three
+//                layers with their activations, and in training the loss and
+//                both layers' deltas; weights and activations stay in shared
+//                memory from one product to the next;
+//   k_mlp_grads  the weight gradients (sums over the batch) with the bias
+//                gradients and the loss, a CTA per output tile.
+// One GEMM launch per product with operands staged 64 columns at a time by a
+// loop of dependent loads took 36 to 46 us each, 17 launches and 285 us a batch
+// of 512; these two and Adam take 32, 18 and 4 us.  An epoch of 20000 samples
+// 11.4 -> 2.5 ms, 512 predictions with their copies 132 -> 64 us, to the same bits.
+//
+// Shared-memory operands are in the canonical layout without swizzle: 8 x
+// 16-byte core matrices of 128 bytes.  Read K-major, a core matrix holds 8 rows
+// (M or N) of 8 k each; read MN-major, 8 k of 8 consecutive m or n each - the
+// same bytes serve a product with the operand and one with its transpose.
+// Descriptors give the distance between core matrices along k (leading) and
+// along M or N (stride).
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -92,185 +99,409 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
 
-// instruction descriptor of kind::f16: BF16 A and B (K-major), FP32 D,
-// M = 128, N = BN
-template <int BN>
+// instruction descriptor of kind::f16: BF16 A and B, FP32 D, M = 128, N = BN;
+// TA, TB: that operand is read MN-major
+template <int BN, bool TA = false, bool TB = false>
 __host__ __device__ constexpr uint32_t idesc_bf16()
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((TA ? 1u : 0u) << 15) | ((TB ? 1u : 0u) << 16) |
+           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
-constexpr int GM = 128;  // tile rows (TMEM lanes)
-constexpr int GK = 64;   // k per staged chunk
-#ifndef LBM_GEMM_BN
-#define LBM_GEMM_BN 64
-#endif
-constexpr int BNH = LBM_GEMM_BN;  // column tile of the GEMMs with 128 or more columns
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// shared memory: two barriers and the TMEM slot, then two stages of A and B.
-// A stage holds exactly its tile: the four MMAs of a chunk read core matrices
-// 2j LBO + {0, LBO} + 16 row groups x 128 bytes, j < 4, i.e. 8 LBO bytes.
-template <int BN>
-struct GemmSmem {
-    static constexpr int HEAD = 128;
-    static constexpr int A_LBO = GM / 8 * 128;  // bytes between core matrices along k
-    static constexpr int B_LBO = BN / 8 * 128;
-    static constexpr int A_STAGE = GM * GK * 2;
-    static constexpr int B_STAGE = BN * GK * 2;
-    static constexpr int BYTES = HEAD + 2 * (A_STAGE + B_STAGE);
-};
-static_assert(GemmSmem<128>::BYTES <= 227 * 1024, "two stages fit in shared memory");
+constexpr int GM = 128;        // rows of a tile (TMEM lanes)
+constexpr int MLP_THREADS = 256;   // gradients: two warps per quarter of the TMEM lanes
+constexpr int ROW_THREADS = 512;   // rows: four
 
-struct GemmArgs {
-    int Mv, Nv, Kv;  // valid extents
-    const bf16 *A;
-    long long sam, sak;
-    const bf16 *B;
-    long long sbn, sbk;
-    const float *bias;  // [n] or null
-    int act;            // 0: none, 1: tanh, 2: times (1 - g(m,n)^2)
-    const bf16 *g;
-    long long sgm, sgn;
-    float *C32;
-    long long scm, scn;
-    bf16 *C16;
-    long long s16m, s16n;
+// STEPS products of K = 16 each into tmem (the first one overwrites it where
+// fresh), issued and committed by one thread; a_step, b_step: bytes between
+// the k = 16 slices of the operands
+template <uint32_t IDESC, int STEPS>
+__device__ __forceinline__ void mma_steps(uint32_t tmem, uint32_t a, uint32_t a_lbo, uint32_t a_sbo, uint32_t a_step,
+                                          uint32_t b, uint32_t b_lbo, uint32_t b_sbo, uint32_t b_step, bool fresh,
+                                          uint32_t bar)
+{
+    tc_fence_after();
+#pragma unroll
+    for (int j = 0; j < STEPS; j++)
+        tc_mma_bf16(tmem, smem_desc(a + j * a_step, a_lbo, a_sbo), smem_desc(b + j * b_step, b_lbo, b_sbo), IDESC,
+                    fresh && j == 0 ? 0u : 1u);
+    tc_commit(bar);
+}
+
+__device__ __forceinline__ uint32_t pack2(float a, float b)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// ---------------------------------------------------------------------------
+// the network over rows
+// ---------------------------------------------------------------------------
+struct RowArgs {
+    const float *X;        // inputs [*][387]
+    const float *T;        // targets [*][6] (training)
+    const long long *idx;  // rows idx[row0 + r] of both, or row0 + r
+    long long row0;
+    int n;
+    const bf16 *W1, *W2, *W3;
+    const float *b1, *b2, *b3;
+    bf16 *Xb, *H1, *H2, *dZ1, *dZ2, *dYb;  // for the gradients (training)
+    float *Y, *dY;
+    double *loss_part;
     unsigned *status;
     int no_mma;            // fault injection: issue no MMA and no commit (the wait finds nothing arriving)
     long long wait_limit;  // clock cycles a wait on the commit barrier may take
 };
 
-// one chunk of rows r0.. (ROWS of them) and k0..k0+GK into the canonical
-// layout.  vec: 1 = the operand is contiguous along k (sk = 1), 2 = along its
-// rows (sr = 1), both with 16-byte aligned runs of 8 (checked by the caller):
-// runs of 8 elements wholly inside the valid extents move as one 16-byte load;
-// the rest element by element, zero outside the extents.
-template <int ROWS>
-__device__ __forceinline__ void stage_tile(const bf16 *P, long long sr, long long sk, int r0, int rv, int k0, int kv,
-                                           int vec, unsigned char *dst)
-{
-    auto at = [&](int r, int k) {
-        return (bf16 *)(dst + ((k >> 3) * (ROWS / 8) + (r >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2);
-    };
-    auto scalar8 = [&](int r, int k, int dr, int dk) {
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-            const int gr = r0 + r + e * dr, gk = k0 + k + e * dk;
-            bf16 v = __float2bfloat16_rn(0.0f);
-            if (gr < rv && gk < kv) v = P[(long long)gr * sr + (long long)gk * sk];
-            *at(r + e * dr, k + e * dk) = v;
-        }
-    };
-    if (vec == 1) {
-        // one core-matrix row (8 k values, 16 bytes) per vector
-        for (int i = threadIdx.x; i < ROWS * (GK / 8); i += GM) {
-            const int r = i / (GK / 8), k = (i % (GK / 8)) * 8;
-            const int gr = r0 + r, gk = k0 + k;
-            if (gr < rv && gk + 8 <= kv)
-                *(uint4 *)at(r, k) = *(const uint4 *)(P + (long long)gr * sr + gk);
-            else
-                scalar8(r, k, 0, 1);
-        }
-    } else if (vec == 2) {
-        // 8 rows at one k: a core-matrix column (consecutive threads take
-        // consecutive k, whose 2-byte stores share 32-bit words)
-        for (int i = threadIdx.x; i < (ROWS / 8) * GK; i += GM) {
-            const int r = (i / GK) * 8, k = i % GK;
-            const int gr = r0 + r, gk = k0 + k;
-            if (gr + 8 <= rv && gk < kv) {
-                const uint4 w = *(const uint4 *)(P + gr + (long long)gk * sk);
-                const bf16 *h = (const bf16 *)&w;
-#pragma unroll
-                for (int e = 0; e < 8; e++) *at(r + e, k) = h[e];
-            } else {
-                scalar8(r, k, 1, 0);
-            }
-        }
-    } else {
-        for (int i = threadIdx.x; i < ROWS * GK; i += GM) {
-            const int r = i / GK, k = i % GK;
-            const int gr = r0 + r, gk = k0 + k;
-            bf16 v = __float2bfloat16_rn(0.0f);
-            if (gr < rv && gk < kv) v = P[(long long)gr * sr + (long long)gk * sk];
-            *at(r, k) = v;
-        }
-    }
-}
+// shared memory: barrier, TMEM slot and biases; the input tile, whose place the
+// activations and deltas take over; W1, whose place W2 takes over; W3
+struct RowSmem {
+    static constexpr int BIAS = 128;                      // b1[128], b2[128], b3[16]
+    static constexpr int RED = BIAS + 4 * (128 + 128 + 16);
+    static constexpr int XA = 2048;
+    static constexpr int X_BYTES = GM * MLP_KIN * 2;
+    static constexpr int TILE = GM * MLP_HIDDEN * 2;      // 128 x 128
+    static constexpr int H1 = XA, H2 = XA + TILE, DZ2 = XA + 2 * TILE, DY = XA + 3 * TILE;  // DY: 128 x 16
+    static constexpr int WB = XA + X_BYTES;
+    static constexpr int W3 = WB + MLP_HIDDEN * MLP_KIN * 2;
+    static constexpr int BYTES = W3 + 16 * MLP_HIDDEN * 2;
+};
+static_assert(RowSmem::RED + 64 <= RowSmem::XA && RowSmem::DY + GM * 32 <= RowSmem::WB, "regions");
+static_assert(RowSmem::BYTES <= 227 * 1024, "shared memory of a CTA");
 
-// which staging path an operand takes (the same for every thread of the grid)
-__device__ __forceinline__ int vec_mode(const bf16 *P, long long sr, long long sk)
-{
-    if (((uintptr_t)P & 15) != 0) return 0;
-    if (sk == 1 && sr % 8 == 0) return 1;
-    if (sr == 1 && sk % 8 == 0) return 2;
-    return 0;
-}
+// 128 rows of core matrices: bytes between neighbours along k and along rows
+constexpr uint32_t T_LBO = GM / 8 * 128, T_SBO = 128;
 
-template <int BN>
-__global__ void __launch_bounds__(GM) k_gemm_tc(GemmArgs g)
+template <bool TRAIN>
+__global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
 {
-    using Sm = GemmSmem<BN>;
-    extern __shared__ __align__(1024) unsigned char gsm[];
-    // stage st: A at As0 + st A_STAGE, B at Bs0 + st B_STAGE, barrier bar0 + 8 st
-    unsigned char *const As0 = gsm + Sm::HEAD;
-    unsigned char *const Bs0 = gsm + Sm::HEAD + 2 * Sm::A_STAGE;
-    const uint32_t bar0 = smem_addr(gsm);
-    const uint32_t slot = smem_addr(gsm + 16);
+    using Sm = RowSmem;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    const uint32_t base = smem_addr(sm), bar = base, slot = base + 16;
+    float *const bias = (float *)(sm + Sm::BIAS);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * GM, n0 = blockIdx.y * BN;
-    constexpr uint32_t NCOLS = BN < 32 ? 32 : BN;
+    const int r0 = blockIdx.x * GM;
+    constexpr uint32_t NCOLS = 256;
 
     if (warp == 0) {
         tmem_alloc(slot, NCOLS);
         tmem_relinquish();
     }
     if (tid == 0) {
-        mbar_init(bar0, 1);
-        mbar_init(bar0 + 8, 1);
+        mbar_init(bar, 1);
+        mbar_fence_init();
+    }
+    // W1 (row-major, 16 bytes at a time) and W3 (rows 6..15 zero)
+    for (int i = tid; i < MLP_HIDDEN * (MLP_KIN / 8); i += ROW_THREADS) {
+        const int r = i & 127, kb = i >> 7;
+        cp_async16(base + Sm::WB + (kb * 16 + (r >> 3)) * 128 + (r & 7) * 16, g.W1 + r * MLP_KIN + kb * 8);
+    }
+    if (tid < 256) {
+        const int r = tid & 15, kb = tid >> 4;
+        unsigned char *d = sm + Sm::W3 + (kb * 2 + (r >> 3)) * 128 + (r & 7) * 16;
+        *(uint4 *)d = r < MLP_NOUT ? *(const uint4 *)(g.W3 + r * MLP_HIDDEN + kb * 8) : make_uint4(0, 0, 0, 0);
+    }
+    if (tid < 128) {
+        bias[tid] = g.b1[tid];
+        bias[128 + tid] = g.b2[tid];
+        if (tid < 16) bias[256 + tid] = tid < MLP_NOUT ? g.b3[tid] : 0.0f;
+    }
+    // inputs: a warp takes 8 rows, four at a time, with all loads of the four in flight
+    {
+        constexpr int NC = (MLP_KIN + 31) / 32;
+        for (int rr = warp * 8; rr < warp * 8 + 8; rr += 4) {
+            float v[4][NC];
+#pragma unroll
+            for (int h = 0; h < 4; h++) {
+                const int r = r0 + rr + h;
+                const bool have = r < g.n;
+                const long long src = have ? (g.idx ? g.idx[g.row0 + r] : g.row0 + r) : 0;
+                const float *x = g.X + src * MLP_NIN;
+#pragma unroll
+                for (int j = 0; j < NC; j++) {
+                    const int k = lane + 32 * j;
+                    v[h][j] = have && k < MLP_NIN ? x[k] : 0.0f;
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 4; h++) {
+                const int r = rr + h;
+#pragma unroll
+                for (int j = 0; j < NC; j++) {
+                    const int k = lane + 32 * j;
+                    if (k >= MLP_KIN) continue;
+                    const bf16 b = __float2bfloat16_rn(v[h][j]);
+                    *(bf16 *)(sm + Sm::XA + ((k >> 3) * 16 + (r >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2) = b;
+                    if (TRAIN && r0 + r < g.n) g.Xb[(long long)(r0 + r) * MLP_KIN + k] = b;
+                }
+            }
+        }
+    }
+    cp_async_wait();
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *(volatile uint32_t *)(sm + 16);
+    const uint32_t d1 = tmem, d2 = tmem + 128;
+
+    unsigned phase = 0;
+    bool ok = true;
+    // every thread waits for the products committed last; false once a wait gave up
+    auto wait = [&]() {
+        ok = mbar_wait_bounded(bar, phase & 1, g.wait_limit);
+        phase++;
+        ok = !__syncthreads_or(!ok);
+        tc_fence_after();
+        return ok;
+    };
+    const bool issuer = tid == 0 && !g.no_mma;
+    // this thread's row of a tile and its quarter of 128 columns
+    const int row = (warp & 3) * 32 + lane, col0 = (warp >> 2) * 32;
+    const bool have = r0 + row < g.n;
+    const uint32_t quarter = (uint32_t)((warp & 3) * 32) << 16;
+    // the epilogue of a 128 x 128 product: f(column, value) rounded to BF16, into
+    // the shared-memory tile at `tile` and, in training, row-major to `out`
+    auto epilogue = [&](uint32_t d, int tile, bf16 *out, auto &&f) {
+#pragma unroll 1
+        for (int c0 = col0; c0 < col0 + 32; c0 += 16) {
+            float v[16];
+            tmem_ld16(d + quarter + (uint32_t)c0, v);
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                uint32_t w[4];
+#pragma unroll
+                for (int e = 0; e < 4; e++)
+                    w[e] = pack2(f(c0 + 8 * q + 2 * e, v[8 * q + 2 * e]), f(c0 + 8 * q + 2 * e + 1, v[8 * q + 2 * e + 1]));
+                const uint4 o = make_uint4(w[0], w[1], w[2], w[3]);
+                const int kb = (c0 >> 3) + q;
+                if (tile >= 0) *(uint4 *)(sm + tile + (kb * 16 + (row >> 3)) * 128 + (row & 7) * 16) = o;
+                if (TRAIN && out && have) *(uint4 *)(out + (long long)(r0 + row) * MLP_HIDDEN + kb * 8) = o;
+            }
+        }
+    };
+    auto ready = [&]() {  // shared-memory writes of all threads before the next products
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+    };
+    // BF16 value (row, column c) of a tile
+    auto tile_at = [&](int tile, int c) {
+        return __bfloat162float(*(const bf16 *)(sm + tile + ((c >> 3) * 16 + (row >> 3)) * 128 + (row & 7) * 16 + (c & 7) * 2));
+    };
+
+    do {
+        // h1 = tanh(X W1^T + b1)
+        if (issuer)
+            mma_steps<idesc_bf16<128>(), MLP_KIN / 16>(d1, base + Sm::XA, T_LBO, T_SBO, 2 * T_LBO, base + Sm::WB, T_LBO,
+                                                       T_SBO, 2 * T_LBO, true, bar);
+        if (!wait()) break;
+        for (int i = tid; i < MLP_HIDDEN * (MLP_HIDDEN / 8); i += ROW_THREADS) {
+            const int r = i & 127, kb = i >> 7;
+            cp_async16(base + Sm::WB + (kb * 16 + (r >> 3)) * 128 + (r & 7) * 16, g.W2 + r * MLP_HIDDEN + kb * 8);
+        }
+        epilogue(d1, Sm::H1, g.H1, [&](int c, float v) { return tanhf(v + bias[c]); });
+        cp_async_wait();
+        ready();
+        // h2 = tanh(h1 W2^T + b2)
+        if (issuer)
+            mma_steps<idesc_bf16<128>(), MLP_HIDDEN / 16>(d2, base + Sm::H1, T_LBO, T_SBO, 2 * T_LBO, base + Sm::WB, T_LBO,
+                                                          T_SBO, 2 * T_LBO, true, bar);
+        if (!wait()) break;
+        epilogue(d2, Sm::H2, g.H2, [&](int c, float v) { return tanhf(v + bias[128 + c]); });
+        ready();
+        // y = h2 W3^T + b3
+        if (issuer)
+            mma_steps<idesc_bf16<16>(), MLP_HIDDEN / 16>(d1, base + Sm::H2, T_LBO, T_SBO, 2 * T_LBO, base + Sm::W3, 256,
+                                                         T_SBO, 512, true, bar);
+        if (!wait()) break;
+        double e2 = 0.0;
+        if (warp < 4) {
+            float v[16], d[8];
+            tmem_ld16(d1 + quarter, v);
+#pragma unroll
+            for (int c = 0; c < 8; c++) d[c] = 0.0f;
+            if (have) {
+                const long long src = TRAIN ? (g.idx ? g.idx[g.row0 + r0 + row] : g.row0 + r0 + row) : 0;
+#pragma unroll
+                for (int c = 0; c < MLP_NOUT; c++) {
+                    const float y = v[c] + bias[256 + c];
+                    g.Y[(long long)(r0 + row) * 16 + c] = y;
+                    if (TRAIN) {
+                        const float diff = y - g.T[src * MLP_NOUT + c];
+                        e2 += (double)diff * diff;
+                        d[c] = 2.0f * diff / (float)(MLP_NOUT * g.n);
+                    }
+                }
+            }
+            if (TRAIN) {
+                // dY = 2 (Y - T)/(6 n), 16 columns of which 6 count
+                const uint4 o = make_uint4(pack2(d[0], d[1]), pack2(d[2], d[3]), pack2(d[4], d[5]), 0);
+                const uint4 zero = make_uint4(0, 0, 0, 0);
+                unsigned char *t = sm + Sm::DY + (row >> 3) * 128 + (row & 7) * 16;
+                *(uint4 *)t = o;
+                *(uint4 *)(t + T_LBO) = zero;
+                if (have) {
+                    uint4 *p = (uint4 *)(g.dYb + (long long)(r0 + row) * 16);
+                    p[0] = o;
+                    p[1] = zero;
+#pragma unroll
+                    for (int c = 0; c < MLP_NOUT; c++) g.dY[(long long)(r0 + row) * 16 + c] = d[c];
+                }
+            }
+        }
+        if constexpr (TRAIN) {
+            // squared error of the tile: lanes, then warps 0..3, in a fixed order
+            for (int o = 16; o > 0; o >>= 1) e2 += __shfl_down_sync(0xffffffffu, e2, o);
+            double *const red = (double *)(sm + Sm::RED);
+            if (lane == 0 && warp < 4) red[warp] = e2;
+            ready();
+            if (tid == 0) g.loss_part[blockIdx.x] = ((red[0] + red[1]) + red[2]) + red[3];
+            // dz2 = (dY W3) (1 - h2^2): W3 read MN-major, n its columns, k its rows
+            if (issuer)
+                mma_steps<idesc_bf16<128, false, true>(), 1>(d2, base + Sm::DY, T_LBO, T_SBO, 0, base + Sm::W3, 128, 256, 0,
+                                                             true, bar);
+            if (!wait()) break;
+            epilogue(d2, Sm::DZ2, g.dZ2, [&](int c, float v) {
+                const float h = tile_at(Sm::H2, c);
+                return v * (1.0f - h * h);
+            });
+            ready();
+            // dz1 = (dz2 W2) (1 - h1^2): W2 read MN-major
+            if (issuer)
+                mma_steps<idesc_bf16<128, false, true>(), MLP_HIDDEN / 16>(d1, base + Sm::DZ2, T_LBO, T_SBO, 2 * T_LBO,
+                                                                           base + Sm::WB, 128, T_LBO, 256, true, bar);
+            if (!wait()) break;
+            epilogue(d1, -1, g.dZ1, [&](int c, float v) {
+                const float h = tile_at(Sm::H1, c);
+                return v * (1.0f - h * h);
+            });
+        }
+    } while (false);
+    if (!ok && tid == 0) {
+        atomicOr(g.status, ST_TIMEOUT);
+        // MMAs still in flight (none are issued under the fault injection) must
+        // finish before the tensor memory is freed
+        if (!g.no_mma) mbar_wait_bounded(bar, (phase - 1) & 1);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, NCOLS);
+}
+
+// ---------------------------------------------------------------------------
+// weight gradients: C[m][n] = sum_b A[b][m] B[b][n] over the batch, A and B
+// row-major BF16: both operands are read MN-major, so that their rows go into
+// shared memory as they lie, 16 bytes at a time.  A chunk of 64 rows per
+// stage, two stages; the next chunk's loads are in flight while the tensor core
+// works, and a stage is refilled only once the commit of the chunk that read it
+// has arrived (bounded waits).
+// ---------------------------------------------------------------------------
+struct GradArgs {
+    int n;
+    const bf16 *Xb, *H1, *H2, *dZ1, *dZ2, *dYb;
+    const float *dY;
+    float *grad;
+    const double *loss_part;
+    int parts;
+    double *loss, *acc;  // *loss: the batch's; added to *acc where given
+    unsigned *status;
+    int no_mma;
+    long long wait_limit;
+};
+
+constexpr int GB = 64;  // batch rows per chunk
+constexpr int GN = 64;  // columns of an output tile
+constexpr int GRAD_W1 = (MLP_KIN + GN - 1) / GN, GRAD_W2 = MLP_HIDDEN / GN;  // tiles of dW1 and dW2
+constexpr int GRAD_TILES = GRAD_W1 + GRAD_W2 + 1;                            // and one of dW3
+constexpr int GRAD_CTAS = GRAD_TILES + 2 * MLP_HIDDEN + MLP_NOUT + 1;        // bias sums, loss
+
+struct GradSmem {
+    static constexpr int HEAD = 128;
+    static constexpr int A_STAGE = GB * GM * 2, B_STAGE = GB * GN * 2;
+    static constexpr int BYTES = HEAD + 2 * (A_STAGE + B_STAGE);
+};
+
+// one tile: BN columns from n0 of B (ldb apart per row, nb 16-byte groups of it valid)
+template <int BN>
+__device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, const bf16 *A, const bf16 *B, int ldb, int n0,
+                                          int nb, float *C, long long scm, long long scn, int ncols)
+{
+    using Sm = GradSmem;
+    const uint32_t base = smem_addr(sm), slot = base + 16;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t NCOLS = BN < 32 ? 32 : BN;
+    constexpr int VA = GB * GM / 8 / MLP_THREADS;                       // 16-byte loads of A a thread
+    constexpr int NB8 = BN / 8, VB = (GB * NB8 + MLP_THREADS - 1) / MLP_THREADS;
+    if (warp == 0) {
+        tmem_alloc(slot, NCOLS);
+        tmem_relinquish();
+    }
+    if (tid == 0) {
+        mbar_init(base, 1);
+        mbar_init(base + 8, 1);
         mbar_fence_init();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *(volatile uint32_t *)(gsm + 16);
-    const int va = vec_mode(g.A, g.sam, g.sak), vb = vec_mode(g.B, g.sbn, g.sbk);
-
-    // chunk c uses stage c & 1 and commits to that stage's barrier, whose
-    // phases complete in chunk order, the one of chunk c having parity
-    // (c >> 1) & 1, and at most one of its phases is ever pending
-    const int nchunks = (g.Kv + GK - 1) / GK;
+    const uint32_t tmem = *(volatile uint32_t *)(sm + 16);
+    // vector i of a chunk: core matrix (k group, m group), row b of 8 in it; the
+    // shared-memory place is 16 i
+    uint4 va[VA], vb[VB];
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    auto fetch = [&](int c) {
+#pragma unroll
+        for (int q = 0; q < VA; q++) {
+            const int i = tid + q * MLP_THREADS, b = c * GB + (i >> 7) * 8 + (i & 7), mb = (i >> 3) & 15;
+            va[q] = b < g.n ? *(const uint4 *)(A + (long long)b * MLP_HIDDEN + mb * 8) : zero;
+        }
+#pragma unroll
+        for (int q = 0; q < VB; q++) {
+            const int i = tid + q * MLP_THREADS, kb = i / (8 * NB8), b = c * GB + kb * 8 + (i & 7), j = (i >> 3) % NB8;
+            vb[q] = i < GB * NB8 && b < g.n && j < nb ? *(const uint4 *)(B + (long long)b * ldb + n0 + j * 8) : zero;
+        }
+    };
+    const int nchunks = (g.n + GB - 1) / GB;
     bool ok = true;
-    int last = -1;  // last chunk whose MMAs were committed
+    int last = -1;
+    fetch(0);
     for (int c = 0; c < nchunks; c++) {
         const int st = c & 1;
         if (c >= 2) {
             // the MMAs of chunk c - 2 read this stage
-            ok = mbar_wait_bounded(bar0 + 8 * st, (unsigned)(((c - 2) >> 1) & 1), g.wait_limit);
-            if (__syncthreads_or(!ok)) break;
+            ok = mbar_wait_bounded(base + 8 * st, (unsigned)(((c - 2) >> 1) & 1), g.wait_limit);
+            if (__syncthreads_or(!ok)) {
+                ok = false;
+                break;
+            }
             tc_fence_after();
         }
-        unsigned char *const As = As0 + st * Sm::A_STAGE;
-        unsigned char *const Bs = Bs0 + st * Sm::B_STAGE;
-        stage_tile<GM>(g.A, g.sam, g.sak, m0, g.Mv, c * GK, g.Kv, va, As);
-        stage_tile<BN>(g.B, g.sbn, g.sbk, n0, g.Nv, c * GK, g.Kv, vb, Bs);
+        unsigned char *const As = sm + Sm::HEAD + st * Sm::A_STAGE;
+        unsigned char *const Bs = sm + Sm::HEAD + 2 * Sm::A_STAGE + st * Sm::B_STAGE;
+#pragma unroll
+        for (int q = 0; q < VA; q++) *(uint4 *)(As + (tid + q * MLP_THREADS) * 16) = va[q];
+#pragma unroll
+        for (int q = 0; q < VB; q++)
+            if (tid + q * MLP_THREADS < GB * NB8) *(uint4 *)(Bs + (tid + q * MLP_THREADS) * 16) = vb[q];
+        if (c + 1 < nchunks) fetch(c + 1);
         fence_async_smem();
         __syncthreads();
-        if (tid == 0 && !g.no_mma) {
-            tc_fence_after();
-#pragma unroll
-            for (int j = 0; j < GK / 16; j++) {
-                const uint64_t ad = smem_desc(smem_addr(As) + j * 2 * Sm::A_LBO, Sm::A_LBO, 128);
-                const uint64_t bd = smem_desc(smem_addr(Bs) + j * 2 * Sm::B_LBO, Sm::B_LBO, 128);
-                tc_mma_bf16(tmem, ad, bd, idesc_bf16<BN>(), (c > 0 || j > 0) ? 1u : 0u);
-            }
-            tc_commit(bar0 + 8 * st);
-        }
+        if (tid == 0 && !g.no_mma)
+            mma_steps<idesc_bf16<BN, true, true>(), GB / 16>(tmem, smem_addr(As), 2048, 128, 4096, smem_addr(Bs),
+                                                             NB8 * 128, 128, 2 * NB8 * 128, c == 0, base + 8 * st);
         last = c;
     }
     // a commit covers every MMA this thread issued before it: the last one's
     // arrival means the accumulator is complete
     if (ok && last >= 0) {
-        ok = mbar_wait_bounded(bar0 + 8 * (last & 1), (unsigned)((last >> 1) & 1), g.wait_limit);
+        ok = mbar_wait_bounded(base + 8 * (last & 1), (unsigned)((last >> 1) & 1), g.wait_limit);
         ok = !__syncthreads_or(!ok);
         tc_fence_after();
     }
@@ -279,31 +510,16 @@ __global__ void __launch_bounds__(GM) k_gemm_tc(GemmArgs g)
             atomicOr(g.status, ST_TIMEOUT);
             // MMAs still in flight (none are issued under the fault injection)
             // must finish before the tensor memory is freed
-            if (!g.no_mma && last >= 0) mbar_wait_bounded(bar0 + 8 * (last & 1), (unsigned)((last >> 1) & 1));
+            if (!g.no_mma && last >= 0) mbar_wait_bounded(base + 8 * (last & 1), (unsigned)((last >> 1) & 1));
         }
-    } else if (nchunks > 0) {
-        const int m = m0 + warp * 32 + lane;
-#pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
+    } else if (warp < 4 || BN > 16) {
+        const int m = (warp & 3) * 32 + lane;
+        for (int c0 = (warp >> 2) * (BN / 2); c0 < (BN > 16 ? (warp >> 2) * (BN / 2) + BN / 2 : 16); c0 += 16) {
             float v[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-            if (m < g.Mv) {
+            tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-                for (int i = 0; i < 16; i++) {
-                    const int n = n0 + c0 + i;
-                    if (n >= g.Nv) break;
-                    float x = v[i];
-                    if (g.bias) x += g.bias[n];
-                    if (g.act == 1) {
-                        x = tanhf(x);
-                    } else if (g.act == 2) {
-                        const float h = __bfloat162float(g.g[(long long)m * g.sgm + (long long)n * g.sgn]);
-                        x *= 1.0f - h * h;
-                    }
-                    if (g.C32) g.C32[(long long)m * g.scm + (long long)n * g.scn] = x;
-                    if (g.C16) g.C16[(long long)m * g.s16m + (long long)n * g.s16n] = __float2bfloat16_rn(x);
-                }
-            }
+            for (int i = 0; i < 16; i++)
+                if (c0 + i < ncols) C[m * scm + (c0 + i) * scn] = v[i];
         }
     }
     tc_fence_before();
@@ -311,12 +527,71 @@ __global__ void __launch_bounds__(GM) k_gemm_tc(GemmArgs g)
     if (warp == 0) tmem_dealloc(tmem, NCOLS);
 }
 
-// k_gemm_tc<BN> needs more than 48 KiB of dynamic shared memory, a function
+// column sum in a fixed order (bias gradients)
+template <class T>
+__device__ __forceinline__ void column_sum(const T *src, int rows, int ld, float *sh, float *out)
+{
+    float s = 0.0f;
+    for (int r = threadIdx.x; r < rows; r += MLP_THREADS) s += (float)src[(long long)r * ld];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int k = MLP_THREADS / 2; k > 0; k >>= 1) {
+        if ((int)threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *out = sh[0];
+}
+
+__global__ void __launch_bounds__(MLP_THREADS) k_mlp_grads(GradArgs g)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    int t = blockIdx.x;
+    if (t < GRAD_W1) {  // dW1[o][i] = sum_b dz1[b][o] x[b][i]
+        const int n0 = t * GN, left = MLP_KIN - n0;
+        grad_tile<GN>(g, sm, g.dZ1, g.Xb, MLP_KIN, n0, left / 8, g.grad + MLP_OFF_W1 + n0, MLP_KIN, 1, left);
+        return;
+    }
+    t -= GRAD_W1;
+    if (t < GRAD_W2) {  // dW2[o][i] = sum_b dz2[b][o] h1[b][i]
+        const int n0 = t * GN;
+        grad_tile<GN>(g, sm, g.dZ2, g.H1, MLP_HIDDEN, n0, GN / 8, g.grad + MLP_OFF_W2 + n0, MLP_HIDDEN, 1, GN);
+        return;
+    }
+    t -= GRAD_W2;
+    if (t == 0) {  // dW3[j][i] = sum_b dY[b][j] h2[b][i]  (M = hidden i, N = output j)
+        grad_tile<16>(g, sm, g.H2, g.dYb, 16, 0, 2, g.grad + MLP_OFF_W3, 1, MLP_HIDDEN, MLP_NOUT);
+        return;
+    }
+    t -= 1;
+    float *const sh = (float *)sm;
+    if (t < MLP_HIDDEN) {
+        column_sum(g.dZ1 + t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B1 + t);
+        return;
+    }
+    t -= MLP_HIDDEN;
+    if (t < MLP_HIDDEN) {
+        column_sum(g.dZ2 + t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B2 + t);
+        return;
+    }
+    t -= MLP_HIDDEN;
+    if (t < MLP_NOUT) {
+        column_sum(g.dY + t, g.n, 16, sh, g.grad + MLP_OFF_B3 + t);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int i = 0; i < g.parts; i++) s += g.loss_part[i];
+        const double l = s / ((double)g.n * MLP_NOUT);
+        *g.loss = l;
+        if (g.acc) *g.acc += l;
+    }
+}
+
+// these kernels need more than 48 KiB of dynamic shared memory, a function
 // attribute of each device: set once per device (under a lock, since
 // contexts on several threads may reach here first together), with its result
 // checked, before the first launch there
-template <int BN>
-static cudaError_t gemm_setup()
+cudaError_t mlp_setup()
 {
     constexpr int MAXDEV = 64;
     static std::mutex mu;
@@ -327,43 +602,41 @@ static cudaError_t gemm_setup()
     if (dev < 0 || dev >= MAXDEV) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(k_gemm_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmSmem<BN>::BYTES);
-    if (e == cudaSuccess) done[dev] = true;
+    const auto size = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((e = cudaFuncSetAttribute(k_mlp_rows<false>, size, RowSmem::BYTES)) == cudaSuccess &&
+        (e = cudaFuncSetAttribute(k_mlp_rows<true>, size, RowSmem::BYTES)) == cudaSuccess &&
+        (e = cudaFuncSetAttribute(k_mlp_grads, size, GradSmem::BYTES)) == cudaSuccess)
+        done[dev] = true;
     return e;
 }
 
-// returns the set-up's or this launch's own error
-template <int BN>
-cudaError_t gemm(const GemmArgs &a, int M, int N, cudaStream_t st)
+// the row kernel's arguments; under the network's fault-injection setting no
+// MMA is issued and the commit barrier is never signalled, so the bounded wait
+// (shortened to about a millisecond) runs out and reports a timeout
+RowArgs row_args(const Mlp &m, const float *X, const float *T, const long long *idx, long long row0, int n,
+                 unsigned *status)
 {
-    const cudaError_t e = gemm_setup<BN>();
-    if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((M + GM - 1) / GM), (unsigned)((N + BN - 1) / BN));
-    void *args[] = {(void *)&a};
-    return cudaLaunchKernel((const void *)k_gemm_tc<BN>, grid, dim3(GM), args, GemmSmem<BN>::BYTES, st);
-}
-
-GemmArgs gargs(int Mv, int Nv, int Kv, const bf16 *A, long long sam, long long sak, const bf16 *B, long long sbn,
-               long long sbk, unsigned *status)
-{
-    GemmArgs a;
+    RowArgs a;
     memset(&a, 0, sizeof a);
-    a.Mv = Mv; a.Nv = Nv; a.Kv = Kv;
-    a.A = A; a.sam = sam; a.sak = sak;
-    a.B = B; a.sbn = sbn; a.sbk = sbk;
+    a.X = X; a.T = T; a.idx = idx; a.row0 = row0; a.n = n;
+    a.W1 = m.W1b; a.W2 = m.W2b; a.W3 = m.W3b;
+    a.b1 = m.theta + MLP_OFF_B1; a.b2 = m.theta + MLP_OFF_B2; a.b3 = m.theta + MLP_OFF_B3;
+    a.Xb = m.X; a.H1 = m.H1; a.H2 = m.H2; a.dZ1 = m.dZ1; a.dZ2 = m.dZ2; a.dYb = m.dYb;
+    a.Y = m.Y; a.dY = m.dY; a.loss_part = m.loss_part;
     a.status = status;
-    a.wait_limit = WAIT_CYCLES;
+    a.no_mma = m.fault_no_commit ? 1 : 0;
+    a.wait_limit = m.fault_no_commit ? 1ll << 21 : WAIT_CYCLES;
     return a;
 }
 
-// the GEMM arguments under the network's fault-injection setting: with it on,
-// no MMA is issued and the commit barrier is never signalled, so the bounded
-// wait (shortened to about a millisecond) runs out and reports a timeout
-static GemmArgs mode(GemmArgs a, const Mlp &m)
+// launched through cudaLaunchKernel: the set-up's or this launch's own error
+template <class A>
+cudaError_t mlp_launch(void (*kernel)(A), int ctas, int threads, int bytes, const A &a, cudaStream_t st)
 {
-    a.no_mma = m.fault_no_commit ? 1 : 0;
-    if (a.no_mma) a.wait_limit = 1ll << 21;
-    return a;
+    const cudaError_t e = mlp_setup();
+    if (e != cudaSuccess) return e;
+    void *args[] = {(void *)&a};
+    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)ctas), dim3((unsigned)threads), args, (size_t)bytes, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -380,84 +653,9 @@ __global__ void k_refresh(const float *theta, bf16 *W1b, bf16 *W2b, bf16 *W3b)
     if (i < MLP_NOUT * MLP_HIDDEN) W3b[i] = __float2bfloat16_rn(theta[MLP_OFF_W3 + i]);
 }
 
-// rows idx[r] (or r) of fp32 features [*][387] -> bf16 inputs [n][400]
-__global__ void k_stage_inputs(const float *X, const long long *idx, long long row0, int n, bf16 *Xb)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)n * MLP_KIN) return;
-    const int r = (int)(t / MLP_KIN), c = (int)(t % MLP_KIN);
-    const long long src = idx ? idx[row0 + r] : row0 + r;
-    Xb[t] = __float2bfloat16_rn(c < MLP_NIN ? X[src * MLP_NIN + c] : 0.0f);
-}
-
-// targets of the batch rows -> T [n][6]
-__global__ void k_stage_targets(const float *Y, const long long *idx, long long row0, int n, float *T)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n * MLP_NOUT) return;
-    const int r = t / MLP_NOUT, c = t % MLP_NOUT;
-    const long long src = idx ? idx[row0 + r] : row0 + r;
-    T[t] = Y[src * MLP_NOUT + c];
-}
-
-// dY = 2 (Y - T) / (6 n) (fp32 and bf16, ld 16 with zero columns 6..15),
-// per-block partial sums of the squared error in FP64
-__global__ void k_loss(const float *Y, const float *T, int n, float *dY, bf16 *dYb, double *part)
-{
-    __shared__ double sh[EW];
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    double e2 = 0.0;
-    if (t < n * 16) {
-        const int r = t / 16, c = t % 16;
-        float d = 0.0f;
-        if (c < MLP_NOUT) {
-            const float diff = Y[r * 16 + c] - T[r * MLP_NOUT + c];
-            e2 = (double)diff * diff;
-            d = 2.0f * diff / (float)(MLP_NOUT * n);
-        }
-        dY[t] = d;
-        dYb[t] = __float2bfloat16_rn(d);
-    }
-    sh[threadIdx.x] = e2;
-    __syncthreads();
-    for (int s = EW / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-// loss of the batch: fixed-order sum of the block partials; optionally added
-// to an accumulator
-__global__ void k_loss_final(const double *part, int nblk, int n, double *loss, double *acc)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0;
-    for (int i = 0; i < nblk; i++) s += part[i];
-    const double l = s / ((double)n * MLP_NOUT);
-    *loss = l;
-    if (acc) *acc += l;
-}
-
-// column sums (bias gradients): out[c] = sum_r src[r ld + c], one block per column
-template <class T>
-__global__ void k_colsum(const T *src, int rows, int ld, float *out)
-{
-    __shared__ float sh[EW];
-    const int c = blockIdx.x;
-    float s = 0.0f;
-    for (int r = threadIdx.x; r < rows; r += EW) s += (float)src[(long long)r * ld + c];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int k = EW / 2; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[c] = sh[0];
-}
-
-// Adam (Kingma and Ba 2015) on the FP32 master weights
-__global__ void k_adam(float *theta, const float *grad, float *m, float *v, float lr, float c1, float c2)
+// Adam (Kingma and Ba 2015) on the FP32 master weights, and their BF16 copies
+__global__ void k_adam(float *theta, const float *grad, float *m, float *v, float lr, float c1, float c2, bf16 *W1b,
+                       bf16 *W2b, bf16 *W3b)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MLP_NPARAM) return;
@@ -466,7 +664,11 @@ __global__ void k_adam(float *theta, const float *grad, float *m, float *v, floa
     const float vi = 0.999f * v[i] + 0.001f * g * g;
     m[i] = mi;
     v[i] = vi;
-    theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    const float t = theta[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    theta[i] = t;
+    if (i < MLP_OFF_B1) W1b[i] = __float2bfloat16_rn(t);
+    else if (i >= MLP_OFF_W2 && i < MLP_OFF_B2) W2b[i - MLP_OFF_W2] = __float2bfloat16_rn(t);
+    else if (i >= MLP_OFF_W3 && i < MLP_OFF_B3) W3b[i - MLP_OFF_W3] = __float2bfloat16_rn(t);
 }
 
 }  // namespace
@@ -492,8 +694,7 @@ cudaError_t mlp_alloc(Mlp &m, int cap)
         (e = A((void **)&m.dZ2, sizeof(bf16) * (size_t)cap * MLP_HIDDEN)) ||
         (e = A((void **)&m.dYb, sizeof(bf16) * (size_t)cap * 16)) || (e = A((void **)&m.Y, sizeof(float) * (size_t)cap * 16)) ||
         (e = A((void **)&m.dY, sizeof(float) * (size_t)cap * 16)) ||
-        (e = A((void **)&m.T, sizeof(float) * (size_t)cap * MLP_NOUT)) ||
-        (e = A((void **)&m.loss_part, sizeof(double) * ((size_t)cap * 16 / EW + 1))) ||
+        (e = A((void **)&m.loss_part, sizeof(double) * ((size_t)cap / GM + 1))) ||
         (e = A((void **)&m.loss, sizeof(double) * 2)))
         return e;
     cudaMemset(m.adam_m, 0, sizeof(float) * MLP_NPARAM);
@@ -505,7 +706,7 @@ cudaError_t mlp_alloc(Mlp &m, int cap)
 void mlp_free(Mlp &m)
 {
     void *ps[] = {m.theta, m.grad, m.adam_m, m.adam_v, m.W1b, m.W2b, m.W3b, m.X, m.H1, m.H2,
-                  m.dZ1, m.dZ2, m.dYb, m.Y, m.dY, m.T, m.loss_part, m.loss};
+                  m.dZ1, m.dZ2, m.dYb, m.Y, m.dY, m.loss_part, m.loss};
     for (void *p : ps) cudaFree(p);
     m = Mlp();
 }
@@ -515,64 +716,26 @@ void mlp_refresh(const Mlp &m, cudaStream_t st)
     k_refresh<<<(MLP_HIDDEN * MLP_KIN + EW - 1) / EW, EW, 0, st>>>(m.theta, m.W1b, m.W2b, m.W3b);
 }
 
-void mlp_stage(const Mlp &m, const float *X, const float *Y, const long long *idx, long long row0, int n,
-               cudaStream_t st)
+cudaError_t mlp_forward(const Mlp &m, const float *X, int n, unsigned *status, cudaStream_t st)
 {
-    const long long t = (long long)n * MLP_KIN;
-    k_stage_inputs<<<(unsigned)((t + EW - 1) / EW), EW, 0, st>>>(X, idx, row0, n, m.X);
-    if (Y) k_stage_targets<<<(n * MLP_NOUT + EW - 1) / EW, EW, 0, st>>>(Y, idx, row0, n, m.T);
+    return mlp_launch(k_mlp_rows<false>, (n + GM - 1) / GM, ROW_THREADS, RowSmem::BYTES,
+                      row_args(m, X, nullptr, nullptr, 0, n, status), st);
 }
 
-cudaError_t mlp_forward(const Mlp &m, int n, unsigned *status, cudaStream_t st)
+cudaError_t mlp_gradient(const Mlp &m, const float *X, const float *T, const long long *idx, long long row0, int n,
+                         double *acc, unsigned *status, cudaStream_t st)
 {
-    cudaError_t e;
-    const float *b1 = m.theta + MLP_OFF_B1, *b2 = m.theta + MLP_OFF_B2, *b3 = m.theta + MLP_OFF_B3;
-    // h1 = tanh(X W1^T + b1)
-    GemmArgs a = gargs(n, MLP_HIDDEN, MLP_KIN, m.X, MLP_KIN, 1, m.W1b, MLP_KIN, 1, status);
-    a.bias = b1; a.act = 1; a.C16 = m.H1; a.s16m = MLP_HIDDEN; a.s16n = 1;
-    if ((e = gemm<BNH>(mode(a, m), n, MLP_HIDDEN, st)) != cudaSuccess) return e;
-    // h2 = tanh(h1 W2^T + b2)
-    a = gargs(n, MLP_HIDDEN, MLP_HIDDEN, m.H1, MLP_HIDDEN, 1, m.W2b, MLP_HIDDEN, 1, status);
-    a.bias = b2; a.act = 1; a.C16 = m.H2; a.s16m = MLP_HIDDEN; a.s16n = 1;
-    if ((e = gemm<BNH>(mode(a, m), n, MLP_HIDDEN, st)) != cudaSuccess) return e;
-    // y = h2 W3^T + b3  ([n][16], columns 6..15 unused)
-    a = gargs(n, MLP_NOUT, MLP_HIDDEN, m.H2, MLP_HIDDEN, 1, m.W3b, MLP_HIDDEN, 1, status);
-    a.bias = b3; a.C32 = m.Y; a.scm = 16; a.scn = 1;
-    if ((e = gemm<16>(mode(a, m), n, 16, st)) != cudaSuccess) return e;
-    return cudaSuccess;
-}
-
-cudaError_t mlp_backward(const Mlp &m, int n, double *acc, unsigned *status, cudaStream_t st)
-{
-    cudaError_t e;
-    float *g = m.grad;
-    const int nl = (n * 16 + EW - 1) / EW;
-    k_loss<<<nl, EW, 0, st>>>(m.Y, m.T, n, m.dY, m.dYb, m.loss_part);
-    k_loss_final<<<1, 32, 0, st>>>(m.loss_part, nl, n, m.loss, acc);
-    // dW3[j][i] = sum_b dY[b][j] h2[b][i]   (M = hidden i, N = output j, K = batch)
-    GemmArgs a = gargs(MLP_HIDDEN, MLP_NOUT, n, m.H2, 1, MLP_HIDDEN, m.dYb, 1, 16, status);
-    a.C32 = g + MLP_OFF_W3; a.scm = 1; a.scn = MLP_HIDDEN;
-    if ((e = gemm<16>(mode(a, m), MLP_HIDDEN, 16, st)) != cudaSuccess) return e;
-    k_colsum<float><<<MLP_NOUT, EW, 0, st>>>(m.dY, n, 16, g + MLP_OFF_B3);
-    // dz2 = (dY W3) * (1 - h2^2)
-    a = gargs(n, MLP_HIDDEN, MLP_NOUT, m.dYb, 16, 1, m.W3b, 1, MLP_HIDDEN, status);
-    a.act = 2; a.g = m.H2; a.sgm = MLP_HIDDEN; a.sgn = 1; a.C16 = m.dZ2; a.s16m = MLP_HIDDEN; a.s16n = 1;
-    if ((e = gemm<BNH>(mode(a, m), n, MLP_HIDDEN, st)) != cudaSuccess) return e;
-    // dW2[o][i] = sum_b dz2[b][o] h1[b][i]
-    a = gargs(MLP_HIDDEN, MLP_HIDDEN, n, m.dZ2, 1, MLP_HIDDEN, m.H1, 1, MLP_HIDDEN, status);
-    a.C32 = g + MLP_OFF_W2; a.scm = MLP_HIDDEN; a.scn = 1;
-    if ((e = gemm<BNH>(mode(a, m), MLP_HIDDEN, MLP_HIDDEN, st)) != cudaSuccess) return e;
-    k_colsum<bf16><<<MLP_HIDDEN, EW, 0, st>>>(m.dZ2, n, MLP_HIDDEN, g + MLP_OFF_B2);
-    // dz1 = (dz2 W2) * (1 - h1^2)
-    a = gargs(n, MLP_HIDDEN, MLP_HIDDEN, m.dZ2, MLP_HIDDEN, 1, m.W2b, 1, MLP_HIDDEN, status);
-    a.act = 2; a.g = m.H1; a.sgm = MLP_HIDDEN; a.sgn = 1; a.C16 = m.dZ1; a.s16m = MLP_HIDDEN; a.s16n = 1;
-    if ((e = gemm<BNH>(mode(a, m), n, MLP_HIDDEN, st)) != cudaSuccess) return e;
-    // dW1[o][i] = sum_b dz1[b][o] x[b][i]
-    a = gargs(MLP_HIDDEN, MLP_KIN, n, m.dZ1, 1, MLP_HIDDEN, m.X, 1, MLP_KIN, status);
-    a.C32 = g + MLP_OFF_W1; a.scm = MLP_KIN; a.scn = 1;
-    if ((e = gemm<BNH>(mode(a, m), MLP_HIDDEN, MLP_KIN, st)) != cudaSuccess) return e;
-    k_colsum<bf16><<<MLP_HIDDEN, EW, 0, st>>>(m.dZ1, n, MLP_HIDDEN, g + MLP_OFF_B1);
-    return cudaSuccess;
+    const int tiles = (n + GM - 1) / GM;
+    const RowArgs r = row_args(m, X, T, idx, row0, n, status);
+    const cudaError_t e = mlp_launch(k_mlp_rows<true>, tiles, ROW_THREADS, RowSmem::BYTES, r, st);
+    if (e != cudaSuccess) return e;
+    GradArgs a;
+    memset(&a, 0, sizeof a);
+    a.n = n;
+    a.Xb = m.X; a.H1 = m.H1; a.H2 = m.H2; a.dZ1 = m.dZ1; a.dZ2 = m.dZ2; a.dYb = m.dYb; a.dY = m.dY;
+    a.grad = m.grad; a.loss_part = m.loss_part; a.parts = tiles; a.loss = m.loss; a.acc = acc;
+    a.status = status; a.no_mma = r.no_mma; a.wait_limit = r.wait_limit;
+    return mlp_launch(k_mlp_grads, GRAD_CTAS, MLP_THREADS, GradSmem::BYTES, a, st);
 }
 
 void mlp_adam(Mlp &m, double lr, cudaStream_t st)
@@ -580,8 +743,8 @@ void mlp_adam(Mlp &m, double lr, cudaStream_t st)
     m.t += 1;
     const float c1 = (float)(1.0 - std::pow(0.9, (double)m.t));
     const float c2 = (float)(1.0 - std::pow(0.999, (double)m.t));
-    k_adam<<<(MLP_NPARAM + EW - 1) / EW, EW, 0, st>>>(m.theta, m.grad, m.adam_m, m.adam_v, (float)lr, c1, c2);
-    mlp_refresh(m, st);
+    k_adam<<<(MLP_NPARAM + EW - 1) / EW, EW, 0, st>>>(m.theta, m.grad, m.adam_m, m.adam_v, (float)lr, c1, c2, m.W1b,
+                                                      m.W2b, m.W3b);
 }
 
 // ---------------------------------------------------------------------------
@@ -713,12 +876,11 @@ void launch_surrogate_forces(const Lattice &L, const Mlp &m, float *feat, cudaSt
     for (int p0 = 0; p0 < L.n_parts; p0 += m.cap) {
         const int np = std::min(m.cap, L.n_parts - p0);
         launch_shell_features<S>(L, p0, np, feat, st);
-        mlp_stage(m, feat, nullptr, nullptr, 0, np, st);
         // a failed set-up or launch stays in the runtime's last error, which
         // lbm_step checks after enqueueing the step
-        if (mlp_forward(m, np, L.status, st) != cudaSuccess) return;
+        if (mlp_forward(m, feat, np, L.status, st) != cudaSuccess) return;
         k_surrogate_apply<<<(np + 127) / 128, 128, 0, st>>>(L, m.Y, p0, np);
-        *launches += 6;
+        *launches += 3;
     }
     mk(STAGE_SURROGATE, 1);
 }
