@@ -106,7 +106,7 @@ static void plan_launch(lbm_ctx *c)
 {
     plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, c->prec == LBM_FP64, &c->fz);
     plan_phi(c->inst_h, c->n_sm, c->prec == LBM_FP64, &c->fz);
-    c->fz.rows = plan_rows(c->inst_h);
+    plan_items(c->inst_h, c->prec == LBM_FP64, &c->fz);
     bool even = true;
     for (const auto &I : c->inst_h) even = even && I.nx % 2 == 0;
     c->fz.pair = even && c->fz.tile == 0;
@@ -137,7 +137,6 @@ static Lattice make_lattice(const lbm_ctx *c)
     Lattice L;
     L.inst = c->inst_d;
     L.n_inst = c->n_inst;
-    L.n_items = c->fz.rows;
     L.buoyancy = 0;
     for (const auto &I : c->inst_h)
         if (I.buoy[0] != 0.0 || I.buoy[1] != 0.0 || I.buoy[2] != 0.0) L.buoyancy = 1;

@@ -32,11 +32,11 @@ constexpr int BOUND_THREADS = 64;
 #ifndef LBM_BOUND_MINB
 #define LBM_BOUND_MINB 2
 #endif
-// CTAs of 256 threads per SM of the one-node collision: 5 (48 registers, no
-// spill) measured faster than 4 (64 registers) and 6 (40, spilling): 123
-// against 127 and 148 us per FP32 256x128x128 launch
+// CTAs of 256 threads per SM of the one-node collision: 4 (64 registers, no
+// spill): 119 us per FP32 256x128x128 launch, 6.5 TB/s of the 184 bytes a node
+// that it moves; 5 and 6 spill and took 137 and 160 us
 #ifndef LBM_COLLIDE_MINB
-#define LBM_COLLIDE_MINB 5
+#define LBM_COLLIDE_MINB 4
 #endif
 
 namespace lbmg {
@@ -520,12 +520,12 @@ __device__ __forceinline__ void collide_body(const Lattice &L, const InstDev &I,
 
 // Node pairs (x even, x + 1) of one row per thread, for 16-bit storage: the
 // pulls along directions with c_x = 0 are one 32-bit load of the pair, every
-// output a pair store (half2, bfloat162 or float2), which halves the
-// per-node load, store, conversion and address instructions.  Each node's
-// arithmetic is that of collide_store_phi (the same expressions; the code
-// generator may fuse a different set of multiply-adds, so the results agree
-// to rounding); a node of the pair that the bulk kernel skips (solid, next to
-// a solid) is computed but not written.
+// output a pair store (half2 or bfloat162), and the arithmetic handles both
+// nodes per instruction (F2), which halves what binds this kernel: issue slots.
+// Each node's arithmetic is that of collide_store_phi (which may leave other
+// multiply-adds fused, so the results agree to rounding); a node of the pair
+// that the bulk kernel skips (solid, next to a solid) is computed but not
+// written.
 template <class S>
 __device__ __forceinline__ void collide_body2(const Lattice &L, const InstDev &I, int cur, int n, int x, int y, int z)
 {
@@ -543,24 +543,28 @@ __device__ __forceinline__ void collide_body2(const Lattice &L, const InstDev &I
     Nbr nb;
     nb.init(x, y, z, I.nx, I.ny, I.nz);
     const int xp2 = x + 2 == I.nx ? 0 : x + 2;
-    R F0[Q], F1[Q];
+    F2 F[Q];
+    {
+        R F0[Q], F1[Q];
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        const FT *row = in.f + i * N + nb.ZO[1 - cz(i)] + nb.YO[1 - cy(i)];
-        if (cx(i) == 0) {
-            ld_pair(row + x, F0[i], F1[i]);
-        } else if (cx(i) == 1) {
-            F0[i] = Store<FT>::ld(row + nb.X[0]);
-            F1[i] = Store<FT>::ld(row + x);
-        } else {
-            F0[i] = Store<FT>::ld(row + x + 1);
-            F1[i] = Store<FT>::ld(row + xp2);
+        for (int i = 0; i < Q; i++) {
+            const FT *row = in.f + i * N + nb.ZO[1 - cz(i)] + nb.YO[1 - cy(i)];
+            if (cx(i) == 0) {
+                ld_pair(row + x, F0[i], F1[i]);
+            } else if (cx(i) == 1) {
+                F0[i] = Store<FT>::ld(row + nb.X[0]);
+                F1[i] = Store<FT>::ld(row + x);
+            } else {
+                F0[i] = Store<FT>::ld(row + x + 1);
+                F1[i] = Store<FT>::ld(row + xp2);
+            }
         }
-    }
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        keep(F0[i]);
-        keep(F1[i]);
+        for (int i = 0; i < Q; i++) {
+            keep(F0[i]);
+            keep(F1[i]);
+            F[i] = f2(F0[i], F1[i]);
+        }
     }
     const bool fluid0 = (fl0 & OWNER_MASK) == OWN_FLUID, fluid1 = (fl1 & OWNER_MASK) == OWN_FLUID;
     const bool a0 = fluid0 && !(fl0 & BOUND_BIT), a1 = fluid1 && !(fl1 & BOUND_BIT);
@@ -572,70 +576,103 @@ __device__ __forceinline__ void collide_body2(const Lattice &L, const InstDev &I
     if (!a0 && !a1) return;
     FluidPar<R> P;
     load_par(I, P);
-    const R phA = pv.x, phB = pv.y;
-    const CollideState<R> cA = collide_state(P, F0, phA, grA);
-    const CollideState<R> cB = collide_state(P, F1, phB, grB);
-    if ((a0 && (!(cA.rr > R(0)) || !(phA == phA))) || (a1 && (!(cB.rr > R(0)) || !(phB == phB))))
+    const F2 gr[3] = {f2(grA.g0, grB.g0), f2(grA.g1, grB.g1), f2(grA.g2, grB.g2)};
+    const Collision<F2> c = collide_setup(CollidePar<F2>(P), F, f2(pv.x, pv.y), gr, f2(grA.k, grB.k));
+    float rA, rB, bA, bB;
+    unpack(c.rr, rA, rB);
+    unpack(c.bq, bA, bB);
+    if ((a0 && (!(rA > R(0)) || !(pv.x == pv.x))) || (a1 && (!(rB > R(0)) || !(pv.y == pv.y))))
         atomicOr(L.status, ST_UNSTABLE);
     if (U) {
-        if (a0) { U[n] = cA.ux; U[Nt + n] = cA.uy; U[2 * Nt + n] = cA.uz; }
-        if (a1) { U[n + 1] = cB.ux; U[Nt + n + 1] = cB.uy; U[2 * Nt + n + 1] = cB.uz; }
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            float uA, uB;
+            unpack(c.u[k], uA, uB);
+            if (a0) U[k * Nt + n] = uA;
+            if (a1) U[k * Nt + n + 1] = uB;
+        }
     }
     FT *const of = out.f + n;
     const bool both = a0 && a1;
-    auto put = [&](auto *p, R v0, R v1) {
-        using T = std::remove_pointer_t<decltype(p)>;
+    auto put = [&](FT *p, F2 v) {
+        float v0, v1;
+        unpack(v, v0, v1);
         if (both) {
             st_pair(p, v0, v1);
         } else if (a0) {
-            Store<T>::st(p, v0);
+            Store<FT>::st(p, v0);
         } else {
-            Store<T>::st(p + 1, v1);
+            Store<FT>::st(p + 1, v1);
         }
     };
-    {
-        if (a0) col_slot<S>(L, g).set(colour_record(P, cA, phA, grA));
-        if (a1) col_slot<S>(L, g + 1).set(colour_record(P, cB, phB, grB));
-    }
-    put(of, collide_rest(P, cA, F0[0]), collide_rest(P, cB, F1[0]));
+    if (a0) col_slot<S>(L, g).set(colour_record(bA, P.eps2, pv.x, grA.g0, grA.g1, grA.g2));
+    if (a1) col_slot<S>(L, g + 1).set(colour_record(bB, P.eps2, pv.y, grB.g0, grB.g1, grB.g2));
+    put(of, collide_rest(c, F[0]));
     PairLoop<R>::run([&](auto ic) {
         constexpr int i = decltype(ic)::value, ib = i + 9;
-        R FiA, FibA, FiB, FibB;
-        collide_pair<R, i>(P, cA, F0[i], F0[ib], FiA, FibA);
-        collide_pair<R, i>(P, cB, F1[i], F1[ib], FiB, FibB);
-        put(of + i * N, FiA, FiB);
-        put(of + ib * N, FibA, FibB);
+        F2 Fi, Fib;
+        collide_pair<i>(c, F[i], F[ib], Fi, Fib);
+        put(of + i * N, Fi);
+        put(of + ib * N, Fib);
     });
 }
 
-// CTAs of 128 threads per SM the node-pair collision is compiled for: 6 (80
-// registers, 60 bytes spilled) measured faster than 4 (128 registers, no
-// spill), 5, 7 and 8 (105, 102, 100 and 109 against 96 us per 256x128x128
-// launch): the pulls of more node pairs in flight outweigh the spill traffic
+// CTAs of 128 threads per SM the node-pair collision is compiled for: 4 (128
+// registers, no spill); 5, 6 and 7 spill and took 3445, 3699 and 3703 us against
+// 3393 on the 96-domain sweep.  With two scalar nodes per thread, the relaxation
+// direction by direction and items of whole rows it was bound by issue and took
+// 3915 us (36 x 200x90x36: 634 -> 545); now 4.8 TB/s.
 #ifndef LBM_COLLIDE2_MINB
-#define LBM_COLLIDE2_MINB 6
+#define LBM_COLLIDE2_MINB 4
 #endif
+// Work items of the collision: consecutive nodes of an instance, whatever their
+// rows (items of whole rows leave lanes idle wherever rows do not fill a CTA: 22%
+// at nx = 200, 25% at 96).  FP64 items are small: its runs are bound by the
+// FP64 pipes of the SMs they reach, and 224 CTAs of 240 nodes on 152 SMs took
+// 66 us for 48x32x32; CTAs of 64 and a third fewer FP64 instructions 31.
 template <class S>
-__global__ void __launch_bounds__(ROW_NODES / 2, LBM_COLLIDE2_MINB) k_collide2(Lattice L, int cur)
+constexpr int COLLIDE_NODES = sizeof(S) == 8 ? 64 : 256;
+
+// the node of item `item` for thread offset j; false past the instance's end
+__device__ __forceinline__ bool item_node(const Lattice &L, long long item, int per_item, int j, const InstDev **Ip,
+                                          int *n, int *x, int *y, int *z)
 {
-    StItem it;
-    st_item(L, blockIdx.x, it);
-    pdl_wait();  // the gradient pass's grad(phi) and curvature
-    const int j = 2 * (int)threadIdx.x;
-    if (j >= it.cnt) return;
-    const InstDev &I = L.inst[it.k];
-    int x, y;
-    item_node(I, it, j, &x, &y);
-    collide_body2<S>(L, I, cur, (it.z * I.ny + y) * I.nx + x, x, y, it.z);
+    int lo = 0, hi = L.n_inst - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (L.inst[mid].item_start <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    const InstDev &I = L.inst[lo];
+    const int m = (int)(item - I.item_start) * per_item + j;
+    if (m >= I.pstride) return false;
+    const int row = I.fd_nx.div(m);
+    *x = m - row * I.nx;
+    *z = I.fd_ny.div(row);
+    *y = row - *z * I.ny;
+    *n = m;
+    *Ip = &I;
+    return true;
 }
 
 template <class S>
-__global__ void __launch_bounds__(ROW_NODES, sizeof(S) == 8 ? 1 : LBM_COLLIDE_MINB) k_collide(Lattice L, int cur)
+__global__ void __launch_bounds__(COLLIDE_NODES<S> / 2, LBM_COLLIDE2_MINB) k_collide2(Lattice L, int cur)
 {
-    for_item_nodes(L, blockIdx.x, [&](const InstDev &I, int n, int x, int y, int z) {
-        pdl_wait();  // the gradient pass's grad(phi) and curvature
-        collide_body<S>(L, I, cur, n, x, y, z);
-    });
+    const InstDev *I;
+    int n, x, y, z;
+    const bool have = item_node(L, blockIdx.x, COLLIDE_NODES<S>, 2 * (int)threadIdx.x, &I, &n, &x, &y, &z);
+    pdl_wait();  // the gradient pass's grad(phi) and curvature
+    if (have) collide_body2<S>(L, *I, cur, n, x, y, z);
+}
+
+template <class S>
+__global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : LBM_COLLIDE_MINB) k_collide(Lattice L, int cur)
+{
+    const InstDev *I;
+    int n, x, y, z;
+    const bool have = item_node(L, blockIdx.x, COLLIDE_NODES<S>, (int)threadIdx.x, &I, &n, &x, &y, &z);
+    pdl_wait();  // the gradient pass's grad(phi) and curvature
+    if (have) collide_body<S>(L, *I, cur, n, x, y, z);
 }
 
 // ---------------------------------------------------------------------------
@@ -1105,34 +1142,18 @@ void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz)
     fz->ph_items = items;
 }
 
-// row-strip work items of the bulk kernels: whole x-rows of one z-plane, at
-// most ROW_NODES nodes per item, or one row cut into segments of at most
-// ROW_NODES nodes
-long long plan_rows(std::vector<InstDev> &inst)
+// the collision's work items
+void plan_items(std::vector<InstDev> &inst, bool fp64, FluidLaunch *fz)
 {
+    const long long per = fp64 ? COLLIDE_NODES<double> : COLLIDE_NODES<float>;
     long long total = 0;
     for (auto &I : inst) {
-        if (I.nx <= ROW_NODES) {
-            I.st_rows = std::min(I.ny, ROW_NODES / I.nx);
-            I.st_seg = I.nx;
-            I.st_nseg = 1;
-        } else {
-            const int nseg = (I.nx + ROW_NODES - 1) / ROW_NODES;
-            int seg = (I.nx + nseg - 1) / nseg;
-            seg = (seg + 1) / 2 * 2;  // even: node pairs never straddle two items
-            I.st_rows = 1;
-            I.st_seg = seg;
-            I.st_nseg = (I.nx + seg - 1) / seg;
-        }
-        I.st_ygroups = (I.ny + I.st_rows - 1) / I.st_rows;
-        I.fd_plane.set(I.st_ygroups * I.st_nseg);
-        I.fd_nseg.set(I.st_nseg);
         I.fd_nx.set(I.nx);
         I.fd_ny.set(I.ny);
-        I.st_item_start = total;
-        total += (long long)I.nz * I.st_ygroups * I.st_nseg;
+        I.item_start = total;
+        total += (I.N + per - 1) / per;
     }
-    return total;
+    fz->items = total;
 }
 
 // launch with programmatic stream serialisation: the kernel may be scheduled
@@ -1158,7 +1179,7 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
                        const FluidLaunch &fz, const SideLane &lane)
 {
     using R = typename Store<S>::real;
-    const dim3 grid((unsigned)fz.rows);  // one CTA per row-strip work item
+    const dim3 grid((unsigned)fz.items);  // one CTA per work item of the collision
     const bool pair = sizeof(S) == 2 && fz.pair;
     // boundary passes: grid-stride over the listed particle nodes and the
     // static list of nodes next to walls
@@ -1209,15 +1230,15 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     if constexpr (BOUNCE_IN_SLOTS<S>) {
         lane.after_collide_bound();
         mk(STAGE_COLLIDE, 0);
-        launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
+        launch_after(k_collide<S>, grid, dim3(COLLIDE_NODES<S>), st, L, cur);
         mk(STAGE_COLLIDE, 1);
     } else {
         bound_pass(k_collide_bound<S>, STAGE_COLLIDE_BOUND);
         if (lane.side && any_bound) cudaEventRecord(lane.b, lane.side);
         lane.after_collide_bound();
         mk(STAGE_COLLIDE, 0);
-        if (pair) launch_after(k_collide2<S>, grid, dim3(ROW_NODES / 2), st, L, cur);
-        else launch_after(k_collide<S>, grid, dim3(ROW_NODES), st, L, cur);
+        if (pair) launch_after(k_collide2<S>, grid, dim3(COLLIDE_NODES<S> / 2), st, L, cur);
+        else launch_after(k_collide<S>, grid, dim3(COLLIDE_NODES<S>), st, L, cur);
         mk(STAGE_COLLIDE, 1);
         if (lane.side && any_bound) cudaStreamWaitEvent(st, lane.b, 0);
     }

@@ -121,12 +121,9 @@ struct InstDev {
     float f_ir0, f_h_ia, f_h_ib;
     float f_wall_u[3];
     float f_cap;  // cap_norm sigma
-    // row-strip work items of the bulk kernels: st_rows whole x-rows of one z-plane per item
-    // (st_nseg = 1, st_seg = nx), or one row cut into st_nseg segments of at
-    // most st_seg nodes; st_ygroups items cover the y rows of a plane
-    long long st_item_start;
-    int st_rows, st_seg, st_nseg, st_ygroups;
-    FastDiv fd_plane, fd_nseg, fd_nx, fd_ny;  // st_ygroups st_nseg, st_nseg, nx, ny
+    // work items of the collision: consecutive nodes
+    long long item_start;
+    FastDiv fd_nx, fd_ny;
     // surrogate inputs: shell gap, velocity and radius scales
     double sh_gap, sh_uref, sh_rref, sh_box;
     // gradient + curvature work items: gc_tiles_x * gc_tiles_y column tiles x
@@ -184,7 +181,6 @@ struct PartDev {
 struct Lattice {
     const InstDev *inst;
     int n_inst;
-    long long n_items;   // row-strip work items of all instances
     int buoyancy;        // some instance has a nonzero buoyancy_a: the immersed fractions are summed
     // boundary lists: entries of list_entry, the static ones in node order
     const long long *static_list;  // static solid nodes next to non-static ones
@@ -682,86 +678,6 @@ __device__ __forceinline__ void wetting_rotate(R *g, const R *ns, R cth, R sth)
     for (int a = 0; a < 3; a++) g[a] = -gm * nc[a];
 }
 
-// ---------------------------------------------------------------------------
-// row-strip work items (all per-node kernels): a strip of one z-plane made of
-// st_rows whole x-rows (at most ROW_NODES nodes), or one segment of a longer row
-// ---------------------------------------------------------------------------
-constexpr int ROW_NODES = 256;  // nodes per work item at most = threads per CTA
-
-struct StItem {
-    int k;       // instance
-    int z, y0;   // plane and first row
-    int nrows;   // rows (whole-row items)
-    int x0, cnt; // first x and number of nodes
-    bool whole;
-};
-
-__device__ __forceinline__ void st_item(const Lattice &L, long long item, StItem &it)
-{
-    int lo = 0, hi = L.n_inst - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (L.inst[mid].st_item_start <= item) lo = mid;
-        else hi = mid - 1;
-    }
-    const InstDev &I = L.inst[lo];
-    const int loc = (int)(item - I.st_item_start);  // < 2^31: rows of one instance
-    const int per_plane = I.st_ygroups * I.st_nseg;
-    it.k = lo;
-    it.z = I.fd_plane.div(loc);
-    const int r = loc - it.z * per_plane;
-    const int yg = I.fd_nseg.div(r), sg = r - yg * I.st_nseg;
-    it.y0 = yg * I.st_rows;
-    it.whole = I.st_nseg == 1;
-    it.nrows = min(I.st_rows, I.ny - it.y0);
-    it.x0 = sg * I.st_seg;
-    it.cnt = it.whole ? it.nrows * I.nx : min(I.st_seg, I.nx - it.x0);
-}
-
-__device__ __forceinline__ int wrap1(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
-
-// first node of the item in the per-node arrays and the 16-byte-aligned start
-// of its flag copy
-__device__ __forceinline__ long long item_node0(const InstDev &I, const StItem &it)
-{
-    return I.node_off + ((long long)it.z * I.ny + it.y0) * I.nx + it.x0;
-}
-
-// node j of a work item
-__device__ __forceinline__ void item_node(const InstDev &I, const StItem &it, int j, int *x, int *y)
-{
-    int r = 0, xx = it.x0 + j;
-    if (it.nrows > 1) {
-        r = I.fd_nx.div(j);
-        xx = j - r * I.nx;
-    }
-    *x = xx;
-    *y = it.y0 + r;
-}
-
-// the nodes of work item `item` (CTAs launched in item order cover a
-// contiguous band of rows, so the neighbour rows they share stay in L2):
-// f(I, n, x, y, z) for the CTA's nodes
-template <class F>
-__device__ __forceinline__ void for_item_nodes(const Lattice &L, long long item, F &&f)
-{
-    StItem it;
-    st_item(L, item, it);
-    const int j = threadIdx.x;
-    if (j >= it.cnt) return;
-    const InstDev &I = L.inst[it.k];
-    if (it.nrows == 1) {
-        // one row or row segment per CTA: y and z are the same for every
-        // thread, which lets the neighbour-row offsets be computed once per CTA
-        const int x = it.x0 + j;
-        f(I, (it.z * I.ny + it.y0) * I.nx + x, x, it.y0, it.z);
-        return;
-    }
-    int x, y;
-    item_node(I, it, j, &x, &y);
-    f(I, (it.z * I.ny + y) * I.nx + x, x, y, it.z);
-}
-
 // kernel stages, in launch order within a step (for per-kernel timing)
 enum Stage {
     STAGE_PHI = 0, STAGE_SOLIDPHI, STAGE_GRAD, STAGE_COLLIDE, STAGE_MEM, STAGE_CAPILLARY, STAGE_DEM,
@@ -803,7 +719,7 @@ struct SideLane {
 constexpr int FORM_PLAIN = 2;  // the launch form of the fluid update (the value the ABI names)
 struct FluidLaunch {
     int tile;           // 0: node-pair bulk collision where possible; 1: one node per thread
-    long long rows;     // row-strip work items (all instances): CTAs of each bulk kernel
+    long long items;    // collision work items (all instances)
     long long ph_items; // order-parameter work items (all instances)
     long long gc_items; // gradient + curvature work items (all instances)
     int gc_rows;        // warps of own nodes per CTA of that kernel (8; FP64: 4 or 8)
@@ -816,8 +732,8 @@ void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector
                    FluidLaunch *fz);
 // plan the work items of the order-parameter kernel into fz
 void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz);
-// plan the row-strip work items of every instance; returns their number
-long long plan_rows(std::vector<InstDev> &inst);
+// plan the collision's work items into fz (and the divisions by nx and ny)
+void plan_items(std::vector<InstDev> &inst, bool fp64, FluidLaunch *fz);
 template <class S>
 void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *launches, const Marker &mk,
                        const FluidLaunch &fz, const SideLane &lane = SideLane());
