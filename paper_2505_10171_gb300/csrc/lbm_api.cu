@@ -615,7 +615,7 @@ static void *device_addressable(const void *p)
 // collision reads no flags, so the boundary bits and lists follow there too;
 // 16-bit storage's does (its boundary bits), so there they wait for it, as the
 // DEM waits for the collision's boundary pass, which reads the particles.  The
-// refill needs the collision's output.  With the surrogate the forces need the
+// refill needs the collision's output and the owners, and runs beside them.  With the surrogate the forces need the
 // collision's velocity, and all that follows stays in the main stream.
 // Profiling keeps one stream (per-kernel events).
 static void enqueue_step(lbm_ctx *c, long long *launches)
@@ -665,9 +665,9 @@ static void enqueue_step(lbm_ctx *c, long long *launches)
                     // (16-bit storage: the collision would zero the stored
                     // velocity of newly covered nodes, so then they follow it)
                     if (early || !q->c->u) launch_geom_owner(*q->L, q->c->side, q->launches, *q->mk);
-                    if (early) launch_geom_surface(*q->L, q->c->side, q->launches, *q->mk);
                 }
                 cudaEventRecord(q->c->ev_join, q->c->side);
+                if (early && !q->sur) launch_geom_surface(*q->L, q->c->side, q->launches, *q->mk);
             };
         }
         // without a side lane the contacts go first: nothing of the step moves a particle before the DEM
@@ -682,8 +682,19 @@ static void enqueue_step(lbm_ctx *c, long long *launches)
         }
         if (sur || !fork) launch_dem<S>(L, c->stream, launches, mk, !sur);
         if (sur || !fork || !(early || !c->u)) launch_geom_owner(L, c->stream, launches, mk);
-        if (sur || !fork || !early) launch_geom_surface(L, c->stream, launches, mk);
+        // boundary bits and lists beside the refill (it reads owners and fresh
+        // bits only): already enqueued there, or forked here
+        const bool surface_done = fork && early && !sur;
+        if (fork && !surface_done) {
+            cudaEventRecord(c->ev_fork, c->stream);
+            cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+        }
+        if (!surface_done) launch_geom_surface(L, fork ? c->side : c->stream, launches, mk);
         launch_refill<S>(L, cur ^ 1, c->stream, launches, mk);
+        if (fork) {
+            cudaEventRecord(c->ev_grad, c->side);
+            cudaStreamWaitEvent(c->stream, c->ev_grad, 0);
+        }
     });
     c->cur ^= 1;
 }
@@ -1832,7 +1843,6 @@ lbm_status lbm_surrogate_predict(lbm_ctx *ctx, const float *X, size_t n, float *
         CU(cudaGetLastError());
         CU(cudaMemcpy2DAsync(Y + r0 * MLP_NOUT, sizeof(float) * MLP_NOUT, ctx->mlp.Y, sizeof(float) * 16,
                              sizeof(float) * MLP_NOUT, nb, cudaMemcpyDeviceToHost, ctx->stream));
-        CU(cudaStreamSynchronize(ctx->stream));
     }
     return check_status(ctx);
 }
@@ -1851,9 +1861,9 @@ lbm_status lbm_surrogate_gradient(lbm_ctx *ctx, const float *X, const float *Y, 
     CU(cudaMemcpyAsync(grad, ctx->mlp.grad, sizeof(float) * MLP_NPARAM, cudaMemcpyDeviceToHost, ctx->stream));
     double l = 0.0;
     CU(cudaMemcpyAsync(&l, ctx->mlp.loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
+    s = check_status(ctx);
     if (loss) *loss = l;
-    return check_status(ctx);
+    return s;
 }
 
 // SplitMix64 (Steele, Lea and Flood 2014) and the Fisher-Yates order of an epoch
@@ -1930,12 +1940,11 @@ lbm_status lbm_surrogate_features(lbm_ctx *ctx, int inst, float *out)
         const int np = std::min(MLP_CAP, I.np - p0);
         dispatch(ctx->prec, [&](auto *tag) {
             using S = std::remove_pointer_t<decltype(tag)>;
-            launch_shell_features<S>(L, I.part_off + p0, np, ctx->feat, ctx->stream);
+            launch_shell_features<S>(L, ctx->mlp, I.part_off + p0, np, ctx->feat, ctx->stream);
         });
         CU(cudaGetLastError());
         CU(cudaMemcpyAsync(out + (size_t)p0 * MLP_NIN, ctx->feat, sizeof(float) * np * MLP_NIN,
                            cudaMemcpyDeviceToHost, ctx->stream));
-        CU(cudaStreamSynchronize(ctx->stream));
     }
     return check_status(ctx);
 }

@@ -25,10 +25,11 @@
 
 #include "lbm_node.cuh"
 
-// Boundary passes, which run beside the bulk kernels: CTAs of 64 threads, so
-// that a short list reaches many SMs (FP64: as many FP64 pipes), 4 times this
-// many per SM
-constexpr int BOUND_THREADS = 64;
+// Boundary passes, which run beside the bulk kernels: CTAs of 64 threads
+// (FP64: one warp), so that a short list reaches many SMs (and FP64 pipes); 4
+// (8) times this many per SM
+template <class S>
+constexpr int BOUND_THREADS = sizeof(S) == 8 ? 32 : 64;
 #ifndef LBM_BOUND_MINB
 #define LBM_BOUND_MINB 2
 #endif
@@ -408,7 +409,7 @@ __device__ __forceinline__ void phi_bound_node(const Lattice &L, int cur, long l
 }
 
 template <class S>
-__global__ void __launch_bounds__(BOUND_THREADS, sizeof(S) == 8 ? 4 : 4 * LBM_BOUND_MINB) k_phi_bound(Lattice L, int cur)
+__global__ void __launch_bounds__(BOUND_THREADS<S>, sizeof(S) == 8 ? 8 : 4 * LBM_BOUND_MINB) k_phi_bound(Lattice L, int cur)
 {
     const long long npb = L.n_parts ? (long long)L.list_n[LIST_FLUID] : 0;
     const long long total = npb + L.n_static_bfl;
@@ -443,7 +444,7 @@ __device__ __forceinline__ void collide_bound_node(const Lattice &L, int cur, lo
 }
 
 template <class S>
-__global__ void __launch_bounds__(BOUND_THREADS, 4 * LBM_BOUND_MINB) k_collide_bound(Lattice L, int cur)
+__global__ void __launch_bounds__(BOUND_THREADS<S>, 4 * LBM_BOUND_MINB) k_collide_bound(Lattice L, int cur)
 {
     const long long npb = L.n_parts ? (long long)L.list_n[LIST_FLUID] : 0;
     const long long total = npb + L.n_static_bfl;
@@ -1206,7 +1207,7 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
             cudaStreamWaitEvent(lane.side, lane.a, 0);
         }
         mk(stage, 0);
-        kernel<<<bgrid, BOUND_THREADS, 0, s>>>(L, cur);
+        kernel<<<bgrid, BOUND_THREADS<S>, 0, s>>>(L, cur);
         mk(stage, 1);
         *launches += 1;
     };

@@ -776,6 +776,7 @@ struct Mlp {
     __nv_bfloat16 *X = nullptr, *H1 = nullptr, *H2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dYb = nullptr;
     float *Y = nullptr, *dY = nullptr;                // [cap][16]
     double *loss_part = nullptr, *loss = nullptr;     // loss[0]: last batch, loss[1]: accumulator
+    double *dirs = nullptr;  // [96][3] unit vectors of the shell points
     int cap = 0;
     long long t = 0;  // Adam steps taken
     bool fault_no_commit = false;  // host-set fault injection (lbm_inject_fault)
@@ -791,7 +792,7 @@ cudaError_t mlp_gradient(const Mlp &m, const float *X, const float *T, const lon
                          double *acc, unsigned *status, cudaStream_t st);
 void mlp_adam(Mlp &m, double lr, cudaStream_t st);
 template <class S>
-void launch_shell_features(const Lattice &L, int p0, int np, float *feat, cudaStream_t st);
+void launch_shell_features(const Lattice &L, const Mlp &m, int p0, int np, float *feat, cudaStream_t st);
 template <class S>
 void launch_surrogate_forces(const Lattice &L, const Mlp &m, float *feat, cudaStream_t st, long long *launches,
                              const Marker &mk);

@@ -695,8 +695,18 @@ cudaError_t mlp_alloc(Mlp &m, int cap)
         (e = A((void **)&m.dYb, sizeof(bf16) * (size_t)cap * 16)) || (e = A((void **)&m.Y, sizeof(float) * (size_t)cap * 16)) ||
         (e = A((void **)&m.dY, sizeof(float) * (size_t)cap * 16)) ||
         (e = A((void **)&m.loss_part, sizeof(double) * ((size_t)cap / GM + 1))) ||
-        (e = A((void **)&m.loss, sizeof(double) * 2)))
+        (e = A((void **)&m.loss, sizeof(double) * 2)) || (e = A((void **)&m.dirs, sizeof(double) * 3 * MLP_SHELL)))
         return e;
+    // directions of the shell points: a Fibonacci sphere
+    double dirs[3 * MLP_SHELL];
+    for (int k = 0; k < MLP_SHELL; k++) {
+        const double ez = 1.0 - (2.0 * k + 1.0) / MLP_SHELL, er = std::sqrt(1.0 - ez * ez);
+        const double az = k * (3.14159265358979323846 * (3.0 - std::sqrt(5.0)));
+        dirs[3 * k] = er * std::cos(az);
+        dirs[3 * k + 1] = er * std::sin(az);
+        dirs[3 * k + 2] = ez;
+    }
+    if ((e = cudaMemcpy(m.dirs, dirs, sizeof dirs, cudaMemcpyHostToDevice))) return e;
     cudaMemset(m.adam_m, 0, sizeof(float) * MLP_NPARAM);
     cudaMemset(m.adam_v, 0, sizeof(float) * MLP_NPARAM);
     cudaMemset(m.loss, 0, sizeof(double) * 2);
@@ -706,7 +716,7 @@ cudaError_t mlp_alloc(Mlp &m, int cap)
 void mlp_free(Mlp &m)
 {
     void *ps[] = {m.theta, m.grad, m.adam_m, m.adam_v, m.W1b, m.W2b, m.W3b, m.X, m.H1, m.H2,
-                  m.dZ1, m.dZ2, m.dYb, m.Y, m.dY, m.loss_part, m.loss};
+                  m.dZ1, m.dZ2, m.dYb, m.Y, m.dY, m.loss_part, m.loss, m.dirs};
     for (void *p : ps) cudaFree(p);
     m = Mlp();
 }
@@ -753,26 +763,41 @@ void mlp_adam(Mlp &m, double lr, cudaStream_t st)
 namespace {
 
 // fields at point X (lattice units, wrapped) as the trilinear mean over the
-// fluid corners of its cell; false when no corner is fluid
+// fluid corners of its cell, whose loads are issued together; false when no
+// corner is fluid
 template <class R>
-__device__ bool interp_fluid(const Lattice &L, const InstDev &I, const double *X, double *phi, double *u)
+__device__ __forceinline__ bool interp_fluid(const Lattice &L, const InstDev &I, const double *X, double *phi, double *u)
 {
-    const int b[3] = {(int)floor(X[0]), (int)floor(X[1]), (int)floor(X[2])};
-    const double f[3] = {X[0] - b[0], X[1] - b[1], X[2] - b[2]};
+    const int n3[3] = {I.nx, I.ny, I.nz};
+    int lo[3], hi[3];
+    double f[3];
+    for (int a = 0; a < 3; a++) {
+        const int b = (int)floor(X[a]);
+        f[a] = X[a] - b;
+        lo[a] = b % n3[a];
+        hi[a] = (b + 1) % n3[a];
+    }
+    const uint8_t *fli = L.flags + I.node_off;
     const R *ph = (const R *)L.phi + I.node_off;
     const R *U = (const R *)L.u + I.node_off;
+    uint8_t fl[8];
+    R p[8], v[3][8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const int n = ((k & 4 ? hi[2] : lo[2]) * I.ny + (k & 2 ? hi[1] : lo[1])) * I.nx + (k & 1 ? hi[0] : lo[0]);
+        fl[k] = fli[n];
+        p[k] = ph[n];
+        for (int a = 0; a < 3; a++) v[a][k] = U[a * L.Ntot + n];
+    }
     double ap = 0.0, au[3] = {0.0, 0.0, 0.0}, ws = 0.0;
-    for (int dz = 0; dz < 2; dz++)
-        for (int dy = 0; dy < 2; dy++)
-            for (int dx = 0; dx < 2; dx++) {
-                const double w = (dx ? f[0] : 1.0 - f[0]) * (dy ? f[1] : 1.0 - f[1]) * (dz ? f[2] : 1.0 - f[2]);
-                const int x = (b[0] + dx) % I.nx, y = (b[1] + dy) % I.ny, z = (b[2] + dz) % I.nz;
-                const int n = (z * I.ny + y) * I.nx + x;
-                if ((L.flags[I.node_off + n] & OWNER_MASK) != OWN_FLUID) continue;
-                ap = ap + w * (double)ph[n];
-                for (int a = 0; a < 3; a++) au[a] = au[a] + w * (double)U[a * L.Ntot + n];
-                ws += w;
-            }
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        if ((fl[k] & OWNER_MASK) != OWN_FLUID) continue;
+        const double w = (k & 1 ? f[0] : 1.0 - f[0]) * (k & 2 ? f[1] : 1.0 - f[1]) * (k & 4 ? f[2] : 1.0 - f[2]);
+        ap = ap + w * (double)p[k];
+        for (int a = 0; a < 3; a++) au[a] = au[a] + w * (double)v[a][k];
+        ws += w;
+    }
     if (ws <= 0.0) return false;
     *phi = ap / ws;
     for (int a = 0; a < 3; a++) u[a] = au[a] / ws;
@@ -780,9 +805,9 @@ __device__ bool interp_fluid(const Lattice &L, const InstDev &I, const double *X
 }
 
 // features of particles p0..p0+gridDim.x-1: 96 shell points (one thread
-// each), then cos(theta), sin(theta), R/R_ref
+// each, directions from the table), then cos(theta), sin(theta), R/R_ref
 template <class R>
-__global__ void __launch_bounds__(128) k_shell(Lattice L, int p0, float *feat)
+__global__ void __launch_bounds__(MLP_SHELL + 32) k_shell(Lattice L, int p0, const double *dirs, float *feat)
 {
     const int p = p0 + blockIdx.x;
     const PartDev &P = L.parts[p];
@@ -790,10 +815,7 @@ __global__ void __launch_bounds__(128) k_shell(Lattice L, int p0, float *feat)
     float *f = feat + (long long)blockIdx.x * MLP_NIN;
     const int k = threadIdx.x;
     if (k < MLP_SHELL) {
-        const double ez = 1.0 - (2.0 * k + 1.0) / MLP_SHELL;
-        const double er = sqrt(1.0 - ez * ez);
-        const double az = k * (3.14159265358979323846 * (3.0 - sqrt(5.0)));
-        const double e[3] = {er * cos(az), er * sin(az), ez};
+        const double e[3] = {dirs[3 * k], dirs[3 * k + 1], dirs[3 * k + 2]};
         const double rs = P.R + I.sh_gap;
         const int n3[3] = {I.nx, I.ny, I.nz};
         double lev[3];
@@ -815,7 +837,9 @@ __global__ void __launch_bounds__(128) k_shell(Lattice L, int p0, float *feat)
             for (int a = 0; a < 3; a++) {
                 const double v = P.x[a] + lev[a] + d[a];
                 if (a == 2 && I.wall_z0 && !(v >= 0.0 && v < n3[2])) in_wall = true;
-                X[a] = v - n3[a] * floor(v / n3[a]);
+                // in [0, n) already, or one period off (the common cases), without a division
+                X[a] = v >= 0.0 && v < n3[a] ? v
+                                             : (v < 0.0 && v >= -n3[a] ? v + n3[a] : v - n3[a] * floor(v / n3[a]));
             }
             if (in_wall) continue;
             double p1 = 0.0, u1[3] = {0.0, 0.0, 0.0};
@@ -826,8 +850,10 @@ __global__ void __launch_bounds__(128) k_shell(Lattice L, int p0, float *feat)
         }
         float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         if (used > 0) {
-            ph /= used;
-            for (int a = 0; a < 3; a++) u[a] /= used;
+            if (nsub > 1) {
+                ph /= used;
+                for (int a = 0; a < 3; a++) u[a] /= used;
+            }
             const double us[3] = {P.v[0] + (P.w[1] * lev[2] - P.w[2] * lev[1]),
                                   P.v[1] + (P.w[2] * lev[0] - P.w[0] * lev[2]),
                                   P.v[2] + (P.w[0] * lev[1] - P.w[1] * lev[0])};
@@ -861,10 +887,10 @@ __global__ void k_surrogate_apply(Lattice L, const float *Y, int p0, int np)
 }  // namespace
 
 template <class S>
-void launch_shell_features(const Lattice &L, int p0, int np, float *feat, cudaStream_t st)
+void launch_shell_features(const Lattice &L, const Mlp &m, int p0, int np, float *feat, cudaStream_t st)
 {
     using R = typename Store<S>::real;
-    k_shell<R><<<np, 128, 0, st>>>(L, p0, feat);
+    k_shell<R><<<np, MLP_SHELL + 32, 0, st>>>(L, p0, m.dirs, feat);
 }
 
 template <class S>
@@ -875,7 +901,7 @@ void launch_surrogate_forces(const Lattice &L, const Mlp &m, float *feat, cudaSt
     mk(STAGE_SURROGATE, 0);
     for (int p0 = 0; p0 < L.n_parts; p0 += m.cap) {
         const int np = std::min(m.cap, L.n_parts - p0);
-        launch_shell_features<S>(L, p0, np, feat, st);
+        launch_shell_features<S>(L, m, p0, np, feat, st);
         // a failed set-up or launch stays in the runtime's last error, which
         // lbm_step checks after enqueueing the step
         if (mlp_forward(m, feat, np, L.status, st) != cudaSuccess) return;
@@ -886,7 +912,7 @@ void launch_surrogate_forces(const Lattice &L, const Mlp &m, float *feat, cudaSt
 }
 
 #define INST(S)                                                                                        \
-    template void launch_shell_features<S>(const Lattice &, int, int, float *, cudaStream_t);          \
+    template void launch_shell_features<S>(const Lattice &, const Mlp &, int, int, float *, cudaStream_t); \
     template void launch_surrogate_forces<S>(const Lattice &, const Mlp &, float *, cudaStream_t, long long *, \
                                              const Marker &);
 INST(double)

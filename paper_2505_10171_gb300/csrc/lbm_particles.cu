@@ -559,8 +559,8 @@ __global__ void __launch_bounds__(32) k_dem(Lattice L, int sum_fluid)
         const double x0 = P.x[lane], xn = P.xn[lane];
         P.x_old[lane] = x0;
         P.xfo[lane] = P.xf[lane];
-        // periodic domain: positions kept in [0, n)
-        const double x1 = ok ? xn - per * floor(xn / per) : x0;
+        // periodic domain: positions kept in [0, n) (the move is below a period)
+        const double x1 = !ok ? x0 : (xn < 0.0 ? xn + per : (xn >= per ? xn - per : xn));
         P.x[lane] = x1;
         P.xf[lane] = (float)x1;
     }
