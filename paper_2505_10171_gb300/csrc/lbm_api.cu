@@ -32,7 +32,7 @@ struct lbm_ctx {
     // (phi, b n) of the current state, one per node
     void *phi = nullptr, *col = nullptr;
     size_t col_sz = 32;  // bytes of one colour record
-    void *grad = nullptr, *u = nullptr;
+    void *grad = nullptr, *nrm = nullptr, *u = nullptr;
     std::vector<PartDev> parts_h;
     PartDev *parts_d = nullptr;
     double *mem_part = nullptr, *cap_part = nullptr, *hist = nullptr;
@@ -78,7 +78,7 @@ struct lbm_ctx {
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_pairs;
     cudaEvent_t ev_open[N_STAGES] = {};
     // launch variant of the fluid update
-    FluidLaunch fz = {0, 0, 0, 0, 8, false};
+    FluidLaunch fz = {0, 0, 0, 0, false};
     int zc_request = 0;        // z-planes per gradient work item, 0: automatic
     std::vector<int> zc_inst;  // per instance (the autotuner's size classes), 0: zc_request
     // drop-speed control: per instance integral (3) and last U_a (3); block partials
@@ -104,7 +104,7 @@ struct lbm_ctx {
 // when every row has an even length
 static void plan_launch(lbm_ctx *c)
 {
-    plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, c->prec == LBM_FP64, &c->fz);
+    plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, &c->fz);
     plan_phi(c->inst_h, c->n_sm, c->prec == LBM_FP64, &c->fz);
     plan_items(c->inst_h, c->prec == LBM_FP64, &c->fz);
     bool even = true;
@@ -151,6 +151,7 @@ static Lattice make_lattice(const lbm_ctx *c)
     L.phi = c->phi;
     L.col = c->col;
     L.grad = c->grad;
+    L.nrm = c->nrm;
     L.u = c->u;
     L.Ntot = c->Ntot;
     L.parts = c->parts_d;
@@ -861,6 +862,7 @@ void lbm_destroy(lbm_ctx *ctx)
     cudaFree(ctx->phi);
     cudaFree(ctx->col);
     cudaFree(ctx->grad);
+    cudaFree(ctx->nrm);
     cudaFree(ctx->static_list);
     cudaFree(ctx->static_bfl);
     cudaFree(ctx->speed_d);
@@ -1043,6 +1045,7 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
         (st = alloc(&ctx->pop[1], ctx->pop_bytes)) || (st = alloc(&ctx->phi, Nt * ctx->real_sz)) ||
         (st = alloc(&ctx->col, Nt * ctx->col_sz)) ||
         (st = alloc(&ctx->grad, 4 * Nt * ctx->real_sz)) ||
+        (prec == LBM_FP64 && (st = alloc(&ctx->nrm, 3 * Nt * ctx->real_sz))) ||
         (st = alloc((void **)&ctx->status, sizeof(unsigned))) ||
         (st = alloc((void **)&ctx->diag_d, sizeof(double) * 2 * n_instances)) ||
         (st = alloc((void **)&ctx->diag_part, sizeof(double) * 2 * DIAG_BLOCKS)) ||

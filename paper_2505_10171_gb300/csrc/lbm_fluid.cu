@@ -8,8 +8,9 @@
 //
 // Kernels of a step: k_phi (z-marching tiles) stores phi;
 // the solid-phi fill over the listed static solid nodes and the step's list
-// of particle-surface solid nodes; k_gradcurv (z-marching tiles:
-// gradient, wetting, normal, curvature); k_collide (or k_collide2).  Nodes next
+// of particle-surface solid nodes; k_gradcurv (z-marching tiles: gradient,
+// wetting, normal, curvature; FP64: k_grad64 and k_curv64); k_collide (or
+// k_collide2).  Nodes next
 // to a solid go to the boundary passes k_phi_bound and k_collide_bound, which
 // run beside the bulk kernels on a second stream.
 //
@@ -679,7 +680,7 @@ __global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : LBM_COL
 // ---------------------------------------------------------------------------
 // gradient, wetting, normal and curvature in one z-marching pass
 // ---------------------------------------------------------------------------
-// A CTA owns a GC_TX x (ROWS RP) column tile and a chunk of z-planes and
+// FP32 arithmetic: a CTA owns a GC_TX x (ROWS RP) column tile and a chunk of z-planes and
 // marches through the chunk's planes of phi (2-node halo).  Both stencils
 // split into in-plane sums of one plane each: with X, Y the differences of the
 // +-x and +-y neighbours, S the sum of the four, A and B the sum and difference
@@ -713,10 +714,6 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // the sums of the gradient carried from plane to plane for one column
 template <class R>
@@ -758,8 +755,8 @@ struct GcPart {
     R x[3], rad, c, s;
 };
 
-// a fluid node next to a solid (region column c, flag planes f0, f1, f2 below,
-// at and above it): the wetting rotation of its gradient g, and
+// a fluid node next to a solid (flag(i): flags of its neighbour i, part(p):
+// particle p): the wetting rotation of its gradient g, and
 // s = 3 sum w_i c_i over its solid neighbours, which take the node's own normal
 // in the curvature (their share is n . s).  The outward solid normal and
 // contact angle: the nearest particle surface if a neighbour belongs to a
@@ -770,16 +767,15 @@ struct GcPart {
 // only where two particles meet.  With the owners' particle records read from
 // memory per direction the pass took 195 us instead of 75 on 256x128x128
 // nodes with eight spheres.
-template <class R, int PW>
-__device__ __forceinline__ void gc_solid(const InstDev &I, const GcPart<R> *parts, const uint8_t *f0,
-                                         const uint8_t *f1, const uint8_t *f2, int c, R phi, int x, int y, int z,
-                                         R *g, R *s)
+template <class R, class Flag, class Part>
+__device__ __forceinline__ void gc_solid(const InstDev &I, const Part &part, const Flag &flag, R phi, int x, int y,
+                                         int z, R *g, R *s)
 {
     int all[3] = {0, 0, 0}, wall[3] = {0, 0, 0};
     unsigned long long met = 0;
 #pragma unroll
     for (int i = 1; i < Q; i++) {
-        const int own = (cz(i) < 0 ? f0 : (cz(i) > 0 ? f2 : f1))[c + cy(i) * PW + cx(i)] & OWNER_MASK;
+        const int own = flag(i) & OWNER_MASK;
         const int k = own == OWN_FLUID ? 0 : (csq(i) == 1 ? 2 : 1);
         const int kw = own == OWN_WALL ? k : 0;
         if (cx(i)) { all[0] += cx(i) * k; wall[0] += cx(i) * kw; }
@@ -798,7 +794,7 @@ __device__ __forceinline__ void gc_solid(const InstDev &I, const GcPart<R> *part
         R bestd = 0;
         bool first = true;
         do {
-            const GcPart<R> &P = parts[__ffsll((long long)met) - 1 - 2];
+            const GcPart<R> &P = part(__ffsll((long long)met) - 1 - 2);
             met &= met - 1;
             R e[3];
             if (sizeof(R) == 8) {
@@ -824,30 +820,27 @@ __device__ __forceinline__ void gc_solid(const InstDev &I, const GcPart<R> *part
     wetting_rotate<R>(g, ns, cth, sth);
 }
 
-// Threads of the pass for arithmetic type R.  Two rows per thread share most of
-// their shared-memory reads (floats: 75 against 72 us with one on 256x128x128
-// nodes, but 1738 against 1993 us on the 96-domain sweep); 8 warps of own
-// nodes beat 4 (80 and 1864 us) and 6 (82 and 1956 us).  FP64 runs are small
-// and bound by the FP64 pipe of the SMs that they reach: one row, and 4 or 8
-// warps by plan_gradcurv's rule (48x32x32: 61 against 90 us).
-template <class R, int ROWS>
+// Threads of the pass.  Two rows per thread share most of their shared-memory
+// reads (75 against 72 us with one on 256x128x128 nodes, but 1738 against
+// 1993 us on the 96-domain sweep); 8 warps of own nodes beat 4 (80 and 1864 us)
+// and 6 (82 and 1956 us).
 struct GcShape {
-    static constexpr int RP = sizeof(R) == 8 ? 1 : 2;
+    static constexpr int RP = 2, ROWS = 8;
     static constexpr int TY = ROWS * RP;
     static constexpr int RING = (GC_TX + 2) * (TY + 2) - GC_TX * TY;  // nodes around the tile
     static constexpr int OWN = GC_TX * ROWS;
     static constexpr int NT = OWN + (RING + 31) / 32 * 32;
 };
 
-// CTAs per SM of the float form: 2 (80 registers); with 3 (56) the march spills
-// and took 139 to 168 us
+// CTAs per SM: 2 (80 registers); with 3 (56) the march spills and took 139 to
+// 168 us
 #ifndef LBM_GC_MINB
 #define LBM_GC_MINB 2
 #endif
-template <class R, int ROWS>
-__global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM_GC_MINB) k_gradcurv(Lattice L)
+__global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L)
 {
-    using Shape = GcShape<R, ROWS>;
+    using R = float;
+    using Shape = GcShape;
     constexpr int RP = Shape::RP, TY = Shape::TY, NT = Shape::NT, OWN = Shape::OWN;
     constexpr int PW = GC_TX + 4, PH = TY + 4, PN = PW * PH;  // phi / flag region (2-node halo)
     constexpr int NW = GC_TX + 2, NH = TY + 2, NN = NW * NH;  // normal region (1-node halo)
@@ -908,7 +901,7 @@ __global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM
         const int r = min(tid + q * NT, PN - 1);
         roff[q] = wrap_any(y0 - 2 + r / PW, ny) * nx + wrap_any(x0 - 2 + r % PW, nx);
     }
-    const R eps2 = sizeof(R) == 8 ? (R)(I.grad_eps * I.grad_eps) : (R)I.f_eps2;
+    const R eps2 = I.f_eps2;
     pdl_trigger();  // the collision may be scheduled as this grid drains
     pdl_wait();     // phi of the order-parameter pass
     R pv[PER];
@@ -939,7 +932,7 @@ __global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM
     };
     for (int p = tid; p < I.np; p += NT) {
         const PartDev &P = L.parts[I.part_off + p];
-        for (int a = 0; a < 3; a++) partS[p].x[a] = sizeof(R) == 8 ? (R)P.x[a] : (R)P.xf[a];
+        for (int a = 0; a < 3; a++) partS[p].x[a] = P.xf[a];
         partS[p].rad = (R)P.R;
         partS[p].c = (R)P.cos_t;
         partS[p].s = (R)P.sin_t;
@@ -986,9 +979,12 @@ __global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM
                     solid = (fl & OWNER_MASK) != OWN_FLUID;
                     if (!solid && (fl & BOUND_BIT)) {
                         R sv[3] = {0, 0, 0};
-                        gc_solid<R, PW>(I, partS, flS[(j - 2) & 3], flS[(j - 1) & 3], flS[j & 3], c,
-                                        phS[(j - 1) & 3][c], wrap_any(gx, nx), wrap_any(gy + r, ny),
-                                        wrap_any(z0 - 3 + j, nz), g, sv);
+                        const uint8_t *f0 = flS[(j - 2) & 3], *f1 = flS[(j - 1) & 3], *f2 = flS[j & 3];
+                        gc_solid<R>(
+                            I, [&](int p) -> const GcPart<R> & { return partS[p]; },
+                            [&](int i) { return (cz(i) < 0 ? f0 : (cz(i) > 0 ? f2 : f1))[c + cy(i) * PW + cx(i)]; },
+                            phS[(j - 1) & 3][c], wrap_any(gx, nx), wrap_any(gy + r, ny), wrap_any(z0 - 3 + j, nz), g,
+                            sv);
                         s0 = sv[0]; s1 = sv[1]; s2 = sv[2];
                     }
                 }
@@ -1052,6 +1048,113 @@ __global__ void __launch_bounds__(GcShape<R, ROWS>::NT, sizeof(R) == 8 ? 1 : LBM
     }
 }
 
+// The FP64 form: a node per thread and two kernels, the normals going through
+// memory.  FP64 instructions have 2 lanes a clock on an SM, so that they are
+// the cost (28 of the gradient, about 45 of the normal, 30 of the curvature; on
+// 48x32x32 nodes 10 us of the whole chip) and the marching tiles' work around
+// their nodes, 1.6 times the normals in a plane and 4 planes more than a chunk
+// has, is what an FP64 run cannot afford: 48x32x32 with a sphere 25 us for
+// both kernels, 59 us marching.
+// One warp a CTA, since the FP64 pipe that a CTA lands on is shared by its SM.
+constexpr int GC64_THREADS = 32;
+__device__ __forceinline__ bool gc64_node(const Lattice &L, const InstDev **I, int *n, int *x, int *y, int *z)
+{
+    constexpr int PER = COLLIDE_NODES<double> / GC64_THREADS;  // CTAs of a work item of the collision
+    return item_node(L, blockIdx.x / PER, COLLIDE_NODES<double>,
+                     (int)(blockIdx.x % PER) * GC64_THREADS + (int)threadIdx.x, I, n, x, y, z);
+}
+
+// gradient, wetting and normal (0 at a solid node); the solid neighbours' share
+// of the curvature into its slot
+__global__ void __launch_bounds__(GC64_THREADS) k_grad64(Lattice L)
+{
+    using R = double;
+    const InstDev *Ip;
+    int n, x, y, z;
+    const bool have = gc64_node(L, &Ip, &n, &x, &y, &z);
+    pdl_trigger();
+    pdl_wait();  // phi of the order-parameter pass
+    if (!have) return;
+    const InstDev &I = *Ip;
+    const uint8_t *const fli = L.flags + I.node_off;
+    const R *const ph = (const R *)L.phi + I.node_off;
+    R *const nrm = (R *)L.nrm + I.node_off;
+    Nbr nb;
+    nb.init(x, y, z, I.nx, I.ny, I.nz);
+    const uint8_t fl = fli[n];
+    R v[Q];
+#pragma unroll
+    for (int i = 0; i < Q; i++) v[i] = ph[nb.at(cx(i), cy(i), cz(i))];
+    if ((fl & OWNER_MASK) != OWN_FLUID) {
+        for (int a = 0; a < 3; a++) nrm[a * L.Ntot + n] = 0;
+        return;
+    }
+    // per axis: difference of the two axis neighbours, and of the diagonal ones
+    R g[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        R axis = 0, diag = 0;
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
+            if (c <= 0) continue;
+            // the neighbour mirrored in this axis
+            const int m = dir_of(a == 0 ? -cx(i) : cx(i), a == 1 ? -cy(i) : cy(i), a == 2 ? -cz(i) : cz(i));
+            if (csq(i) == 1) axis = v[i] - v[m];
+            else diag += v[i] - v[m];
+        }
+        g[a] = fma(R(1.0 / 6.0), axis, R(1.0 / 12.0) * diag);
+    }
+    R sv[3] = {0, 0, 0};
+    if (fl & BOUND_BIT) {
+        auto part = [&](int p) {
+            const PartDev &P = L.parts[I.part_off + p];
+            return GcPart<R>{{P.x[0], P.x[1], P.x[2]}, P.R, P.cos_t, P.sin_t};
+        };
+        gc_solid<R>(
+            I, part, [&](int i) { return fli[nb.at(cx(i), cy(i), cz(i))]; }, v[0], x, y, z, g, sv);
+    }
+    const R im = frsqrt(fma(g[0], g[0], fma(g[1], g[1], fma(g[2], g[2], (R)(I.grad_eps * I.grad_eps)))));
+    R share = 0;
+    for (int a = 0; a < 3; a++) {
+        const R na = g[a] * im;
+        nrm[a * L.Ntot + n] = na;
+        share = fma(na, sv[a], share);
+    }
+    ((GradRec<R> *)L.grad)[I.node_off + n] = GradRec<R>{g[0], g[1], g[2], share};
+}
+
+// curvature
+__global__ void __launch_bounds__(GC64_THREADS) k_curv64(Lattice L)
+{
+    using R = double;
+    const InstDev *Ip;
+    int n, x, y, z;
+    const bool have = gc64_node(L, &Ip, &n, &x, &y, &z);
+    pdl_trigger();  // the collision may be scheduled as this grid drains
+    pdl_wait();     // the normals
+    if (!have) return;
+    const InstDev &I = *Ip;
+    const R *const nrm = (const R *)L.nrm + I.node_off;
+    R *const k = &((GradRec<R> *)L.grad)[I.node_off + n].k;
+    Nbr nb;
+    nb.init(x, y, z, I.nx, I.ny, I.nz);
+    const uint8_t fl = L.flags[I.node_off + n];
+    const R share = *k;
+    R axis = 0, diag = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
+            if (c == 0) continue;
+            const R na = nrm[a * L.Ntot + nb.at(cx(i), cy(i), cz(i))];
+            R &sum = csq(i) == 1 ? axis : diag;
+            sum = c > 0 ? sum + na : sum - na;
+        }
+    if ((fl & OWNER_MASK) == OWN_FLUID) *k = share + fma(R(1.0 / 6.0), axis, R(1.0 / 12.0) * diag);
+}
+
 // Cost of marching chunks of zc planes (and `halo` planes more) through column
 // tiles of tx x ty nodes over all instances, in plane iterations: the waves of
 // CTAs, counted as full ones (a CTA of the last wave runs as long as any) and
@@ -1070,38 +1173,28 @@ static double march_cost(const std::vector<InstDev> &inst, int tx, int ty, int z
 }
 constexpr int ZC_MAX = 64;
 
-// The gradient pass's work items.  Where no z-chunk is asked for, the planes
-// per item (and for FP64 the tile's height, by the threads that march) of the
-// least cost.  Slots are the resident CTAs; one per SM for FP64, whose CTAs
-// share their SM's FP64 pipe.  128x64x64 FP32, 4 planes against 16: 24 against
-// 37 us; 48x32x32 FP64: 61 us against 270 with 16 planes.  Every choice gives
-// the same bits.
-void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool fp64,
+// The FP32 gradient pass's work items.  Where no z-chunk is asked for, the
+// planes per item of the least cost; slots are the resident CTAs.  128x64x64, 4
+// planes against 16: 24 against 37 us.  Every choice gives the same bits.
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm,
                    FluidLaunch *fz)
 {
-    const double slots = n_sm * (fp64 ? 1.0 : (double)LBM_GC_MINB);
-    int rows = 8, zc_auto = 16;
+    const double slots = n_sm * (double)LBM_GC_MINB;
+    int zc_auto = 16;
     double least = -1.0;
-    for (int r : {8, 4}) {
-        if (r == 4 && !fp64) continue;
-        const int ty = fp64 ? r : GcShape<float, 8>::TY;
-        const double threads = r == 8 ? GcShape<double, 8>::NT : GcShape<double, 4>::NT;
-        for (int zc = ZC_MAX; zc >= 2; zc--) {
-            const double cost = march_cost(inst, GC_TX, ty, zc, 4, slots) * threads;
-            if (least < 0.0 || cost < least) {
-                least = cost;
-                rows = r;
-                zc_auto = zc;
-            }
+    for (int zc = ZC_MAX; zc >= 2; zc--) {
+        const double cost = march_cost(inst, GC_TX, GcShape::TY, zc, 4, slots);
+        if (least < 0.0 || cost < least) {
+            least = cost;
+            zc_auto = zc;
         }
     }
-    const int ty = fp64 ? rows : GcShape<float, 8>::TY;
     long long items = 0;
     for (size_t k = 0; k < inst.size(); k++) {
         InstDev &I = inst[k];
         const int req = k < zc_inst.size() && zc_inst[k] > 0 ? zc_inst[k] : zc_request;
         I.gc_tiles_x = (I.nx + GC_TX - 1) / GC_TX;
-        I.gc_tiles_y = (I.ny + ty - 1) / ty;
+        I.gc_tiles_y = (I.ny + GcShape::TY - 1) / GcShape::TY;
         const int zc = std::min(req > 0 ? req : zc_auto, I.nz);
         I.gc_nchunks = (I.nz + zc - 1) / zc;
         I.gc_zc = (I.nz + I.gc_nchunks - 1) / I.gc_nchunks;
@@ -1111,7 +1204,6 @@ void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector
         items += (long long)I.gc_tiles_x * I.gc_tiles_y * I.gc_nchunks;
     }
     fz->gc_items = items;
-    fz->gc_rows = rows;
 }
 
 // The order-parameter pass's work items, planned alike: one plane of halo
@@ -1221,11 +1313,12 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     if (lane.side && any_bound) cudaStreamWaitEvent(st, lane.b, 0);
     mk(STAGE_GRAD, 0);
     if constexpr (sizeof(R) == 8) {
-        if (fz.gc_rows == 4)
-            launch_after(k_gradcurv<R, 4>, dim3((unsigned)fz.gc_items), dim3(GcShape<R, 4>::NT), st, L);
-    }
-    if (fz.gc_rows == 8)
-        launch_after(k_gradcurv<R, 8>, dim3((unsigned)fz.gc_items), dim3(GcShape<R, 8>::NT), st, L);
+        const dim3 warps((unsigned)(fz.items * (COLLIDE_NODES<double> / GC64_THREADS)));
+        launch_after(k_grad64, warps, dim3(GC64_THREADS), st, L);
+        launch_after(k_curv64, warps, dim3(GC64_THREADS), st, L);
+        *launches += 1;
+    } else
+        launch_after(k_gradcurv, dim3((unsigned)fz.gc_items), dim3(GcShape::NT), st, L);
     mk(STAGE_GRAD, 1);
     lane.after_grad();
     if constexpr (BOUNCE_IN_SLOTS<S>) {

@@ -35,6 +35,13 @@ __host__ __device__ constexpr int cx(int i) { return i == 0 ? 0 : (i <= 9 ? hx(i
 __host__ __device__ constexpr int cy(int i) { return i == 0 ? 0 : (i <= 9 ? hy(i - 1) : -hy(i - 10)); }
 __host__ __device__ constexpr int cz(int i) { return i == 0 ? 0 : (i <= 9 ? hz(i - 1) : -hz(i - 10)); }
 __host__ __device__ constexpr int opp(int i) { return i == 0 ? 0 : (i <= 9 ? i + 9 : i - 9); }
+// the direction with c = (x, y, z)
+__host__ __device__ constexpr int dir_of(int x, int y, int z)
+{
+    for (int i = 0; i < Q; i++)
+        if (cx(i) == x && cy(i) == y && cz(i) == z) return i;
+    return -1;
+}
 __host__ __device__ constexpr int csq(int i) { return cx(i) * cx(i) + cy(i) * cy(i) + cz(i) * cz(i); }
 template <class T>
 __host__ __device__ constexpr T wgt(int i)
@@ -193,6 +200,7 @@ struct Lattice {
     void *phi;           // [Ntot] real: the order parameter of the step (outside a step: of the last one)
     void *col;           // [Ntot] ColRec<real>: colour record (phi, b n) of the stored state
     void *grad;          // [Ntot] GradRec<real>: corrected grad(phi) and curvature of fluid nodes
+    void *nrm;           // [3][Ntot] double: the normals between the FP64 gradient and curvature kernels
     void *u;             // [3][Ntot] real (store_velocity)
     long long Ntot;
     PartDev *parts;
@@ -722,13 +730,12 @@ struct FluidLaunch {
     long long items;    // collision work items (all instances)
     long long ph_items; // order-parameter work items (all instances)
     long long gc_items; // gradient + curvature work items (all instances)
-    int gc_rows;        // warps of own nodes per CTA of that kernel (8; FP64: 4 or 8)
     bool pair;          // every instance has an even nx: node-pair kernels for 16-bit storage
 };
 // plan the work items of the gradient + curvature kernel into fz (z-planes per
 // item: zc_inst[k] for instance k where set (> 0), else zc_request where set,
-// else chosen from the grid's size and the n_sm SMs; fp64: double arithmetic)
-void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool fp64,
+// else chosen from the grid's size and the n_sm SMs); FP64 runs have no tiles
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm,
                    FluidLaunch *fz);
 // plan the work items of the order-parameter kernel into fz
 void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz);
