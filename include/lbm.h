@@ -324,7 +324,8 @@ lbm_status lbm_diagnostics(lbm_ctx *ctx, int inst, double *out);
  * bulk collision takes two nodes of a row per thread (pair loads and stores),
  * one node per thread otherwise; tile 1: one node per thread always.
  * zchunk: z-planes per work item of the gradient pass (0: chosen from the
- * size of the grid; FP64 runs take a node per thread instead).  Every shape
+ * size of the grid; FP64 contexts and those of up to 655360 nodes take a node
+ * per thread instead).  Every shape
  * computes the same update; the node-pair collision agrees with the one-node
  * collision to the rounding of the storage type (the code generator may fuse
  * a different set of multiply-adds), the z-chunk gives the same bits.  Invalid

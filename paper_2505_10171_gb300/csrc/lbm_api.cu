@@ -1045,7 +1045,8 @@ lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision p
         (st = alloc(&ctx->pop[1], ctx->pop_bytes)) || (st = alloc(&ctx->phi, Nt * ctx->real_sz)) ||
         (st = alloc(&ctx->col, Nt * ctx->col_sz)) ||
         (st = alloc(&ctx->grad, 4 * Nt * ctx->real_sz)) ||
-        (prec == LBM_FP64 && (st = alloc(&ctx->nrm, 3 * Nt * ctx->real_sz))) ||
+        ((prec == LBM_FP64 || ctx->Ntot <= GRAD_NODES_MAX) &&
+         (st = alloc(&ctx->nrm, 3 * Nt * ctx->real_sz))) ||
         (st = alloc((void **)&ctx->status, sizeof(unsigned))) ||
         (st = alloc((void **)&ctx->diag_d, sizeof(double) * 2 * n_instances)) ||
         (st = alloc((void **)&ctx->diag_part, sizeof(double) * 2 * DIAG_BLOCKS)) ||

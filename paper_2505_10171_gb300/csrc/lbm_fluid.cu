@@ -9,8 +9,8 @@
 // Kernels of a step: k_phi (z-marching tiles) stores phi;
 // the solid-phi fill over the listed static solid nodes and the step's list
 // of particle-surface solid nodes; k_gradcurv (z-marching tiles: gradient,
-// wetting, normal, curvature; FP64: k_grad64 and k_curv64); k_collide (or
-// k_collide2).  Nodes next
+// wetting, normal, curvature; FP64 and small grids: k_grad_nodes and
+// k_curv_nodes); k_collide (or k_collide2).  Nodes next
 // to a solid go to the boundary passes k_phi_bound and k_collide_bound, which
 // run beside the bulk kernels on a second stream.
 //
@@ -714,6 +714,10 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // the sums of the gradient carried from plane to plane for one column
 template <class R>
@@ -1048,30 +1052,42 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
     }
 }
 
-// The FP64 form: a node per thread and two kernels, the normals going through
-// memory.  FP64 instructions have 2 lanes a clock on an SM, so that they are
-// the cost (28 of the gradient, about 45 of the normal, 30 of the curvature; on
-// 48x32x32 nodes 10 us of the whole chip) and the marching tiles' work around
-// their nodes, 1.6 times the normals in a plane and 4 planes more than a chunk
-// has, is what an FP64 run cannot afford: 48x32x32 with a sphere 25 us for
-// both kernels, 59 us marching.
-// One warp a CTA, since the FP64 pipe that a CTA lands on is shared by its SM.
-constexpr int GC64_THREADS = 32;
-__device__ __forceinline__ bool gc64_node(const Lattice &L, const InstDev **I, int *n, int *x, int *y, int *z)
+// The form without tiles: a node per thread and two kernels, the normals going
+// through memory, with the roundings of the marching form (the same bits).
+//
+// FP64: FP64 instructions have 2 lanes a clock on an SM, so that they are the
+// cost (about 35 of the gradient, 45 of the normal, 40 of the curvature; on
+// 48x32x32 nodes some 10 us of the whole chip), and the marching tiles' work
+// around their nodes, 1.6 times the normals in a plane and 4 planes more than a
+// chunk has, is what a run cannot afford: 48x32x32 with a sphere 25 us for both
+// kernels, 59 us marching.  One warp a CTA, since the FP64 pipe that a CTA lands
+// on is shared by its SM.
+//
+// FP32 arithmetic: bound by latency on a small grid, where a march of some 10
+// planes with a barrier each is a chain that few CTAs walk, and by loads (48 a
+// node) and 28 bytes a node more on a large one.  Marching against this form,
+// with the events' 5 us: 48x32x32 21 and 11 us, 4 x 48^3 (0.44 M nodes) 29 and
+// 19, 16 x 40x33x29 (0.61 M) 39 and 26, 96x96x64 (0.59 M) 21 and 21, 96^3
+// (0.88 M) 25 and 27, 256x128x64 35 and 49, 256x128x128 73 and 115: taken up
+// to GRAD_NODES_MAX nodes of a context.
+template <class R>
+constexpr int GN_THREADS = sizeof(R) == 8 ? 32 : 128;
+template <class R>
+__device__ __forceinline__ bool gn_node(const Lattice &L, const InstDev **I, int *n, int *x, int *y, int *z)
 {
-    constexpr int PER = COLLIDE_NODES<double> / GC64_THREADS;  // CTAs of a work item of the collision
-    return item_node(L, blockIdx.x / PER, COLLIDE_NODES<double>,
-                     (int)(blockIdx.x % PER) * GC64_THREADS + (int)threadIdx.x, I, n, x, y, z);
+    constexpr int PER = COLLIDE_NODES<R> / GN_THREADS<R>;  // CTAs of a work item of the collision
+    return item_node(L, blockIdx.x / PER, COLLIDE_NODES<R>,
+                     (int)(blockIdx.x % PER) * GN_THREADS<R> + (int)threadIdx.x, I, n, x, y, z);
 }
 
 // gradient, wetting and normal (0 at a solid node); the solid neighbours' share
 // of the curvature into its slot
-__global__ void __launch_bounds__(GC64_THREADS) k_grad64(Lattice L)
+template <class R>
+__global__ void __launch_bounds__(GN_THREADS<R>) k_grad_nodes(Lattice L)
 {
-    using R = double;
     const InstDev *Ip;
     int n, x, y, z;
-    const bool have = gc64_node(L, &Ip, &n, &x, &y, &z);
+    const bool have = gn_node<R>(L, &Ip, &n, &x, &y, &z);
     pdl_trigger();
     pdl_wait();  // phi of the order-parameter pass
     if (!have) return;
@@ -1089,48 +1105,53 @@ __global__ void __launch_bounds__(GC64_THREADS) k_grad64(Lattice L)
         for (int a = 0; a < 3; a++) nrm[a * L.Ntot + n] = 0;
         return;
     }
-    // per axis: difference of the two axis neighbours, and of the diagonal ones
+    auto at = [&](int dx, int dy, int dz) { return v[dir_of(dx, dy, dz)]; };
+    const R twelfth = R(1.0 / 12.0), sixth = R(1.0 / 6.0);
     R g[3];
+    {
+        const R d1 = sub_rn(at(1, 1, 0), at(-1, -1, 0)), d2 = sub_rn(at(1, -1, 0), at(-1, 1, 0));
+        const R X = sub_rn(at(1, 0, 0), at(-1, 0, 0)), Y = sub_rn(at(0, 1, 0), at(0, -1, 0));
+        R hx[2], hy[2], q[2];  // of the planes below and above
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        R axis = 0, diag = 0;
-#pragma unroll
-        for (int i = 1; i < Q; i++) {
-            const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
-            if (c <= 0) continue;
-            // the neighbour mirrored in this axis
-            const int m = dir_of(a == 0 ? -cx(i) : cx(i), a == 1 ? -cy(i) : cy(i), a == 2 ? -cz(i) : cz(i));
-            if (csq(i) == 1) axis = v[i] - v[m];
-            else diag += v[i] - v[m];
+        for (int k = 0; k < 2; k++) {
+            const int dz = 2 * k - 1;
+            hx[k] = mul_rn(twelfth, sub_rn(at(1, 0, dz), at(-1, 0, dz)));
+            hy[k] = mul_rn(twelfth, sub_rn(at(0, 1, dz), at(0, -1, dz)));
+            q[k] = fma_rn(sixth, at(0, 0, dz),
+                          mul_rn(twelfth, add_rn(add_rn(at(1, 0, dz), at(-1, 0, dz)), add_rn(at(0, 1, dz), at(0, -1, dz)))));
         }
-        g[a] = fma(R(1.0 / 6.0), axis, R(1.0 / 12.0) * diag);
+        g[0] = add_rn(fma_rn(sixth, X, fma_rn(twelfth, add_rn(d1, d2), hx[0])), hx[1]);
+        g[1] = add_rn(fma_rn(sixth, Y, fma_rn(twelfth, sub_rn(d1, d2), hy[0])), hy[1]);
+        g[2] = sub_rn(q[1], q[0]);
     }
     R sv[3] = {0, 0, 0};
     if (fl & BOUND_BIT) {
         auto part = [&](int p) {
             const PartDev &P = L.parts[I.part_off + p];
-            return GcPart<R>{{P.x[0], P.x[1], P.x[2]}, P.R, P.cos_t, P.sin_t};
+            if constexpr (sizeof(R) == 8) return GcPart<R>{{P.x[0], P.x[1], P.x[2]}, P.R, P.cos_t, P.sin_t};
+            else return GcPart<R>{{P.xf[0], P.xf[1], P.xf[2]}, (R)P.R, (R)P.cos_t, (R)P.sin_t};
         };
         gc_solid<R>(
             I, part, [&](int i) { return fli[nb.at(cx(i), cy(i), cz(i))]; }, v[0], x, y, z, g, sv);
     }
-    const R im = frsqrt(fma(g[0], g[0], fma(g[1], g[1], fma(g[2], g[2], (R)(I.grad_eps * I.grad_eps)))));
-    R share = 0;
+    const R eps2 = sizeof(R) == 8 ? (R)(I.grad_eps * I.grad_eps) : (R)I.f_eps2;
+    const R im = frsqrt(fma_rn(g[0], g[0], fma_rn(g[1], g[1], fma_rn(g[2], g[2], eps2))));
+    R nn[3];
     for (int a = 0; a < 3; a++) {
-        const R na = g[a] * im;
-        nrm[a * L.Ntot + n] = na;
-        share = fma(na, sv[a], share);
+        nn[a] = mul_rn(g[a], im);
+        nrm[a * L.Ntot + n] = nn[a];
     }
+    const R share = fma_rn(nn[0], sv[0], fma_rn(nn[1], sv[1], mul_rn(nn[2], sv[2])));
     ((GradRec<R> *)L.grad)[I.node_off + n] = GradRec<R>{g[0], g[1], g[2], share};
 }
 
 // curvature
-__global__ void __launch_bounds__(GC64_THREADS) k_curv64(Lattice L)
+template <class R>
+__global__ void __launch_bounds__(GN_THREADS<R>) k_curv_nodes(Lattice L)
 {
-    using R = double;
     const InstDev *Ip;
     int n, x, y, z;
-    const bool have = gc64_node(L, &Ip, &n, &x, &y, &z);
+    const bool have = gn_node<R>(L, &Ip, &n, &x, &y, &z);
     pdl_trigger();  // the collision may be scheduled as this grid drains
     pdl_wait();     // the normals
     if (!have) return;
@@ -1141,18 +1162,26 @@ __global__ void __launch_bounds__(GC64_THREADS) k_curv64(Lattice L)
     nb.init(x, y, z, I.nx, I.ny, I.nz);
     const uint8_t fl = L.flags[I.node_off + n];
     const R share = *k;
-    R axis = 0, diag = 0;
+    // normals' components where the curvature takes them: n_a of the neighbours with c_a != 0
+    auto at = [&](int a, int dx, int dy, int dz) { return nrm[a * L.Ntot + nb.at(dx, dy, dz)]; };
+    const R twelfth = R(1.0 / 12.0), sixth = R(1.0 / 6.0);
+    R e[3];
 #pragma unroll
-    for (int a = 0; a < 3; a++)
+    for (int dz = -1; dz <= 1; dz++)
+        e[dz + 1] = add_rn(sub_rn(at(0, 1, 0, dz), at(0, -1, 0, dz)), sub_rn(at(1, 0, 1, dz), at(1, 0, -1, dz)));
+    R U[2], W[2];  // of the planes below and above
 #pragma unroll
-        for (int i = 1; i < Q; i++) {
-            const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
-            if (c == 0) continue;
-            const R na = nrm[a * L.Ntot + nb.at(cx(i), cy(i), cz(i))];
-            R &sum = csq(i) == 1 ? axis : diag;
-            sum = c > 0 ? sum + na : sum - na;
-        }
-    if ((fl & OWNER_MASK) == OWN_FLUID) *k = share + fma(R(1.0 / 6.0), axis, R(1.0 / 12.0) * diag);
+    for (int m = 0; m < 2; m++) {
+        const int dz = 2 * m - 1;
+        U[m] = mul_rn(twelfth, e[2 * m]);
+        W[m] = fma_rn(sixth, at(2, 0, 0, dz),
+                      mul_rn(twelfth, add_rn(add_rn(at(2, 1, 0, dz), at(2, -1, 0, dz)),
+                                             add_rn(at(2, 0, 1, dz), at(2, 0, -1, dz)))));
+    }
+    const R diag = add_rn(sub_rn(add_rn(at(0, 1, 1, 0), at(1, 1, 1, 0)), add_rn(at(0, -1, -1, 0), at(1, -1, -1, 0))),
+                          sub_rn(sub_rn(at(0, 1, -1, 0), at(1, 1, -1, 0)), sub_rn(at(0, -1, 1, 0), at(1, -1, 1, 0))));
+    const R kp = fma_rn(sixth, e[1], fma_rn(twelfth, diag, sub_rn(U[0], W[0])));
+    if ((fl & OWNER_MASK) == OWN_FLUID) *k = add_rn(add_rn(kp, add_rn(U[1], W[1])), share);
 }
 
 // Cost of marching chunks of zc planes (and `halo` planes more) through column
@@ -1312,10 +1341,10 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     mk(STAGE_PHI, 1);
     if (lane.side && any_bound) cudaStreamWaitEvent(st, lane.b, 0);
     mk(STAGE_GRAD, 0);
-    if constexpr (sizeof(R) == 8) {
-        const dim3 warps((unsigned)(fz.items * (COLLIDE_NODES<double> / GC64_THREADS)));
-        launch_after(k_grad64, warps, dim3(GC64_THREADS), st, L);
-        launch_after(k_curv64, warps, dim3(GC64_THREADS), st, L);
+    if (L.nrm) {
+        const dim3 ctas((unsigned)(fz.items * (COLLIDE_NODES<R> / GN_THREADS<R>)));
+        launch_after(k_grad_nodes<R>, ctas, dim3(GN_THREADS<R>), st, L);
+        launch_after(k_curv_nodes<R>, ctas, dim3(GN_THREADS<R>), st, L);
         *launches += 1;
     } else
         launch_after(k_gradcurv, dim3((unsigned)fz.gc_items), dim3(GcShape::NT), st, L);

@@ -200,7 +200,7 @@ struct Lattice {
     void *phi;           // [Ntot] real: the order parameter of the step (outside a step: of the last one)
     void *col;           // [Ntot] ColRec<real>: colour record (phi, b n) of the stored state
     void *grad;          // [Ntot] GradRec<real>: corrected grad(phi) and curvature of fluid nodes
-    void *nrm;           // [3][Ntot] double: the normals between the FP64 gradient and curvature kernels
+    void *nrm;           // [3][Ntot] real: the normals between the gradient and curvature kernels (null: one marching pass)
     void *u;             // [3][Ntot] real (store_velocity)
     long long Ntot;
     PartDev *parts;
@@ -732,9 +732,12 @@ struct FluidLaunch {
     long long gc_items; // gradient + curvature work items (all instances)
     bool pair;          // every instance has an even nx: node-pair kernels for 16-bit storage
 };
+// The gradient pass takes a node per thread in FP64 runs and up to this many
+// nodes of a context, marching tiles beyond (measured beside the kernels)
+constexpr long long GRAD_NODES_MAX = 640 * 1024;
 // plan the work items of the gradient + curvature kernel into fz (z-planes per
 // item: zc_inst[k] for instance k where set (> 0), else zc_request where set,
-// else chosen from the grid's size and the n_sm SMs); FP64 runs have no tiles
+// else chosen from the grid's size and the n_sm SMs); used where L.nrm is null
 void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm,
                    FluidLaunch *fz);
 // plan the work items of the order-parameter kernel into fz
