@@ -7,17 +7,22 @@
 //
 // The products are small (0.14 GFLOP forward for 1000 rows), so what they cost
 // is latency: launches, round trips to memory, and barriers.  Two kernels:
-//   k_mlp_rows   a CTA takes 128 rows through the whole network: inputs gathered
+//   k_mlp_rows   a CTA takes 32 rows through the whole network: inputs gathered
 //                and rounded to BF16 on the way into shared memory, the three
 //                layers with their activations, and in training the loss and
 //                both layers' deltas; weights and activations stay in shared
 //                memory from one product to the next;
 //   k_mlp_grads  the weight gradients (sums over the batch) with the bias
 //                gradients and the loss, a CTA per output tile.
+// The rows are the N side of the products and the layer's units the M side, so
+// that a CTA may have few rows (a batch of 512 is 16 CTAs) and yet every lane of
+// the tensor memory a value.
 // One GEMM launch per product with operands staged 64 columns at a time by a
 // loop of dependent loads took 36 to 46 us each, 17 launches and 285 us a batch
-// of 512; these two and Adam take 32, 18 and 4 us.  An epoch of 20000 samples
-// 11.4 -> 2.5 ms, 512 predictions with their copies 132 -> 64 us, to the same bits.
+// of 512; with 128 rows to a CTA (the M side) the two kernels and Adam took 31,
+// 18 and 4 us, now 21, 16 and 4.  An epoch of 20000 samples 11.4 -> 2.5 ->
+// 2.06 ms, 512 predictions with their copies 132 -> 61 -> 58 us, to the same
+// bits.
 //
 // Shared-memory operands are in the canonical layout without swizzle: 8 x
 // 16-byte core matrices of 128 bytes.  Read K-major, a core matrix holds 8 rows
@@ -91,6 +96,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
+// 8 columns
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v)
+{
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
+}
+
 // shared-memory matrix descriptor: start address, leading (k) and stride
 // (row-group) byte offsets, descriptor version 1, no swizzle
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
@@ -112,11 +130,23 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+// the same with the last 16 - bytes of them zero
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait_group()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-constexpr int GM = 128;        // rows of a tile (TMEM lanes)
+constexpr int GM = 128;        // M of a product (TMEM lanes)
+constexpr int NR = 32;         // rows of a CTA of the row kernel
 constexpr int MLP_THREADS = 256;   // gradients: two warps per quarter of the TMEM lanes
-constexpr int ROW_THREADS = 512;   // rows: four
+constexpr int ROW_THREADS = 512;   // rows: four, of 8 rows each
 
 // STEPS products of K = 16 each into tmem (the first one overwrites it where
 // fresh), issued and committed by one thread; a_step, b_step: bytes between
@@ -159,24 +189,41 @@ struct RowArgs {
     long long wait_limit;  // clock cycles a wait on the commit barrier may take
 };
 
-// shared memory: barrier, TMEM slot and biases; the input tile, whose place the
-// activations and deltas take over; W1, whose place W2 takes over; W3
+// shared memory: barrier, TMEM slot and biases; the input tile; activations and
+// deltas; the weights.  W3 has 16 rows (6..15 zero); a product with it on the M
+// side reads 128, whose results past the sixth are not used: up to 1920 bytes
+// behind the last slice's, kept in bounds by W3_BYTES
 struct RowSmem {
     static constexpr int BIAS = 128;                      // b1[128], b2[128], b3[16]
     static constexpr int RED = BIAS + 4 * (128 + 128 + 16);
     static constexpr int XA = 2048;
-    static constexpr int X_BYTES = GM * MLP_KIN * 2;
-    static constexpr int TILE = GM * MLP_HIDDEN * 2;      // 128 x 128
-    static constexpr int H1 = XA, H2 = XA + TILE, DZ2 = XA + 2 * TILE, DY = XA + 3 * TILE;  // DY: 128 x 16
-    static constexpr int WB = XA + X_BYTES;
-    static constexpr int W3 = WB + MLP_HIDDEN * MLP_KIN * 2;
-    static constexpr int BYTES = W3 + 16 * MLP_HIDDEN * 2;
+    static constexpr int TILE = NR * MLP_HIDDEN * 2;      // 32 x 128
+    static constexpr int H1 = XA + NR * MLP_KIN * 2, H2 = H1 + TILE, DZ2 = H2 + TILE, DY = DZ2 + TILE;  // DY: 32 x 16
+    static constexpr int W1 = DY + NR * 16 * 2;
+    static constexpr int W2 = W1 + MLP_HIDDEN * MLP_KIN * 2;
+    static constexpr int W3 = W2 + MLP_HIDDEN * MLP_HIDDEN * 2;
+    static constexpr int W3_BYTES = 16 * MLP_HIDDEN * 2 + 2048;
+    static constexpr int BYTES = W3 + W3_BYTES;
 };
-static_assert(RowSmem::RED + 64 <= RowSmem::XA && RowSmem::DY + GM * 32 <= RowSmem::WB, "regions");
+static_assert(RowSmem::RED + 128 <= RowSmem::XA, "regions");
+static_assert((MLP_HIDDEN / 8 - 1) * 256 + GM / 8 * 128 <= RowSmem::W3_BYTES, "rows read past W3");
 static_assert(RowSmem::BYTES <= 227 * 1024, "shared memory of a CTA");
 
-// 128 rows of core matrices: bytes between neighbours along k and along rows
-constexpr uint32_t T_LBO = GM / 8 * 128, T_SBO = 128;
+// bytes between neighbouring core matrices along k and along rows: 128 rows of
+// weights, NR rows of the batch
+constexpr uint32_t T_LBO = GM / 8 * 128, R_LBO = NR / 8 * 128, T_SBO = 128;
+
+// a weight matrix of 128 rows and K columns, row-major, into shared memory.  A
+// warp takes 8 rows by 64 bytes: whole sectors, and whole core matrices
+template <int K>
+__device__ __forceinline__ void load_weights(uint32_t dst, const bf16 *W, int tid)
+{
+    constexpr int KB = K / 8, QUADS = (KB + 3) / 4;
+    for (int i = tid; i < QUADS * 16 * 32; i += ROW_THREADS) {
+        const int r = (i & 7) + 8 * ((i >> 5) & 15), kb = ((i >> 3) & 3) + 4 * (i >> 9);
+        if (kb < KB) cp_async16(dst + (kb * 16 + (r >> 3)) * 128 + (r & 7) * 16, W + r * K + kb * 8);
+    }
+}
 
 template <bool TRAIN>
 __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
@@ -186,8 +233,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
     const uint32_t base = smem_addr(sm), bar = base, slot = base + 16;
     float *const bias = (float *)(sm + Sm::BIAS);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int r0 = blockIdx.x * GM;
-    constexpr uint32_t NCOLS = 256;
+    const int r0 = blockIdx.x * NR;
+    constexpr uint32_t NCOLS = 2 * NR;
 
     if (warp == 0) {
         tmem_alloc(slot, NCOLS);
@@ -197,50 +244,63 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
         mbar_init(bar, 1);
         mbar_fence_init();
     }
-    // W1 (row-major, 16 bytes at a time) and W3 (rows 6..15 zero)
-    for (int i = tid; i < MLP_HIDDEN * (MLP_KIN / 8); i += ROW_THREADS) {
-        const int r = i & 127, kb = i >> 7;
-        cp_async16(base + Sm::WB + (kb * 16 + (r >> 3)) * 128 + (r & 7) * 16, g.W1 + r * MLP_KIN + kb * 8);
+    // inputs: a warp takes 2 rows, all loads in flight
+    constexpr int NC = (MLP_KIN + 31) / 32;
+    float v[2][NC];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int r = r0 + warp * 2 + h;
+        const bool have = r < g.n;
+        const long long src = have ? (g.idx ? g.idx[g.row0 + r] : g.row0 + r) : 0;
+        const float *x = g.X + src * MLP_NIN;
+#pragma unroll
+        for (int j = 0; j < NC; j++) {
+            const int k = lane + 32 * j;
+            v[h][j] = have && k < MLP_NIN ? x[k] : 0.0f;
+        }
     }
+    load_weights<MLP_KIN>(base + Sm::W1, g.W1, tid);
+    load_weights<MLP_HIDDEN>(base + Sm::W2, g.W2, tid);
     if (tid < 256) {
         const int r = tid & 15, kb = tid >> 4;
         unsigned char *d = sm + Sm::W3 + (kb * 2 + (r >> 3)) * 128 + (r & 7) * 16;
         *(uint4 *)d = r < MLP_NOUT ? *(const uint4 *)(g.W3 + r * MLP_HIDDEN + kb * 8) : make_uint4(0, 0, 0, 0);
+    } else if (tid < 256 + NR * 2) {
+        *(uint4 *)(sm + Sm::DY + (tid - 256) * 16) = make_uint4(0, 0, 0, 0);
     }
     if (tid < 128) {
         bias[tid] = g.b1[tid];
         bias[128 + tid] = g.b2[tid];
         if (tid < 16) bias[256 + tid] = tid < MLP_NOUT ? g.b3[tid] : 0.0f;
     }
-    // inputs: a warp takes 8 rows, four at a time, with all loads of the four in flight
+    // this thread's unit (TMEM lane) and its 8 rows (TMEM columns) of the CTA's
+    const int unit = (warp & 3) * 32 + lane, row = (warp >> 2) * 8;
+    const bool out_unit = unit < MLP_NOUT;
+    float target[8];
+    if (TRAIN && out_unit) {
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int r = r0 + row + j;
+            target[j] = r < g.n ? g.T[(g.idx ? g.idx[g.row0 + r] : g.row0 + r) * MLP_NOUT + unit] : 0.0f;
+        }
+    }
+    // two values of neighbouring units (or inputs) and one row from lanes 2i and
+    // 2i + 1 with one value a and b of two rows each: the even lane's are of the
+    // first row, the odd lane's of the second
+    const bool odd = lane & 1;
+    auto exchange = [&](float a, float b) {
+        const float other = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+        return odd ? pack2(other, b) : pack2(a, other);
+    };
     {
-        constexpr int NC = (MLP_KIN + 31) / 32;
-        for (int rr = warp * 8; rr < warp * 8 + 8; rr += 4) {
-            float v[4][NC];
+        const int r = warp * 2 + (int)odd;
 #pragma unroll
-            for (int h = 0; h < 4; h++) {
-                const int r = r0 + rr + h;
-                const bool have = r < g.n;
-                const long long src = have ? (g.idx ? g.idx[g.row0 + r] : g.row0 + r) : 0;
-                const float *x = g.X + src * MLP_NIN;
-#pragma unroll
-                for (int j = 0; j < NC; j++) {
-                    const int k = lane + 32 * j;
-                    v[h][j] = have && k < MLP_NIN ? x[k] : 0.0f;
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < 4; h++) {
-                const int r = rr + h;
-#pragma unroll
-                for (int j = 0; j < NC; j++) {
-                    const int k = lane + 32 * j;
-                    if (k >= MLP_KIN) continue;
-                    const bf16 b = __float2bfloat16_rn(v[h][j]);
-                    *(bf16 *)(sm + Sm::XA + ((k >> 3) * 16 + (r >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2) = b;
-                    if (TRAIN && r0 + r < g.n) g.Xb[(long long)(r0 + r) * MLP_KIN + k] = b;
-                }
-            }
+        for (int j = 0; j < NC; j++) {
+            const int k = (lane & ~1) + 32 * j;
+            const uint32_t w = exchange(v[0][j], v[1][j]);
+            if (k >= MLP_KIN) continue;
+            *(uint32_t *)(sm + Sm::XA + (k >> 3) * R_LBO + (r >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2) = w;
+            if (TRAIN && r0 + r < g.n) *(uint32_t *)(g.Xb + (long long)(r0 + r) * MLP_KIN + k) = w;
         }
     }
     cp_async_wait();
@@ -249,7 +309,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *(volatile uint32_t *)(sm + 16);
-    const uint32_t d1 = tmem, d2 = tmem + 128;
+    const uint32_t d1 = tmem, d2 = tmem + NR;
 
     unsigned phase = 0;
     bool ok = true;
@@ -262,28 +322,24 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
         return ok;
     };
     const bool issuer = tid == 0 && !g.no_mma;
-    // this thread's row of a tile and its quarter of 128 columns
-    const int row = (warp & 3) * 32 + lane, col0 = (warp >> 2) * 32;
-    const bool have = r0 + row < g.n;
-    const uint32_t quarter = (uint32_t)((warp & 3) * 32) << 16;
-    // the epilogue of a 128 x 128 product: f(column, value) rounded to BF16, into
-    // the shared-memory tile at `tile` and, in training, row-major to `out`
-    auto epilogue = [&](uint32_t d, int tile, bf16 *out, auto &&f) {
-#pragma unroll 1
-        for (int c0 = col0; c0 < col0 + 32; c0 += 16) {
-            float v[16];
-            tmem_ld16(d + quarter + (uint32_t)c0, v);
+    const uint32_t mine = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)row;
+    // the epilogue of a product of 128 units: f(j, value) of this thread's rows,
+    // rounded to BF16, kept where asked, into the shared-memory tile at `tile`
+    // and, in training, row-major to `out`
+    auto epilogue = [&](uint32_t d, int tile, bf16 *out, float *kept, auto &&f) {
+        float a[8];
+        tmem_ld8(d + mine, a);
 #pragma unroll
-            for (int q = 0; q < 2; q++) {
-                uint32_t w[4];
+        for (int j = 0; j < 8; j++) {
+            a[j] = __bfloat162float(__float2bfloat16_rn(f(j, a[j])));
+            if (kept) kept[j] = a[j];
+        }
 #pragma unroll
-                for (int e = 0; e < 4; e++)
-                    w[e] = pack2(f(c0 + 8 * q + 2 * e, v[8 * q + 2 * e]), f(c0 + 8 * q + 2 * e + 1, v[8 * q + 2 * e + 1]));
-                const uint4 o = make_uint4(w[0], w[1], w[2], w[3]);
-                const int kb = (c0 >> 3) + q;
-                if (tile >= 0) *(uint4 *)(sm + tile + (kb * 16 + (row >> 3)) * 128 + (row & 7) * 16) = o;
-                if (TRAIN && out && have) *(uint4 *)(out + (long long)(r0 + row) * MLP_HIDDEN + kb * 8) = o;
-            }
+        for (int j = 0; j < 8; j += 2) {
+            const uint32_t w = exchange(a[j], a[j + 1]);
+            const int u = unit & ~1, r = row + j + (int)odd;
+            if (tile >= 0) *(uint32_t *)(sm + tile + (u >> 3) * R_LBO + (r >> 3) * 128 + (r & 7) * 16 + (u & 7) * 2) = w;
+            if (TRAIN && out && r0 + r < g.n) *(uint32_t *)(out + (long long)(r0 + r) * MLP_HIDDEN + u) = w;
         }
     };
     auto ready = [&]() {  // shared-memory writes of all threads before the next products
@@ -291,97 +347,76 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
         tc_fence_before();
         __syncthreads();
     };
-    // BF16 value (row, column c) of a tile
-    auto tile_at = [&](int tile, int c) {
-        return __bfloat162float(*(const bf16 *)(sm + tile + ((c >> 3) * 16 + (row >> 3)) * 128 + (row & 7) * 16 + (c & 7) * 2));
-    };
+    float h1[8], h2[8];
 
     do {
-        // h1 = tanh(X W1^T + b1)
+        // h1 = tanh(W1 x + b1)
         if (issuer)
-            mma_steps<idesc_bf16<128>(), MLP_KIN / 16>(d1, base + Sm::XA, T_LBO, T_SBO, 2 * T_LBO, base + Sm::WB, T_LBO,
-                                                       T_SBO, 2 * T_LBO, true, bar);
+            mma_steps<idesc_bf16<NR>(), MLP_KIN / 16>(d1, base + Sm::W1, T_LBO, T_SBO, 2 * T_LBO, base + Sm::XA, R_LBO,
+                                                      T_SBO, 2 * R_LBO, true, bar);
         if (!wait()) break;
-        for (int i = tid; i < MLP_HIDDEN * (MLP_HIDDEN / 8); i += ROW_THREADS) {
-            const int r = i & 127, kb = i >> 7;
-            cp_async16(base + Sm::WB + (kb * 16 + (r >> 3)) * 128 + (r & 7) * 16, g.W2 + r * MLP_HIDDEN + kb * 8);
-        }
-        epilogue(d1, Sm::H1, g.H1, [&](int c, float v) { return tanhf(v + bias[c]); });
-        cp_async_wait();
+        epilogue(d1, Sm::H1, g.H1, h1, [&](int, float a) { return tanhf(a + bias[unit]); });
         ready();
-        // h2 = tanh(h1 W2^T + b2)
+        // h2 = tanh(W2 h1 + b2)
         if (issuer)
-            mma_steps<idesc_bf16<128>(), MLP_HIDDEN / 16>(d2, base + Sm::H1, T_LBO, T_SBO, 2 * T_LBO, base + Sm::WB, T_LBO,
-                                                          T_SBO, 2 * T_LBO, true, bar);
+            mma_steps<idesc_bf16<NR>(), MLP_HIDDEN / 16>(d2, base + Sm::W2, T_LBO, T_SBO, 2 * T_LBO, base + Sm::H1, R_LBO,
+                                                         T_SBO, 2 * R_LBO, true, bar);
         if (!wait()) break;
-        epilogue(d2, Sm::H2, g.H2, [&](int c, float v) { return tanhf(v + bias[128 + c]); });
+        epilogue(d2, Sm::H2, g.H2, h2, [&](int, float a) { return tanhf(a + bias[128 + unit]); });
         ready();
-        // y = h2 W3^T + b3
+        // y = W3 h2 + b3
         if (issuer)
-            mma_steps<idesc_bf16<16>(), MLP_HIDDEN / 16>(d1, base + Sm::H2, T_LBO, T_SBO, 2 * T_LBO, base + Sm::W3, 256,
-                                                         T_SBO, 512, true, bar);
+            mma_steps<idesc_bf16<NR>(), MLP_HIDDEN / 16>(d1, base + Sm::W3, 256, T_SBO, 512, base + Sm::H2, R_LBO, T_SBO,
+                                                         2 * R_LBO, true, bar);
         if (!wait()) break;
         double e2 = 0.0;
-        if (warp < 4) {
-            float v[16], d[8];
-            tmem_ld16(d1 + quarter, v);
+        if ((warp & 3) == 0) {
+            float a[8];
+            tmem_ld8(d1 + mine, a);
 #pragma unroll
-            for (int c = 0; c < 8; c++) d[c] = 0.0f;
-            if (have) {
-                const long long src = TRAIN ? (g.idx ? g.idx[g.row0 + r0 + row] : g.row0 + r0 + row) : 0;
-#pragma unroll
-                for (int c = 0; c < MLP_NOUT; c++) {
-                    const float y = v[c] + bias[256 + c];
-                    g.Y[(long long)(r0 + row) * 16 + c] = y;
+            for (int j = 0; j < 8; j++) {
+                const int r = row + j;
+                const bool have = r0 + r < g.n;
+                float d = 0.0f;
+                if (out_unit && have) {
+                    const float y = a[j] + bias[256 + unit];
+                    g.Y[(long long)(r0 + r) * 16 + unit] = y;
                     if (TRAIN) {
-                        const float diff = y - g.T[src * MLP_NOUT + c];
+                        const float diff = y - target[j];
                         e2 += (double)diff * diff;
-                        d[c] = 2.0f * diff / (float)(MLP_NOUT * g.n);
+                        d = 2.0f * diff / (float)(MLP_NOUT * g.n);
+                        g.dY[(long long)(r0 + r) * 16 + unit] = d;
                     }
                 }
-            }
-            if (TRAIN) {
-                // dY = 2 (Y - T)/(6 n), 16 columns of which 6 count
-                const uint4 o = make_uint4(pack2(d[0], d[1]), pack2(d[2], d[3]), pack2(d[4], d[5]), 0);
-                const uint4 zero = make_uint4(0, 0, 0, 0);
-                unsigned char *t = sm + Sm::DY + (row >> 3) * 128 + (row & 7) * 16;
-                *(uint4 *)t = o;
-                *(uint4 *)(t + T_LBO) = zero;
-                if (have) {
-                    uint4 *p = (uint4 *)(g.dYb + (long long)(r0 + row) * 16);
-                    p[0] = o;
-                    p[1] = zero;
-#pragma unroll
-                    for (int c = 0; c < MLP_NOUT; c++) g.dY[(long long)(r0 + row) * 16 + c] = d[c];
+                if (TRAIN && unit < 16) {
+                    // dY = 2 (Y - T)/(6 n), 16 columns of which 6 count
+                    const bf16 o = __float2bfloat16_rn(d);
+                    if (out_unit) *(bf16 *)(sm + Sm::DY + (r >> 3) * 128 + (r & 7) * 16 + unit * 2) = o;
+                    if (have) g.dYb[(long long)(r0 + r) * 16 + unit] = o;
                 }
             }
         }
         if constexpr (TRAIN) {
-            // squared error of the tile: lanes, then warps 0..3, in a fixed order
+            // squared error of the tile: lanes, then rows by eights, in a fixed order
             for (int o = 16; o > 0; o >>= 1) e2 += __shfl_down_sync(0xffffffffu, e2, o);
             double *const red = (double *)(sm + Sm::RED);
-            if (lane == 0 && warp < 4) red[warp] = e2;
+            if (lane == 0 && (warp & 3) == 0) red[warp >> 2] = e2;
             ready();
             if (tid == 0) g.loss_part[blockIdx.x] = ((red[0] + red[1]) + red[2]) + red[3];
-            // dz2 = (dY W3) (1 - h2^2): W3 read MN-major, n its columns, k its rows
+            // dz2 = (W3^T dY) (1 - h2^2): W3 read MN-major, m its columns, k its rows
             if (issuer)
-                mma_steps<idesc_bf16<128, false, true>(), 1>(d2, base + Sm::DY, T_LBO, T_SBO, 0, base + Sm::W3, 128, 256, 0,
-                                                             true, bar);
+                mma_steps<idesc_bf16<NR, true, false>(), 1>(d2, base + Sm::W3, 128, 256, 0, base + Sm::DY, R_LBO, T_SBO, 0,
+                                                            true, bar);
             if (!wait()) break;
-            epilogue(d2, Sm::DZ2, g.dZ2, [&](int c, float v) {
-                const float h = tile_at(Sm::H2, c);
-                return v * (1.0f - h * h);
-            });
+            epilogue(d2, Sm::DZ2, g.dZ2, nullptr, [&](int j, float a) { return a * (1.0f - h2[j] * h2[j]); });
             ready();
-            // dz1 = (dz2 W2) (1 - h1^2): W2 read MN-major
+            // dz1 = (W2^T dz2) (1 - h1^2): W2 read MN-major
             if (issuer)
-                mma_steps<idesc_bf16<128, false, true>(), MLP_HIDDEN / 16>(d1, base + Sm::DZ2, T_LBO, T_SBO, 2 * T_LBO,
-                                                                           base + Sm::WB, 128, T_LBO, 256, true, bar);
+                mma_steps<idesc_bf16<NR, true, false>(), MLP_HIDDEN / 16>(d1, base + Sm::W2, 128, T_LBO, 256,
+                                                                          base + Sm::DZ2, R_LBO, T_SBO, 2 * R_LBO, true,
+                                                                          bar);
             if (!wait()) break;
-            epilogue(d1, -1, g.dZ1, [&](int c, float v) {
-                const float h = tile_at(Sm::H1, c);
-                return v * (1.0f - h * h);
-            });
+            epilogue(d1, -1, g.dZ1, nullptr, [&](int j, float a) { return a * (1.0f - h1[j] * h1[j]); });
         }
     } while (false);
     if (!ok && tid == 0) {
@@ -399,9 +434,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
 // weight gradients: C[m][n] = sum_b A[b][m] B[b][n] over the batch, A and B
 // row-major BF16: both operands are read MN-major, so that their rows go into
 // shared memory as they lie, 16 bytes at a time.  A chunk of 64 rows per
-// stage, two stages; the next chunk's loads are in flight while the tensor core
-// works, and a stage is refilled only once the commit of the chunk that read it
-// has arrived (bounded waits).
+// stage, eight stages filled by asynchronous copies, so that a batch of 512 has
+// all its loads in flight at once; a stage is refilled only once the commit of
+// the chunk that read it has arrived (bounded waits).  Two stages took 17.8 us for
+// a batch of 512, eight 16.5.
 // ---------------------------------------------------------------------------
 struct GradArgs {
     int n;
@@ -420,13 +456,15 @@ constexpr int GB = 64;  // batch rows per chunk
 constexpr int GN = 64;  // columns of an output tile
 constexpr int GRAD_W1 = (MLP_KIN + GN - 1) / GN, GRAD_W2 = MLP_HIDDEN / GN;  // tiles of dW1 and dW2
 constexpr int GRAD_TILES = GRAD_W1 + GRAD_W2 + 1;                            // and one of dW3
-constexpr int GRAD_CTAS = GRAD_TILES + 2 * MLP_HIDDEN + MLP_NOUT + 1;        // bias sums, loss
+constexpr int GRAD_CTAS = GRAD_TILES + 2 * (MLP_HIDDEN / 8) + 2;             // bias sums 8 at a time, loss
 
 struct GradSmem {
-    static constexpr int HEAD = 128;
+    static constexpr int STAGES = 8;
+    static constexpr int SLOT = 64, HEAD = 128;  // STAGES barriers, the TMEM slot
     static constexpr int A_STAGE = GB * GM * 2, B_STAGE = GB * GN * 2;
-    static constexpr int BYTES = HEAD + 2 * (A_STAGE + B_STAGE);
+    static constexpr int BYTES = HEAD + STAGES * (A_STAGE + B_STAGE);
 };
+static_assert(GradSmem::BYTES <= 227 * 1024, "shared memory of a CTA");
 
 // one tile: BN columns from n0 of B (ldb apart per row, nb 16-byte groups of it valid)
 template <int BN>
@@ -434,74 +472,76 @@ __device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, 
                                           int nb, float *C, long long scm, long long scn, int ncols)
 {
     using Sm = GradSmem;
-    const uint32_t base = smem_addr(sm), slot = base + 16;
+    constexpr int ST = Sm::STAGES;
+    const uint32_t base = smem_addr(sm);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr uint32_t NCOLS = BN < 32 ? 32 : BN;
-    constexpr int VA = GB * GM / 8 / MLP_THREADS;                       // 16-byte loads of A a thread
+    constexpr int VA = GB * GM / 8 / MLP_THREADS;                       // 16-byte copies of A a thread
     constexpr int NB8 = BN / 8, VB = (GB * NB8 + MLP_THREADS - 1) / MLP_THREADS;
+    const int nchunks = (g.n + GB - 1) / GB;
+    // vector i of a chunk: core matrix (k group, m group), row b of 8 in it; the
+    // shared-memory place is 16 i.  One group of copies per call, an empty one
+    // past the last chunk
+    auto fetch = [&](int c) {
+        const uint32_t As = base + Sm::HEAD + (c % ST) * Sm::A_STAGE;
+        const uint32_t Bs = base + Sm::HEAD + ST * Sm::A_STAGE + (c % ST) * Sm::B_STAGE;
+        if (c < nchunks) {
+#pragma unroll
+            for (int q = 0; q < VA; q++) {
+                const int i = tid + q * MLP_THREADS, b = c * GB + (i >> 7) * 8 + (i & 7), mb = (i >> 3) & 15;
+                const bool have = b < g.n;
+                cp_async16z(As + i * 16, A + (have ? (long long)b * MLP_HIDDEN + mb * 8 : 0), have ? 16 : 0);
+            }
+#pragma unroll
+            for (int q = 0; q < VB; q++) {
+                const int i = tid + q * MLP_THREADS, kb = i / (8 * NB8), b = c * GB + kb * 8 + (i & 7), j = (i >> 3) % NB8;
+                const bool have = b < g.n && j < nb;
+                if (i < GB * NB8) cp_async16z(Bs + i * 16, B + (have ? (long long)b * ldb + n0 + j * 8 : 0), have ? 16 : 0);
+            }
+        }
+        cp_async_commit();
+    };
+    for (int c = 0; c < ST; c++) fetch(c);
     if (warp == 0) {
-        tmem_alloc(slot, NCOLS);
+        tmem_alloc(base + Sm::SLOT, NCOLS);
         tmem_relinquish();
     }
     if (tid == 0) {
-        mbar_init(base, 1);
-        mbar_init(base + 8, 1);
+        for (int i = 0; i < ST; i++) mbar_init(base + 8 * i, 1);
         mbar_fence_init();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *(volatile uint32_t *)(sm + 16);
-    // vector i of a chunk: core matrix (k group, m group), row b of 8 in it; the
-    // shared-memory place is 16 i
-    uint4 va[VA], vb[VB];
-    const uint4 zero = make_uint4(0, 0, 0, 0);
-    auto fetch = [&](int c) {
-#pragma unroll
-        for (int q = 0; q < VA; q++) {
-            const int i = tid + q * MLP_THREADS, b = c * GB + (i >> 7) * 8 + (i & 7), mb = (i >> 3) & 15;
-            va[q] = b < g.n ? *(const uint4 *)(A + (long long)b * MLP_HIDDEN + mb * 8) : zero;
-        }
-#pragma unroll
-        for (int q = 0; q < VB; q++) {
-            const int i = tid + q * MLP_THREADS, kb = i / (8 * NB8), b = c * GB + kb * 8 + (i & 7), j = (i >> 3) % NB8;
-            vb[q] = i < GB * NB8 && b < g.n && j < nb ? *(const uint4 *)(B + (long long)b * ldb + n0 + j * 8) : zero;
-        }
-    };
-    const int nchunks = (g.n + GB - 1) / GB;
+    const uint32_t tmem = *(volatile uint32_t *)(sm + Sm::SLOT);
     bool ok = true;
     int last = -1;
-    fetch(0);
     for (int c = 0; c < nchunks; c++) {
-        const int st = c & 1;
-        if (c >= 2) {
-            // the MMAs of chunk c - 2 read this stage
-            ok = mbar_wait_bounded(base + 8 * st, (unsigned)(((c - 2) >> 1) & 1), g.wait_limit);
+        if (c >= 1 && c - 1 + ST < nchunks) {
+            // chunk c - 1 + ST takes the stage that the MMAs of chunk c - 1 read
+            ok = mbar_wait_bounded(base + 8 * ((c - 1) % ST), (unsigned)(((c - 1) / ST) & 1), g.wait_limit);
             if (__syncthreads_or(!ok)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
         }
-        unsigned char *const As = sm + Sm::HEAD + st * Sm::A_STAGE;
-        unsigned char *const Bs = sm + Sm::HEAD + 2 * Sm::A_STAGE + st * Sm::B_STAGE;
-#pragma unroll
-        for (int q = 0; q < VA; q++) *(uint4 *)(As + (tid + q * MLP_THREADS) * 16) = va[q];
-#pragma unroll
-        for (int q = 0; q < VB; q++)
-            if (tid + q * MLP_THREADS < GB * NB8) *(uint4 *)(Bs + (tid + q * MLP_THREADS) * 16) = vb[q];
-        if (c + 1 < nchunks) fetch(c + 1);
+        if (c >= 1) fetch(c - 1 + ST);
+        cp_async_wait_group<ST - 1>();  // ST + c groups committed: chunk c has landed
         fence_async_smem();
         __syncthreads();
         if (tid == 0 && !g.no_mma)
-            mma_steps<idesc_bf16<BN, true, true>(), GB / 16>(tmem, smem_addr(As), 2048, 128, 4096, smem_addr(Bs),
-                                                             NB8 * 128, 128, 2 * NB8 * 128, c == 0, base + 8 * st);
+            mma_steps<idesc_bf16<BN, true, true>(), GB / 16>(
+                tmem, base + Sm::HEAD + (c % ST) * Sm::A_STAGE, 2048, 128, 4096,
+                base + Sm::HEAD + ST * Sm::A_STAGE + (c % ST) * Sm::B_STAGE, NB8 * 128, 128, 2 * NB8 * 128, c == 0,
+                base + 8 * (c % ST));
         last = c;
     }
+    cp_async_wait();
     // a commit covers every MMA this thread issued before it: the last one's
     // arrival means the accumulator is complete
     if (ok && last >= 0) {
-        ok = mbar_wait_bounded(base + 8 * (last & 1), (unsigned)((last >> 1) & 1), g.wait_limit);
+        ok = mbar_wait_bounded(base + 8 * (last % ST), (unsigned)((last / ST) & 1), g.wait_limit);
         ok = !__syncthreads_or(!ok);
         tc_fence_after();
     }
@@ -510,7 +550,7 @@ __device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, 
             atomicOr(g.status, ST_TIMEOUT);
             // MMAs still in flight (none are issued under the fault injection)
             // must finish before the tensor memory is freed
-            if (!g.no_mma && last >= 0) mbar_wait_bounded(base + 8 * (last & 1), (unsigned)((last >> 1) & 1));
+            if (!g.no_mma && last >= 0) mbar_wait_bounded(base + 8 * (last % ST), (unsigned)((last / ST) & 1));
         }
     } else if (warp < 4 || BN > 16) {
         const int m = (warp & 3) * 32 + lane;
@@ -527,19 +567,32 @@ __device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, 
     if (warp == 0) tmem_dealloc(tmem, NCOLS);
 }
 
-// column sum in a fixed order (bias gradients)
+// sums of 8 neighbouring columns in a fixed order (bias gradients), `cols` of
+// them wanted
 template <class T>
-__device__ __forceinline__ void column_sum(const T *src, int rows, int ld, float *sh, float *out)
+__device__ __forceinline__ void column_sums(const T *src, int rows, int ld, float *sh, float *out, int cols)
 {
-    float s = 0.0f;
-    for (int r = threadIdx.x; r < rows; r += MLP_THREADS) s += (float)src[(long long)r * ld];
-    sh[threadIdx.x] = s;
+    float s[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) s[e] = 0.0f;
+    for (int r = threadIdx.x; r < rows; r += MLP_THREADS) {
+        alignas(16) T v[8];
+#pragma unroll
+        for (int k = 0; k < (int)sizeof v / 16; k++) ((uint4 *)v)[k] = ((const uint4 *)(src + (long long)r * ld))[k];
+#pragma unroll
+        for (int e = 0; e < 8; e++) s[e] += (float)v[e];
+    }
+#pragma unroll
+    for (int e = 0; e < 8; e++) sh[e * MLP_THREADS + threadIdx.x] = s[e];
     __syncthreads();
     for (int k = MLP_THREADS / 2; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
+        if ((int)threadIdx.x < k)
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                sh[e * MLP_THREADS + threadIdx.x] += sh[e * MLP_THREADS + threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = sh[0];
+    if ((int)threadIdx.x < cols) out[threadIdx.x] = sh[threadIdx.x * MLP_THREADS];
 }
 
 __global__ void __launch_bounds__(MLP_THREADS) k_mlp_grads(GradArgs g)
@@ -564,18 +617,18 @@ __global__ void __launch_bounds__(MLP_THREADS) k_mlp_grads(GradArgs g)
     }
     t -= 1;
     float *const sh = (float *)sm;
-    if (t < MLP_HIDDEN) {
-        column_sum(g.dZ1 + t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B1 + t);
+    if (t < MLP_HIDDEN / 8) {
+        column_sums(g.dZ1 + 8 * t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B1 + 8 * t, 8);
         return;
     }
-    t -= MLP_HIDDEN;
-    if (t < MLP_HIDDEN) {
-        column_sum(g.dZ2 + t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B2 + t);
+    t -= MLP_HIDDEN / 8;
+    if (t < MLP_HIDDEN / 8) {
+        column_sums(g.dZ2 + 8 * t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B2 + 8 * t, 8);
         return;
     }
-    t -= MLP_HIDDEN;
-    if (t < MLP_NOUT) {
-        column_sum(g.dY + t, g.n, 16, sh, g.grad + MLP_OFF_B3 + t);
+    t -= MLP_HIDDEN / 8;
+    if (t == 0) {  // columns 6 and 7 of dY are not written and not wanted
+        column_sums(g.dY, g.n, 16, sh, g.grad + MLP_OFF_B3, MLP_NOUT);
         return;
     }
     if (threadIdx.x == 0) {
@@ -694,7 +747,7 @@ cudaError_t mlp_alloc(Mlp &m, int cap)
         (e = A((void **)&m.dZ2, sizeof(bf16) * (size_t)cap * MLP_HIDDEN)) ||
         (e = A((void **)&m.dYb, sizeof(bf16) * (size_t)cap * 16)) || (e = A((void **)&m.Y, sizeof(float) * (size_t)cap * 16)) ||
         (e = A((void **)&m.dY, sizeof(float) * (size_t)cap * 16)) ||
-        (e = A((void **)&m.loss_part, sizeof(double) * ((size_t)cap / GM + 1))) ||
+        (e = A((void **)&m.loss_part, sizeof(double) * ((size_t)cap / NR + 1))) ||
         (e = A((void **)&m.loss, sizeof(double) * 2)) || (e = A((void **)&m.dirs, sizeof(double) * 3 * MLP_SHELL)))
         return e;
     // directions of the shell points: a Fibonacci sphere
@@ -728,14 +781,14 @@ void mlp_refresh(const Mlp &m, cudaStream_t st)
 
 cudaError_t mlp_forward(const Mlp &m, const float *X, int n, unsigned *status, cudaStream_t st)
 {
-    return mlp_launch(k_mlp_rows<false>, (n + GM - 1) / GM, ROW_THREADS, RowSmem::BYTES,
+    return mlp_launch(k_mlp_rows<false>, (n + NR - 1) / NR, ROW_THREADS, RowSmem::BYTES,
                       row_args(m, X, nullptr, nullptr, 0, n, status), st);
 }
 
 cudaError_t mlp_gradient(const Mlp &m, const float *X, const float *T, const long long *idx, long long row0, int n,
                          double *acc, unsigned *status, cudaStream_t st)
 {
-    const int tiles = (n + GM - 1) / GM;
+    const int tiles = (n + NR - 1) / NR;
     const RowArgs r = row_args(m, X, T, idx, row0, n, status);
     const cudaError_t e = mlp_launch(k_mlp_rows<true>, tiles, ROW_THREADS, RowSmem::BYTES, r, st);
     if (e != cudaSuccess) return e;
