@@ -20,9 +20,11 @@
 // One GEMM launch per product with operands staged 64 columns at a time by a
 // loop of dependent loads took 36 to 46 us each, 17 launches and 285 us a batch
 // of 512; with 128 rows to a CTA (the M side) the two kernels and Adam took 31,
-// 18 and 4 us, now 21, 16 and 4.  An epoch of 20000 samples 11.4 -> 2.5 ->
-// 2.06 ms, 512 predictions with their copies 132 -> 61 -> 58 us, to the same
-// bits.
+// 18 and 4 us, now 21, 16 and 4.  Each is scheduled while the one before drains,
+// and does before its wait what does not depend on it (the rows' gather, Adam's
+// moments).  An epoch of 20000 samples 11.4 -> 2.5 -> 2.06 ms, with the
+// overlap 1.53 ms; 512 predictions with their copies 132 -> 61 -> 56 us, to the
+// same bits.
 //
 // Shared-memory operands are in the canonical layout without swizzle: 8 x
 // 16-byte core matrices of 128 bytes.  Read K-major, a core matrix holds 8 rows
@@ -244,6 +246,15 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
         mbar_init(bar, 1);
         mbar_fence_init();
     }
+    // A training batch's inputs and targets do not depend on the kernels before,
+    // so their gather runs before the wait for those; a prediction's inputs may
+    // be the preceding kernel's.  Programmatic launches (also of the other two
+    // kernels) are triggered only after the own wait, so that a kernel running
+    // ahead of its wait knows the last but one to be complete.
+    if (!TRAIN) {
+        pdl_wait();
+        pdl_trigger();
+    }
     // inputs: a warp takes 2 rows, all loads in flight
     constexpr int NC = (MLP_KIN + 31) / 32;
     float v[2][NC];
@@ -258,20 +269,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
             const int k = lane + 32 * j;
             v[h][j] = have && k < MLP_NIN ? x[k] : 0.0f;
         }
-    }
-    load_weights<MLP_KIN>(base + Sm::W1, g.W1, tid);
-    load_weights<MLP_HIDDEN>(base + Sm::W2, g.W2, tid);
-    if (tid < 256) {
-        const int r = tid & 15, kb = tid >> 4;
-        unsigned char *d = sm + Sm::W3 + (kb * 2 + (r >> 3)) * 128 + (r & 7) * 16;
-        *(uint4 *)d = r < MLP_NOUT ? *(const uint4 *)(g.W3 + r * MLP_HIDDEN + kb * 8) : make_uint4(0, 0, 0, 0);
-    } else if (tid < 256 + NR * 2) {
-        *(uint4 *)(sm + Sm::DY + (tid - 256) * 16) = make_uint4(0, 0, 0, 0);
-    }
-    if (tid < 128) {
-        bias[tid] = g.b1[tid];
-        bias[128 + tid] = g.b2[tid];
-        if (tid < 16) bias[256 + tid] = tid < MLP_NOUT ? g.b3[tid] : 0.0f;
     }
     // this thread's unit (TMEM lane) and its 8 rows (TMEM columns) of the CTA's
     const int unit = (warp & 3) * 32 + lane, row = (warp >> 2) * 8;
@@ -292,16 +289,45 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) k_mlp_rows(RowArgs g)
         const float other = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
         return odd ? pack2(other, b) : pack2(a, other);
     };
-    {
-        const int r = warp * 2 + (int)odd;
+    uint32_t xw[NC];
+    const int xr = warp * 2 + (int)odd;
+    auto store_inputs = [&]() {
 #pragma unroll
         for (int j = 0; j < NC; j++) {
             const int k = (lane & ~1) + 32 * j;
-            const uint32_t w = exchange(v[0][j], v[1][j]);
-            if (k >= MLP_KIN) continue;
-            *(uint32_t *)(sm + Sm::XA + (k >> 3) * R_LBO + (r >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2) = w;
-            if (TRAIN && r0 + r < g.n) *(uint32_t *)(g.Xb + (long long)(r0 + r) * MLP_KIN + k) = w;
+            xw[j] = exchange(v[0][j], v[1][j]);
+            if (k < MLP_KIN)
+                *(uint32_t *)(sm + Sm::XA + (k >> 3) * R_LBO + (xr >> 3) * 128 + (xr & 7) * 16 + (k & 7) * 2) = xw[j];
         }
+    };
+    if (TRAIN) {
+        store_inputs();
+        pdl_wait();
+        pdl_trigger();
+    }
+    load_weights<MLP_KIN>(base + Sm::W1, g.W1, tid);
+    load_weights<MLP_HIDDEN>(base + Sm::W2, g.W2, tid);
+    if (tid < 256) {
+        const int r = tid & 15, kb = tid >> 4;
+        unsigned char *d = sm + Sm::W3 + (kb * 2 + (r >> 3)) * 128 + (r & 7) * 16;
+        *(uint4 *)d = r < MLP_NOUT ? *(const uint4 *)(g.W3 + r * MLP_HIDDEN + kb * 8) : make_uint4(0, 0, 0, 0);
+    } else if (tid < 256 + NR * 2) {
+        *(uint4 *)(sm + Sm::DY + (tid - 256) * 16) = make_uint4(0, 0, 0, 0);
+    }
+    if (tid < 128) {
+        bias[tid] = g.b1[tid];
+        bias[128 + tid] = g.b2[tid];
+        if (tid < 16) bias[256 + tid] = tid < MLP_NOUT ? g.b3[tid] : 0.0f;
+    }
+    if (TRAIN) {
+        if (r0 + xr < g.n)
+#pragma unroll
+            for (int j = 0; j < NC; j++) {
+                const int k = (lane & ~1) + 32 * j;
+                if (k < MLP_KIN) *(uint32_t *)(g.Xb + (long long)(r0 + xr) * MLP_KIN + k) = xw[j];
+            }
+    } else {
+        store_inputs();
     }
     cp_async_wait();
     fence_async_smem();
@@ -465,6 +491,7 @@ struct GradSmem {
     static constexpr int BYTES = HEAD + STAGES * (A_STAGE + B_STAGE);
 };
 static_assert(GradSmem::BYTES <= 227 * 1024, "shared memory of a CTA");
+static_assert(MLP_KIN % 16 == 0 && MLP_OFF_W1 % 4 == 0 && MLP_OFF_W2 % 4 == 0, "16-byte stores of gradient rows");
 
 // one tile: BN columns from n0 of B (ldb apart per row, nb 16-byte groups of it valid)
 template <int BN>
@@ -501,7 +528,6 @@ __device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, 
         }
         cp_async_commit();
     };
-    for (int c = 0; c < ST; c++) fetch(c);
     if (warp == 0) {
         tmem_alloc(base + Sm::SLOT, NCOLS);
         tmem_relinquish();
@@ -510,6 +536,9 @@ __device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, 
         for (int i = 0; i < ST; i++) mbar_init(base + 8 * i, 1);
         mbar_fence_init();
     }
+    pdl_wait();  // the batch's activations and deltas
+    pdl_trigger();
+    for (int c = 0; c < ST; c++) fetch(c);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -557,9 +586,16 @@ __device__ __forceinline__ void grad_tile(const GradArgs &g, unsigned char *sm, 
         for (int c0 = (warp >> 2) * (BN / 2); c0 < (BN > 16 ? (warp >> 2) * (BN / 2) + BN / 2 : 16); c0 += 16) {
             float v[16];
             tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+            if (BN > 16) {  // rows of C (scn 1), whole groups of 16 columns
+                if (c0 < ncols)
 #pragma unroll
-            for (int i = 0; i < 16; i++)
-                if (c0 + i < ncols) C[m * scm + (c0 + i) * scn] = v[i];
+                    for (int i = 0; i < 16; i += 4)
+                        *(float4 *)(C + m * scm + c0 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; i++)
+                    if (c0 + i < ncols) C[m * scm + (c0 + i) * scn] = v[i];
+            }
         }
     }
     tc_fence_before();
@@ -617,6 +653,8 @@ __global__ void __launch_bounds__(MLP_THREADS) k_mlp_grads(GradArgs g)
     }
     t -= 1;
     float *const sh = (float *)sm;
+    pdl_wait();
+    pdl_trigger();
     if (t < MLP_HIDDEN / 8) {
         column_sums(g.dZ1 + 8 * t, g.n, MLP_HIDDEN, sh, g.grad + MLP_OFF_B1 + 8 * t, 8);
         return;
@@ -682,14 +720,30 @@ RowArgs row_args(const Mlp &m, const float *X, const float *T, const long long *
     return a;
 }
 
-// launched through cudaLaunchKernel: the set-up's or this launch's own error
+// with programmatic stream serialisation: the kernel may be scheduled while its
+// predecessor in the stream drains (it calls pdl_wait first)
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), int ctas, int threads, int bytes, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+// the set-up's or this launch's own error
 template <class A>
 cudaError_t mlp_launch(void (*kernel)(A), int ctas, int threads, int bytes, const A &a, cudaStream_t st)
 {
     const cudaError_t e = mlp_setup();
-    if (e != cudaSuccess) return e;
-    void *args[] = {(void *)&a};
-    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)ctas), dim3((unsigned)threads), args, (size_t)bytes, st);
+    return e != cudaSuccess ? e : launch_after(kernel, ctas, threads, bytes, st, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -711,13 +765,18 @@ __global__ void k_adam(float *theta, const float *grad, float *m, float *v, floa
                        bf16 *W2b, bf16 *W3b)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= MLP_NPARAM) return;
+    const bool have = i < MLP_NPARAM;
+    // the moments and weights are this kernel's own: loaded before the gradients are waited for
+    const float m0 = have ? m[i] : 0.0f, v0 = have ? v[i] : 0.0f, t0 = have ? theta[i] : 0.0f;
+    pdl_wait();
+    pdl_trigger();
+    if (!have) return;
     const float g = grad[i];
-    const float mi = 0.9f * m[i] + 0.1f * g;
-    const float vi = 0.999f * v[i] + 0.001f * g * g;
+    const float mi = 0.9f * m0 + 0.1f * g;
+    const float vi = 0.999f * v0 + 0.001f * g * g;
     m[i] = mi;
     v[i] = vi;
-    const float t = theta[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    const float t = t0 - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
     theta[i] = t;
     if (i < MLP_OFF_B1) W1b[i] = __float2bfloat16_rn(t);
     else if (i >= MLP_OFF_W2 && i < MLP_OFF_B2) W2b[i - MLP_OFF_W2] = __float2bfloat16_rn(t);
@@ -806,8 +865,8 @@ void mlp_adam(Mlp &m, double lr, cudaStream_t st)
     m.t += 1;
     const float c1 = (float)(1.0 - std::pow(0.9, (double)m.t));
     const float c2 = (float)(1.0 - std::pow(0.999, (double)m.t));
-    k_adam<<<(MLP_NPARAM + EW - 1) / EW, EW, 0, st>>>(m.theta, m.grad, m.adam_m, m.adam_v, (float)lr, c1, c2, m.W1b,
-                                                      m.W2b, m.W3b);
+    launch_after(k_adam, (MLP_NPARAM + EW - 1) / EW, EW, 0, st, m.theta, m.grad, m.adam_m, m.adam_v, (float)lr, c1, c2,
+                 m.W1b, m.W2b, m.W3b);
 }
 
 // ---------------------------------------------------------------------------
