@@ -324,7 +324,7 @@ lbm_status lbm_diagnostics(lbm_ctx *ctx, int inst, double *out);
  * bulk collision takes two nodes of a row per thread (pair loads and stores),
  * one node per thread otherwise; tile 1: one node per thread always.
  * zchunk: z-planes per work item of the gradient pass (0: chosen from the
- * size of the grid; FP64 contexts and those of up to 655360 nodes take a node
+ * size of the grid; FP64 contexts and those of up to 786432 nodes take a node
  * per thread instead).  Every shape
  * computes the same update; the node-pair collision agrees with the one-node
  * collision to the rounding of the storage type (the code generator may fuse
@@ -359,9 +359,10 @@ long long lbm_last_launch_count(const lbm_ctx *ctx);
 lbm_status lbm_profile(lbm_ctx *ctx, int enable);
 
 /* Read the per-kernel record since lbm_profile(ctx, 1): for stage k
- * (order parameter, solid phi, gradient+wetting, collision [four-kernel
- * form], momentum exchange, capillary force, DEM, geometry owner, geometry
- * boundary, refill, fused fluid kernel, particle-region phi/gradient)
+ * (order parameter, solid phi, gradient + wetting + curvature, collision,
+ * momentum exchange, capillary force, DEM, geometry owner, geometry boundary,
+ * refill, three unused ones, surrogate, order-parameter boundary pass,
+ * collision boundary pass, contacts)
  * out[2k] = launches, out[2k+1] = total device milliseconds; at most
  * max_stages stages are written.  Synchronises. */
 lbm_status lbm_profile_read(lbm_ctx *ctx, double *out, int max_stages);

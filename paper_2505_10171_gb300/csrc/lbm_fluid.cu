@@ -698,10 +698,13 @@ __global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : LBM_COL
 // then).  The first 32 ROWS threads own RP rows of one column each; further
 // threads take the nodes around the tile, whose normals the curvature needs.
 //
-// Bound by instruction issue (62% of the slots at 22 resident warps per SM), not
-// by memory: 24 bytes a node, most of which stay in L2.  The form with three
-// stored planes and 48 reads a node executed 14.2 warp instructions per node,
-// this one 11.3: 96-domain sweep (1.5e8 nodes) 2796 -> 1738 us, 64 x 96x48x48
+// Bound by the chain of a plane's iteration (shared-memory reads, the normal's
+// inverse root, a barrier: 58% of the issue slots at 20 to 24 resident warps per
+// SM), not by memory: 24 bytes a node, most of which stay in L2.  With the two
+// rows in two-float instructions it executes a fifth fewer and takes as long
+// (75.5 against 73 us on 256x128x128, 1720 against 1746 us in the sweep).  The
+// form with three stored planes and 48 reads a node executed 14.2 warp
+// instructions per node, this one 9.6: 96-domain sweep (1.5e8 nodes) 2796 -> 1738 us, 64 x 96x48x48
 // 254 -> 204 us, 128x64x64 37 -> 24 us, 256x128x128 75 us either way.
 constexpr int GC_TX = 32;
 
@@ -1066,10 +1069,11 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
 // FP32 arithmetic: bound by latency on a small grid, where a march of some 10
 // planes with a barrier each is a chain that few CTAs walk, and by loads (48 a
 // node) and 28 bytes a node more on a large one.  Marching against this form,
-// with the events' 5 us: 48x32x32 21 and 11 us, 4 x 48^3 (0.44 M nodes) 29 and
-// 19, 16 x 40x33x29 (0.61 M) 39 and 26, 96x96x64 (0.59 M) 21 and 21, 96^3
-// (0.88 M) 25 and 27, 256x128x64 35 and 49, 256x128x128 73 and 115: taken up
-// to GRAD_NODES_MAX nodes of a context.
+// with the events' 5 us: 48x32x32 21 and 11 us; 0.44 M nodes as 4 x 48^3 29 and
+// 19; 0.7 M as one domain 24 and 23 (201x91x37) or 21 and 23 (128x80x72), as 6
+// x 48^3 38 and 25, as 19 x 40x33x29 49 and 29; 0.88 M as 96^3 25 and 27, as 8
+// x 48^3 35 and 31; 256x128x64 35 and 49; 256x128x128 73 and 115: taken up to
+// GRAD_NODES_MAX nodes of a context.
 template <class R>
 constexpr int GN_THREADS = sizeof(R) == 8 ? 32 : 128;
 template <class R>

@@ -734,7 +734,7 @@ struct FluidLaunch {
 };
 // The gradient pass takes a node per thread in FP64 runs and up to this many
 // nodes of a context, marching tiles beyond (measured beside the kernels)
-constexpr long long GRAD_NODES_MAX = 640 * 1024;
+constexpr long long GRAD_NODES_MAX = 768 * 1024;
 // plan the work items of the gradient + curvature kernel into fz (z-planes per
 // item: zc_inst[k] for instance k where set (> 0), else zc_request where set,
 // else chosen from the grid's size and the n_sm SMs); used where L.nrm is null

@@ -7,7 +7,7 @@ from paper_2505_10171_gb300 import workloads as W
 from test_gpu_grad_fp64 import DOMAINS, workload
 
 pytestmark = pytest.mark.gpu
-NODES_MAX = 640 * 1024
+NODES_MAX = 768 * 1024
 
 
 @pytest.fixture(scope="module", autouse=True)
