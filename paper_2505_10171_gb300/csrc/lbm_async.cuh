@@ -1,5 +1,5 @@
 // Shared-memory barriers and bulk asynchronous copies (PTX) of the
-// tensor-core GEMM of the surrogate network.
+// tensor-core products of the surrogate network.
 // Every wait is bounded (about one second) so that a kernel can report a
 // missing arrival instead of hanging.
 #pragma once

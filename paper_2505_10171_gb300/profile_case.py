@@ -4,7 +4,7 @@ The drop + spheres workload cropped to 256 x 128 x 64 (2.1 M nodes: the FP32
 populations, 320 MB, exceed the L2 size, so DRAM figures stay meaningful),
 20 steps to develop the flow, then 3 steps with per-stage event timing
 (every kernel launched eagerly, one stream), then one surrogate forward pass
-of 4096 rows through the tensor-core GEMMs.  Prints the per-stage times in
+of 4096 rows through the tensor-core products.  Prints the per-stage times in
 microseconds per launch.
 
     python -m paper_2505_10171_gb300.profile_case fp32
