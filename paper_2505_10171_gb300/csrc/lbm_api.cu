@@ -45,6 +45,10 @@ struct lbm_ctx {
     double *cap_pts = nullptr;  // Lagrangian surface-point table, then in single precision
     double *crec = nullptr;     // DEM contact records
     unsigned *status = nullptr;
+    struct Answer {
+        double loss;
+        unsigned status;
+    } *answer = nullptr;  // page-locked; with the network
     int mem_blocks = 1, mem_side = 1, geom_blocks = 1, geom_side = 1;
     int cur = 0;
     long long steps = 0;
@@ -814,14 +818,38 @@ static const char *status_text(unsigned s)
     return "device status";
 }
 
+static lbm_status status_of(lbm_ctx *ctx, unsigned s)
+{
+    if (s) return fail(ctx, (s & ST_TIMEOUT) && !(s & ST_UNSTABLE) ? LBM_ERR_TIMEOUT : LBM_ERR_UNSTABLE,
+                       status_text(s));
+    return LBM_OK;
+}
+
 static lbm_status check_status(lbm_ctx *ctx)
 {
     unsigned s = 0;
     CU(cudaMemcpyAsync(&s, ctx->status, sizeof s, cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
-    if (s) return fail(ctx, (s & ST_TIMEOUT) && !(s & ST_UNSTABLE) ? LBM_ERR_TIMEOUT : LBM_ERR_UNSTABLE,
-                       status_text(s));
+    return status_of(ctx, s);
+}
+
+// The same for a call that ends in a copy to the caller's memory, in one round
+// trip to the device: the status word (and the network's loss) go to page-locked
+// memory before that copy, and are looked at once it has arrived.  Copied to the
+// stack each was a synchronisation of its own: 512 predictions 55 against 47 us, a
+// gradient of 512 rows 94 against 80 us.
+static lbm_status send_status(lbm_ctx *ctx, bool loss = false)
+{
+    CU(cudaMemcpyAsync(&ctx->answer->status, ctx->status, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
+    if (loss)
+        CU(cudaMemcpyAsync(&ctx->answer->loss, ctx->mlp.loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     return LBM_OK;
+}
+
+static lbm_status sent_status(lbm_ctx *ctx)
+{
+    CU(cudaStreamSynchronize(ctx->stream));
+    return status_of(ctx, ctx->answer->status);
 }
 
 static void drop_graph(lbm_ctx *c)
@@ -862,6 +890,7 @@ void lbm_destroy(lbm_ctx *ctx)
     cudaFree(ctx->phi);
     cudaFree(ctx->col);
     cudaFree(ctx->grad);
+    cudaFreeHost(ctx->answer);
     cudaFree(ctx->nrm);
     cudaFree(ctx->static_list);
     cudaFree(ctx->static_bfl);
@@ -1756,6 +1785,7 @@ static lbm_status ensure_mlp(lbm_ctx *ctx)
     CU(cudaStreamSynchronize(ctx->stream));
     cudaError_t e = mlp_alloc(ctx->mlp, MLP_CAP);
     if (e == cudaSuccess && !ctx->feat) e = cudaMalloc((void **)&ctx->feat, sizeof(float) * MLP_CAP * MLP_NIN);
+    if (e == cudaSuccess && !ctx->answer) e = cudaMallocHost((void **)&ctx->answer, sizeof *ctx->answer);
     if (e != cudaSuccess) {
         mlp_free(ctx->mlp);
         cudaGetLastError();
@@ -1845,10 +1875,11 @@ lbm_status lbm_surrogate_predict(lbm_ctx *ctx, const float *X, size_t n, float *
         if (s != LBM_OK) return s;
         CU(mlp_forward(ctx->mlp, Xd, nb, ctx->status, ctx->stream));
         CU(cudaGetLastError());
+        if ((s = send_status(ctx)) != LBM_OK) return s;
         CU(cudaMemcpy2DAsync(Y + r0 * MLP_NOUT, sizeof(float) * MLP_NOUT, ctx->mlp.Y, sizeof(float) * 16,
                              sizeof(float) * MLP_NOUT, nb, cudaMemcpyDeviceToHost, ctx->stream));
     }
-    return check_status(ctx);
+    return sent_status(ctx);
 }
 
 lbm_status lbm_surrogate_gradient(lbm_ctx *ctx, const float *X, const float *Y, size_t n, float *grad,
@@ -1862,11 +1893,10 @@ lbm_status lbm_surrogate_gradient(lbm_ctx *ctx, const float *X, const float *Y, 
     if (s != LBM_OK) return s;
     CU(mlp_gradient(ctx->mlp, Xd, Yd, nullptr, 0, (int)n, nullptr, ctx->status, ctx->stream));
     CU(cudaGetLastError());
+    if ((s = send_status(ctx, true)) != LBM_OK) return s;
     CU(cudaMemcpyAsync(grad, ctx->mlp.grad, sizeof(float) * MLP_NPARAM, cudaMemcpyDeviceToHost, ctx->stream));
-    double l = 0.0;
-    CU(cudaMemcpyAsync(&l, ctx->mlp.loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    s = check_status(ctx);
-    if (loss) *loss = l;
+    s = sent_status(ctx);
+    if (loss) *loss = ctx->answer->loss;
     return s;
 }
 
@@ -1947,10 +1977,11 @@ lbm_status lbm_surrogate_features(lbm_ctx *ctx, int inst, float *out)
             launch_shell_features<S>(L, ctx->mlp, I.part_off + p0, np, ctx->feat, ctx->stream);
         });
         CU(cudaGetLastError());
+        if ((s = send_status(ctx)) != LBM_OK) return s;
         CU(cudaMemcpyAsync(out + (size_t)p0 * MLP_NIN, ctx->feat, sizeof(float) * np * MLP_NIN,
                            cudaMemcpyDeviceToHost, ctx->stream));
     }
-    return check_status(ctx);
+    return sent_status(ctx);
 }
 
 lbm_status lbm_inject_fault(lbm_ctx *ctx, int fault)

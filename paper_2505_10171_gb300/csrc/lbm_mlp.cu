@@ -23,8 +23,8 @@
 // 18 and 4 us, now 21, 16 and 4.  Each is scheduled while the one before drains,
 // and does before its wait what does not depend on it (the rows' gather, Adam's
 // moments).  An epoch of 20000 samples 11.4 -> 2.5 -> 2.06 ms, with the
-// overlap 1.53 ms; 512 predictions with their copies 132 -> 61 -> 56 us, to the
-// same bits.
+// overlap 1.53 ms; 512 predictions with their copies 132 -> 61 -> 56 us (and 47
+// with one synchronisation), to the same bits.
 //
 // Shared-memory operands are in the canonical layout without swizzle: 8 x
 // 16-byte core matrices of 128 bytes.  Read K-major, a core matrix holds 8 rows
