@@ -685,20 +685,22 @@ __device__ __forceinline__ uint8_t set_boundary(const Lattice &L, const InstDev 
 // change only within one link of a node whose owner changed, i.e. within
 // the particle's last displacement and one link of its surface: the other
 // nodes of the cube cost a distance (all: the bits of every node and no lists,
-// when particles are added).  512 spheres R = 3: 80 us with 18 flags read for every node,
-// now 43.
+// when particles are added); the cube is cut to what the surface reaches (19 -> 11
+// nodes a side there).  512 spheres R = 3: 80 us with 18 flags read for every
+// node, 43 with the whole cube's distances, now 22.
 __global__ void __launch_bounds__(PART_THREADS) k_geom_surface(Lattice L, FastDiv fd, int all)
 {
     const PartDev &P = L.parts[blockIdx.y];
     const InstDev &I = L.inst[P.inst];
-    Region reg;
-    reg.init(P.xf, (int)fd.d, I.nx, I.ny, I.nz);
     const int mine = 2 + P.local;
     const float m0 = min_image_r<float>(P.xf[0] - P.xfo[0], I.nx), m1 = min_image_r<float>(P.xf[1] - P.xfo[1], I.ny),
                 m2 = min_image_r<float>(P.xf[2] - P.xfo[2], I.nz);
     // one link is at most sqrt 2; 0.1 covers the single-precision distance
     const float reach = sqrtf(m0 * m0 + m1 * m1 + m2 * m2) + 1.52f;
     const float lo = fmaxf(P.Rf - reach, 0.0f), hi = P.Rf + reach, lo2 = P.Rf > reach ? lo * lo : -1.0f, hi2 = hi * hi;
+    // nodes within hi of the centre lie floor(hi) below to floor(hi) + 1 above its floor
+    Region reg;
+    reg.init(P.xf, all ? (int)fd.d : min((int)fd.d, 2 * (int)hi + 3), I.nx, I.ny, I.nz);
     const long long count = reg.count();
     const int lane = threadIdx.x & 31;
     auto append = [&](bool take, long long e, long long *list, unsigned long long *n) {
