@@ -108,7 +108,7 @@ struct lbm_ctx {
 // when every row has an even length
 static void plan_launch(lbm_ctx *c)
 {
-    plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, &c->fz);
+    plan_gradcurv(c->inst_h, c->zc_request, c->zc_inst, c->n_sm, c->prec == LBM_FP32, &c->fz);
     plan_phi(c->inst_h, c->n_sm, c->prec == LBM_FP64, &c->fz);
     plan_items(c->inst_h, c->prec == LBM_FP64, &c->fz);
     bool even = true;

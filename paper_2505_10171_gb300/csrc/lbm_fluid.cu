@@ -34,11 +34,15 @@ constexpr int BOUND_THREADS = sizeof(S) == 8 ? 32 : 64;
 #ifndef LBM_BOUND_MINB
 #define LBM_BOUND_MINB 2
 #endif
-// CTAs of 256 threads per SM of the one-node collision: 4 (64 registers, no
-// spill): 119 us per FP32 256x128x128 launch, 6.5 TB/s of the 184 bytes a node
-// that it moves; 5 and 6 spill and took 137 and 160 us
+// CTAs of 256 threads per SM of the one-node collision.  FP32 storage: 5 (48
+// registers, no spill), 119 us per 256x128x128 launch, 6.6 TB/s of the 188 bytes
+// a node that it moves; 4 (64) 125 us.  16-bit storage: 4 (64 registers), as the
+// gathered form spills with 48
 #ifndef LBM_COLLIDE_MINB
 #define LBM_COLLIDE_MINB 4
+#endif
+#ifndef LBM_COLLIDE_MINB_F32
+#define LBM_COLLIDE_MINB_F32 5
 #endif
 
 namespace lbmg {
@@ -77,6 +81,13 @@ __host__ __device__ constexpr int five(int dx, int dy)
 //   four neighbours),  D the diagonal differences,  k = 1/(36 sqrt 2),
 // the plane adds E/18 + k D to its own nodes' sum, k E + V to those above and
 // k E - V to those below: 26 scalar reads a node instead of 19 16-byte ones.
+// FP32 storage sums direction by direction (BY_DIRECTION): there a staged node
+// holds the nine values that its record gives along the directions, a_k and
+// (a_k +- a_l)/sqrt 2, formed once instead of by every node that pulls them, in
+// a ring of three or four planes, and the 18 values and 19 p of a node are read
+// where they are wanted: with p and the plane below carried in registers
+// (80, spilling) the pass took 111 us on 256x128x128 and 347 on 64 x 96x48x48,
+// with nothing carried (72) 94 and 285.
 // The 19 pulled offsets of the next plane are loaded as soon as this plane's
 // are used, so that they are in flight for a whole iteration.
 // Bound by the latency of those loads (96 bytes a node FP32, 58 of 16-bit
@@ -84,11 +95,26 @@ __host__ __device__ constexpr int five(int dx, int dy)
 // FP32 472 -> 284 us (4.8 TB/s), 96-domain FP16 sweep 4297 -> 2692 us,
 // 256x128x128 107 -> 93 us (FP16 92 -> 83: two waves of CTAs and little more),
 // against the form that loaded every record where it was wanted.  Three CTAs
-// per SM (80 registers); two 104 to 119 us, four (64, spilling) 213.
+// per SM (80 registers); two 104 to 119 us, four (64, spilling) 213 (by
+// direction 114 and 114).
 constexpr int PH_TX = 32, PH_TY = 8;
 #ifndef LBM_PHI_MINB
 #define LBM_PHI_MINB 3
 #endif
+
+// direction i as one of the values +-a_k, +-(a_k +- a_l)/sqrt 2 that it pulls
+// from its own plane (four) or a neighbouring one (five): which, and whether
+// with the positive sign
+__host__ __device__ constexpr int dir_along(int i)
+{
+    if (cz(i) == 0) return csq(i) == 1 ? (cx(i) ? 0 : 1) : (cx(i) == cy(i) ? 2 : 3);
+    if (csq(i) == 1) return 0;
+    return cx(i) ? (cx(i) == cz(i) ? 1 : 2) : (cy(i) == cz(i) ? 3 : 4);
+}
+__host__ __device__ constexpr bool dir_forward(int i)
+{
+    return cx(i) ? cx(i) > 0 : (cy(i) ? cy(i) > 0 : cz(i) > 0);
+}
 
 template <class S>
 __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MINB)
@@ -96,7 +122,13 @@ __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MIN
 {
     using R = typename Store<S>::real;
     constexpr int NT = PH_TX * PH_TY, PW = PH_TX + 2, PN = PW * (PH_TY + 2), PER = (PN + NT - 1) / NT;
-    __shared__ R recS[2][4][PN];
+    constexpr bool DIR = BY_DIRECTION<S>;
+    // staged planes, a ring each: p and a_0, a_1, a_2; by direction p, what nodes
+    // of the same plane pull (a_0, a_1, (a_0 +- a_1)/sqrt 2) and what those of the
+    // planes beside it do (a_2, (a_0 +- a_2)/sqrt 2, (a_1 +- a_2)/sqrt 2)
+    constexpr int SLOTS = DIR ? 4 : 2;
+    __shared__ R recS[SLOTS][DIR ? 1 : 4][PN];
+    __shared__ R sameS[DIR ? 3 : 1][DIR ? 4 : 1][DIR ? PN : 1], sideS[DIR ? 4 : 1][DIR ? 5 : 1][DIR ? PN : 1];
     pdl_trigger();  // the gradient pass may be scheduled as this grid drains
 
     const long long item = blockIdx.x;
@@ -147,15 +179,31 @@ __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MIN
 #pragma unroll
         for (int q = 0; q < PER; q++) rv[q] = rec[zo + roff[q]];
     };
-    auto store = [&](int j) {
+    int at1 = 2, at0 = 0, atn = 1;  // sameS: slots of the planes j - 1, j and j + 1
+    auto store = [&](int j, int same) {
 #pragma unroll
         for (int q = 0; q < PER; q++) {
             const int r = tid + q * NT;
             if (r < PN) {
-                recS[j & 1][0][r] = rv[q].p;
-                recS[j & 1][1][r] = rv[q].a0;
-                recS[j & 1][2][r] = rv[q].a1;
-                recS[j & 1][3][r] = rv[q].a2;
+                const int slot = j & (SLOTS - 1);
+                const R a0 = rv[q].a0, a1 = rv[q].a1, a2 = rv[q].a2;
+                recS[slot][0][r] = rv[q].p;
+                if constexpr (DIR) {
+                    const R h = R(0.70710678118654752440);
+                    sameS[same][0][r] = a0;
+                    sameS[same][1][r] = a1;
+                    sameS[same][2][r] = mul_rn(h, add_rn(a0, a1));
+                    sameS[same][3][r] = mul_rn(h, sub_rn(a0, a1));
+                    sideS[slot][0][r] = a2;
+                    sideS[slot][1][r] = mul_rn(h, add_rn(a0, a2));
+                    sideS[slot][2][r] = mul_rn(h, sub_rn(a0, a2));
+                    sideS[slot][3][r] = mul_rn(h, add_rn(a1, a2));
+                    sideS[slot][4][r] = mul_rn(h, sub_rn(a1, a2));
+                } else {
+                    recS[slot][1][r] = a0;
+                    recS[slot][2][r] = a1;
+                    recS[slot][3][r] = a2;
+                }
             }
         }
     };
@@ -172,13 +220,13 @@ __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MIN
         fl = fli[zt * plane + off[1][1]];
     };
     fetch();
-    store(0);
+    store(0, at0);
     pull(z0);
     __syncthreads();
 
     const R k18 = R(1.0 / 18.0), kd = R(0.70710678118654752440 / 36.0);
-    // p of the last plane ([y][x], sources of the target as off) and the five of
-    // the plane before that a target above pulls from; sums of a to come
+    // gathered sums: p of the last plane ([y][x], sources of the target as off) and
+    // the five of the plane before that a target above pulls from; sums of a to come
     R p1[3][3], p2[5];
     R above = 0, own = 0;  // of the plane after the last: what is below gives; of the last plane: all but its plane above
 #pragma unroll
@@ -190,57 +238,85 @@ __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MIN
     for (int j = 0; j < zc + 2; j++) {
         // plane z0-1+j is staged; the target is plane z0-2+j
         if (j < zc + 1) fetch();
-        const R *s = recS[j & 1][0] + c;
-        R p0[3][3];
+        R p0[3][3], E = 0, V = 0, D = 0;
+        if constexpr (!DIR) {
+            const R *s = recS[j & 1][0] + c;
 #pragma unroll
-        for (int b = 0; b < 3; b++)
+            for (int b = 0; b < 3; b++)
 #pragma unroll
-            for (int a = 0; a < 3; a++) p0[b][a] = s[(1 - b) * PW + 1 - a];
-        const R *a0 = s + PN, *a1 = a0 + PN, *a2 = a1 + PN;
-        const R E = (a0[-1] - a0[1]) + (a1[-PW] - a1[PW]);
-        const R V = k18 * a2[0] + kd * ((a2[-1] + a2[1]) + (a2[-PW] + a2[PW]));
-        const R D = ((a0[-PW - 1] + a1[-PW - 1]) - (a0[PW + 1] + a1[PW + 1])) +
-                    ((a0[PW - 1] - a1[PW - 1]) - (a0[-PW + 1] - a1[-PW + 1]));
+                for (int a = 0; a < 3; a++) p0[b][a] = s[(1 - b) * PW + 1 - a];
+            const R *a0 = s + PN, *a1 = a0 + PN, *a2 = a1 + PN;
+            E = (a0[-1] - a0[1]) + (a1[-PW] - a1[PW]);
+            V = k18 * a2[0] + kd * ((a2[-1] + a2[1]) + (a2[-PW] + a2[PW]));
+            D = ((a0[-PW - 1] + a1[-PW - 1]) - (a0[PW + 1] + a1[PW + 1])) +
+                ((a0[PW - 1] - a1[PW - 1]) - (a0[-PW + 1] - a1[-PW + 1]));
+        }
         if (j >= 2) {
-            const R T = own + (kd * E - V);
             R f[Q];
 #pragma unroll
             for (int i = 0; i < Q; i++) f[i] = Store<S>::cvt(F[i]);
             const int zt = z0 - 2 + j;
             const bool write = inside && !(fl & (OWNER_MASK | BOUND_BIT));  // fluid, no solid beside it
             if (j < zc + 1) pull(zt + 1);
-            // p (1 + F) and F summed by weight: rest, axes, diagonals
-            R ga = 0, gd = 0, fa = 0, fd = 0;
+            R num, den;
+            if constexpr (DIR) {
+                // G_i = p (1 + F_i) + (c_i . a)/|c_i|, then the two sums over i
+                R sG = 0, sF = 0;
 #pragma unroll
-            for (int i = 1; i < Q; i++) {
-                const R p = cz(i) == 0 ? p1[cy(i) + 1][cx(i) + 1]
-                                       : (cz(i) < 0 ? p0[cy(i) + 1][cx(i) + 1] : p2[five(cx(i), cy(i))]);
-                const R g = p + p * f[i];
-                if (csq(i) == 1) {
-                    ga += g;
-                    fa += f[i];
-                } else {
-                    gd += g;
-                    fd += f[i];
+                for (int i = 0; i < Q; i++) {
+                    const int at = c - cy(i) * PW - cx(i), slot = (j - 1 - cz(i)) & 3, k = dir_along(i);
+                    const R p = recS[slot][0][at], e = add_rn(R(1), f[i]);
+                    R G = mul_rn(p, e);
+                    if (i > 0) {
+                        const R t = cz(i) == 0 ? sameS[at1][k][at] : sideS[slot][k][at];
+                        G = fma_rn(p, e, dir_forward(i) ? t : -t);
+                    }
+                    sF = fma_rn(wgt<R>(i), f[i], sF);
+                    sG = fma_rn(wgt<R>(i), G, sG);
                 }
+                num = sG;
+                den = add_rn(R(1), sF);
+            } else {
+                // p (1 + F) and F summed by weight: rest, axes, diagonals
+                const R T = own + (kd * E - V);
+                R ga = 0, gd = 0, fa = 0, fd = 0;
+#pragma unroll
+                for (int i = 1; i < Q; i++) {
+                    const R p = cz(i) == 0 ? p1[cy(i) + 1][cx(i) + 1]
+                                           : (cz(i) < 0 ? p0[cy(i) + 1][cx(i) + 1] : p2[five(cx(i), cy(i))]);
+                    const R g = p + p * f[i];
+                    if (csq(i) == 1) {
+                        ga += g;
+                        fa += f[i];
+                    } else {
+                        gd += g;
+                        fd += f[i];
+                    }
+                }
+                num = R(1.0 / 3.0) * (p1[1][1] + p1[1][1] * f[0]) + (k18 * ga + (R(1.0 / 36.0) * gd + T));
+                den = R(1) + (R(1.0 / 3.0) * f[0] + (k18 * fa + R(1.0 / 36.0) * fd));
             }
-            const R num = R(1.0 / 3.0) * (p1[1][1] + p1[1][1] * f[0]) + (k18 * ga + (R(1.0 / 36.0) * gd + T));
-            const R den = R(1) + (R(1.0 / 3.0) * f[0] + (k18 * fa + R(1.0 / 36.0) * fd));
             if (write) phi[zt * plane + off[1][1]] = num / den;
         }
-        own = above + (k18 * E + kd * D);
-        above = kd * E + V;
-        p2[0] = p1[1][1];
-        p2[1] = p1[1][0];
-        p2[2] = p1[1][2];
-        p2[3] = p1[0][1];
-        p2[4] = p1[2][1];
+        if constexpr (!DIR) {
+            own = above + (k18 * E + kd * D);
+            above = kd * E + V;
+            p2[0] = p1[1][1];
+            p2[1] = p1[1][0];
+            p2[2] = p1[1][2];
+            p2[3] = p1[0][1];
+            p2[4] = p1[2][1];
 #pragma unroll
-        for (int b = 0; b < 3; b++)
+            for (int b = 0; b < 3; b++)
 #pragma unroll
-            for (int a = 0; a < 3; a++) p1[b][a] = p0[b][a];
-        if (j < zc + 1) store(j + 1);
+                for (int a = 0; a < 3; a++) p1[b][a] = p0[b][a];
+        }
+        if (j < zc + 1) store(j + 1, atn);
         __syncthreads();
+        const int last = at1;
+        at1 = at0;
+        at0 = atn;
+        atn = last;
     }
 }
 
@@ -668,7 +744,7 @@ __global__ void __launch_bounds__(COLLIDE_NODES<S> / 2, LBM_COLLIDE2_MINB) k_col
 }
 
 template <class S>
-__global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : LBM_COLLIDE_MINB) k_collide(Lattice L, int cur)
+__global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : (sizeof(S) == 4 ? LBM_COLLIDE_MINB_F32 : LBM_COLLIDE_MINB)) k_collide(Lattice L, int cur)
 {
     const InstDev *I;
     int n, x, y, z;
@@ -681,8 +757,10 @@ __global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : LBM_COL
 // gradient, wetting, normal and curvature in one z-marching pass
 // ---------------------------------------------------------------------------
 // FP32 arithmetic: a CTA owns a GC_TX x (ROWS RP) column tile and a chunk of z-planes and
-// marches through the chunk's planes of phi (2-node halo).  Both stencils
-// split into in-plane sums of one plane each: with X, Y the differences of the
+// marches through the chunk's planes of phi (2-node halo).  FP32 storage (DIR)
+// takes both stencils direction by direction from the planes around a node, kept
+// in two rings.  16-bit storage splits them into in-plane sums of one plane
+// each: with X, Y the differences of the
 // +-x and +-y neighbours, S the sum of the four, A and B the sum and difference
 // of the two diagonal differences of a plane,
 //   gx(z) = X/6 + A/12 + [X(z+1) + X(z-1)]/12,   gy alike with Y and B,
@@ -704,23 +782,12 @@ __global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : LBM_COL
 // rows in two-float instructions it executes a fifth fewer and takes as long
 // (75.5 against 73 us on 256x128x128, 1720 against 1746 us in the sweep).  The
 // form with three stored planes and 48 reads a node executed 14.2 warp
-// instructions per node, this one 9.6: 96-domain sweep (1.5e8 nodes) 2796 -> 1738 us, 64 x 96x48x48
-// 254 -> 204 us, 128x64x64 37 -> 24 us, 256x128x128 75 us either way.
+// instructions per node, this one 9.6: 96-domain sweep (1.5e8 nodes) 2796 -> 1738 us, 256x128x128
+// 75 -> 73 us.  By direction the 48 reads stay: 64 x 96x48x48 254 -> 217 us by
+// one barrier a plane instead of three and planes without flags passed by
+// (184 with gathered sums), 256x128x128 75 -> 78 us, the walls of a 64x64x1024
+// tube 89 -> 119 us (98).
 constexpr int GC_TX = 32;
-
-// Operations rounded as written: a tile's own nodes and those around it run
-// two copies of the code below, which the compiler would otherwise be free to
-// contract into different multiply-adds, and a node's normal must have the
-// same bits in every tile (with the copies contracted apart, a symmetric drop
-// took up a sideways drift of 1e-4 of its speed).
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // the sums of the gradient carried from plane to plane for one column
 template <class R>
@@ -774,27 +841,40 @@ struct GcPart {
 // only where two particles meet.  With the owners' particle records read from
 // memory per direction the pass took 195 us instead of 75 on 256x128x128
 // nodes with eight spheres.
-template <class R, class Flag, class Part>
-__device__ __forceinline__ void gc_solid(const InstDev &I, const Part &part, const Flag &flag, R phi, int x, int y,
-                                         int z, R *g, R *s)
+// DIR: the substrate's sum in floating point, direction by direction; returns
+// a bit per solid neighbour, direction i at bit i.
+template <bool DIR, class R, class Flag, class Part>
+__device__ __forceinline__ unsigned gc_solid(const InstDev &I, const Part &part, const Flag &flag, R phi, int x, int y,
+                                             int z, R *g, R *s)
 {
     int all[3] = {0, 0, 0}, wall[3] = {0, 0, 0};
+    R ws[3] = {0, 0, 0};
+    unsigned solid = 0;
     unsigned long long met = 0;
 #pragma unroll
     for (int i = 1; i < Q; i++) {
         const int own = flag(i) & OWNER_MASK;
         const int k = own == OWN_FLUID ? 0 : (csq(i) == 1 ? 2 : 1);
         const int kw = own == OWN_WALL ? k : 0;
-        if (cx(i)) { all[0] += cx(i) * k; wall[0] += cx(i) * kw; }
-        if (cy(i)) { all[1] += cy(i) * k; wall[1] += cy(i) * kw; }
-        if (cz(i)) { all[2] += cz(i) * k; wall[2] += cz(i) * kw; }
+        if constexpr (DIR) {
+            if (k) solid |= 1u << i;
+            const R w = kw ? wgt<R>(i) : R(0);
+            if (cx(i)) ws[0] = sub_rn(ws[0], cx(i) * w);
+            if (cy(i)) ws[1] = sub_rn(ws[1], cy(i) * w);
+            if (cz(i)) ws[2] = sub_rn(ws[2], cz(i) * w);
+        } else {
+            if (cx(i)) { all[0] += cx(i) * k; wall[0] += cx(i) * kw; }
+            if (cy(i)) { all[1] += cy(i) * k; wall[1] += cy(i) * kw; }
+            if (cz(i)) { all[2] += cz(i) * k; wall[2] += cz(i) * kw; }
+        }
         met |= 1ull << own;
     }
-    for (int a = 0; a < 3; a++) s[a] = R(1.0 / 12.0) * all[a];
+    if constexpr (!DIR)
+        for (int a = 0; a < 3; a++) s[a] = R(1.0 / 12.0) * all[a];
     const R wet_max = sizeof(R) == 8 ? (R)I.wet_max : (R)I.f_wet_max;
-    if (!(fabs(phi) < wet_max)) return;
+    if (!(fabs(phi) < wet_max)) return solid;
     met &= ~(1ull << OWN_FLUID | 1ull << OWN_WALL | 1ull << OWN_PRESS);  // a pressure face carries no contact angle
-    R d[3] = {R(-wall[0]), R(-wall[1]), R(-wall[2])};
+    R d[3] = {DIR ? ws[0] : R(-wall[0]), DIR ? ws[1] : R(-wall[1]), DIR ? ws[2] : R(-wall[2])};
     R cth = (R)I.cos_tw, sth = (R)I.sin_tw;
     if (met) {
         // lowest index first: it wins a tie
@@ -822,17 +902,62 @@ __device__ __forceinline__ void gc_solid(const InstDev &I, const Part &part, con
         } while (met);
     }
     const R l = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    if (l == R(0)) return;
+    if (l == R(0)) return solid;
     const R ns[3] = {d[0] / l, d[1] / l, d[2] / l};
     wetting_rotate<R>(g, ns, cth, sth);
+    return solid;
+}
+
+// The sums direction by direction.  at(dx, dy, dz): phi of that neighbour;
+// gradient 3 sum_i w_i c_i phi
+template <class R, class At>
+__device__ __forceinline__ void dir_gradient(const At &at, R *g)
+{
+    g[0] = g[1] = g[2] = 0;
+#pragma unroll
+    for (int i = 1; i < Q; i++) {
+        const R p = at(cx(i), cy(i), cz(i)), w = R(3) * wgt<R>(i);
+        if (cx(i)) g[0] = fma_rn(cx(i) * w, p, g[0]);
+        if (cy(i)) g[1] = fma_rn(cy(i) * w, p, g[1]);
+        if (cz(i)) g[2] = fma_rn(cz(i) * w, p, g[2]);
+    }
+}
+
+// nf(a, i): component a of the normal of neighbour i (the node's own normal where
+// that is solid); curvature 3 sum_i w_i c_i . n over opposite pairs, as
+// w_i c_i . (n_i - n_ib)
+template <class R, class NF>
+__device__ __forceinline__ R dir_curvature(const NF &nf)
+{
+    R k = 0;
+#pragma unroll
+    for (int i = 1; i <= 9; i++) {
+        R t = 0;
+        if (cx(i)) t = sub_rn(nf(0, i), nf(0, i + 9));
+        if (cy(i)) {
+            const R d = sub_rn(nf(1, i), nf(1, i + 9));
+            t = cx(i) ? (cy(i) > 0 ? add_rn(t, d) : sub_rn(t, d)) : d;
+        }
+        if (cz(i)) {
+            const R d = sub_rn(nf(2, i), nf(2, i + 9));
+            t = cx(i) || cy(i) ? (cz(i) > 0 ? add_rn(t, d) : sub_rn(t, d)) : d;
+        }
+        k = fma_rn(wgt<R>(i), t, k);
+    }
+    return mul_rn(R(3), k);
 }
 
 // Threads of the pass.  Two rows per thread share most of their shared-memory
 // reads (75 against 72 us with one on 256x128x128 nodes, but 1738 against
 // 1993 us on the 96-domain sweep); 8 warps of own nodes beat 4 (80 and 1864 us)
 // and 6 (82 and 1956 us).
+// By direction a node reads the three planes around it for each sum (18 + 30
+// values; two rows share few of them), one row a thread: 78 us on 256x128x128 and
+// 218 on 64 x 96x48x48, with two rows 83 and 225, with 12 rows of threads 80 and
+// 227.
+template <bool DIR>
 struct GcShape {
-    static constexpr int RP = 2, ROWS = 8;
+    static constexpr int RP = DIR ? 1 : 2, ROWS = 8;
     static constexpr int TY = ROWS * RP;
     static constexpr int RING = (GC_TX + 2) * (TY + 2) - GC_TX * TY;  // nodes around the tile
     static constexpr int OWN = GC_TX * ROWS;
@@ -840,21 +965,27 @@ struct GcShape {
 };
 
 // CTAs per SM: 2 (80 registers); with 3 (56) the march spills and took 139 to
-// 168 us
+// 168 us.  By direction 3 (56, no spill); 2 took as long on one domain and 6%
+// more on 64, 4 spill and took a quarter longer
 #ifndef LBM_GC_MINB
 #define LBM_GC_MINB 2
 #endif
-__global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L)
+#ifndef LBM_GC_MINB_DIR
+#define LBM_GC_MINB_DIR 3
+#endif
+template <bool DIR>
+__global__ void __launch_bounds__(GcShape<DIR>::NT, DIR ? LBM_GC_MINB_DIR : LBM_GC_MINB) k_gradcurv(Lattice L)
 {
     using R = float;
-    using Shape = GcShape;
+    using Shape = GcShape<DIR>;
     constexpr int RP = Shape::RP, TY = Shape::TY, NT = Shape::NT, OWN = Shape::OWN;
     constexpr int PW = GC_TX + 4, PH = TY + 4, PN = PW * PH;  // phi / flag region (2-node halo)
     constexpr int NW = GC_TX + 2, NH = TY + 2, NN = NW * NH;  // normal region (1-node halo)
     constexpr int PER = (PN + NT - 1) / NT;                   // region values per thread
     __shared__ R phS[4][PN];
     __shared__ uint8_t flS[4][PN];
-    __shared__ R nS[2][3][NN];
+    constexpr int NS = DIR ? 4 : 2;                           // normal planes kept
+    __shared__ R nS[NS][3][NN];
     __shared__ GcPart<R> partS[MAX_PART];
 
     const long long item = blockIdx.x;
@@ -952,6 +1083,9 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
     R kp[RP], ud[RP];              // curvature of the last normal plane but for the plane above; its U - V
     R corr1[RP], corr2[RP];        // the solid neighbours' share of it, planes z0-4+j and z0-5+j
     unsigned fl1 = 0, fl2 = 0;     // own fluid nodes of those planes, a bit per row
+    unsigned sol1[RP], sol2[RP];   // by direction: their solid neighbours
+#pragma unroll
+    for (int r = 0; r < RP; r++) sol1[r] = sol2[r] = 0;
 #pragma unroll
     for (int r = 0; r < RP; r++) kp[r] = ud[r] = corr1[r] = corr2[r] = 0;
     unsigned inside = 0;           // own nodes inside the domain
@@ -962,21 +1096,40 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
     for (int j = 0; j < zc + 5; j++) {
         if (j < zc + 3) fetch();
         R corr[RP];
+        unsigned sol[RP];
 #pragma unroll
-        for (int r = 0; r < RP; r++) corr[r] = 0;
+        for (int r = 0; r < RP; r++) {
+            corr[r] = 0;
+            sol[r] = 0;
+        }
         unsigned fluid = 0;
         if (j < zc + 4) {
             // (1) gradient and normal of plane z0-3+j; 0 for a solid node
-            const R *pl = phS[j & 3] + pc;
-            R v[RP + 2][3];
+            // (by direction: from the rows of the three planes around it)
+            R v[RP + 2][3], vm[DIR ? RP + 2 : 1][3], vp[DIR ? RP + 2 : 1][3];
+            {
+                const R *pl = phS[(DIR ? j - 1 : j) & 3] + pc;
 #pragma unroll
-            for (int r = 0; r < RP + 2; r++)
-                if (r < 3 || own) load_row(pl + (r - 1) * PW, v[r]);
+                for (int r = 0; r < RP + 2; r++)
+                    if (r < 3 || own) load_row(pl + (r - 1) * PW, v[r]);
+            }
+            if constexpr (DIR) {
+                const R *pm = phS[(j - 2) & 3] + pc, *pp = phS[j & 3] + pc;
+#pragma unroll
+                for (int r = 0; r < RP + 2; r++)
+                    if (r < 3 || own) {
+                        load_row(pm + (r - 1) * PW, vm[r]);
+                        load_row(pp + (r - 1) * PW, vp[r]);
+                    }
+            }
 #pragma unroll
             for (int r = 0; r < RP; r++) {
                 if (r > 0 && !own) break;
                 R g[3], nn[3];
-                col[r].advance(v[r], v[r + 1], v[r + 2], g);
+                if constexpr (DIR)
+                    dir_gradient<R>([&](int dx, int dy, int dz) { return (dz < 0 ? vm : (dz > 0 ? vp : v))[r + 1 + dy][1 + dx]; }, g);
+                else
+                    col[r].advance(v[r], v[r + 1], v[r + 2], g);
                 if (j < 2) continue;
                 bool solid = false;
                 R s0 = 0, s1 = 0, s2 = 0;
@@ -987,7 +1140,7 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
                     if (!solid && (fl & BOUND_BIT)) {
                         R sv[3] = {0, 0, 0};
                         const uint8_t *f0 = flS[(j - 2) & 3], *f1 = flS[(j - 1) & 3], *f2 = flS[j & 3];
-                        gc_solid<R>(
+                        sol[r] = gc_solid<DIR, R>(
                             I, [&](int p) -> const GcPart<R> & { return partS[p]; },
                             [&](int i) { return (cz(i) < 0 ? f0 : (cz(i) > 0 ? f2 : f1))[c + cy(i) * PW + cx(i)]; },
                             phS[(j - 1) & 3][c], wrap_any(gx, nx), wrap_any(gy + r, ny), wrap_any(z0 - 3 + j, nz), g,
@@ -995,23 +1148,47 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
                         s0 = sv[0]; s1 = sv[1]; s2 = sv[2];
                     }
                 }
-                const R im = frsqrt(fma_rn(g[0], g[0], fma_rn(g[1], g[1], fma_rn(g[2], g[2], eps2))));
-                nn[0] = mul_rn(g[0], im);
-                nn[1] = mul_rn(g[1], im);
-                nn[2] = mul_rn(g[2], im);
+                if constexpr (DIR) {
+                    dir_normal(g, eps2, nn);
+                } else {
+                    const R im = frsqrt(fma_rn(g[0], g[0], fma_rn(g[1], g[1], fma_rn(g[2], g[2], eps2))));
+                    nn[0] = mul_rn(g[0], im);
+                    nn[1] = mul_rn(g[1], im);
+                    nn[2] = mul_rn(g[2], im);
+                }
                 if (solid) nn[0] = nn[1] = nn[2] = 0;
                 if (own) {
                     const bool here = !solid && (inside >> r & 1u);
                     if (here && j >= 3 && j < zc + 3) out[(j - 3) * plane + r * nx].set_gradient(g);
                     if (here) fluid |= 1u << r;
-                    corr[r] = fma_rn(nn[0], s0, fma_rn(nn[1], s1, mul_rn(nn[2], s2)));
+                    if constexpr (!DIR) corr[r] = fma_rn(nn[0], s0, fma_rn(nn[1], s1, mul_rn(nn[2], s2)));
                 }
-                R *d = &nS[j & 1][0][nc + r * NW];
+                R *d = &nS[j & (NS - 1)][0][nc + r * NW];
                 d[0] = nn[0];
                 d[NN] = nn[1];
                 d[2 * NN] = nn[2];
             }
         }
+        if constexpr (DIR) {
+            // (2) curvature of plane z0-5+j from the normals of the planes around it
+            if (j >= 5 && own) {
+                const R *n0 = nS[(j - 3) & 3][0] + nc, *n1 = nS[(j - 2) & 3][0] + nc, *n2 = nS[(j - 1) & 3][0] + nc;
+#pragma unroll
+                for (int r = 0; r < RP; r++) {
+                    auto normal = [&](int i) { return (cz(i) < 0 ? n0 : (cz(i) > 0 ? n2 : n1)) + (r + cy(i)) * NW + cx(i); };
+                    // a warp takes one of the two ways, not both in turn
+                    R k;
+                    if (__any_sync(0xffffffffu, sol2[r] != 0))
+                        k = dir_curvature<R>([&](int a, int i) {
+                            const R *q = sol2[r] >> i & 1u ? n1 + r * NW : normal(i);
+                            return q[a * NN];
+                        });
+                    else
+                        k = dir_curvature<R>([&](int a, int i) { return normal(i)[a * NN]; });
+                    if (fl2 >> r & 1u) out[(j - 5) * plane + r * nx].k = k;
+                }
+            }
+        } else
         // (2) curvature of plane z0-5+j: the in-plane sums of the normals of plane z0-4+j
         if (j >= 3 && own) {
             const R *a = nS[(j - 1) & 1][0] + nc, *b = a + NN, *d = b + NN;
@@ -1047,6 +1224,8 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
         for (int r = 0; r < RP; r++) {
             corr2[r] = corr1[r];
             corr1[r] = corr[r];
+            sol2[r] = sol1[r];
+            sol1[r] = sol[r];
         }
         fl2 = fl1;
         fl1 = fluid;
@@ -1073,7 +1252,8 @@ __global__ void __launch_bounds__(GcShape::NT, LBM_GC_MINB) k_gradcurv(Lattice L
 // 19; 0.7 M as one domain 24 and 23 (201x91x37) or 21 and 23 (128x80x72), as 6
 // x 48^3 38 and 25, as 19 x 40x33x29 49 and 29; 0.88 M as 96^3 25 and 27, as 8
 // x 48^3 35 and 31; 256x128x64 35 and 49; 256x128x128 73 and 115: taken up to
-// GRAD_NODES_MAX nodes of a context.
+// GRAD_NODES_MAX nodes of a context.  (Marching with gathered sums; by direction
+// it takes some 5 to 20% longer.)
 template <class R>
 constexpr int GN_THREADS = sizeof(R) == 8 ? 32 : 128;
 template <class R>
@@ -1086,7 +1266,7 @@ __device__ __forceinline__ bool gn_node(const Lattice &L, const InstDev **I, int
 
 // gradient, wetting and normal (0 at a solid node); the solid neighbours' share
 // of the curvature into its slot
-template <class R>
+template <class R, bool DIR>
 __global__ void __launch_bounds__(GN_THREADS<R>) k_grad_nodes(Lattice L)
 {
     const InstDev *Ip;
@@ -1112,7 +1292,9 @@ __global__ void __launch_bounds__(GN_THREADS<R>) k_grad_nodes(Lattice L)
     auto at = [&](int dx, int dy, int dz) { return v[dir_of(dx, dy, dz)]; };
     const R twelfth = R(1.0 / 12.0), sixth = R(1.0 / 6.0);
     R g[3];
-    {
+    if constexpr (DIR) {
+        dir_gradient<R>(at, g);
+    } else {
         const R d1 = sub_rn(at(1, 1, 0), at(-1, -1, 0)), d2 = sub_rn(at(1, -1, 0), at(-1, 1, 0));
         const R X = sub_rn(at(1, 0, 0), at(-1, 0, 0)), Y = sub_rn(at(0, 1, 0), at(0, -1, 0));
         R hx[2], hy[2], q[2];  // of the planes below and above
@@ -1135,22 +1317,24 @@ __global__ void __launch_bounds__(GN_THREADS<R>) k_grad_nodes(Lattice L)
             if constexpr (sizeof(R) == 8) return GcPart<R>{{P.x[0], P.x[1], P.x[2]}, P.R, P.cos_t, P.sin_t};
             else return GcPart<R>{{P.xf[0], P.xf[1], P.xf[2]}, (R)P.R, (R)P.cos_t, (R)P.sin_t};
         };
-        gc_solid<R>(
+        gc_solid<DIR, R>(
             I, part, [&](int i) { return fli[nb.at(cx(i), cy(i), cz(i))]; }, v[0], x, y, z, g, sv);
     }
     const R eps2 = sizeof(R) == 8 ? (R)(I.grad_eps * I.grad_eps) : (R)I.f_eps2;
-    const R im = frsqrt(fma_rn(g[0], g[0], fma_rn(g[1], g[1], fma_rn(g[2], g[2], eps2))));
     R nn[3];
-    for (int a = 0; a < 3; a++) {
-        nn[a] = mul_rn(g[a], im);
-        nrm[a * L.Ntot + n] = nn[a];
+    if constexpr (DIR) {
+        dir_normal(g, eps2, nn);
+    } else {
+        const R im = frsqrt(fma_rn(g[0], g[0], fma_rn(g[1], g[1], fma_rn(g[2], g[2], eps2))));
+        for (int a = 0; a < 3; a++) nn[a] = mul_rn(g[a], im);
     }
+    for (int a = 0; a < 3; a++) nrm[a * L.Ntot + n] = nn[a];
     const R share = fma_rn(nn[0], sv[0], fma_rn(nn[1], sv[1], mul_rn(nn[2], sv[2])));
     ((GradRec<R> *)L.grad)[I.node_off + n] = GradRec<R>{g[0], g[1], g[2], share};
 }
 
 // curvature
-template <class R>
+template <class R, bool DIR>
 __global__ void __launch_bounds__(GN_THREADS<R>) k_curv_nodes(Lattice L)
 {
     const InstDev *Ip;
@@ -1164,7 +1348,21 @@ __global__ void __launch_bounds__(GN_THREADS<R>) k_curv_nodes(Lattice L)
     R *const k = &((GradRec<R> *)L.grad)[I.node_off + n].k;
     Nbr nb;
     nb.init(x, y, z, I.nx, I.ny, I.nz);
-    const uint8_t fl = L.flags[I.node_off + n];
+    const uint8_t *const fli = L.flags + I.node_off;
+    const uint8_t fl = fli[n];
+    if constexpr (DIR) {
+        if ((fl & OWNER_MASK) != OWN_FLUID) return;
+        auto normal = [&](int a, int i) { return nrm[a * L.Ntot + nb.at(cx(i), cy(i), cz(i))]; };
+        if (fl & BOUND_BIT) {
+            unsigned solid = 0;
+#pragma unroll
+            for (int i = 1; i < Q; i++)
+                if ((fli[nb.at(cx(i), cy(i), cz(i))] & OWNER_MASK) != OWN_FLUID) solid |= 1u << i;
+            *k = dir_curvature<R>([&](int a, int i) { return solid >> i & 1u ? nrm[a * L.Ntot + n] : normal(a, i); });
+        } else
+            *k = dir_curvature<R>(normal);
+        return;
+    }
     const R share = *k;
     // normals' components where the curvature takes them: n_a of the neighbours with c_a != 0
     auto at = [&](int a, int dx, int dy, int dz) { return nrm[a * L.Ntot + nb.at(dx, dy, dz)]; };
@@ -1209,14 +1407,15 @@ constexpr int ZC_MAX = 64;
 // The FP32 gradient pass's work items.  Where no z-chunk is asked for, the
 // planes per item of the least cost; slots are the resident CTAs.  128x64x64, 4
 // planes against 16: 24 against 37 us.  Every choice gives the same bits.
-void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm,
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool dir,
                    FluidLaunch *fz)
 {
-    const double slots = n_sm * (double)LBM_GC_MINB;
+    const double slots = n_sm * (double)(dir ? LBM_GC_MINB_DIR : LBM_GC_MINB);
+    const int TY = dir ? GcShape<true>::TY : GcShape<false>::TY;
     int zc_auto = 16;
     double least = -1.0;
     for (int zc = ZC_MAX; zc >= 2; zc--) {
-        const double cost = march_cost(inst, GC_TX, GcShape::TY, zc, 4, slots);
+        const double cost = march_cost(inst, GC_TX, TY, zc, 4, slots);
         if (least < 0.0 || cost < least) {
             least = cost;
             zc_auto = zc;
@@ -1227,7 +1426,7 @@ void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector
         InstDev &I = inst[k];
         const int req = k < zc_inst.size() && zc_inst[k] > 0 ? zc_inst[k] : zc_request;
         I.gc_tiles_x = (I.nx + GC_TX - 1) / GC_TX;
-        I.gc_tiles_y = (I.ny + GcShape::TY - 1) / GcShape::TY;
+        I.gc_tiles_y = (I.ny + TY - 1) / TY;
         const int zc = std::min(req > 0 ? req : zc_auto, I.nz);
         I.gc_nchunks = (I.nz + zc - 1) / zc;
         I.gc_zc = (I.nz + I.gc_nchunks - 1) / I.gc_nchunks;
@@ -1347,11 +1546,11 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     mk(STAGE_GRAD, 0);
     if (L.nrm) {
         const dim3 ctas((unsigned)(fz.items * (COLLIDE_NODES<R> / GN_THREADS<R>)));
-        launch_after(k_grad_nodes<R>, ctas, dim3(GN_THREADS<R>), st, L);
-        launch_after(k_curv_nodes<R>, ctas, dim3(GN_THREADS<R>), st, L);
+        launch_after(k_grad_nodes<R, BY_DIRECTION<S>>, ctas, dim3(GN_THREADS<R>), st, L);
+        launch_after(k_curv_nodes<R, BY_DIRECTION<S>>, ctas, dim3(GN_THREADS<R>), st, L);
         *launches += 1;
     } else
-        launch_after(k_gradcurv, dim3((unsigned)fz.gc_items), dim3(GcShape::NT), st, L);
+        launch_after(k_gradcurv<BY_DIRECTION<S>>, dim3((unsigned)fz.gc_items), dim3(GcShape<BY_DIRECTION<S>>::NT), st, L);
     mk(STAGE_GRAD, 1);
     lane.after_grad();
     if constexpr (BOUNCE_IN_SLOTS<S>) {

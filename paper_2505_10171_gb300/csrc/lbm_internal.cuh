@@ -20,6 +20,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <vector>
 
 namespace lbmg {
@@ -432,6 +433,44 @@ struct Region {
     }
 };
 
+// FP32 storage sums the order parameter, the gradient, the curvature and the
+// moments of the collision direction by direction, in the order of the
+// directions; the other types gather terms (fewer instructions or FP64 operations).
+// A regrouped FP32 sum moves phi by some 1e-7, and the wetting rotation
+// applies where |phi| < wet_max: a node whose phi lies that close to the cut
+// falls on its other side, turns its normal (by 60 degrees at a wall of 150) and
+// moves phi by up to 8e-4 from there on.  A run in FP32 follows one order of
+// summation for good, so that its results stay the same from one version of
+// these kernels to the next.  (In 16-bit storage the offsets' own rounding is
+// coarser than any regrouping; in FP64 no node comes that close.)
+template <class S>
+constexpr bool BY_DIRECTION = std::is_same_v<S, float>;
+
+// Operations rounded as written.  Several copies of the gradient's arithmetic
+// (a tile's own nodes, those around it, the form without tiles) must give a
+// node the same bits, and the compiler would be free to contract each into
+// different multiply-adds (with the copies contracted apart, a symmetric drop
+// took up a sideways drift of 1e-4 of its speed).
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// regularised interface normal n = g/sqrt(|g|^2 + eps^2) of FP32 storage;
+// returns the norm
+template <class R>
+__device__ __forceinline__ R dir_normal(const R *g, R eps2, R *nn)
+{
+    const R m2 = add_rn(fma_rn(g[2], g[2], fma_rn(g[0], g[0], mul_rn(g[1], g[1]))), eps2);
+    const R im = frsqrt(m2);
+    for (int a = 0; a < 3; a++) nn[a] = mul_rn(g[a], im);
+    return mul_rn(m2, im);
+}
+
 // The colour record of a node of the stored state (see the top of this
 // file): the order parameter phi of the collision that produced it and
 // a = b n, one 16-byte (FP64: 32-byte) aligned record, so that a pulled source
@@ -666,8 +705,9 @@ __device__ __forceinline__ typename Store<S>::real gather_colour(const Nbr &nb, 
             const bool fluid = own[i] == OWN_FLUID;
             const ColRec<R> s = {fluid ? r[k].p : cn.p, fluid ? r[k].a0 : cn.a0, fluid ? r[k].a1 : cn.a1,
                                  fluid ? r[k].a2 : cn.a2};
-            const R t = col_rec(i, s);
-            g += wgt<R>(i) * (s.p * (R(1) + F[i]) + (fluid || own[i] == OWN_PRESS ? t : -t));
+            const R t = col_rec(i, s), st = fluid || own[i] == OWN_PRESS ? t : -t;
+            if constexpr (BY_DIRECTION<S>) g = fma_rn(wgt<R>(i), fma_rn(s.p, add_rn(R(1), F[i]), st), g);
+            else g += wgt<R>(i) * (s.p * (R(1) + F[i]) + st);
         }
     }
     return g;
@@ -766,7 +806,7 @@ constexpr long long GRAD_NODES_MAX = 768 * 1024;
 // plan the work items of the gradient + curvature kernel into fz (z-planes per
 // item: zc_inst[k] for instance k where set (> 0), else zc_request where set,
 // else chosen from the grid's size and the n_sm SMs); used where L.nrm is null
-void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm,
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool dir,
                    FluidLaunch *fz);
 // plan the work items of the order-parameter kernel into fz
 void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz);

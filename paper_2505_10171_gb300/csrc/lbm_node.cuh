@@ -1,7 +1,8 @@
 // Per-node arithmetic of the collision (Sec. IV of arXiv 2505.10171): velocity
 // and force, MRT with Guo forcing in its two-relaxation-time form, recolouring.
-// One template for every kernel and arithmetic: V is float, double, or F2, two
-// floats that an instruction handles at once (a node pair of 16-bit storage).
+// The gathered form is one template: V is double, float (16-bit storage), or
+// F2, two floats that an instruction handles at once (a node pair of 16-bit
+// storage).  FP32 storage relaxes direction by direction (BY_DIRECTION).
 #pragma once
 
 #include <type_traits>
@@ -245,6 +246,83 @@ __device__ __forceinline__ ColRec<R> colour_record(R bq, R eps2, R phi, R g0, R 
     return ColRec<R>{phi, b * g0, b * g1, b * g2};
 }
 
+// The form of FP32 storage: moments summed and pairs relaxed direction by
+// direction.  The collision is bound by memory there (119 us per 256x128x128
+// launch either way), so the gathered form has nothing to give, and it rounds
+// otherwise (see BY_DIRECTION).
+template <class R>
+struct DirCollision {
+    R sF, rr, u[3], f[3], om, omp, uu, uF, cpe, cpo, bq;
+};
+
+// g, kap: corrected grad(phi) and curvature
+template <class R>
+__device__ __forceinline__ DirCollision<R> dir_setup(const FluidPar<R> &P, const R (&F)[Q], R phi, const R (&g)[3], R kap)
+{
+    DirCollision<R> c;
+    R sF = 0, jx = 0, jy = 0, jz = 0;
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        const R w = wgt<R>(i);
+        sF += w * F[i];
+        if (cx(i)) jx += w * cx(i) * F[i];
+        if (cy(i)) jy += w * cy(i) * F[i];
+        if (cz(i)) jz += w * cz(i) * F[i];
+    }
+    c.sF = sF;
+    c.rr = R(1) + sF;  // rho / rho0
+    // force density: CSF -1/2 sigma kappa grad(phi) plus phase-weighted body forces
+    const R hs = R(-0.5) * P.sigma * kap;
+    const R pa = R(0.5) * (R(1) + phi), pb = R(0.5) * (R(1) - phi);
+    // (which product is rounded by itself is part of the results: it differs in x)
+    c.f[0] = fma_rn(pb, P.bb[0], fma_rn(pa, P.ba[0], mul_rn(hs, g[0])));
+    c.f[1] = fma_rn(pb, P.bb[1], fma_rn(hs, g[1], mul_rn(pa, P.ba[1])));
+    c.f[2] = fma_rn(pb, P.bb[2], fma_rn(hs, g[2], mul_rn(pa, P.ba[2])));
+    // velocity: rho u = sum c f + F/2
+    const R rho = P.rho0 * c.rr;
+    const R irho = frcp(rho);
+    c.u[0] = (P.rho0 * jx + R(0.5) * c.f[0]) * irho;
+    c.u[1] = (P.rho0 * jy + R(0.5) * c.f[1]) * irho;
+    c.u[2] = (P.rho0 * jz + R(0.5) * c.f[2]) * irho;
+    // relaxation rates: harmonic-mean viscosity, tau = eta/(rho cs2) + 1/2
+    const R inv_eta = (R(1) + phi) * P.h_ia + (R(1) - phi) * P.h_ib;
+    const R tau = R(3) * frcp(inv_eta * rho) + R(0.5);
+    c.om = frcp(tau);
+    c.omp = R(8) * (R(2) - c.om) * frcp(R(8) - c.om);
+    c.uu = c.u[0] * c.u[0] + c.u[1] * c.u[1] + c.u[2] * c.u[2];
+    c.uF = c.u[0] * c.f[0] + c.u[1] * c.f[1] + c.u[2] * c.f[2];
+    c.cpe = R(1) - R(0.5) * c.om;
+    c.cpo = R(1) - R(0.5) * c.omp;
+    c.bq = R(0.5) * P.beta * c.rr * (R(1) - phi * phi);
+    return c;
+}
+
+template <class R>
+__device__ __forceinline__ R dir_rest(const FluidPar<R> &P, const DirCollision<R> &c, R F0)
+{
+    const R feq0 = c.sF + c.rr * (R(-1.5) * c.uu);
+    const R fb0 = R(-3) * c.uF * P.ir0;
+    return F0 - c.om * (F0 - feq0) + c.cpe * fb0;
+}
+
+// opposite pair (i, i + 9), relaxed in its even and odd parts
+template <int i, class R>
+__device__ __forceinline__ void dir_pair(const FluidPar<R> &P, const DirCollision<R> &c, R Fi_in, R Fib_in, R &Fi, R &Fib)
+{
+    const R cu = cx(i) * c.u[0] + cy(i) * c.u[1] + cz(i) * c.u[2];
+    const R cF = cx(i) * c.f[0] + cy(i) * c.f[1] + cz(i) * c.f[2];
+    const R eqp = c.sF + c.rr * (R(4.5) * cu * cu - R(1.5) * c.uu);
+    const R eqm = c.rr * R(3) * cu;
+    const R fbp = (R(9) * cu * cF - R(3) * c.uF) * P.ir0;
+    const R fbm = R(3) * cF * P.ir0;
+    const R fp = R(0.5) * (Fi_in + Fib_in);
+    const R fm = R(0.5) * (Fi_in - Fib_in);
+    const R dp = -c.om * (fp - eqp) + c.cpe * fbp;
+    const R dm = -c.omp * (fm - eqm) + c.cpo * fbm;
+    Fi = Fi_in + dp + dm;
+    Fib = Fib_in + dp - dm;
+}
+
 // force, velocity, MRT with Guo forcing, recolouring and the write of node n.
 // The recolouring of Sec. IV gives G*_i = phi (1 + F*_i) + b (c_i . n)/|c_i|
 // with b = beta/2 (rho/rho0)(1 - phi^2): the state is complete with F* and
@@ -261,18 +339,39 @@ __device__ __forceinline__ void collide_store_phi(const FluidPar<typename Store<
     const int N = out.N;
     FT *const of = out.f + n;  // F_0 of this node; F_i at of + i N
     const R g[3] = {gr.g0, gr.g1, gr.g2};
-    const Collision<R> c = collide_setup(CollidePar<R>(P), F, phi, g, gr.k);
-    if (status && (!(c.rr > R(0)) || !(phi == phi))) atomicOr(status, ST_UNSTABLE);
-    if (U) { U[n] = c.u[0]; U[Ustride + n] = c.u[1]; U[2 * Ustride + n] = c.u[2]; }
-    C.set(colour_record(c.bq, P.eps2, phi, g[0], g[1], g[2]));
-    Store<FT>::st(of, collide_rest(c, F[0]));
-    PairLoop<R>::run([&](auto ic) {
-        constexpr int i = decltype(ic)::value, ib = i + 9;
-        R Fi, Fib;
-        collide_pair<i>(c, F[i], F[ib], Fi, Fib);
-        Store<FT>::st(of + i * N, Fi);
-        Store<FT>::st(of + ib * N, Fib);
-    });
+    auto store_moments = [&](R rr, const R *u) {
+        if (status && (!(rr > R(0)) || !(phi == phi))) atomicOr(status, ST_UNSTABLE);
+        if (U) { U[n] = u[0]; U[Ustride + n] = u[1]; U[2 * Ustride + n] = u[2]; }
+    };
+    if constexpr (BY_DIRECTION<S>) {
+        // the gradient as the product of its norm and normal, as it was formed
+        R nn[3];
+        const R m = dir_normal(g, P.eps2, nn);
+        const R gm[3] = {nn[0] * m, nn[1] * m, nn[2] * m};
+        const DirCollision<R> c = dir_setup(P, F, phi, gm, gr.k);
+        store_moments(c.rr, c.u);
+        C.set(ColRec<R>{phi, c.bq * nn[0], c.bq * nn[1], c.bq * nn[2]});
+        Store<FT>::st(of, dir_rest(P, c, F[0]));
+        PairLoop<R>::run([&](auto ic) {
+            constexpr int i = decltype(ic)::value, ib = i + 9;
+            R Fi, Fib;
+            dir_pair<i>(P, c, F[i], F[ib], Fi, Fib);
+            Store<FT>::st(of + i * N, Fi);
+            Store<FT>::st(of + ib * N, Fib);
+        });
+    } else {
+        const Collision<R> c = collide_setup(CollidePar<R>(P), F, phi, g, gr.k);
+        store_moments(c.rr, c.u);
+        C.set(colour_record(c.bq, P.eps2, phi, g[0], g[1], g[2]));
+        Store<FT>::st(of, collide_rest(c, F[0]));
+        PairLoop<R>::run([&](auto ic) {
+            constexpr int i = decltype(ic)::value, ib = i + 9;
+            R Fi, Fib;
+            collide_pair<i>(c, F[i], F[ib], Fi, Fib);
+            Store<FT>::st(of + i * N, Fi);
+            Store<FT>::st(of + ib * N, Fib);
+        });
+    }
 }
 
 }  // namespace lbmg

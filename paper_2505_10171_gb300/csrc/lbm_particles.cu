@@ -130,10 +130,10 @@ __global__ void __launch_bounds__(MEM_THREADS) k_mem(Lattice L, int cur, FastDiv
             D0[a] = d;
         }
         const R r0 = sizeof(R) == 8 ? (R)I.rho0 : (R)I.f_rho0;
-        R rr = 1;
+        R sF = 0;  // the offsets' sum first: added to 1 one by one, each would be rounded at 1
 #pragma unroll
-        for (int i = 0; i < Q; i++) rr += wgt<R>(i) * F[i];
-        const R r6 = R(6) * rr;
+        for (int i = 0; i < Q; i++) sF += wgt<R>(i) * F[i];
+        const R r6 = R(6) * (R(1) + sF);
         // lever and wall velocity of a link, and c.u_w
         auto link = [&](int i, const R *lev, const R *uw, R cu) {
             const R wt = wgt<R>(i) * r0;
@@ -231,9 +231,10 @@ __device__ __forceinline__ void surface_point(const Lattice &L, int pt, double *
     for (int a = 0; a < 4; a++) t[a] = L.cap_pts[4 * pt + a];
 }
 
-template <class R, bool BUOY>
+template <class S, bool BUOY>
 __global__ void __launch_bounds__(CAP_THREADS) k_capillary(Lattice L)
 {
+    using R = typename Store<S>::real;
     const int p = blockIdx.y;
     const PartDev &P = L.parts[p];
     const InstDev &I = L.inst[P.inst];
@@ -279,11 +280,15 @@ __global__ void __launch_bounds__(CAP_THREADS) k_capillary(Lattice L)
         for (int k = 0; k < 8; k++) {
             if ((fl[k] & OWNER_MASK) != OWN_FLUID) continue;
             const R wgt_ = (k & 1 ? fr[0] : R(1) - fr[0]) * (k & 2 ? fr[1] : R(1) - fr[1]) * (k & 4 ? fr[2] : R(1) - fr[2]);
+            R g[3] = {gc[k].g0, gc[k].g1, gc[k].g2};
+            if constexpr (BY_DIRECTION<S>) {  // as the collision takes it
+                R nn[3];
+                const R m = dir_normal(g, I.f_eps2, nn);
+                for (int a = 0; a < 3; a++) g[a] = mul_rn(nn[a], m);
+            }
             ws += wgt_;
             phs += wgt_ * pc[k];
-            gs[0] += wgt_ * gc[k].g0;
-            gs[1] += wgt_ * gc[k].g1;
-            gs[2] += wgt_ * gc[k].g2;
+            for (int a = 0; a < 3; a++) gs[a] += wgt_ * g[a];
         }
         if (ws > R(0)) {
             const R phv = phs / ws;
@@ -928,13 +933,12 @@ void launch_momentum_exchange(const Lattice &L, int cur, cudaStream_t st, long l
 template <class S>
 void launch_capillary(const Lattice &L, cudaStream_t st, long long *launches, const Marker &mk)
 {
-    using R = typename Store<S>::real;
     if (L.n_parts == 0) return;
     mk(STAGE_CAPILLARY, 0);
     if (L.buoyancy)
-        k_capillary<R, true><<<dim3(CAP_BLOCKS, L.n_parts), CAP_THREADS, 0, st>>>(L);
+        k_capillary<S, true><<<dim3(CAP_BLOCKS, L.n_parts), CAP_THREADS, 0, st>>>(L);
     else
-        k_capillary<R, false><<<dim3(CAP_BLOCKS, L.n_parts), CAP_THREADS, 0, st>>>(L);
+        k_capillary<S, false><<<dim3(CAP_BLOCKS, L.n_parts), CAP_THREADS, 0, st>>>(L);
     mk(STAGE_CAPILLARY, 1);
     *launches += 1;
 }
