@@ -1390,12 +1390,19 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
         long long **lists[2] = {&ctx->static_list, &ctx->static_bfl};
         long long *counts[2] = {&ctx->n_static, &ctx->n_static_bfl};
         cudaError_t e = cudaSuccess;
+        // (a call that ran out of memory half way leaves the first list: another
+        // solid map since then may need a longer one)
+        for (int mode = 0; mode < 2; mode++) {
+            cudaFree(*lists[mode]);
+            *lists[mode] = nullptr;
+            *counts[mode] = 0;
+        }
         for (int mode = 0; mode < 2 && e == cudaSuccess; mode++) {
             long long h = 0;
             launch_static_count(L, blocks, offs, mode, ctx->stream);
             e = cudaMemcpyAsync(&h, offs + nb, sizeof h, cudaMemcpyDeviceToHost, ctx->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-            if (e == cudaSuccess && h > 0 && !*lists[mode]) e = cudaMalloc((void **)lists[mode], sizeof(long long) * h);
+            if (e == cudaSuccess && h > 0) e = cudaMalloc((void **)lists[mode], sizeof(long long) * h);
             if (e == cudaSuccess && h > 0) launch_static_fill(L, offs, *lists[mode], mode, ctx->stream);
             if (e == cudaSuccess) *counts[mode] = h;
         }
@@ -1404,6 +1411,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
         if (e == cudaSuccess) launch_first_lists(L, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // before offs goes
         cudaFree(offs);
+        if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next call
         CU(e);
         CU(cudaGetLastError());
         ctx->static_ready = true;
