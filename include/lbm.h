@@ -334,11 +334,14 @@ lbm_status lbm_set_fluid_kernel(lbm_ctx *ctx, int form, int tile, int zchunk);
 
 /* Autotuner of the launch shape, on the context's own instances.  Instances
  * fall into size classes by nz (<= 64, <= 96, <= 128, larger); for each class
- * present, the z-planes per work item of the gradient pass are chosen from 8,
- * 16 and 32 (the other classes held at their current choice), then the
- * bulk-kernel variant (tile 0, 1).  Each candidate is re-planned, its step
+ * present, the z-planes per work item of the gradient pass are chosen from the
+ * number that zchunk 0 stands for and two of 8, 16 and 32 (the other classes held
+ * at their current choice; the first is kept unless another is 1% faster), then
+ * the bulk-kernel variant (tile 0, 1).  Each candidate is re-planned, its step
  * graph captured and warmed up for 2 steps, then timed over `steps` (>= 2)
- * steps with CUDA events on the context stream; the fastest is kept.  The
+ * steps with CUDA events on the context stream; the fastest is kept.  Where the
+ * z-chunk has no effect (FP64 contexts and those of up to 786432 nodes) the
+ * candidates are 8, 16 and 32, the same kernels for each.  The
  * simulation advances by all the trial steps (every shape computes the same
  * update).  *tile receives the variant; zchunks (may be NULL) one z-chunk per
  * instance; ms_best (may be NULL) the ms per step of the chosen shape.

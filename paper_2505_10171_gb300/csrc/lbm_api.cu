@@ -2106,8 +2106,18 @@ lbm_status lbm_autotune(lbm_ctx *ctx, int steps, int *tile, int *zchunks, double
     ctx->zc_inst.assign(ctx->n_inst, 0);
     bool present[4] = {false, false, false, false};
     for (const auto &I : ctx->inst_h) present[size_class(I.nz)] = true;
-    const int cand[3] = {8, 16, 32};
-    double best = -1.0;
+    // where the pass marches, the planned chunk first, in the place of the
+    // candidate nearest to it, to be left for one that gains more than the runs
+    // of a shape differ (elsewhere the chunk has no effect)
+    int cand[3] = {8, 16, 32};
+    if (!ctx->nrm) {
+        const int planned = planned_zchunk(ctx->inst_h, ctx->n_sm, ctx->prec == LBM_FP32);
+        int near = 0;
+        for (int k = 1; k < 3; k++)
+            if (std::fabs(std::log((double)cand[k] / planned)) < std::fabs(std::log((double)cand[near] / planned))) near = k;
+        cand[near] = cand[0];
+        cand[0] = planned;
+    }
     for (int c = 0; c < 4 && st == LBM_OK; c++) {
         if (!present[c]) continue;
         int bz = 0;
@@ -2117,17 +2127,15 @@ lbm_status lbm_autotune(lbm_ctx *ctx, int steps, int *tile, int *zchunks, double
                 if (size_class(ctx->inst_h[k].nz) == c) ctx->zc_inst[k] = z;
             double ms = 0.0;
             if ((st = time_shape(&ms)) != LBM_OK) break;
-            if (bc < 0.0 || ms < bc) {
+            if (bc < 0.0 || ms < (ctx->nrm ? 1.0 : 0.99) * bc) {
                 bc = ms;
                 bz = z;
             }
         }
         for (int k = 0; k < ctx->n_inst; k++)
             if (size_class(ctx->inst_h[k].nz) == c) ctx->zc_inst[k] = bz;
-        best = bc;
     }
     // 2. the bulk-kernel variant
-    (void)best;
     int bt = 0;
     double bestt = -1.0;
     for (int t = 0; t < 2 && st == LBM_OK; t++) {

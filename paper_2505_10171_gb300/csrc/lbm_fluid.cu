@@ -1407,20 +1407,27 @@ constexpr int ZC_MAX = 64;
 // The FP32 gradient pass's work items.  Where no z-chunk is asked for, the
 // planes per item of the least cost; slots are the resident CTAs.  128x64x64, 4
 // planes against 16: 24 against 37 us.  Every choice gives the same bits.
-void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool dir,
-                   FluidLaunch *fz)
+int planned_zchunk(const std::vector<InstDev> &inst, int n_sm, bool dir)
 {
     const double slots = n_sm * (double)(dir ? LBM_GC_MINB_DIR : LBM_GC_MINB);
     const int TY = dir ? GcShape<true>::TY : GcShape<false>::TY;
-    int zc_auto = 16;
+    int planned = 16;
     double least = -1.0;
     for (int zc = ZC_MAX; zc >= 2; zc--) {
         const double cost = march_cost(inst, GC_TX, TY, zc, 4, slots);
         if (least < 0.0 || cost < least) {
             least = cost;
-            zc_auto = zc;
+            planned = zc;
         }
     }
+    return planned;
+}
+
+void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool dir,
+                   FluidLaunch *fz)
+{
+    const int TY = dir ? GcShape<true>::TY : GcShape<false>::TY;
+    const int zc_auto = planned_zchunk(inst, n_sm, dir);
     long long items = 0;
     for (size_t k = 0; k < inst.size(); k++) {
         InstDev &I = inst[k];

@@ -803,9 +803,12 @@ struct FluidLaunch {
 // The gradient pass takes a node per thread in FP64 runs and up to this many
 // nodes of a context, marching tiles beyond (measured beside the kernels)
 constexpr long long GRAD_NODES_MAX = 768 * 1024;
+// z-planes per work item of the gradient + curvature kernel for a grid's size and
+// the n_sm SMs; dir: FP32 storage
+int planned_zchunk(const std::vector<InstDev> &inst, int n_sm, bool dir);
 // plan the work items of the gradient + curvature kernel into fz (z-planes per
 // item: zc_inst[k] for instance k where set (> 0), else zc_request where set,
-// else chosen from the grid's size and the n_sm SMs); used where L.nrm is null
+// else planned_zchunk); used where L.nrm is null
 void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector<int> &zc_inst, int n_sm, bool dir,
                    FluidLaunch *fz);
 // plan the work items of the order-parameter kernel into fz
