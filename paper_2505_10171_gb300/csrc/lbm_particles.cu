@@ -510,19 +510,39 @@ __global__ void __launch_bounds__(CONTACT_THREADS) k_contacts(Lattice L)
 
 // The step of a particle, by one warp: the fluid forces from the block partials
 // of the momentum-exchange and capillary kernels (lanes over a fixed block
-// stride, then warp_sums; sum_fluid 0: the surrogate has set them), contacts
+// stride, then warp_sums, WARPS of them for the momentum exchange's and their
+// sums in order; sum_fluid 0: the surrogate has set them), contacts
 // added in a fixed order (substrate, then partners in increasing index), the
 // velocity-Verlet correction with lane a and 3 + a on axis a, and the record
 // in the record ring.  It also empties the boundary and refill lists that the
 // geometry kernels after it fill.  One warp a CTA: the particles' FP64 chains
 // run on as many SMs (a CTA of 8 warps per instance, contacts included, took
-// 28 us for 8 particles and 17 for one; now 14, and 6 for the contacts).
-template <class T, bool BUOY>
-__global__ void __launch_bounds__(32) k_dem(Lattice L, int sum_fluid)
+// 28 us for 8 particles and 17 for one; now 14, and 6 for the contacts).  A large
+// sphere has a partial for each 64 nodes of its cube (R = 8: 145, 16: 792, 60:
+// 30518), a round trip for every 32 that a warp takes: the kernel took 14, 31 and
+// 843 us with one warp, 14, 17 and 126 with eight (sixteen 15, 18 and 120).
+constexpr int DEM_WARPS = 8;
+constexpr int DEM_ONE_WARP = 96;  // partials that one warp takes
+template <class T, bool BUOY, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_dem(Lattice L, int sum_fluid)
 {
     const int pg = blockIdx.x, lane = threadIdx.x;
-    if (pg == 0 && lane < 4) L.list_n[lane] = 0;
     PartDev &P = L.parts[pg];
+    __shared__ double wide[WARPS > 1 ? WARPS : 1][MEM_PART];
+    if constexpr (WARPS > 1) {
+        if (sum_fluid) {
+            double m[16];
+            for (int a = 0; a < 16; a++) m[a] = 0.0;
+            for (int b = threadIdx.x; b < L.mem_blocks; b += 32 * WARPS)
+                for (int a = 0; a < MEM_PART; a++) m[a] += L.mem_part[((long long)pg * L.mem_blocks + b) * MEM_PART + a];
+            warp_sums<16>(m);
+            const int l = threadIdx.x & 31;
+            if (l % 2 == 0 && l / 2 < MEM_PART) wide[threadIdx.x >> 5][l / 2] = m[0];
+            __syncthreads();
+        }
+        if (threadIdx.x >= 32) return;  // the first warp goes on
+    }
+    if (pg == 0 && lane < 4) L.list_n[lane] = 0;
     const InstDev &I = L.inst[P.inst];
     const int np = I.np, p = P.local;
     const double *rec = L.crec + (long long)I.crec_off * 12;
@@ -534,11 +554,19 @@ __global__ void __launch_bounds__(32) k_dem(Lattice L, int sum_fluid)
         constexpr int NC = BUOY ? 8 : 6;  // capillary partials used
         for (int b = lane; b < CAP_BLOCKS; b += 32)
             for (int a = 0; a < NC; a++) c[a] += L.cap_part[((long long)pg * CAP_BLOCKS + b) * CAP_PART + a];
-        for (int b = lane; b < L.mem_blocks; b += 32)
-            for (int a = 0; a < MEM_PART; a++) m[a] += L.mem_part[((long long)pg * L.mem_blocks + b) * MEM_PART + a];
-        warp_sums<16>(m);
+        if constexpr (WARPS > 1) {
+            if (lane < MEM_PART) {
+                double t = wide[0][lane];
+                for (int w = 1; w < WARPS; w++) t += wide[w][lane];
+                s[lane] = t;
+            }
+        } else {
+            for (int b = lane; b < L.mem_blocks; b += 32)
+                for (int a = 0; a < MEM_PART; a++) m[a] += L.mem_part[((long long)pg * L.mem_blocks + b) * MEM_PART + a];
+            warp_sums<16>(m);
+            if (lane % 2 == 0 && lane / 2 < MEM_PART) s[lane / 2] = m[0];
+        }
         warp_sums<8>(c);
-        if (lane % 2 == 0 && lane / 2 < 12) s[lane / 2] = m[0];
         if (lane % 4 == 0) s[12 + lane / 4] = c[0];
         __syncwarp();
         if (lane < 3) {
@@ -959,10 +987,10 @@ void launch_dem(const Lattice &L, cudaStream_t st, long long *launches, const Ma
     using R = typename Store<S>::real;
     if (L.n_parts == 0) return;
     mk(STAGE_DEM, 0);
-    if (L.buoyancy)
-        k_dem<R, true><<<L.n_parts, 32, 0, st>>>(L, sum_fluid ? 1 : 0);
-    else
-        k_dem<R, false><<<L.n_parts, 32, 0, st>>>(L, sum_fluid ? 1 : 0);
+    const bool wide = sum_fluid && L.mem_blocks > DEM_ONE_WARP;
+    auto kernel = L.buoyancy ? (wide ? k_dem<R, true, DEM_WARPS> : k_dem<R, true, 1>)
+                             : (wide ? k_dem<R, false, DEM_WARPS> : k_dem<R, false, 1>);
+    kernel<<<L.n_parts, wide ? 32 * DEM_WARPS : 32, 0, st>>>(L, sum_fluid ? 1 : 0);
     mk(STAGE_DEM, 1);
     *launches += 1;
 }
