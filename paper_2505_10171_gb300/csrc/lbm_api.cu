@@ -82,7 +82,7 @@ struct lbm_ctx {
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_pairs;
     cudaEvent_t ev_open[N_STAGES] = {};
     // launch variant of the fluid update
-    FluidLaunch fz = {0, 0, 0, 0, false};
+    FluidLaunch fz = {0, 0, 0, 0, 0, false};
     int zc_request = 0;        // z-planes per gradient work item, 0: automatic
     std::vector<int> zc_inst;  // per instance (the autotuner's size classes), 0: zc_request
     // drop-speed control: per instance integral (3) and last U_a (3); block partials

@@ -6,7 +6,7 @@
 // divergence (curvature) -> CSF + body force -> MRT with Guo forcing, evaluated
 // in its two-relaxation-time form -> recolouring -> write.
 //
-// Kernels of a step: k_phi (z-marching tiles) stores phi;
+// Kernels of a step: k_phi (z-marching tiles; narrow domains: k_phi_nodes) stores phi;
 // the solid-phi fill over the listed static solid nodes and the step's list
 // of particle-surface solid nodes; k_gradcurv (z-marching tiles: gradient,
 // wetting, normal, curvature; FP64 and small grids: k_grad_nodes and
@@ -733,6 +733,57 @@ __device__ __forceinline__ bool item_node(const Lattice &L, long long item, int 
     return true;
 }
 
+// The form without tiles, for domains that fill few of the tiles' lanes or planes:
+// a node per thread, direction by direction, every record loaded where it is
+// wanted.  Bound by the latency of those loads and by L1 (19 records of 16 bytes a
+// node).  Marching against this form, FP32 (FP16), by the share of the tiles'
+// work that is nodes, nx ny nz over 256 tiles nz + 2 planes: 0.25 (8x8x16384) 82
+// and 34 us (70, 27); 0.33 (1024x1024x1) 49 and 35 (42, 27); 0.45 (34x34x1024) 58
+// and 41 (50, 33); 0.47 (512 x 16^3) 102 and 85 (92, 84); 0.57 (42x42x1024) 70 and
+// 57 (60, 52); 0.60 (64 x 40^3) 135 and 131 (117, 125); 0.75 (48x48x1024) 72 and 69
+// (62, 65); 1 (256x128x128) 94 and 113 (82, 114).  FP64 keeps the tiles, which
+// spare it instructions.
+// Four CTAs per SM (64 registers); three 43 us on 34x34x1024, two 43.
+constexpr int PN_NODES = 256;
+constexpr double PN_SHARE = 0.58;
+#ifndef LBM_PHI_NODES_MINB
+#define LBM_PHI_NODES_MINB 4
+#endif
+template <class S>
+__global__ void __launch_bounds__(PN_NODES, LBM_PHI_NODES_MINB) k_phi_nodes(Lattice L, int cur)
+{
+    using R = typename Store<S>::real;
+    int lo = 0, hi = L.n_inst - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (L.inst[mid].pn_item_start <= (long long)blockIdx.x) lo = mid;
+        else hi = mid - 1;
+    }
+    const InstDev &I = L.inst[lo];
+    const int n = (int)((long long)blockIdx.x - I.pn_item_start) * PN_NODES + (int)threadIdx.x;
+    pdl_trigger();  // the gradient pass may be scheduled as this grid drains
+    if (n >= I.pstride) return;
+    const int row = I.fd_nx.div(n), z = I.fd_ny.div(row), x = n - row * I.nx, y = row - z * I.ny;
+    Nbr nb;
+    nb.init(x, y, z, I.nx, I.ny, I.nz);
+    const Pop<S> in(L.pop[cur], I);
+    const ColRec<R> *const rec = (const ColRec<R> *)L.col + I.node_off;
+    const uint8_t fl = L.flags[I.node_off + n];
+    R sF = 0, sG = 0;
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        const int s = nb.at(-cx(i), -cy(i), -cz(i));
+        const R F = in.F(i, s), e = add_rn(R(1), F);
+        const ColRec<R> r = rec[s];
+        const R G = i ? fma_rn(r.p, e, col_rec(i, r)) : mul_rn(r.p, e);
+        sF = fma_rn(wgt<R>(i), F, sF);
+        sG = fma_rn(wgt<R>(i), G, sG);
+    }
+    R v = sG / add_rn(R(1), sF);
+    keep(v);
+    if (!(fl & (OWNER_MASK | BOUND_BIT))) ((R *)L.phi)[I.node_off + n] = v;
+}
+
 template <class S>
 __global__ void __launch_bounds__(COLLIDE_NODES<S> / 2, LBM_COLLIDE2_MINB) k_collide2(Lattice L, int cur)
 {
@@ -1446,32 +1497,48 @@ void plan_gradcurv(std::vector<InstDev> &inst, int zc_request, const std::vector
 }
 
 // The order-parameter pass's work items, planned alike: one plane of halo
-// staged on each side of a chunk
+// staged on each side of a chunk.  An instance's form follows from its own shape
+// (its results must not depend on what else a context holds).
+static bool phi_by_node(const InstDev &I, bool fp64)
+{
+    const double tiles = (double)((I.nx + PH_TX - 1) / PH_TX) * ((I.ny + PH_TY - 1) / PH_TY);
+    return !fp64 && (double)I.nx * I.ny * I.nz < PN_SHARE * (PH_TX * PH_TY) * tiles * (I.nz + 2);
+}
+
 void plan_phi(std::vector<InstDev> &inst, int n_sm, bool fp64, FluidLaunch *fz)
 {
     const double slots = n_sm * (fp64 ? 1.0 : (double)LBM_PHI_MINB);
+    std::vector<InstDev> tiled;
+    for (const auto &I : inst)
+        if (!phi_by_node(I, fp64)) tiled.push_back(I);
     int best = 16;
     double least = -1.0;
     for (int zc = ZC_MAX; zc >= 2; zc--) {
-        const double cost = march_cost(inst, PH_TX, PH_TY, zc, 2, slots);
+        const double cost = march_cost(tiled, PH_TX, PH_TY, zc, 2, slots);
         if (least < 0.0 || cost < least) {
             least = cost;
             best = zc;
         }
     }
-    long long items = 0;
+    long long items = 0, nodes = 0;
     for (auto &I : inst) {
         I.ph_tiles_x = (I.nx + PH_TX - 1) / PH_TX;
         const int tiles_y = (I.ny + PH_TY - 1) / PH_TY;
+        I.pn_item_start = nodes;
+        I.ph_item_start = items;
+        if (phi_by_node(I, fp64)) {
+            nodes += (I.N + PN_NODES - 1) / PN_NODES;
+            continue;
+        }
         const int zc = std::min(best, I.nz);
         I.ph_nchunks = (I.nz + zc - 1) / zc;
         I.ph_zc = (I.nz + I.ph_nchunks - 1) / I.ph_nchunks;
         I.fd_ph_nchunks.set(I.ph_nchunks);
         I.fd_ph_tiles_x.set(I.ph_tiles_x);
-        I.ph_item_start = items;
         items += (long long)I.ph_tiles_x * tiles_y * I.ph_nchunks;
     }
     fz->ph_items = items;
+    fz->pn_items = nodes;
 }
 
 // the collision's work items
@@ -1547,7 +1614,10 @@ void launch_fluid_step(const Lattice &L, int cur, cudaStream_t st, long long *la
     if (lane.side && any_bound) cudaEventRecord(lane.b, lane.side);
     lane.after_phi_bound();
     mk(STAGE_PHI, 0);
-    k_phi<S><<<(unsigned)fz.ph_items, PH_TX * PH_TY, 0, st>>>(L, cur);
+    if constexpr (sizeof(S) < 8)
+        if (fz.pn_items > 0) k_phi_nodes<S><<<(unsigned)fz.pn_items, PN_NODES, 0, st>>>(L, cur);
+    if (fz.ph_items > 0) k_phi<S><<<(unsigned)fz.ph_items, PH_TX * PH_TY, 0, st>>>(L, cur);
+    if (fz.pn_items > 0 && fz.ph_items > 0) *launches += 1;
     mk(STAGE_PHI, 1);
     if (lane.side && any_bound) cudaStreamWaitEvent(st, lane.b, 0);
     mk(STAGE_GRAD, 0);

@@ -144,6 +144,7 @@ struct InstDev {
     long long ph_item_start;
     int ph_tiles_x, ph_nchunks, ph_zc;
     FastDiv fd_ph_nchunks, fd_ph_tiles_x;
+    long long pn_item_start;  // the same of the instances that it takes a node per thread
     // drop-speed control (body force on phase a): component mask, interval,
     // target velocity, PI gains, base force
     int sp_mask, sp_interval;
@@ -796,7 +797,8 @@ constexpr int FORM_PLAIN = 2;  // the launch form of the fluid update (the value
 struct FluidLaunch {
     int tile;           // 0: node-pair bulk collision where possible; 1: one node per thread
     long long items;    // collision work items (all instances)
-    long long ph_items; // order-parameter work items (all instances)
+    long long ph_items; // order-parameter work items (all instances): marching tiles
+    long long pn_items; // and a node per thread
     long long gc_items; // gradient + curvature work items (all instances)
     bool pair;          // every instance has an even nx: node-pair kernels for 16-bit storage
 };
