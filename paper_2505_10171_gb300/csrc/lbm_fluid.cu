@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(PH_TX *PH_TY, sizeof(S) == 8 ? 1 : LBM_PHI_MIN
 #pragma unroll
         for (int i = 0; i < Q; i++) {
             const S *const base = pf + (i * N + zo[cz(i) + 1]);
-            F[i] = pop_load(base + off[cy(i) + 1][cx(i) + 1]);
+            F[i] = pop_load_beside_writes(base + off[cy(i) + 1][cx(i) + 1]);
         }
         fl = fli[zt * plane + off[1][1]];
     };
@@ -454,10 +454,7 @@ __device__ __forceinline__ const InstDev &list_node(const Lattice &L, long long 
 // nodes like all others and has no boundary pass.  (16-bit storage would round
 // the offset there; its collision takes these nodes in k_collide_bound.)  The
 // bulk order-parameter pass may load such a slot while it is written: for a
-// node next to a solid, whose value it drops.
-template <class S>
-constexpr bool BOUNCE_IN_SLOTS = sizeof(S) >= 4;
-
+// node next to a solid, whose value it drops (pop_load_beside_writes).
 template <class S>
 __device__ __forceinline__ void phi_bound_node(const Lattice &L, int cur, long long e)
 {
@@ -773,7 +770,7 @@ __global__ void __launch_bounds__(PN_NODES, LBM_PHI_NODES_MINB) k_phi_nodes(Latt
 #pragma unroll
     for (int i = 0; i < Q; i++) {
         const int s = nb.at(-cx(i), -cy(i), -cz(i));
-        const R F = in.F(i, s), e = add_rn(R(1), F);
+        const R F = in.F_beside_writes(i, s), e = add_rn(R(1), F);
         const ColRec<R> r = rec[s];
         const R G = i ? fma_rn(r.p, e, col_rec(i, r)) : mul_rn(r.p, e);
         sF = fma_rn(wgt<R>(i), F, sF);

@@ -256,6 +256,19 @@ __device__ __forceinline__ T pop_load(const T *p)
     return __ldg(p);
 }
 
+// The boundary pass of the order parameter keeps bounced offsets in slots of solid
+// nodes (FP32 and FP64 storage); its own threads and the bulk pass beside it load
+// such a slot while it may be written, for a node that drops the value.  Those
+// loads are plain ones: the read-only path is for memory that nothing writes
+// while a kernel runs.  (Same time either way.)
+template <class S>
+constexpr bool BOUNCE_IN_SLOTS = sizeof(S) >= 4;
+template <class T>
+__device__ __forceinline__ T pop_load_beside_writes(const T *p)
+{
+    return BOUNCE_IN_SLOTS<T> ? *p : pop_load(p);
+}
+
 template <class S>
 struct Store;
 template <>
@@ -305,6 +318,10 @@ struct Pop {
     {
     }
     __device__ __forceinline__ R F(int i, int m) const { return Store<FT>::ld(f + i * N + m); }
+    __device__ __forceinline__ R F_beside_writes(int i, int m) const
+    {
+        return Store<FT>::cvt(pop_load_beside_writes(f + i * N + m));
+    }
     __device__ __forceinline__ void setF(int i, int m, R v) const { Store<FT>::st(f + i * N + m, v); }
 };
 
@@ -600,8 +617,8 @@ __device__ __forceinline__ void gather_links(const InstDev &I, const PartDev *pa
     for (int i = 0; i < Q; i++) {
         const int s = nb.at(-cx(i), -cy(i), -cz(i));
         own[i] = fli[s];
-        F[i] = in.F(i, s);
-        oF[i] = in.F(i, n);
+        F[i] = in.F_beside_writes(i, s);
+        oF[i] = in.F_beside_writes(i, n);
     }
     R sF = 0;
     unsigned long long met = 0;
