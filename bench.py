@@ -51,16 +51,22 @@ def population_bytes_per_node(stage, prec):
 
 
 def design_bytes_per_node(stage, prec):
+    """moved_bytes_per_node of a gradient record of five reals (normal, norm,
+    curvature), which the kernels had before it became four."""
+    e, r = ELEM[prec], REAL[prec]
+    return {"phi": 19 * e + 5 * r, "grad_wetting": 6 * r, "collide": 38 * e + 10 * r}.get(stage, 0)
+
+
+def moved_bytes_per_node(stage, prec):
     """Every byte a kernel reads or writes per node, each once: populations
     plus the per-node reals (phi, the colour record of 4, the gradient record of
     4: grad phi and kappa), flags left out.  Order parameter: 19 F + the sources'
-    records + phi out; gradient pass: phi in, its record out; collision: 19 F,
-    phi and the gradient record in, 19 F + record out.  The gradient pass and the
-    collision count one real more, the fifth of the gradient record's former
-    layout (2% of the collision's bytes), so that the fractions of older runs
-    compare."""
+    records + phi out; gradient pass: phi in, its record out (FP64, in two
+    kernels: the normals out and in and the curvature's slot in and out besides);
+    collision: 19 F, phi and the gradient record in, 19 F + record out."""
     e, r = ELEM[prec], REAL[prec]
-    return {"phi": 19 * e + 5 * r, "grad_wetting": 6 * r, "collide": 38 * e + 10 * r}.get(stage, 0)
+    grad = 13 * r if prec == "fp64" else 5 * r
+    return {"phi": 19 * e + 5 * r, "grad_wetting": grad, "collide": 38 * e + 9 * r}.get(stage, 0)
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant
@@ -343,10 +349,10 @@ def main():
     dom = max(prof, key=lambda k: prof[k]["ms"])
     dom_ms = prof[dom]["ms"] / max(1, prof[dom]["launches"])
     dom_bytes = population_bytes_per_node(dom, args.precision) * N
-    dom_design = design_bytes_per_node(dom, args.precision) * N
+    dom_design = moved_bytes_per_node(dom, args.precision) * N
     achieved = dom_bytes / (dom_ms * 1e-3) / 1e9 if dom_bytes else None
     step_bytes = method_bytes_per_lu(args.precision) * N
-    design_step = sum(design_bytes_per_node(k, args.precision) for k in ("phi", "grad_wetting", "collide"))
+    design_step = sum(moved_bytes_per_node(k, args.precision) for k in ("phi", "grad_wetting", "collide"))
     roofline = dict(bound="hbm", kernel=dom, achieved=achieved, peak=hbm, unit="GB/s",
                     frac=(achieved / hbm) if achieved else None,
                     traffic=ncu_traffic(dom, args.precision), peak_source=peak_src,
@@ -435,7 +441,7 @@ def extra_measure(torch, lbm, W, args, stream, N):
         col = prof["collide"]
         cms = col["ms"] / max(1, col["launches"])
         out[prec] = dict(value=N * K / (ms_g * 1e-3) / 1e6, value_profiled=N * K / (ms * 1e-3) / 1e6,
-                         collide_ms=cms, collide_gbs=design_bytes_per_node("collide", prec) * N / (cms * 1e-3) / 1e9,
+                         collide_ms=cms, collide_gbs=moved_bytes_per_node("collide", prec) * N / (cms * 1e-3) / 1e9,
                          steps=K)
     # the non-tensor arithmetic ceiling of the 16-bit modes (their collision
     # is issue-bound): measured FP32 FMA throughput against the nominal rate
