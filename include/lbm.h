@@ -176,8 +176,10 @@ enum {
  * records (uneven sizes allowed).  stream is a cudaStream_t (NULL: the
  * library creates its own).  Validates every parameter (nu > 0, beta in
  * [0, 1], sizes > 0, finite values) -> LBM_ERR_ARG; allocates all lattice
- * memory -> LBM_ERR_OOM.  Populations start at rest with phi = -1 everywhere
- * until lbm_init_fields. */
+ * memory -> LBM_ERR_OOM.  A node takes 38 population elements, a byte and 9
+ * reals (4 bytes, FP64 8), 3 reals more in FP64 contexts and those of up to
+ * 786432 nodes, and 3 more where an instance stores the velocity.  Populations
+ * start at rest with phi = -1 everywhere until lbm_init_fields. */
 lbm_status lbm_create(const lbm_params *params, int n_instances, lbm_precision prec,
                       void *stream, lbm_ctx **out);
 

@@ -1228,6 +1228,21 @@ lbm_status lbm_init_fields_device(lbm_ctx *ctx, int inst, const double *phi, con
     return LBM_OK;
 }
 
+// Nodes of a particle of radius R that a step can list at most.  A listed node is
+// within one link of the particle's surface, or has been on the other side of it
+// before a move below GEOM_MARGIN - 1 along each axis: the largest list is the
+// uncovered nodes', from R to R + sqrt(3) (GEOM_MARGIN - 1) of the centre.  The unit
+// cubes around nodes do not overlap and reach sqrt(3)/2 further, so that many fit
+// into that shell at most; and into a cube of 2 R + 5 a side, which is less for small R.
+// (The cubes alone took 276 MB for a sphere of R = 100, now 22.)
+static long long surface_nodes(double R)
+{
+    const double half = 0.5 * std::sqrt(3.0), out = R + std::sqrt(3.0) * (GEOM_MARGIN - 1) + half, in = std::max(0.0, R - half);
+    const double shell = 4.0 / 3.0 * M_PI * (out * out * out - in * in * in);
+    const long long side = 2 * (long long)std::ceil(R) + 5;
+    return std::min((long long)std::ceil(shell) + 1, side * side * side);
+}
+
 lbm_status lbm_add_particles(lbm_ctx *ctx, int inst, int n, const lbm_particle *parts)
 {
     if (!ctx) return LBM_ERR_ARG;
@@ -1351,9 +1366,8 @@ lbm_status lbm_add_particles(lbm_ctx *ctx, int inst, int n, const lbm_particle *
     ctx->parts_d = nullptr;
     ctx->mem_part = ctx->cap_part = ctx->hist = ctx->crec = nullptr;
     CU(cudaMalloc((void **)&ctx->parts_d, sizeof(PartDev) * np));
-    // the nodes of a particle and within one link of it lie in a cube of this side
-    const long long ls = 2 * (long long)std::ceil(Rmax) + 5;
-    ctx->list_cap = (long long)np * ls * ls * ls;
+    ctx->list_cap = 0;
+    for (auto &q : all) ctx->list_cap += surface_nodes(q.R);
     CU(cudaMalloc((void **)&ctx->lists, sizeof(long long) * 4 * (size_t)ctx->list_cap));
     if (!ctx->list_n) CU(cudaMalloc((void **)&ctx->list_n, sizeof(unsigned long long) * 4));
     CU(cudaMalloc((void **)&ctx->mem_part, sizeof(double) * MEM_PART * np * ctx->mem_blocks));
