@@ -11,8 +11,8 @@
 // of particle-surface solid nodes; k_gradcurv (z-marching tiles: gradient,
 // wetting, normal, curvature; FP64 and small grids: k_grad_nodes and
 // k_curv_nodes); k_collide (or k_collide2).  Nodes next
-// to a solid go to the boundary passes k_phi_bound and k_collide_bound, which
-// run beside the bulk kernels on a second stream.
+// to a solid go to the boundary pass k_phi_bound and, in 16-bit storage, to
+// k_collide_bound, which run beside the bulk kernels on a second stream.
 //
 // The state between steps is the total offsets F* (pop[cur]) with one colour
 // record per node: phi (the order parameter its collision used) and b n (the
@@ -1300,8 +1300,9 @@ __global__ void __launch_bounds__(GcShape<DIR>::NT, DIR ? LBM_GC_MINB_DIR : LBM_
 // 19; 0.7 M as one domain 24 and 23 (201x91x37) or 21 and 23 (128x80x72), as 6
 // x 48^3 38 and 25, as 19 x 40x33x29 49 and 29; 0.88 M as 96^3 25 and 27, as 8
 // x 48^3 35 and 31; 256x128x64 35 and 49; 256x128x128 73 and 115: taken up to
-// GRAD_NODES_MAX nodes of a context.  (Marching with gathered sums; by direction
-// it takes some 5 to 20% longer.)
+// GRAD_NODES_MAX nodes of a context.  (Marching with gathered sums.  A uniform
+// field in FP32, by direction: 4 x 48^3 19 and 19, 6 x 48^3 22 and 25, 19 x
+// 40x33x29 32 and 28, 96^3 22 and 26, 256x128x64 41 and 52.)
 template <class R>
 constexpr int GN_THREADS = sizeof(R) == 8 ? 32 : 128;
 template <class R>

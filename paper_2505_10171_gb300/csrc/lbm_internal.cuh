@@ -275,7 +275,6 @@ template <>
 struct Store<double> {
     using real = double;
     static __device__ __forceinline__ double ld(const double *p) { return pop_load(p); }
-    static __device__ __forceinline__ double lds(const double *p) { return *p; }  // shared memory
     static __device__ __forceinline__ double cvt(double v) { return v; }
     static __device__ __forceinline__ void st(double *p, double v) { *p = v; }
 };
@@ -283,7 +282,6 @@ template <>
 struct Store<float> {
     using real = float;
     static __device__ __forceinline__ float ld(const float *p) { return pop_load(p); }
-    static __device__ __forceinline__ float lds(const float *p) { return *p; }  // shared memory
     static __device__ __forceinline__ float cvt(float v) { return v; }
     static __device__ __forceinline__ void st(float *p, float v) { *p = v; }
 };
@@ -291,7 +289,6 @@ template <>
 struct Store<__half> {
     using real = float;
     static __device__ __forceinline__ float ld(const __half *p) { return __half2float(pop_load(p)); }
-    static __device__ __forceinline__ float lds(const __half *p) { return __half2float(*p); }  // shared memory
     static __device__ __forceinline__ float cvt(__half v) { return __half2float(v); }
     static __device__ __forceinline__ void st(__half *p, float v) { *p = __float2half_rn(v); }
 };
@@ -299,7 +296,6 @@ template <>
 struct Store<__nv_bfloat16> {
     using real = float;
     static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(pop_load(p)); }
-    static __device__ __forceinline__ float lds(const __nv_bfloat16 *p) { return __bfloat162float(*p); }  // shared memory
     static __device__ __forceinline__ float cvt(__nv_bfloat16 v) { return __bfloat162float(v); }
     static __device__ __forceinline__ void st(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
@@ -339,12 +335,6 @@ __device__ __forceinline__ void ld_pair(const __nv_bfloat16 *p, float &a, float 
     a = __low2float(v);
     b = __high2float(v);
 }
-__device__ __forceinline__ void ld_pair(const float *p, float &a, float &b)
-{
-    const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
-    a = v.x;
-    b = v.y;
-}
 __device__ __forceinline__ void st_pair(__half *p, float a, float b)
 {
     *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(a, b);
@@ -353,7 +343,6 @@ __device__ __forceinline__ void st_pair(__nv_bfloat16 *p, float a, float b)
 {
     *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
-__device__ __forceinline__ void st_pair(float *p, float a, float b) { *reinterpret_cast<float2 *>(p) = make_float2(a, b); }
 
 // minimum-image displacement on a periodic axis of n nodes (|d| < 3n/2): the
 // same value as d - n floor(d/n + 1/2) without a double-precision division
@@ -572,14 +561,6 @@ struct Colour {
     {
     }
     __device__ __forceinline__ ColRec<R> at(int m) const { return c[m]; }
-    // G*_i = phi (1 + F*_i) + (c_i . a)/|c_i| of the record at m
-    __device__ __forceinline__ R G(int i, int m, R F) const
-    {
-        const ColRec<R> r = c[m];
-        R g = r.p * (R(1) + F);
-        if (i) g += col_rec(i, r);
-        return g;
-    }
 };
 
 template <class S>
@@ -670,7 +651,7 @@ __device__ __forceinline__ void gather_links(const InstDev &I, const PartDev *pa
         // in FP64, whose every instruction counts, one lever for all links instead
         // of 32 instructions a link (48x32x32 with a wall and a sphere: order-
         // parameter boundary pass 28 -> 12 us).  FP32 keeps the other form: with
-        // both the pass spills (66 against 61 us in a tube of radius 40)
+        // both the pass spills more (66 against 61 us in a tube of radius 40)
         R d[3];
         if (sizeof(R) == 8 && node_lever<R>(I, x, y, z, c, d)) {
             const R u0 = v[0] + (w[1] * d[2] - w[2] * d[1]), u1 = v[1] + (w[2] * d[0] - w[0] * d[2]),

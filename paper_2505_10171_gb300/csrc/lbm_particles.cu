@@ -756,8 +756,9 @@ __device__ __forceinline__ uint8_t set_boundary(const Lattice &L, const InstDev 
 // change only within one link of a node whose owner changed, i.e. within
 // the particle's last displacement and one link of its surface: the other
 // nodes of the cube cost a distance (all: the bits of every node and no lists,
-// when particles are added); the cube is cut to what the surface reaches (19 -> 11
-// nodes a side there).  512 spheres R = 3: 80 us with 18 flags read for every
+// when particles are added); the cube is cut to what the surface reaches (23 -> 11
+// nodes a side there; its nodes are found by integer division, no slower than
+// by a precomputed one).  512 spheres R = 3: 80 us with 18 flags read for every
 // node, 43 with the whole cube's distances, now 22.
 __global__ void __launch_bounds__(PART_THREADS) k_geom_surface(Lattice L, FastDiv fd, int all)
 {
