@@ -831,10 +831,9 @@ __global__ void __launch_bounds__(COLLIDE_NODES<S>, sizeof(S) == 8 ? 4 : (sizeof
 // (75.5 against 73 us on 256x128x128, 1720 against 1746 us in the sweep).  The
 // form with three stored planes and 48 reads a node executed 14.2 warp
 // instructions per node, this one 9.6: 96-domain sweep (1.5e8 nodes) 2796 -> 1738 us, 256x128x128
-// 75 -> 73 us.  By direction the 48 reads stay: 64 x 96x48x48 254 -> 217 us by
+// 75 -> 73 us.  By direction the 48 reads stay: 64 x 96x48x48 254 -> 212 us by
 // one barrier a plane instead of three and planes without flags passed by
-// (184 with gathered sums), 256x128x128 75 -> 78 us, the walls of a 64x64x1024
-// tube 89 -> 119 us (98).
+// (184 with gathered sums), 256x128x128 75 -> 74 us.
 constexpr int GC_TX = 32;
 
 // the sums of the gradient carried from plane to plane for one column
@@ -889,8 +888,9 @@ struct GcPart {
 // only where two particles meet.  With the owners' particle records read from
 // memory per direction the pass took 195 us instead of 75 on 256x128x128
 // nodes with eight spheres.
-// DIR: the substrate's sum in floating point, direction by direction; returns
-// a bit per solid neighbour, direction i at bit i.
+// DIR: the substrate's sum in floating point, direction by direction, for nodes
+// that the wetting turns only (the walls of a 64x64x1024 tube: the pass 119 us with
+// it for every node, 93 so); returns a bit per solid neighbour, direction i at bit i.
 template <bool DIR, class R, class Flag, class Part>
 __device__ __forceinline__ unsigned gc_solid(const InstDev &I, const Part &part, const Flag &flag, R phi, int x, int y,
                                              int z, R *g, R *s)
@@ -899,13 +899,19 @@ __device__ __forceinline__ unsigned gc_solid(const InstDev &I, const Part &part,
     R ws[3] = {0, 0, 0};
     unsigned solid = 0;
     unsigned long long met = 0;
+    const R wet_max = sizeof(R) == 8 ? (R)I.wet_max : (R)I.f_wet_max;
+    if constexpr (DIR) {
+#pragma unroll
+        for (int i = 1; i < Q; i++)
+            if ((flag(i) & OWNER_MASK) != OWN_FLUID) solid |= 1u << i;
+        if (!(fabs(phi) < wet_max)) return solid;
+    }
 #pragma unroll
     for (int i = 1; i < Q; i++) {
         const int own = flag(i) & OWNER_MASK;
         const int k = own == OWN_FLUID ? 0 : (csq(i) == 1 ? 2 : 1);
         const int kw = own == OWN_WALL ? k : 0;
         if constexpr (DIR) {
-            if (k) solid |= 1u << i;
             const R w = kw ? wgt<R>(i) : R(0);
             if (cx(i)) ws[0] = sub_rn(ws[0], cx(i) * w);
             if (cy(i)) ws[1] = sub_rn(ws[1], cy(i) * w);
@@ -919,8 +925,7 @@ __device__ __forceinline__ unsigned gc_solid(const InstDev &I, const Part &part,
     }
     if constexpr (!DIR)
         for (int a = 0; a < 3; a++) s[a] = R(1.0 / 12.0) * all[a];
-    const R wet_max = sizeof(R) == 8 ? (R)I.wet_max : (R)I.f_wet_max;
-    if (!(fabs(phi) < wet_max)) return solid;
+    if (!DIR && !(fabs(phi) < wet_max)) return solid;
     met &= ~(1ull << OWN_FLUID | 1ull << OWN_WALL | 1ull << OWN_PRESS);  // a pressure face carries no contact angle
     R d[3] = {DIR ? ws[0] : R(-wall[0]), DIR ? ws[1] : R(-wall[1]), DIR ? ws[2] : R(-wall[2])};
     R cth = (R)I.cos_tw, sth = (R)I.sin_tw;
@@ -1000,9 +1005,9 @@ __device__ __forceinline__ R dir_curvature(const NF &nf)
 // 1993 us on the 96-domain sweep); 8 warps of own nodes beat 4 (80 and 1864 us)
 // and 6 (82 and 1956 us).
 // By direction a node reads the three planes around it for each sum (18 + 30
-// values; two rows share few of them), one row a thread: 78 us on 256x128x128 and
-// 218 on 64 x 96x48x48, with two rows 83 and 225, with 12 rows of threads 80 and
-// 227.
+// values; two rows share few of them), one row a thread: 74 us on 256x128x128 and
+// 212 on 64 x 96x48x48 (78 and 218 when two rows took 83 and 225, and 12 rows of
+// threads 80 and 227).
 template <bool DIR>
 struct GcShape {
     static constexpr int RP = DIR ? 1 : 2, ROWS = 8;
