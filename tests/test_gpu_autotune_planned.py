@@ -19,6 +19,6 @@ def test_planned_chunk_is_kept_where_it_is_fastest():
     from paper_2505_10171_gb300 import lbm
     c = lbm.Context(dict(W.COMMON, nx=32, ny=8, nz=4096), "fp32")
     c.lbm_init_fields(np.full(32 * 8 * 4096, -1.0), None, None)
-    _, zchunks, _ = c.lbm_autotune(100)
+    _, zchunks, _ = c.lbm_autotune(1000)
     c.close()
     assert zchunks == [9]
